@@ -96,10 +96,13 @@ struct Cfg {
     static constexpr int kGroupFloats = 144;
     static constexpr int kRingFloatsPerWarp = 2 * kGroupFloats;
     // vector mode (wgrad): ONE ring for the CTA, filled by the two loader warps: per chunk 128 row factors 1/S_a and BN column
-    // factors 1/S_b, kVecDepth chunks deep, handed over kVecBlock chunks at a time
+    // factors 1/S_b, kVecDepth chunks deep, handed over kVecBlock chunks at a time.  A slot is laid out for the fragments of the
+    // promotion warps: rows [32-row quarter][row % 8][row / 8 % 4]; columns [column half][column % 4][column / 4], the four
+    // residues kVecQuad floats apart (16 bytes more than their data: their 16-byte reads hit distinct banks)
     static constexpr int kVecDepth = 16, kVecBlock = 4, kVecAhead = 8;
-    static constexpr int kVecSlotFloats = 128 + BN;
-    static constexpr int kSbInvBytes = (SCALE == 2) ? kVecDepth * kVecSlotFloats * 4 : kNumEpiWarps * kRingFloatsPerWarp * 4;
+    static constexpr int kVecQuad = BN / 8 + 4;
+    static constexpr int kVecSlotFloats = 128 + 8 * kVecQuad;
+    static constexpr int kSbInvBytes = (SCALE == 2) ? (kVecDepth * kVecSlotFloats * 4 + 1023) / 1024 * 1024 : kNumEpiWarps * kRingFloatsPerWarp * 4;
     // block mode (fwd / dgrad) writes its output through per-warp 2 KB staging tiles and TMA stores
     static constexpr bool kTmaOut = (SCALE == 1);
     static constexpr int kOutStageBytes = kTmaOut ? kNumEpiWarps * 2048 : 0;
@@ -170,6 +173,50 @@ __device__ __forceinline__ void store32(const GemmArgs &g, int64_t row, int col,
     }
 }
 
+// 4 x 4 transpose of words over the four lanes of a quad: afterwards w[k] is lane k's former w[lane % 4].
+__device__ __forceinline__ void quad_transpose(uint32_t (&w)[4], int lane)
+{
+#pragma unroll
+    for (int m = 1; m <= 2; m <<= 1) {
+        const bool up = (lane & m) != 0;
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            if (k & m) continue;
+            const uint32_t got = __shfl_xor_sync(0xFFFFFFFFu, up ? w[k] : w[k + m], m);
+            if (up) w[k] = got; else w[k + m] = got;
+        }
+    }
+}
+
+// Stores a fragment of 16 rows x 32 columns in the register order of tmem_ld_frag: rows `row` and `row + 8`, columns
+// col + 4 i + lane % 4.  The lanes of a quad swap so that each stores four consecutive columns of every sixteen.
+template <bool OUT_F32>
+__device__ __forceinline__ void store_frag(const GemmArgs &g, int64_t row, int col, const float *v, int lane)
+{
+#pragma unroll
+    for (int b = 0; b < 2; ++b) {
+        const int64_t r = row + 8 * b;
+#pragma unroll
+        for (int k = 0; k < 2; ++k) {
+            const int c = col + 16 * k + 4 * (lane & 3);
+            uint32_t w[4];
+#pragma unroll
+            for (int i = 0; i < 4; ++i) w[i] = __float_as_uint(v[2 * (4 * k + i) + b]);
+            quad_transpose(w, lane);
+            if (r < g.Mo && c < g.No) {
+                float4 o = make_float4(__uint_as_float(w[0]), __uint_as_float(w[1]), __uint_as_float(w[2]), __uint_as_float(w[3]));
+                if (OUT_F32) {
+                    float4 *dst = reinterpret_cast<float4 *>(static_cast<float *>(g.out) + r * g.ldo + c);
+                    if (g.accumulate) { const float4 p = *dst; o.x += p.x; o.y += p.y; o.z += p.z; o.w += p.w; }
+                    *dst = o;
+                } else {
+                    *reinterpret_cast<uint2 *>(static_cast<__nv_bfloat16 *>(g.out) + r * g.ldo + c) = make_uint2(pack_bf16x2(o.x, o.y), pack_bf16x2(o.z, o.w));
+                }
+            }
+        }
+    }
+}
+
 template <MmaKind KIND, int BN, int SCALE, bool OUT_F32>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmO,
@@ -178,10 +225,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     using C = Cfg<KIND, BN, SCALE>;
     constexpr int S = C::kStages;
     constexpr int HALF = BN / 2;     // columns handled by one epilogue warp
-    // columns per tensor-memory load: 16 in vector mode (wgrad: the promotion loop holds the column reciprocals next to the
-    // staging registers and runs 1.5-4 % faster with the smaller groups), 32 otherwise (fwd / dgrad: 2.5 % faster than 16)
+    // registers per tensor-memory load: 16 in vector mode (wgrad: 16 rows x 32 columns as a fragment), 32 otherwise (32 rows x
+    // 32 columns; fwd / dgrad: 2.5 % faster than 16)
     constexpr int GC = (SCALE == SCALE_VEC_B) ? 16 : 32;
     constexpr int G = HALF / GC;     // groups handled by one epilogue warp per chunk
+    constexpr int D = (SCALE == SCALE_VEC_B) ? (G < 6 ? G : 4) : 2;   // groups of staging registers next to the accumulators
 
     extern __shared__ uint8_t smem_raw[];
     // operand tiles need 1024-byte alignment for the 128-byte swizzle
@@ -378,12 +426,25 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             request();                       // position cc + kVecAhead
             cp_async_wait<C::kVecAhead>();   // this lane's copies of position cc have landed
             const uint32_t d = cc % C::kVecDepth;
-            float4 *mine = reinterpret_cast<float4 *>(scale_ring + d * C::kVecSlotFloats + (rows_side ? 0 : 128) + 4 * lane);
-            const float4 v = mine[0];
-            mine[0] = make_float4(rcp_approx(v.x), rcp_approx(v.y), rcp_approx(v.z), rcp_approx(v.w));
-            if (!rows_side && 128 + 4 * lane < BN) {
-                const float4 w = mine[32];
-                mine[32] = make_float4(rcp_approx(w.x), rcp_approx(w.y), rcp_approx(w.z), rcp_approx(w.w));
+            // raw factors of four consecutive lines per lane -> reciprocals in the fragment order of the slot
+            float *slot = scale_ring + d * C::kVecSlotFloats;
+            const float4 *raw = reinterpret_cast<const float4 *>(slot + (rows_side ? 0 : 128) + 4 * lane);
+            const float4 v = raw[0];
+            float4 w = v;
+            if (!rows_side && 128 + 4 * lane < BN) w = raw[32];
+            __syncwarp();                    // every lane has read its raw values
+            if (rows_side) {
+                // rows 4*lane .. +3: quarter lane / 8, row / 8 = lane / 2 % 4, row % 8 = 4 * (lane % 2) + t
+                float *dst = slot + (lane >> 3) * 32 + (lane & 1) * 16 + ((lane >> 1) & 3);
+                dst[0] = rcp_approx(v.x); dst[4] = rcp_approx(v.y); dst[8] = rcp_approx(v.z); dst[12] = rcp_approx(v.w);
+            } else {
+                auto put = [&](int col, const float4 &x) {   // col: a multiple of four
+                    const int hh = col / HALF;
+                    float *dst = slot + 128 + 4 * hh * C::kVecQuad + (col - hh * HALF) / 4;
+                    dst[0] = rcp_approx(x.x); dst[C::kVecQuad] = rcp_approx(x.y); dst[2 * C::kVecQuad] = rcp_approx(x.z); dst[3 * C::kVecQuad] = rcp_approx(x.w);
+                };
+                put(4 * lane, v);
+                if (128 + 4 * lane < BN) put(128 + 4 * lane, w);
             }
             __syncwarp();
             // a block is published when its last slot (or the last chunk of all) is ready
@@ -472,18 +533,27 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             for (int c = 0; c < nacc; ++c, ++cc) {
                 const uint32_t a = cc & 1u;
                 float f[G];
-                // vector mode: this chunk's slot of the CTA's factor ring (filled by warps 2 and 3), taken over a block at a time
+                // Vector mode: this chunk's slot of the CTA's factor ring (filled by warps 2 and 3), taken over a block at a time.
+                // A thread's fragment is 4 rows (lane / 4 + 8 b) x HALF / 4 columns (4 j + lane % 4), so it needs 4 + HALF / 4 factors:
+                // 9 shared-memory reads of 16 bytes per chunk and warp.  With a row per lane (the 32x32b loads of fwd / dgrad) it was
+                // one broadcast read per four columns, 33 in all: about 600 cycles of the shared-memory pipe per 128 x 256 chunk, next to
+                // the 770 that the operands' way in and out takes.
                 const uint32_t vd = cc % C::kVecDepth;
                 const float *vslot = scale_ring + vd * C::kVecSlotFloats;
-                const float *slot = vslot + 128 + h * HALF;   // this warp's column reciprocals
                 if (SCALE == SCALE_VEC_B && (cc % C::kVecBlock) == 0) {
                     const bool got = mbar_wait(vfull_bar(vd / C::kVecBlock), (cc / C::kVecDepth) & 1u, abort_flag, g.wait_limit_ns);
                     if (!__all_sync(0xFFFFFFFFu, got)) { ok = false; break; }
                 }
+                float4 rf = make_float4(0.0f, 0.0f, 0.0f, 0.0f), cf[2][2];   // row factors; column factors of two 32-column blocks
+                const float4 *cfs = reinterpret_cast<const float4 *>(vslot + 128 + (4 * h + (lane & 3)) * C::kVecQuad);
+                if (SCALE == SCALE_VEC_B) {
+                    rf = *reinterpret_cast<const float4 *>(vslot + q * 32 + (lane >> 2) * 4);
+                    cf[0][0] = cfs[0]; cf[0][1] = cfs[1];
+                    cf[1][0] = cfs[2]; cf[1][1] = cfs[3];
+                }
 #pragma unroll
                 for (int gi = 0; gi < G; ++gi) {
                     if (SCALE == SCALE_BLOCK_B) f[gi] = (kBlocksPerWarp == 1 || ((col0 + 32 * gi) >> 7) == blk0) ? fq[0][0] : fq[kBlocksPerWarp - 1][0];
-                    else f[gi] = vslot[q * 32 + lane];
                 }
                 if (SCALE == SCALE_BLOCK_B) {
 #pragma unroll
@@ -498,10 +568,14 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 }
                 tc_fence_after_sync();
                 const uint32_t taddr = tmem_base + ((uint32_t)(q * 32) << 16) + a * BN + h * HALF;
-                // two 32-column groups in registers next to the accumulators
-                uint32_t v[2][GC];
-                tmem_ld_cols(taddr, v[0]);
-                if (G > 1) tmem_ld_cols(taddr + GC, v[1]);
+                uint32_t v[D][GC];
+                auto load_group = [&](int gi, uint32_t (&dst)[GC]) {
+                    // vector mode: rows 16 * (gi % 2) .., columns 32 * (gi / 2) ..
+                    if constexpr (SCALE == SCALE_VEC_B) tmem_ld_frag(taddr + ((uint32_t)(16 * (gi & 1)) << 16) + 32 * (gi >> 1), dst);
+                    else tmem_ld_cols(taddr + GC * gi, dst);
+                };
+#pragma unroll
+                for (int gi = 0; gi < D; ++gi) load_group(gi, v[gi]);
                 if (SCALE != SCALE_NONE) {
                     // In the shadow of the first load.  Block mode: with the last chunk of a group of four the register
                     // queue is empty; the next group's slot (requested four chunks ago) is turned into the next four
@@ -534,33 +608,40 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         for (int i = 0; i < GC / 2; ++i)
                             acc[(GC / 2) * gi + i] = __ffma2_rn(make_float2(__uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1])), ff, acc[(GC / 2) * gi + i]);
                     } else {
-                        const float2 ff = make_float2(f[0], f[0]);
-                        const float4 *sbv = reinterpret_cast<const float4 *>(slot + GC * gi);
+                        // group gi: rows 16 * (gi % 2) + {lane / 4, + 8}, columns 32 * (gi / 2) + 4 i + lane % 4
+                        const float2 r2 = (gi & 1) ? make_float2(rf.z, rf.w) : make_float2(rf.x, rf.y);
 #pragma unroll
-                        for (int i = 0; i < GC / 4; ++i) {
-                            const float4 s4 = sbv[i];   // reciprocal column scales, broadcast read
-                            const float2 r0 = make_float2(s4.x, s4.y);
-                            const float2 r1 = make_float2(s4.z, s4.w);
-                            const float2 p0 = __fmul2_rn(make_float2(__uint_as_float(cur[4 * i]), __uint_as_float(cur[4 * i + 1])), r0);
-                            const float2 p1 = __fmul2_rn(make_float2(__uint_as_float(cur[4 * i + 2]), __uint_as_float(cur[4 * i + 3])), r1);
-                            acc[(GC / 2) * gi + 2 * i] = __ffma2_rn(p0, ff, acc[(GC / 2) * gi + 2 * i]);
-                            acc[(GC / 2) * gi + 2 * i + 1] = __ffma2_rn(p1, ff, acc[(GC / 2) * gi + 2 * i + 1]);
+                        for (int i = 0; i < 8; ++i) {
+                            const float4 c4 = cf[(gi >> 1) & 1][i >> 2];
+                            const float c = (i & 3) == 0 ? c4.x : (i & 3) == 1 ? c4.y : (i & 3) == 2 ? c4.z : c4.w;
+                            const float2 p = __fmul2_rn(make_float2(__uint_as_float(cur[2 * i]), __uint_as_float(cur[2 * i + 1])), r2);
+                            acc[8 * gi + i].x = fmaf(p.x, c, acc[8 * gi + i].x);
+                            acc[8 * gi + i].y = fmaf(p.y, c, acc[8 * gi + i].y);
                         }
                     }
                 };
-                // Two loads are in flight from the start; each group's FMAs free its registers for the load two groups
-                // on.  A load is waited for one group after it was issued, before the next one is issued (the wait covers
-                // every outstanding load of the thread), so that its latency lies under that group's FMAs and no group is
-                // consumed before its load has been waited for.  The buffer goes back to the MMA warp when the last load
-                // has landed; the last group follows the release.
                 tmem_ld_wait();
-                if (G <= 2) release_buffer();
+                if (G <= D) release_buffer();
 #pragma unroll
                 for (int gi = 0; gi < G; ++gi) {
-                    consume_group(gi, v[gi & 1]);
-                    if (gi >= 1 && gi + 1 < G) tmem_ld_wait();                   // group gi+1 has landed
-                    if (gi + 2 < G) tmem_ld_cols(taddr + GC * (gi + 2), v[gi & 1]);
-                    if (G > 2 && gi + 2 == G) release_buffer();                  // ... and it was the chunk's last load
+                    consume_group(gi, v[gi % D]);
+                    if constexpr (SCALE == SCALE_VEC_B) {
+                        // D loads from the start, the others as registers become free, and one wait for all of them: the buffer goes
+                        // back after G - D groups' worth of multiplications (waiting for the last load later, with the buffer handed back
+                        // later too: 2-4 % slower)
+                        if ((gi & 1) && (gi >> 1) + 2 < G / 2) { cf[(gi >> 1) & 1][0] = cfs[gi + 3]; cf[(gi >> 1) & 1][1] = cfs[gi + 4]; }
+                        if (gi + D < G) load_group(gi + D, v[gi % D]);
+                        if (gi + D == G - 1) { tmem_ld_wait(); release_buffer(); }
+                    } else {
+                        // Two loads are in flight from the start; each group's FMAs free its registers for the load two groups
+                        // on.  A load is waited for one group after it was issued, before the next one is issued (the wait covers
+                        // every outstanding load of the thread), so that its latency lies under that group's FMAs and no group is
+                        // consumed before its load has been waited for.  The buffer goes back to the MMA warp when the last load
+                        // has landed; the last group follows the release.
+                        if (gi >= 1 && gi + 1 < G) tmem_ld_wait();                   // group gi+1 has landed
+                        if (gi + 2 < G) load_group(gi + 2, v[gi & 1]);
+                        if (G > 2 && gi + 2 == G) release_buffer();                  // ... and it was the chunk's last load
+                    }
                 }
                 if (SCALE == SCALE_VEC_B && (cc % C::kVecBlock) == C::kVecBlock - 1) {
                     __syncwarp();                        // every lane has read the block's slots
@@ -614,18 +695,32 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                             write_out = (old == (uint32_t)wi.nsl - 1u);
                             if (write_out) {
                                 __threadfence();
+                                // half a warp's share at a time, all its loads of a slice in flight together: 2 L2 round trips per
+                                // slice (one per 16 bytes before: 25 us at the end of every sliced launch)
 #pragma unroll
-                                for (int j4 = 0; j4 < HALF / 4; ++j4) {
-                                    float4 v = __ldcg(reinterpret_cast<const float4 *>(first + j4 * 128));
-                                    for (int sl = 1; sl < wi.nsl; ++sl) {
-                                        const float4 u = __ldcg(reinterpret_cast<const float4 *>(first + (size_t)sl * kNumEpiWarps * kWarpFloats + j4 * 128));
-                                        v.x += u.x; v.y += u.y; v.z += u.z; v.w += u.w;
+                                for (int b0 = 0; b0 < HALF / 4; b0 += HALF / 8) {
+                                    for (int sl = 0; sl < wi.nsl; ++sl) {
+                                        const float *src = first + (size_t)sl * kNumEpiWarps * kWarpFloats + b0 * 128;
+                                        float4 u[HALF / 8];
+#pragma unroll
+                                        for (int j = 0; j < HALF / 8; ++j) u[j] = __ldcg(reinterpret_cast<const float4 *>(src + j * 128));
+#pragma unroll
+                                        for (int j = 0; j < HALF / 8; ++j) {
+                                            float *d = av + 4 * (b0 + j);
+                                            if (sl == 0) { d[0] = u[j].x; d[1] = u[j].y; d[2] = u[j].z; d[3] = u[j].w; }
+                                            else { d[0] += u[j].x; d[1] += u[j].y; d[2] += u[j].z; d[3] += u[j].w; }
+                                        }
                                     }
-                                    av[4 * j4] = v.x; av[4 * j4 + 1] = v.y; av[4 * j4 + 2] = v.z; av[4 * j4 + 3] = v.w;
                                 }
                             }
                         }
-                        if (write_out && row_ok) {
+                        if constexpr (SCALE == SCALE_VEC_B) {
+                            if (write_out) {
+#pragma unroll
+                                for (int gi = 0; gi < G; ++gi)
+                                    store_frag<OUT_F32>(g, row0 + 16 * (gi & 1) + (lane >> 2), col0 + 32 * (gi >> 1), reinterpret_cast<const float *>(acc) + 16 * gi, lane);
+                            }
+                        } else if (write_out && row_ok) {
 #pragma unroll
                             for (int gi = 0; gi < HALF / 32; ++gi) store32<OUT_F32>(g, row, col0 + 32 * gi, reinterpret_cast<const float *>(acc) + 32 * gi);
                         }

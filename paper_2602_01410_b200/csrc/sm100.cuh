@@ -281,6 +281,19 @@ __device__ __forceinline__ void tmem_ld_cols(uint32_t taddr, uint32_t (&r)[16])
         : "r"(taddr)
         : "memory");
 }
+// Load 16 lanes x 32 columns (lane base a multiple of 16 within the warp's 32) as a fragment: thread T gets r[2i] = lane T/4,
+// column 4i + T%4 and r[2i+1] = lane T/4 + 8, the same column.  (Half the rate of the 32x32b shape; the 16x256b shape, whose
+// fragments hold column pairs, has a quarter of it: 134 / 256 / 512 cycles measured for 128 x 256 words on one SM.)
+__device__ __forceinline__ void tmem_ld_frag(uint32_t taddr, uint32_t (&r)[16])
+{
+    asm volatile(
+        "tcgen05.ld.sync.aligned.16x128b.x8.b32 "
+        "{%0, %1, %2, %3, %4, %5, %6, %7, %8, %9, %10, %11, %12, %13, %14, %15}, [%16];"
+        : "=r"(r[0]), "=r"(r[1]), "=r"(r[2]), "=r"(r[3]), "=r"(r[4]), "=r"(r[5]), "=r"(r[6]), "=r"(r[7]), "=r"(r[8]),
+          "=r"(r[9]), "=r"(r[10]), "=r"(r[11]), "=r"(r[12]), "=r"(r[13]), "=r"(r[14]), "=r"(r[15])
+        : "r"(taddr)
+        : "memory");
+}
 // Wait for this thread's outstanding tcgen05.ld.  ptxas tracks the destination registers of the
 // asynchronous load up to this instruction, so uses of them stay behind it.
 __device__ __forceinline__ void tmem_ld_wait() { asm volatile("tcgen05.wait::ld.sync.aligned;" ::: "memory"); }
