@@ -90,7 +90,7 @@ struct Cfg {
     static constexpr int kABytes = BM * 128;
     static constexpr int kBBytes = BN * 128;
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = (BN >= 256) ? 4 : 5;
+    static constexpr int kStages = (BN >= 256 || SCALE == 1) ? 4 : 5;
     // block mode (fwd / dgrad) fetches four chunks of scale factors per instruction into two alternating group slots:
     // [4 chunks][32 rows] S_a, then [2 blocks][4 chunks] S_b
     static constexpr int kGroupFloats = 144;
@@ -103,9 +103,11 @@ struct Cfg {
     static constexpr int kVecQuad = BN / 8 + 4;
     static constexpr int kVecSlotFloats = 128 + 8 * kVecQuad;
     static constexpr int kSbInvBytes = (SCALE == 2) ? (kVecDepth * kVecSlotFloats * 4 + 1023) / 1024 * 1024 : kNumEpiWarps * kRingFloatsPerWarp * 4;
-    // block mode (fwd / dgrad) writes its output through per-warp 2 KB staging tiles and TMA stores
+    // block mode (fwd / dgrad) writes its output through kOutSlots 2 KB staging tiles per warp and TMA stores; where shared
+    // memory has room for a warp's whole bf16 tile no store is waited for before the next tile's sums
     static constexpr bool kTmaOut = (SCALE == 1);
-    static constexpr int kOutStageBytes = kTmaOut ? kNumEpiWarps * 2048 : 0;
+    static constexpr int kOutSlots = (BN == 192) ? 3 : 1;
+    static constexpr int kOutStageBytes = kTmaOut ? kNumEpiWarps * kOutSlots * 2048 : 0;
     static constexpr int kSmemBytes = kStages * kStageBytes + kSbInvBytes + kOutStageBytes + 256 + 1024;  // + barriers + alignment slack
     static_assert(kSmemBytes <= 232448, "shared memory budget");
     static_assert(kStageBytes % 1024 == 0 && kSbInvBytes % 1024 == 0, "staging tiles must stay 1024-byte aligned");
@@ -229,7 +231,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // 32 columns; fwd / dgrad: 2.5 % faster than 16)
     constexpr int GC = (SCALE == SCALE_VEC_B) ? 16 : 32;
     constexpr int G = HALF / GC;     // groups handled by one epilogue warp per chunk
-    constexpr int D = (SCALE == SCALE_VEC_B) ? (G < 6 ? G : 4) : 2;   // groups of staging registers next to the accumulators
+    constexpr int D = (SCALE == SCALE_VEC_B) ? (G < 6 ? G : 4) : (BN == 192) ? G : 2;   // groups of staging registers next to the accumulators
+    // (192-wide tiles: 96 accumulators leave room for the whole chunk, so the buffer goes back before any multiplication)
 
     extern __shared__ uint8_t smem_raw[];
     // operand tiles need 1024-byte alignment for the 128-byte swizzle
@@ -310,7 +313,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         }
     } else if (warp == 1) {
         // ================= MMA issuer =================
-        if (lane == 0) {
+        // Block mode: an elected lane, under which the operands of the tcgen05 instructions stay in uniform registers (issue of a chunk
+        // 204 -> 55 cycles, 2-4 % of the FP4 kernels); in vector mode it costs the promotion warps registers and gains nothing.
+        if (SCALE == SCALE_BLOCK_B ? elect_one() : lane == 0) {
             uint32_t it = 0, cc = 0;
             bool ok = true;
             const uint32_t sfa = tmem_base + C::kSfCol0, sfb = tmem_base + C::kSfCol0 + 16;
@@ -464,7 +469,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         // ([2 blocks][4 chunks] at float 128 of the group).  Vector mode reads the CTA's ring of ready factors.
         float *ring = scale_ring + e * C::kRingFloatsPerWarp;
         const uint32_t ring_u32 = smem_u32(ring);
-        const uint32_t stage_u32 = out_stage0 + e * 2048;   // this warp's staging tile: 32 rows x 64 bytes
+        const uint32_t stage_u32 = out_stage0 + e * (C::kOutSlots * 2048);   // this warp's staging tiles: 32 rows x 64 bytes each
         uint32_t cc = 0;
         bool ok = true;
         for (int w = blockIdx.x; w < g.num_items && ok; w += gridDim.x) {
@@ -582,7 +587,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     // factors and the slot of the group just finished is refilled two groups ahead.  One warp barrier
                     // per four chunks: between the copies of all lanes and the reads of all lanes.
                     if (SCALE == SCALE_BLOCK_B) {
-                        if ((c & 3) == 3) {
+                        if ((c & 3) == 3 && c + 1 < nacc) {
                             cp_async_wait<0>();
                             __syncwarp();
                             load_factors((c >> 2) + 1);
@@ -625,7 +630,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
                 for (int gi = 0; gi < G; ++gi) {
                     consume_group(gi, v[gi % D]);
-                    if constexpr (SCALE == SCALE_VEC_B) {
+                    if constexpr (D == G) {
+                        // the whole chunk was loaded at once
+                    } else if constexpr (SCALE == SCALE_VEC_B) {
                         // D loads from the start, the others as registers become free, and one wait for all of them: the buffer goes
                         // back after G - D groups' worth of multiplications (waiting for the last load later, with the buffer handed back
                         // later too: 2-4 % slower)
@@ -658,7 +665,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         constexpr int kPerBox = OUT_F32 ? 16 : 32;   // output columns per 64-byte box row
 #pragma unroll
                         for (int b = 0; b < HALF / kPerBox; ++b) {
-                            if (lane == 0) bulk_wait_read0();     // the previous box has left the staging tile
+                            if (lane == 0) bulk_wait_read<C::kOutSlots - 1>();     // the box that was in this staging tile has left it
                             __syncwarp();
                             const float *src = reinterpret_cast<const float *>(acc) + b * kPerBox;
 #pragma unroll
@@ -667,12 +674,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                                 if (OUT_F32) o = make_uint4(__float_as_uint(src[4 * j]), __float_as_uint(src[4 * j + 1]), __float_as_uint(src[4 * j + 2]), __float_as_uint(src[4 * j + 3]));
                                 else o = make_uint4(pack_bf16x2(src[8 * j], src[8 * j + 1]), pack_bf16x2(src[8 * j + 2], src[8 * j + 3]),
                                                     pack_bf16x2(src[8 * j + 4], src[8 * j + 5]), pack_bf16x2(src[8 * j + 6], src[8 * j + 7]));
-                                st_shared_v4(stage_u32 + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4), o);
+                                st_shared_v4(stage_u32 + (b % C::kOutSlots) * 2048 + lane * 64 + ((j ^ ((lane >> 1) & 3)) << 4), o);
                             }
                             fence_proxy_async();
                             __syncwarp();
                             const int col = col0 + b * kPerBox;
-                            if (lane == 0 && col < g.No && row0 < g.Mo) { tma_store_2d(&tmO, stage_u32, col, row0); bulk_commit(); }
+                            if (lane == 0) {
+                                if (col < g.No && row0 < g.Mo) tma_store_2d(&tmO, stage_u32 + (b % C::kOutSlots) * 2048, col, row0);
+                                bulk_commit();   // one group per box, empty outside the matrix: the wait above counts groups
+                            }
                         }
                     } else {
                         bool write_out = true;
@@ -972,13 +982,13 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         return f32 ? launch_gemm<MmaKind::F16, 256, SCALE_NONE, true>(tmA, tmB, tmO, g, idesc, st)
                    : launch_gemm<MmaKind::F16, 256, SCALE_NONE, false>(tmA, tmB, tmO, g, idesc, st);
     }
-    if (fmt_a == SNIP_FMT_FP4_E2M1 && fmt_b == SNIP_FMT_FP4_E2M1 && (Kc % 128) != 0) {
-        // Packed FP4 on both sides, contraction length ending in a 64-wide tile: kind::mxf4 on the packed bytes
-        // (fetched as plain u8, exact extents).  Whole chunks take the path below instead: the per-chunk
-        // promotion, not the tensor pipe, sets the pace of these kernels, and there a 128x256 tile of
-        // kind::f8f6f4 (FP4 codes expanded by the TMA unit, still fetched packed from L2) does a third more
-        // columns per hand-off than the 128x192 tile that tensor memory allows next to kind::mxf4's scale
-        // factors: measured 10-20 % faster on the 7B shapes.
+    if (fmt_a == SNIP_FMT_FP4_E2M1 && fmt_b == SNIP_FMT_FP4_E2M1 && (scale_mode == SCALE_BLOCK_B || (Kc % 128) != 0)) {
+        // Packed FP4 on both sides, forward / input gradient, or a contraction length ending in a 64-wide tile: kind::mxf4 on the
+        // packed bytes (fetched as plain u8, exact extents).  Its 128x192 tile (what tensor memory allows next to the scale
+        // factors) does a quarter less per hand-off than the 128x256 tile of kind::f8f6f4, but a chunk's sums fit in the promotion
+        // warps' registers at once, and with half the operand bytes and a quarter of the tensor time it stays below the power
+        // cap: 16384x12288x4096 755 -> 673 us, 8192x3200x8640 215 -> 193 us, 8192x2048x256 16.4 -> 14.5 us.  The weight gradient over
+        // whole chunks takes the path below: with two operations per element the wider tile is as fast or faster.
         constexpr int BN = 192;
         rc = make_operand_map(&tmA, a_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, Mo, Kc / 2, Kc / 2, 128, BM);
         if (rc) return rc;
@@ -988,7 +998,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         g.stage_tx_bytes = (BM + BN) * 128 + tx_skew;
         return launch_gemm_scale<MmaKind::MXF4, BN>(scale_mode, f32, tmA, tmB, tmO, g, idesc, st);
     }
-    // FP8 x FP8, the mixed pairs and FP4 x FP4 over whole chunks: kind::f8f6f4; FP4 operands are expanded by
+    // FP8 x FP8, the mixed pairs and the FP4 x FP4 weight gradient over whole chunks: kind::f8f6f4; FP4 operands are expanded by
     // the TMA unit to one 16-byte-aligned group per 16 elements, which is the layout this MMA kind reads
     constexpr int BN = 256;
     const bool a4 = fmt_a == SNIP_FMT_FP4_E2M1, b4 = fmt_b == SNIP_FMT_FP4_E2M1;
