@@ -488,19 +488,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             // Block mode: the scale factors of four consecutive chunks with two instructions per warp.  Lane L
             // fetches 16 bytes = S_a of rows 4*(L%8) .. +3 of chunk 4*gn + L/8 (the warp's 32 rows lie inside or
             // outside the matrix together: row counts are multiples of 64); lanes 0..3 (0..7 with two blocks)
-            // fetch S_b of one chunk each.  Group gn lands in slot gn % 2.
+            // fetch S_b of one chunk each.  Group gn lands in slot gn % 2; groups are requested in order, so the source pointers
+            // only step (64-bit index products and bounds per request: 3-6 % of the FP4 kernels).
             constexpr int kBlocksPerWarp = ((HALF % 128) == 0) ? 1 : 2;
+            const float *pa = g.sa + (int64_t)(lane >> 3) * g.sa_chunk_stride + row0 + (lane & 7) * 4;
+            const float *pb = g.sb + (int64_t)min(blk0 + (lane >> 2), blk_last) * g.sb_blk_stride + (int64_t)(lane & 3) * g.sb_chunk_stride;
+            const int64_t pa_step = 4 * g.sa_chunk_stride, pb_step = 4 * g.sb_chunk_stride;
+            int left_a = (row0 < g.Mo) ? nacc - (lane >> 3) : 0, left_b = (lane < 4 * kBlocksPerWarp) ? nacc - (lane & 3) : 0;
             auto prefetch_group = [&](int gn) {
-                if (4 * gn < nacc) {
-                    const uint32_t slot = ring_u32 + (gn & 1) * C::kGroupFloats * 4;
-                    const int ci = lane >> 3, r4 = (lane & 7) * 4, chunk = 4 * gn + ci;
-                    if (row0 < g.Mo && chunk < nacc)
-                        cp_async_16(slot + (ci * 32 + r4) * 4, g.sa + (int64_t)chunk * g.sa_chunk_stride + row0 + r4);
-                    if (lane < 4 * kBlocksPerWarp) {
-                        const int blk = min(blk0 + (lane >> 2), blk_last), cb = 4 * gn + (lane & 3);
-                        if (cb < nacc) cp_async_4(slot + (128 + lane) * 4, g.sb + (int64_t)blk * g.sb_blk_stride + (int64_t)cb * g.sb_chunk_stride);
-                    }
-                }
+                const uint32_t slot = ring_u32 + (gn & 1) * C::kGroupFloats * 4;
+                if (left_a > 0) cp_async_16(slot + lane * 16, pa);
+                if (left_b > 0) cp_async_4(slot + (128 + lane) * 4, pb);
+                pa += pa_step; pb += pb_step; left_a -= 4; left_b -= 4;
                 cp_async_commit();
             };
 
