@@ -39,7 +39,64 @@ struct DualOut {
     uint64_t seed = 0;
 };
 
+// A linear-layer call enqueues a chain of kernels by programmatic dependent launch: quantizers, then GEMMs.
+//   CHAIN_NONE  : a call of its own (starts after the kernel ahead of it on the stream; a quantizer launches its own statistics
+//                 reduction)
+//   CHAIN_FIRST : starts after the kernel ahead of it has completed, then lets the next one start beside it
+//   CHAIN_BESIDE: independent of the members ahead of it: starts at once and waits for the one ahead only before it ends, so that
+//                 "the last member has completed" keeps meaning "all of them have"
+//   CHAIN_AFTER : its prologue runs beside the members ahead of it, its work after they have completed
+enum ChainRole { CHAIN_NONE = 0, CHAIN_FIRST = 1, CHAIN_BESIDE = 2, CHAIN_AFTER = 3 };
+
+// Statistics partials left by the quantizers of a chain; the GEMM behind them reduces them in warps it has to spare (otherwise a
+// launch per quantizer, in the way of everything behind it).
+struct StatJob {
+    const void *partials;   // CtaPartial[n] (quant_device.cuh)
+    snip_stats_t *out;
+    int32_t n;
+};
+struct StatJobs {
+    StatJob job[6];
+    int32_t count = 0;
+};
+
+// Workspace of one GEMM: status word, and (optional) arrival counters and partial sums of sliced tiles.  cleared: the status word and
+// the counters are already zero, or will be by the time the kernel starts.
+struct GemmWs {
+    uint32_t *status = nullptr;
+    uint32_t *counters = nullptr;
+    float *partials = nullptr;
+    bool cleared = false;
+};
+
+// What a chain passes along: the first quantizer clears `zero_words` words at `zero` (GEMM status word and slice counters).
+struct ChainLink {
+    int role = CHAIN_NONE;
+    uint32_t *zero = nullptr;
+    int32_t zero_words = 0;
+    StatJobs *jobs = nullptr;   // quantizers append, the next GEMM takes them
+};
+
 // Fails with SNIP_ERR_UNSUPPORTED unless the current device is compute capability 10.x.
 int require_sm100();
+
+// Launch with (pdl) or without the attribute that lets the kernel start beside the one ahead of it (griddepcontrol in the kernel
+// decides what waits).
+template <typename... KArgs, typename... Args>
+int launch_chained(void (*kern)(KArgs...), int grid, int threads, size_t smem_bytes, cudaStream_t st, bool pdl, const Args &...args)
+{
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)grid);
+    cfg.blockDim = dim3((unsigned)threads);
+    cfg.dynamicSmemBytes = smem_bytes;
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = pdl ? 1 : 0;
+    SNIP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
+    return SNIP_OK;
+}
 
 }  // namespace snip

@@ -20,6 +20,7 @@
 #include <atomic>
 
 #include "common.cuh"
+#include "quant_device.cuh"
 #include "sm100.cuh"
 
 namespace snip {
@@ -58,6 +59,8 @@ struct GemmArgs {
     int32_t split_first, nsplit, num_items;
     float *partials;           // [tail tile r][slice j][epilogue warp][column quad][row lane][4]: FP32 sums of a slice
     uint32_t *counters;        // [tail tile r][epilogue warp]: slices that have delivered their sums (zero at launch)
+    int32_t chain;             // ChainRole
+    StatJobs stats;            // reductions left by the quantizers ahead
 };
 
 struct WorkItem {
@@ -277,6 +280,9 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
+    // everything up to here touches nothing that a kernel ahead on the stream writes
+    if (g.chain != CHAIN_BESIDE) pdl_wait();
+    pdl_launch_dependents();
 
     if (KIND == MmaKind::MXF4) {
         // constant scale factors 2^0 (UE8M0 byte 127) for every row of A and B
@@ -370,7 +376,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 }
             }
         }
-      } else if (SCALE == SCALE_VEC_B) {
+      } else if (SCALE != SCALE_VEC_B) {
+        // ================= warp 2: statistics of the quantizers ahead =================
+        if (warp == 2)
+            for (int i = blockIdx.x; i < g.stats.count; i += gridDim.x) reduce_stats_warp(g.stats.job[i], lane);
+      } else {
         // ================= warps 2, 3: scale loaders of the weight-gradient product =================
         // Both factors of a chunk are vectors here (1/S_a per output row, 1/S_b per output column).  Warp 2 brings the 128
         // row scales, warp 3 the BN column scales of every chunk into one ring for the CTA (cp.async, kVecAhead chunks
@@ -456,6 +466,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             if (lane == 0 && ((cc % C::kVecBlock) == C::kVecBlock - 1 || cc + 1 == total)) mbar_arrive(vfull_bar(d / C::kVecBlock));
         }
         cp_async_wait<0>();
+        if (warp == 2)
+            for (int i = blockIdx.x; i < g.stats.count; i += gridDim.x) reduce_stats_warp(g.stats.job[i], lane);
       }
     } else {
         reg_alloc<232>();    // needs (232-168)*256 = 16384 <= 16384 (an unsatisfiable request would block forever)
@@ -743,6 +755,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 
     // ---- teardown: every role ends here, tensor memory is always released ------------------
     __syncwarp();
+    if (g.chain == CHAIN_BESIDE) pdl_wait();
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag) {
@@ -830,7 +843,7 @@ int sm_count()
 }
 
 template <MmaKind KIND, int BN, int SCALE, bool OUT_F32>
-int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc, cudaStream_t st)
+int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc, bool cleared, cudaStream_t st)
 {
     using C = Cfg<KIND, BN, SCALE>;
     auto kern = gemm_kernel<KIND, BN, SCALE, OUT_F32>;
@@ -850,24 +863,22 @@ int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
         while (ns > 1 && (num_kstages / ns < kMinSliceStages || rest * ns > kMaxSlicedItems)) --ns;
         if (ns > 1) {
             ga.split_first = full; ga.nsplit = ns; ga.num_items = full + rest * ns;
-            SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)rest * kNumEpiWarps * sizeof(uint32_t), st));
+            if (!cleared) SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)rest * kNumEpiWarps * sizeof(uint32_t), st));
         }
     }
     const int grid = ga.num_items < sms ? ga.num_items : sms;
-    kern<<<grid, kGemmThreads, C::kSmemBytes, st>>>(tmA, tmB, tmO, ga, idesc);
-    SNIP_CUDA_TRY(cudaGetLastError());
-    return SNIP_OK;
+    return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, tmA, tmB, tmO, ga, idesc);
 }
 
 template <MmaKind KIND, int BN>
 int launch_gemm_scale(int scale, bool out_f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g,
-                      uint32_t idesc, cudaStream_t st)
+                      uint32_t idesc, bool cleared, cudaStream_t st)
 {
     if (scale == SCALE_BLOCK_B)
-        return out_f32 ? launch_gemm<KIND, BN, SCALE_BLOCK_B, true>(tmA, tmB, tmO, g, idesc, st)
-                       : launch_gemm<KIND, BN, SCALE_BLOCK_B, false>(tmA, tmB, tmO, g, idesc, st);
-    return out_f32 ? launch_gemm<KIND, BN, SCALE_VEC_B, true>(tmA, tmB, tmO, g, idesc, st)
-                   : launch_gemm<KIND, BN, SCALE_VEC_B, false>(tmA, tmB, tmO, g, idesc, st);
+        return out_f32 ? launch_gemm<KIND, BN, SCALE_BLOCK_B, true>(tmA, tmB, tmO, g, idesc, cleared, st)
+                       : launch_gemm<KIND, BN, SCALE_BLOCK_B, false>(tmA, tmB, tmO, g, idesc, cleared, st);
+    return out_f32 ? launch_gemm<KIND, BN, SCALE_VEC_B, true>(tmA, tmB, tmO, g, idesc, cleared, st)
+                   : launch_gemm<KIND, BN, SCALE_VEC_B, false>(tmA, tmB, tmO, g, idesc, cleared, st);
 }
 
 }  // namespace
@@ -876,6 +887,20 @@ size_t gemm_ws_bytes() { return 256; }
 // Workspace with which the weight-gradient product may slice the tiles of its last wave along the contraction:
 // status word, arrival counters, one FP32 tile per slice.
 size_t gemm_ws_bytes_sliced() { return kSliceCountersOffset + kSliceCountersBytes + (size_t)kMaxSlicedItems * BM * 256 * sizeof(float); }
+
+// The parts of a workspace of gemm_ws_bytes() or gemm_ws_bytes_sliced(), for one GEMM.
+GemmWs gemm_ws(void *ws, size_t ws_bytes)
+{
+    GemmWs w;
+    w.status = static_cast<uint32_t *>(ws);
+    if (ws_bytes >= gemm_ws_bytes_sliced()) {
+        w.counters = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(ws) + kSliceCountersOffset);
+        w.partials = reinterpret_cast<float *>(static_cast<uint8_t *>(ws) + kSliceCountersOffset + kSliceCountersBytes);
+    }
+    return w;
+}
+// What a chain's first kernel clears of it: status word and counters.
+int32_t gemm_ws_zero_words() { return (int32_t)((kSliceCountersOffset + kSliceCountersBytes) / sizeof(uint32_t)); }
 
 // Testing hooks (snip_debug_set): process-wide, off by default.
 namespace {
@@ -895,6 +920,8 @@ void gemm_debug_hooks(uint64_t *wait_limit_ns, int *tx_skew)
 int gemm_pair_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, int64_t Mo, int64_t No, int64_t Kc, const float *sa,
                    int64_t sa_chunk_stride, const float *sb, int64_t sb_chunk_stride, int64_t sb_blk_stride, int scale_mode, void *out,
                    int out_dtype, int accumulate, uint32_t *status, uint64_t wait_limit_ns, int tx_skew, cudaStream_t st);
+
+int launch_stat_jobs(const StatJobs &jobs, cudaStream_t st);   // quantize.cu
 
 // Zeroes the status word of a GEMM workspace (enqueued; allocates nothing).
 int gemm_clear_status(void *ws, cudaStream_t st)
@@ -924,14 +951,14 @@ int transpose_bf16(const void *in, void *out, int64_t rows, int64_t cols, cudaSt
 // scale_mode: SCALE_NONE for BF16, SCALE_BLOCK_B (fwd / dgrad), SCALE_VEC_B (wgrad).
 int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, int64_t Mo, int64_t No, int64_t Kc, const float *sa,
               int64_t sa_chunk_stride, const float *sb, int64_t sb_chunk_stride, int64_t sb_blk_stride, int scale_mode, void *out,
-              int out_dtype, int accumulate, void *ws, size_t ws_bytes, cudaStream_t st, bool clear_status)
+              int out_dtype, int accumulate, const GemmWs &w, cudaStream_t st, const ChainLink &link)
 {
     if (!a_codes || !b_codes || !out) return SNIP_ERR_ARG;
     if (!valid_dim(Mo) || !valid_dim(No) || !valid_dim(Kc) || Mo > INT32_MAX || No > INT32_MAX || Kc > INT32_MAX) return SNIP_ERR_SHAPE;
     if (out_dtype != SNIP_OUT_BF16 && out_dtype != SNIP_OUT_FP32) return SNIP_ERR_ARG;
     if (accumulate && out_dtype != SNIP_OUT_FP32) return SNIP_ERR_UNSUPPORTED;
-    if (!ws || ws_bytes < gemm_ws_bytes()) return SNIP_ERR_WORKSPACE;
-    if (!aligned16(a_codes) || !aligned16(b_codes) || !aligned16(out) || !aligned16(ws)) return SNIP_ERR_ALIGN;
+    if (!w.status) return SNIP_ERR_WORKSPACE;
+    if (!aligned16(a_codes) || !aligned16(b_codes) || !aligned16(out) || !aligned16(w.status)) return SNIP_ERR_ALIGN;
     const bool a16 = fmt_a == SNIP_FMT_BF16, b16 = fmt_b == SNIP_FMT_BF16;
     if (a16 != b16) return SNIP_ERR_UNSUPPORTED;
     if (!a16 && (!sa || !sb)) return SNIP_ERR_ARG;
@@ -940,19 +967,21 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     if (rc != SNIP_OK) return rc;
     // The status word starts at zero for this call unless the caller runs several GEMMs against one word
     // and has cleared it itself (an earlier GEMM's timeout must survive the later ones).
-    if (clear_status) { rc = gemm_clear_status(ws, st); if (rc) return rc; }
+    if (!w.cleared) { rc = gemm_clear_status(w.status, st); if (rc) return rc; }
 
     GemmArgs g;
     g.Mo = (int32_t)Mo; g.No = (int32_t)No; g.Kc = (int32_t)Kc;
     g.sa = sa; g.sa_chunk_stride = sa_chunk_stride;
     g.sb = sb; g.sb_chunk_stride = sb_chunk_stride; g.sb_blk_stride = sb_blk_stride;
     g.out = out; g.ldo = No; g.accumulate = accumulate;
-    g.status = static_cast<uint32_t *>(ws);
+    g.status = w.status;
+    g.chain = link.role;
+    if (link.jobs) g.stats = *link.jobs;
     g.split_first = 0; g.nsplit = 1; g.num_items = 0;   // set per launch
     g.partials = nullptr; g.counters = nullptr;
-    if (!a16 && scale_mode == SCALE_VEC_B && ws_bytes >= gemm_ws_bytes_sliced() && g_slicing.load()) {
-        g.counters = reinterpret_cast<uint32_t *>(static_cast<uint8_t *>(ws) + kSliceCountersOffset);
-        g.partials = reinterpret_cast<float *>(static_cast<uint8_t *>(ws) + kSliceCountersOffset + kSliceCountersBytes);
+    if (!a16 && scale_mode == SCALE_VEC_B && w.partials && g_slicing.load()) {
+        g.counters = w.counters;
+        g.partials = w.partials;
     }
     g.stage_tx_bytes = 0;
     g.wait_limit_ns = (uint64_t)g_wait_limit_ns.load();
@@ -962,9 +991,12 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // The CTA-pair kernels (gemm_pair.cu) are an alternative form of the same product, kept for comparison: they
     // run only when asked for through snip_debug_set (on the 7B shapes they are slower than the kernels below).
     const int choice = g_kernel_choice.load();
-    if (!a16 && choice == 2)
+    if (!a16 && choice == 2) {
+        rc = launch_stat_jobs(g.stats, st);   // these kernels do not reduce statistics
+        if (rc) return rc;
         return gemm_pair_impl(fmt_a, fmt_b, a_codes, b_codes, Mo, No, Kc, sa, sa_chunk_stride, sb, sb_chunk_stride, sb_blk_stride, scale_mode,
                               out, out_dtype, accumulate, g.status, g.wait_limit_ns, tx_skew, st);
+    }
 
     CUtensorMap tmA, tmB, tmO;
     // output boxes of 32 rows x 64 bytes for the TMA stores of the block-mode epilogue
@@ -978,8 +1010,8 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         if (rc) return rc;
         const uint32_t idesc = make_idesc(1, 1, BM, 256);
         g.stage_tx_bytes = (BM + 256) * 128 + tx_skew;
-        return f32 ? launch_gemm<MmaKind::F16, 256, SCALE_NONE, true>(tmA, tmB, tmO, g, idesc, st)
-                   : launch_gemm<MmaKind::F16, 256, SCALE_NONE, false>(tmA, tmB, tmO, g, idesc, st);
+        return f32 ? launch_gemm<MmaKind::F16, 256, SCALE_NONE, true>(tmA, tmB, tmO, g, idesc, w.cleared, st)
+                   : launch_gemm<MmaKind::F16, 256, SCALE_NONE, false>(tmA, tmB, tmO, g, idesc, w.cleared, st);
     }
     if (fmt_a == SNIP_FMT_FP4_E2M1 && fmt_b == SNIP_FMT_FP4_E2M1 && (scale_mode == SCALE_BLOCK_B || (Kc % 128) != 0)) {
         // Packed FP4 on both sides, forward / input gradient, or a contraction length ending in a 64-wide tile: kind::mxf4 on the
@@ -995,7 +1027,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         if (rc) return rc;
         const uint32_t idesc = make_idesc_block_scaled(1, 1, BM, BN);
         g.stage_tx_bytes = (BM + BN) * 128 + tx_skew;
-        return launch_gemm_scale<MmaKind::MXF4, BN>(scale_mode, f32, tmA, tmB, tmO, g, idesc, st);
+        return launch_gemm_scale<MmaKind::MXF4, BN>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
     }
     // FP8 x FP8, the mixed pairs and the FP4 x FP4 weight gradient over whole chunks: kind::f8f6f4; FP4 operands are expanded by
     // the TMA unit to one 16-byte-aligned group per 16 elements, which is the layout this MMA kind reads
@@ -1018,7 +1050,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // an FP4 operand expanded by the TMA unit occupies 128 B per row in shared memory but reports
     // only its 64 packed source bytes to the barrier
     g.stage_tx_bytes = BM * (a4 ? 64 : 128) + BN * (b4 ? 64 : 128) + tx_skew;
-    return launch_gemm_scale<MmaKind::F8F6F4, BN>(scale_mode, f32, tmA, tmB, tmO, g, idesc, st);
+    return launch_gemm_scale<MmaKind::F8F6F4, BN>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
 }
 
 }  // namespace snip
@@ -1054,8 +1086,9 @@ extern "C" int snip_gemm_quantized(int op, const snip_qtensor_t *a, const snip_q
         sa_cs = Mo; sb_cs = No; sb_bs = 0; mode = SCALE_VEC_B;
     }
     if (!q) mode = SCALE_NONE;
+    if (!ws || ws_bytes < gemm_ws_bytes()) return SNIP_ERR_WORKSPACE;
     return gemm_impl(a->fmt, b->fmt, a->codes, b->codes, Mo, No, Kc, sa, sa_cs, sb, sb_cs, sb_bs, mode, out, out_dtype, accumulate,
-                     ws, ws_bytes, static_cast<cudaStream_t>(stream), true);
+                     gemm_ws(ws, ws_bytes), static_cast<cudaStream_t>(stream), ChainLink());
 }
 
 extern "C" int snip_debug_set(int key, long long value)

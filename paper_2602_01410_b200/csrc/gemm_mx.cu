@@ -22,6 +22,7 @@
 #include <string.h>
 
 #include "common.cuh"
+#include "quant_device.cuh"
 #include "sm100.cuh"
 
 namespace snip {
@@ -48,6 +49,8 @@ struct MxArgs {
     uint32_t *status;
     const float *amax_a, *amax_b;   // two-level option: the tensors' magnitude bounds (device); else null
     uint64_t wait_limit_ns;    // bound of every device-side wait
+    int32_t chain;             // ChainRole
+    StatJobs stats;            // reductions left by the quantizers ahead
 };
 
 template <MmaKind KIND>
@@ -133,6 +136,9 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     __syncthreads();
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
+    // everything up to here touches nothing that a kernel ahead on the stream writes
+    if (g.chain != CHAIN_BESIDE) pdl_wait();
+    pdl_launch_dependents();
 
     if (warp == 0) {
         // ================= producer: operand tiles and scale-factor atoms =================
@@ -225,6 +231,9 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                 }
             }
         }
+    } else if (warp == 2) {
+        // ================= statistics of the quantizers ahead =================
+        for (int i = blockIdx.x; i < g.stats.count; i += gridDim.x) reduce_stats_warp(g.stats.job[i], lane);
     } else if (warp >= 4) {
         // ================= epilogue: drain, round, store =================
         const int e = warp - 4, q = warp & 3, h = e >> 2;
@@ -289,6 +298,7 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
     // ---- teardown ----
     __syncwarp();
+    if (g.chain == CHAIN_BESIDE) pdl_wait();
     tc_fence_before_sync();
     __syncthreads();
     if (*abort_flag) {
@@ -313,9 +323,7 @@ int launch_mx(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap 
     SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
     const int num_tiles = (int)(ceil_div(g.Mo, BM) * ceil_div(g.No, BN));
     const int grid = num_tiles < sms ? num_tiles : sms;
-    kern<<<grid, kThreads, C::kSmemBytes, st>>>(tmA, tmB, tmO, g, idesc);
-    SNIP_CUDA_TRY(cudaGetLastError());
-    return SNIP_OK;
+    return launch_chained(kern, grid, kThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, tmA, tmB, tmO, g, idesc);
 }
 
 }  // namespace
@@ -323,22 +331,23 @@ int launch_mx(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap 
 int make_tiled_map_2d(CUtensorMap *map, const void *ptr, int dtype, int64_t rows, int64_t inner_elems, int64_t row_bytes, int box_x_elems,
                       int box_rows, int swizzle);
 int gemm_clear_status(void *ws, cudaStream_t st);
+GemmWs gemm_ws(void *ws, size_t ws_bytes);
 int gemm_sm_count();
 void gemm_debug_hooks(uint64_t *wait_limit_ns, int *tx_skew);   // testing hooks of snip_debug_set (gemm.cu)
 
 // a_codes [Mo][Kc], b_codes [No][Kc] contraction-major; sfa / sfb: UE8M0 atoms [line tile][chunk][512].
 int gemm_mx_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, const void *sfa, const void *sfb, int64_t Mo, int64_t No,
-                 int64_t Kc, void *out, int out_dtype, void *ws, size_t ws_bytes, cudaStream_t st, bool clear_status)
+                 int64_t Kc, void *out, int out_dtype, const GemmWs &w, cudaStream_t st, const ChainLink &link)
 {
     if (!a_codes || !b_codes || !sfa || !sfb || !out) return SNIP_ERR_ARG;
     if (!valid_dim(Mo) || !valid_dim(No) || !valid_dim(Kc) || Mo > INT32_MAX || No > INT32_MAX || Kc > INT32_MAX) return SNIP_ERR_SHAPE;
     if (out_dtype != SNIP_OUT_BF16 && out_dtype != SNIP_OUT_FP32) return SNIP_ERR_ARG;
     if (fmt_a == SNIP_FMT_BF16 || fmt_b == SNIP_FMT_BF16) return SNIP_ERR_UNSUPPORTED;
-    if (!ws || ws_bytes < 256) return SNIP_ERR_WORKSPACE;
-    if (!aligned16(a_codes) || !aligned16(b_codes) || !aligned16(sfa) || !aligned16(sfb) || !aligned16(out) || !aligned16(ws)) return SNIP_ERR_ALIGN;
+    if (!w.status) return SNIP_ERR_WORKSPACE;
+    if (!aligned16(a_codes) || !aligned16(b_codes) || !aligned16(sfa) || !aligned16(sfb) || !aligned16(out) || !aligned16(w.status)) return SNIP_ERR_ALIGN;
     int rc = require_sm100();
     if (rc != SNIP_OK) return rc;
-    if (clear_status) { rc = gemm_clear_status(ws, st); if (rc) return rc; }   // see gemm_impl
+    if (!w.cleared) { rc = gemm_clear_status(w.status, st); if (rc) return rc; }   // see gemm_impl
     const bool f32 = out_dtype == SNIP_OUT_FP32;
     const bool a4 = fmt_a == SNIP_FMT_FP4_E2M1, b4 = fmt_b == SNIP_FMT_FP4_E2M1;
 
@@ -347,7 +356,9 @@ int gemm_mx_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes,
     g.sfa = static_cast<const uint8_t *>(sfa);
     g.sfb = static_cast<const uint8_t *>(sfb);
     g.n_atoms_b = (int32_t)ceil_div(No, 128);
-    g.status = static_cast<uint32_t *>(ws);
+    g.status = w.status;
+    g.chain = link.role;
+    if (link.jobs) g.stats = *link.jobs;
     int tx_skew = 0;
     gemm_debug_hooks(&g.wait_limit_ns, &tx_skew);
     g.amax_a = g.amax_b = nullptr;
@@ -382,24 +393,26 @@ int gemm_mx_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes,
 // Two-level option: packed E2M1 codes, E4M3 scale bytes per 16-long tile as atoms [line tile][chunk][half][512], and the
 // two tensors' magnitude bounds (device pointers).  out = (sum of block-scaled products) / (enc_a * enc_b), enc = 2688 / bound.
 int gemm_nvfp4_impl(const void *a_codes, const void *b_codes, const void *sfa, const void *sfb, const float *amax_a, const float *amax_b,
-                    int64_t Mo, int64_t No, int64_t Kc, void *out, int out_dtype, void *ws, size_t ws_bytes, cudaStream_t st, bool clear_status)
+                    int64_t Mo, int64_t No, int64_t Kc, void *out, int out_dtype, const GemmWs &w, cudaStream_t st, const ChainLink &link)
 {
     if (!a_codes || !b_codes || !sfa || !sfb || !amax_a || !amax_b || !out) return SNIP_ERR_ARG;
     if (!valid_dim(Mo) || !valid_dim(No) || !valid_dim(Kc) || Mo > INT32_MAX || No > INT32_MAX || Kc > INT32_MAX) return SNIP_ERR_SHAPE;
     if (out_dtype != SNIP_OUT_BF16 && out_dtype != SNIP_OUT_FP32) return SNIP_ERR_ARG;
-    if (!ws || ws_bytes < 256) return SNIP_ERR_WORKSPACE;
-    if (!aligned16(a_codes) || !aligned16(b_codes) || !aligned16(sfa) || !aligned16(sfb) || !aligned16(out) || !aligned16(ws)) return SNIP_ERR_ALIGN;
+    if (!w.status) return SNIP_ERR_WORKSPACE;
+    if (!aligned16(a_codes) || !aligned16(b_codes) || !aligned16(sfa) || !aligned16(sfb) || !aligned16(out) || !aligned16(w.status)) return SNIP_ERR_ALIGN;
     if ((reinterpret_cast<uintptr_t>(amax_a) & 3u) || (reinterpret_cast<uintptr_t>(amax_b) & 3u)) return SNIP_ERR_ALIGN;
     int rc = require_sm100();
     if (rc != SNIP_OK) return rc;
-    if (clear_status) { rc = gemm_clear_status(ws, st); if (rc) return rc; }
+    if (!w.cleared) { rc = gemm_clear_status(w.status, st); if (rc) return rc; }
     const bool f32 = out_dtype == SNIP_OUT_FP32;
     MxArgs g;
     g.Mo = (int32_t)Mo; g.No = (int32_t)No; g.Kc = (int32_t)Kc;
     g.sfa = static_cast<const uint8_t *>(sfa);
     g.sfb = static_cast<const uint8_t *>(sfb);
     g.n_atoms_b = (int32_t)ceil_div(No, 128);
-    g.status = static_cast<uint32_t *>(ws);
+    g.status = w.status;
+    g.chain = link.role;
+    if (link.jobs) g.stats = *link.jobs;
     int tx_skew = 0;
     gemm_debug_hooks(&g.wait_limit_ns, &tx_skew);
     g.amax_a = amax_a; g.amax_b = amax_b;
@@ -444,7 +457,8 @@ extern "C" int snip_gemm_mx(int op, const snip_qtensor_t *a, const void *sf_a, c
             return SNIP_ERR_UNSUPPORTED;
         Mo = a->cols; No = b->cols; Kc = a->rows;
     }
-    return gemm_mx_impl(a->fmt, b->fmt, a->codes, b->codes, sf_a, sf_b, Mo, No, Kc, out, out_dtype, ws, ws_bytes, static_cast<cudaStream_t>(stream), true);
+    if (!ws || ws_bytes < 256) return SNIP_ERR_WORKSPACE;
+    return gemm_mx_impl(a->fmt, b->fmt, a->codes, b->codes, sf_a, sf_b, Mo, No, Kc, out, out_dtype, gemm_ws(ws, 256), static_cast<cudaStream_t>(stream), ChainLink());
 }
 
 extern "C" int snip_gemm_nvfp4(int op, const snip_qtensor_t *a, const void *sf_a, const float *amax_a, const snip_qtensor_t *b, const void *sf_b,
@@ -467,5 +481,6 @@ extern "C" int snip_gemm_nvfp4(int op, const snip_qtensor_t *a, const void *sf_a
         if (a->block != SNIP_BLOCK_COL_16x1 || b->block != SNIP_BLOCK_COL_16x1) return SNIP_ERR_UNSUPPORTED;
         Mo = a->cols; No = b->cols; Kc = a->rows;
     }
-    return gemm_nvfp4_impl(a->codes, b->codes, sf_a, sf_b, amax_a, amax_b, Mo, No, Kc, out, out_dtype, ws, ws_bytes, static_cast<cudaStream_t>(stream), true);
+    if (!ws || ws_bytes < 256) return SNIP_ERR_WORKSPACE;
+    return gemm_nvfp4_impl(a->codes, b->codes, sf_a, sf_b, amax_a, amax_b, Mo, No, Kc, out, out_dtype, gemm_ws(ws, 256), static_cast<cudaStream_t>(stream), ChainLink());
 }

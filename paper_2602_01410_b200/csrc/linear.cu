@@ -9,23 +9,24 @@ int quantize_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt
                   float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st);
 int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, int64_t Mo, int64_t No, int64_t Kc, const float *sa,
               int64_t sa_chunk_stride, const float *sb, int64_t sb_chunk_stride, int64_t sb_blk_stride, int scale_mode, void *out,
-              int out_dtype, int accumulate, void *ws, size_t ws_bytes, cudaStream_t st, bool clear_status);
-int gemm_clear_status(void *ws, cudaStream_t st);
+              int out_dtype, int accumulate, const GemmWs &w, cudaStream_t st, const ChainLink &link);
+GemmWs gemm_ws(void *ws, size_t ws_bytes);
+int32_t gemm_ws_zero_words();
 int quantize_impl_ex(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags, int pow2, void *sf,
-                     void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st);
+                     void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st,
+                     const ChainLink &link);
 int gemm_mx_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, const void *sfa, const void *sfb, int64_t Mo, int64_t No,
-                 int64_t Kc, void *out, int out_dtype, void *ws, size_t ws_bytes, cudaStream_t st, bool clear_status);
+                 int64_t Kc, void *out, int out_dtype, const GemmWs &w, cudaStream_t st, const ChainLink &link);
 int transpose_bf16(const void *in, void *out, int64_t rows, int64_t cols, cudaStream_t st);
 size_t gemm_ws_bytes();
 size_t gemm_ws_bytes_sliced();   // with room for the weight-gradient product's contraction slices
 int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int kind, int pow2, const DualOut &oa, const DualOut &ob,
-                       void *ws, size_t ws_bytes, cudaStream_t st);
+                       void *ws, size_t ws_bytes, cudaStream_t st, const ChainLink &link);
 int quantize_nvfp4_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, const float *tensor_amax, void *codes_a, void *sf_a,
                              snip_stats_t *stats_a, void *codes_b, void *sf_b, snip_stats_t *stats_b, int rounding, uint64_t seed, void *ws,
-                             size_t ws_bytes, cudaStream_t st);
+                             size_t ws_bytes, cudaStream_t st, const ChainLink &link);
 int gemm_nvfp4_impl(const void *a_codes, const void *b_codes, const void *sfa, const void *sfb, const float *amax_a, const float *amax_b,
-                    int64_t Mo, int64_t No, int64_t Kc, void *out, int out_dtype, void *ws, size_t ws_bytes, cudaStream_t st, bool clear_status);
-int gemm_clear_status(void *ws, cudaStream_t st);
+                    int64_t Mo, int64_t No, int64_t Kc, void *out, int out_dtype, const GemmWs &w, cudaStream_t st, const ChainLink &link);
 
 namespace {
 
@@ -129,15 +130,23 @@ int linear_impl(int op, const void *A, const void *B, void *out, int64_t M, int6
 
     int rc;
     const void *ga = A, *gb = B;
+    // quantizers and GEMM form a chain: no statistics or clearing launches of their own, no gaps
+    StatJobs jobs;
+    ChainLink first, beside, after;
+    first.role = CHAIN_FIRST; first.zero = static_cast<uint32_t *>(gws); first.zero_words = gemm_ws_zero_words(); first.jobs = &jobs;
+    beside.role = CHAIN_BESIDE; beside.jobs = &jobs;
+    after.role = CHAIN_AFTER; after.jobs = &jobs;
+    GemmWs gw = gemm_ws(gws, mx ? gemm_ws_bytes() : gemm_ws_bytes_sliced());
     if (q) {
         rc = quantize_impl_ex(A, p.rows_a, p.cols_a, p.cols_a, fmt_a, p.block_a, (p.tr_a ? SNIP_Q_TRANSPOSED : 0u) | (stats_a ? SNIP_Q_STATS : 0u),
-                              mx ? 1 : 0, sf_a, codes_a, scales_a, stats_a, nullptr, sws_a, sws_a_bytes, st);
+                              mx ? 1 : 0, sf_a, codes_a, scales_a, stats_a, nullptr, sws_a, sws_a_bytes, st, first);
         if (rc) return rc;
         rc = quantize_impl_ex(B, p.rows_b, p.cols_b, p.cols_b, fmt_b, p.block_b, (p.tr_b ? SNIP_Q_TRANSPOSED : 0u) | (stats_b ? SNIP_Q_STATS : 0u),
-                              mx ? 1 : 0, sf_b, codes_b, scales_b, stats_b, nullptr, sws_b, sws_b_bytes, st);
+                              mx ? 1 : 0, sf_b, codes_b, scales_b, stats_b, nullptr, sws_b, sws_b_bytes, st, beside);
+        gw.cleared = true;
         if (rc) return rc;
         ga = codes_a; gb = codes_b;
-        if (mx) return gemm_mx_impl(fmt_a, fmt_b, ga, gb, sf_a, sf_b, p.Mo, p.No, p.Kc, out, out_dtype, gws, gemm_ws_bytes(), st, true);
+        if (mx) return gemm_mx_impl(fmt_a, fmt_b, ga, gb, sf_a, sf_b, p.Mo, p.No, p.Kc, out, out_dtype, gw, st, after);
     } else {
         // BF16 tag: identity quantization; only operands whose contraction index is not contiguous are copied
         if (p.tr_a) { rc = transpose_bf16(A, codes_a, p.rows_a, p.cols_a, st); if (rc) return rc; ga = codes_a; }
@@ -150,7 +159,7 @@ int linear_impl(int op, const void *A, const void *B, void *out, int64_t M, int6
     else if (op == SNIP_OP_DGRAD) { sb_bs = 1; sb_cs = ceil_div(K, 128); }
     else { sb_bs = 0; sb_cs = p.No; }
     return gemm_impl(fmt_a, fmt_b, ga, gb, p.Mo, p.No, p.Kc, scales_a, sa_cs, scales_b, sb_cs, sb_bs, q ? p.scale_mode : SCALE_NONE, out,
-                     out_dtype, accumulate, gws, gemm_ws_bytes_sliced(), st, true);
+                     out_dtype, accumulate, gw, st, q ? after : ChainLink());
 }
 
 
@@ -163,8 +172,8 @@ struct FwdBwdCarve {
     void *codes[6];
     float *scales[6];
     void *sf[6];
-    void *stats_ws;
-    size_t stats_ws_bytes;
+    void *stats_ws[3];
+    size_t stats_ws_bytes[3];
     size_t total;
 };
 
@@ -188,13 +197,11 @@ FwdBwdCarve carve_fwd_bwd(void *ws, int64_t M, int64_t N, int64_t K, const int (
         f.sf[i] = mx ? c.take(sf_bytes(rows[i], cols[i])) : nullptr;
     }
     size_t sb = 0;
-    for (int i = 0; i < 6; i += 2) {
-        size_t w = 0;
-        snip_quantize_dual_workspace(rows[i], cols[i], &w);
-        if (w > sb) sb = w;
+    for (int i = 0; i < 6; i += 2) {   // the statistics of all three tensors are reduced together, behind the last quantizer
+        snip_quantize_dual_workspace(rows[i], cols[i], &sb);
+        f.stats_ws[i / 2] = c.take(sb);
+        f.stats_ws_bytes[i / 2] = sb;
     }
-    f.stats_ws = c.take(sb);
-    f.stats_ws_bytes = sb;
     f.total = c.off;
     return f;
 }
@@ -288,28 +295,39 @@ extern "C" int snip_linear_fwd_bwd(const void *X, const void *W, const void *dY,
         const int sr = (i >= 4 && dy_rounding == SNIP_ROUND_STOCHASTIC && fmt[i] == SNIP_FMT_FP4_E2M1) ? 1 : 0;
         return DualOut{fmt[i], f.codes[i], f.scales[i], f.sf[i], stats6 ? stats6 + i : nullptr, sr, dy_seed};
     };
+    // One chain: the three quantizers side by side (each tensor is read once and leaves both of its copies), then the three GEMMs, which
+    // are independent of one another: the next one takes the SMs that the last wave of the one ahead leaves idle.  The first quantizer
+    // clears the status word (one for the three GEMMs) and the slice counters, the first GEMM reduces the statistics.
+    StatJobs jobs;
+    ChainLink quant[3], mult[3];
+    for (int i = 0; i < 3; ++i) {
+        quant[i].role = i ? CHAIN_BESIDE : CHAIN_FIRST;
+        quant[i].jobs = &jobs;
+        mult[i].role = i ? CHAIN_BESIDE : CHAIN_AFTER;
+    }
+    quant[0].zero = static_cast<uint32_t *>(f.gws);
+    quant[0].zero_words = gemm_ws_zero_words();
+    mult[0].jobs = &jobs;
+    GemmWs gw = gemm_ws(f.gws, gemm_ws_bytes_sliced());
+    gw.cleared = true;
     auto gemm = [&](int op, int ia, int ib, void *out) -> int {
         const LinearPlan p = plan_for(op, M, N, K);
-        if (mx) return gemm_mx_impl(fmt[ia], fmt[ib], f.codes[ia], f.codes[ib], f.sf[ia], f.sf[ib], p.Mo, p.No, p.Kc, out, out_dtype, f.gws, gemm_ws_bytes(), st, false);
+        const ChainLink &link = mult[op];
+        if (mx) return gemm_mx_impl(fmt[ia], fmt[ib], f.codes[ia], f.codes[ib], f.sf[ia], f.sf[ib], p.Mo, p.No, p.Kc, out, out_dtype, gw, st, link);
         int64_t sb_cs, sb_bs;
         if (op == SNIP_OP_FWD) { sb_bs = ceil_div(K, 128); sb_cs = 1; }
         else if (op == SNIP_OP_DGRAD) { sb_bs = 1; sb_cs = ceil_div(K, 128); }
         else { sb_bs = 0; sb_cs = p.No; }
         return gemm_impl(fmt[ia], fmt[ib], f.codes[ia], f.codes[ib], p.Mo, p.No, p.Kc, f.scales[ia], p.Mo, f.scales[ib], sb_cs, sb_bs, p.scale_mode, out,
-                         out_dtype, 0, f.gws, gemm_ws_bytes_sliced(), st, false);
+                         out_dtype, 0, gw, st, link);
     };
-    // one status word serves the three GEMMs of this call: cleared once, so that a timeout of the first is not erased
-    rc = gemm_clear_status(f.gws, st);
+    rc = quantize_dual_impl(X, M, K, K, kind_xdy, mx, out_of(0), out_of(1), f.stats_ws[0], f.stats_ws_bytes[0], st, quant[0]);
     if (rc) return rc;
-    // forward: X and W are read once each and leave both of their quantized copies behind
-    rc = quantize_dual_impl(X, M, K, K, kind_xdy, mx, out_of(0), out_of(1), f.stats_ws, f.stats_ws_bytes, st);
+    rc = quantize_dual_impl(W, N, K, K, kind_w, mx, out_of(2), out_of(3), f.stats_ws[1], f.stats_ws_bytes[1], st, quant[1]);
     if (rc) return rc;
-    rc = quantize_dual_impl(W, N, K, K, kind_w, mx, out_of(2), out_of(3), f.stats_ws, f.stats_ws_bytes, st);
+    rc = quantize_dual_impl(dY, M, N, N, kind_xdy, mx, out_of(4), out_of(5), f.stats_ws[2], f.stats_ws_bytes[2], st, quant[2]);
     if (rc) return rc;
     rc = gemm(SNIP_OP_FWD, 0, 2, Y);
-    if (rc) return rc;
-    // backward: dY is read once; dgrad and wgrad consume the stored copies
-    rc = quantize_dual_impl(dY, M, N, N, kind_xdy, mx, out_of(4), out_of(5), f.stats_ws, f.stats_ws_bytes, st);
     if (rc) return rc;
     rc = gemm(SNIP_OP_DGRAD, 4, 3, dX);
     if (rc) return rc;
@@ -324,8 +342,8 @@ struct NvCarve {
     void *gws;
     void *codes[6];
     void *sf[6];
-    void *stats_ws;
-    size_t stats_ws_bytes, total;
+    void *stats_ws[3];
+    size_t stats_ws_bytes[3], total;
 };
 NvCarve carve_nvfp4(void *ws, int64_t M, int64_t N, int64_t K)
 {
@@ -340,12 +358,11 @@ NvCarve carve_nvfp4(void *ws, int64_t M, int64_t N, int64_t K)
         snip_quantize_nvfp4_sizes(rows[i], cols[i], &cb, &fb);
         f.codes[i] = c.take(cb);
         f.sf[i] = c.take(fb);
-        size_t w = 0;
-        snip_quantize_dual_workspace(rows[i], cols[i], &w);
-        if (w > sb) sb = w;
+        if (i & 1) continue;
+        snip_quantize_dual_workspace(rows[i], cols[i], &sb);
+        f.stats_ws[i / 2] = c.take(sb);
+        f.stats_ws_bytes[i / 2] = sb;
     }
-    f.stats_ws = c.take(sb);
-    f.stats_ws_bytes = sb;
     f.total = c.off;
     return f;
 }
@@ -375,20 +392,31 @@ extern "C" int snip_linear_fwd_bwd_nvfp4(const void *X, const void *W, const voi
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const float *bx = bounds3, *bw = bounds3 + 1, *bdy = bounds3 + 2;
     auto stat = [&](int i) { return stats6 ? stats6 + i : nullptr; };
-    int rc = gemm_clear_status(f.gws, st);   // one status word for the three GEMMs
+    // the chain of snip_linear_fwd_bwd: three quantizers side by side, three GEMMs behind them
+    StatJobs jobs;
+    ChainLink quant[3], mult[3];
+    for (int i = 0; i < 3; ++i) {
+        quant[i].role = i ? CHAIN_BESIDE : CHAIN_FIRST;
+        quant[i].jobs = &jobs;
+        mult[i].role = i ? CHAIN_BESIDE : CHAIN_AFTER;
+    }
+    quant[0].zero = static_cast<uint32_t *>(f.gws);
+    quant[0].zero_words = 1;
+    mult[0].jobs = &jobs;
+    GemmWs gw = gemm_ws(f.gws, gemm_ws_bytes());
+    gw.cleared = true;
+    int rc = quantize_nvfp4_dual_impl(X, M, K, K, bx, f.codes[0], f.sf[0], stat(0), f.codes[1], f.sf[1], stat(1), SNIP_ROUND_NEAREST_EVEN, 0,
+                                      f.stats_ws[0], f.stats_ws_bytes[0], st, quant[0]);
     if (rc) return rc;
-    rc = quantize_nvfp4_dual_impl(X, M, K, K, bx, f.codes[0], f.sf[0], stat(0), f.codes[1], f.sf[1], stat(1), SNIP_ROUND_NEAREST_EVEN, 0, f.stats_ws,
-                                  f.stats_ws_bytes, st);
+    rc = quantize_nvfp4_dual_impl(W, N, K, K, bw, f.codes[2], f.sf[2], stat(2), f.codes[3], f.sf[3], stat(3), SNIP_ROUND_NEAREST_EVEN, 0, f.stats_ws[1],
+                                  f.stats_ws_bytes[1], st, quant[1]);
     if (rc) return rc;
-    rc = quantize_nvfp4_dual_impl(W, N, K, K, bw, f.codes[2], f.sf[2], stat(2), f.codes[3], f.sf[3], stat(3), SNIP_ROUND_NEAREST_EVEN, 0, f.stats_ws,
-                                  f.stats_ws_bytes, st);
+    rc = quantize_nvfp4_dual_impl(dY, M, N, N, bdy, f.codes[4], f.sf[4], stat(4), f.codes[5], f.sf[5], stat(5), dy_rounding, dy_seed, f.stats_ws[2],
+                                  f.stats_ws_bytes[2], st, quant[2]);
     if (rc) return rc;
-    rc = gemm_nvfp4_impl(f.codes[0], f.codes[2], f.sf[0], f.sf[2], bx, bw, M, N, K, Y, out_dtype, f.gws, gemm_ws_bytes(), st, false);
+    rc = gemm_nvfp4_impl(f.codes[0], f.codes[2], f.sf[0], f.sf[2], bx, bw, M, N, K, Y, out_dtype, gw, st, mult[0]);
     if (rc) return rc;
-    rc = quantize_nvfp4_dual_impl(dY, M, N, N, bdy, f.codes[4], f.sf[4], stat(4), f.codes[5], f.sf[5], stat(5), dy_rounding, dy_seed, f.stats_ws,
-                                  f.stats_ws_bytes, st);
+    rc = gemm_nvfp4_impl(f.codes[4], f.codes[3], f.sf[4], f.sf[3], bdy, bw, M, K, N, dX, out_dtype, gw, st, mult[1]);
     if (rc) return rc;
-    rc = gemm_nvfp4_impl(f.codes[4], f.codes[3], f.sf[4], f.sf[3], bdy, bw, M, K, N, dX, out_dtype, f.gws, gemm_ws_bytes(), st, false);
-    if (rc) return rc;
-    return gemm_nvfp4_impl(f.codes[5], f.codes[1], f.sf[5], f.sf[1], bdy, bx, N, K, M, dW, out_dtype, f.gws, gemm_ws_bytes(), st, false);
+    return gemm_nvfp4_impl(f.codes[5], f.codes[1], f.sf[5], f.sf[1], bdy, bx, N, K, M, dW, out_dtype, gw, st, mult[2]);
 }

@@ -10,6 +10,35 @@
 
 namespace snip {
 
+struct CtaPartial {  // statistics of one CTA, reduced in fixed order
+    double sumsq_x;
+    double sumsq_err;
+    float amax;
+    float pad[3];
+};
+
+// Fixed-order reduction of one set of per-CTA partials by one warp (each lane a fixed strided subset, then shuffles).
+__device__ __forceinline__ void reduce_stats_warp(const StatJob &job, int lane)
+{
+    const CtaPartial *p = static_cast<const CtaPartial *>(job.partials);
+    double dx = 0.0, de = 0.0;
+    float am = 0.0f;
+#pragma unroll 4
+    for (int i = lane; i < job.n; i += 32) {
+        const double2 v = __ldcg(reinterpret_cast<const double2 *>(p + i));
+        dx += v.x;
+        de += v.y;
+        am = fmaxf(am, __ldcg(&p[i].amax));
+    }
+#pragma unroll
+    for (int off = 16; off > 0; off >>= 1) {
+        dx += __shfl_xor_sync(0xFFFFFFFFu, dx, off);
+        de += __shfl_xor_sync(0xFFFFFFFFu, de, off);
+        am = fmaxf(am, __shfl_xor_sync(0xFFFFFFFFu, am, off));
+    }
+    if (lane == 0) { job.out->sumsq_x = dx; job.out->sumsq_err = de; job.out->amax = am; job.out->reserved = 0; }
+}
+
 __device__ __forceinline__ float bf16lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 

@@ -33,13 +33,6 @@ namespace {
 constexpr int kTile = 128;
 constexpr int kThreads = 256;
 
-struct CtaPartial {  // one per CTA, reduced in fixed order by stats_reduce_kernel
-    double sumsq_x;
-    double sumsq_err;
-    float amax;
-    float pad[3];
-};
-
 struct QuantArgs {
     const uint16_t *x;
     int32_t rows, cols, ld;   // 32-bit (checked on the host): index products are 32 x 32 -> 64-bit multiplies
@@ -54,7 +47,23 @@ struct QuantArgs {
     uint32_t *sf;         // optional: UE8M0 bytes of 1/S in 512-byte atoms for hardware block scaling; null if unused
                           // (two-level option: the E4M3 scale bytes, two atoms per 128x128 tile)
     const float *tensor_amax;   // two-level option: bound of the tensor's magnitudes (device); else unused
+    int chain;            // ChainRole
+    uint32_t *zero;       // words this launch clears for the kernels behind it
+    int32_t zero_words;
 };
+
+// Start of every quantizer: wait for the kernel ahead on the stream (unless independent of it), let the one behind be scheduled
+// (it waits for this grid where it has to), clear what the chain asks for.
+__device__ __forceinline__ void chain_begin(const QuantArgs &a)
+{
+    if (a.chain != CHAIN_BESIDE) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.zero_words; i += gridDim.x * blockDim.x) a.zero[i] = 0u;
+}
+__device__ __forceinline__ void chain_end(const QuantArgs &a)
+{
+    if (a.chain == CHAIN_BESIDE) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // Scratch shared memory of one CTA (next to the tile slot).
 struct QuantShared {
@@ -819,12 +828,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_kernel(const Qu
     QuantShared &sh = *reinterpret_cast<QuantShared *>(smem + kStageBytes);
     QuantShared32 *s32 = reinterpret_cast<QuantShared32 *>(smem + kSmemBytes);   // present only for the 32-long tile kinds
     const uint4 *slot = reinterpret_cast<const uint4 *>(smem) + threadIdx.x;
-    // this grid may have been scheduled before the kernel ahead of it on the stream has finished (see
-    // launch_persistent): nothing is read or written before that kernel is complete
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    // the statistics reduction that follows on the stream may be scheduled now; it waits for this
-    // grid to finish before it reads anything (programmatic dependent launch)
-    if (STATS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_begin(a);
     ThreadStats ts;
     TileWalk w((int)a.tiles_r, (int)a.tiles_c);
     if (w.valid()) prefetch_tile(a, w.r, w.c, smem);
@@ -840,6 +844,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_kernel(const Qu
         __syncthreads();  // the scratch arrays are reused by the next tile
     }
     if (STATS) finish_stats<false>(ts, sh, a.partials, nullptr);
+    chain_end(a);
 }
 
 // Two outputs from one read (the tile kinds a tensor is consumed with, paper Fig. 5): `a` as stored
@@ -855,8 +860,7 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSm) quantize_dual_kernel
     QuantShared &sh = *reinterpret_cast<QuantShared *>(smem + kStageBytes);
     QuantShared32 *s32 = reinterpret_cast<QuantShared32 *>(smem + kSmemBytes);   // present only with SUB32
     const uint4 *slot = reinterpret_cast<const uint4 *>(smem) + threadIdx.x;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (STATS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_begin(d.a);
     ThreadStats ts;
     TileWalk w((int)d.a.tiles_r, (int)d.a.tiles_c);
     if (w.valid()) prefetch_tile(d.a, w.r, w.c, smem);
@@ -874,6 +878,7 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSm) quantize_dual_kernel
         __syncthreads();
     }
     if (STATS) finish_stats<true>(ts, sh, d.a.partials, d.b.partials);
+    chain_end(d.a);
 }
 
 // Two-level option, both copies from one read: a = 1x16 tiles as stored, b = 16x1 tiles transposed, E2M1 codes.
@@ -884,8 +889,7 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSm) quantize_nvfp4_dual_
     QuantShared &sh = *reinterpret_cast<QuantShared *>(smem + kStageBytes);
     QuantShared32 *s32 = reinterpret_cast<QuantShared32 *>(smem + kSmemBytes);   // holds this kernel's QuantShared16
     const uint4 *slot = reinterpret_cast<const uint4 *>(smem) + threadIdx.x;
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    if (STATS) asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_begin(d.a);
     TwoLevel tw;
     {
         const float bound = *d.a.tensor_amax;
@@ -909,6 +913,7 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSm) quantize_nvfp4_dual_
         __syncthreads();
     }
     if (STATS) finish_stats<true>(ts, sh, d.a.partials, d.b.partials);
+    chain_end(d.a);
 }
 
 // Fixed-order reduction of the per-CTA partials into one snip_stats_t (deterministic: every thread
@@ -1037,6 +1042,26 @@ void launch_fmt32(const QuantArgs &a, int block, bool codes, bool stats, dim3 gr
     }
 }
 
+// The statistics reduction behind a quantizer: launched at once, or left to the GEMM that ends the chain.
+int launch_reduce(const ReduceSets &sets, int nsets, int64_t nparts, const ChainLink &link, cudaStream_t st)
+{
+    if (link.jobs) {
+        for (int i = 0; i < nsets; ++i) link.jobs->job[link.jobs->count++] = {sets.partials[i], sets.out[i], (int32_t)nparts};
+        return SNIP_OK;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3((unsigned)nsets);
+    cfg.blockDim = dim3(1024);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SNIP_CUDA_TRY(cudaLaunchKernelEx(&cfg, stats_reduce_kernel, sets, nparts));
+    return SNIP_OK;
+}
+
 // CTAs of a persistent launch over ntiles tiles: kCtasPerSm per SM (what the kernels' shared memory and
 // registers allow), never more than there are tiles.
 int64_t persistent_ctas(int64_t ntiles, int per_sm = kCtasPerSm)
@@ -1055,9 +1080,21 @@ size_t stats_ws_bytes(int64_t rows, int64_t cols, bool rowstats)
 
 }  // namespace
 
+namespace {
+__global__ void stat_jobs_kernel(const StatJobs jobs) { reduce_stats_warp(jobs.job[blockIdx.x], threadIdx.x); }
+}  // namespace
+// The reductions of a chain as a launch of their own.
+int launch_stat_jobs(const StatJobs &jobs, cudaStream_t st)
+{
+    if (jobs.count == 0) return SNIP_OK;
+    stat_jobs_kernel<<<jobs.count, 32, 0, st>>>(jobs);
+    SNIP_CUDA_TRY(cudaGetLastError());
+    return SNIP_OK;
+}
+
 // Internal entry used by snip_quantize and by the linear-layer calls.
 int quantize_impl_ex(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags, int pow2, void *sf,
-                     void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st);
+                     void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st, const ChainLink &link = ChainLink());
 
 int quantize_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags,
                   void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes,
@@ -1068,19 +1105,19 @@ int quantize_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt
 
 int quantize_impl_full(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags, int pow2, void *sf, int sr,
                        uint64_t seed, void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes,
-                       cudaStream_t st);
+                       cudaStream_t st, const ChainLink &link = ChainLink());
 
 // pow2 = 1 selects the power-of-two scale rule; sf (optional, needs pow2) receives the UE8M0 atoms.
 int quantize_impl_ex(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags, int pow2, void *sf,
-                     void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st)
+                     void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st, const ChainLink &link)
 {
-    return quantize_impl_full(x, rows, cols, ld, fmt, block, flags, pow2, sf, 0, 0, codes, scales, stats, row_stats, ws, ws_bytes, st);
+    return quantize_impl_full(x, rows, cols, ld, fmt, block, flags, pow2, sf, 0, 0, codes, scales, stats, row_stats, ws, ws_bytes, st, link);
 }
 
 // sr = 1: stochastic rounding with `seed` (FP4 codes, 1x128 tiles as stored or 128x1 tiles transposed, no per-row sums).
 int quantize_impl_full(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags, int pow2, void *sf, int sr,
                        uint64_t seed, void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes,
-                       cudaStream_t st)
+                       cudaStream_t st, const ChainLink &link)
 {
     if (sf) {
         const bool tr = (flags & SNIP_Q_TRANSPOSED) != 0;
@@ -1118,6 +1155,8 @@ int quantize_impl_full(const void *x, int64_t rows, int64_t cols, int64_t ld, in
     a.rows = (int32_t)rows; a.cols = (int32_t)cols; a.ld = (int32_t)ld;
     a.pow2 = pow2; a.sf = static_cast<uint32_t *>(sf);
     a.seed = seed;
+    a.tensor_amax = nullptr;
+    a.chain = link.role; a.zero = link.zero; a.zero_words = link.zero_words;
     a.codes = want_codes ? static_cast<uint8_t *>(codes) : nullptr;
     a.scales = want_codes ? scales : nullptr;
     a.partials = any_stats ? static_cast<CtaPartial *>(ws) : nullptr;
@@ -1143,17 +1182,8 @@ int quantize_impl_full(const void *x, int64_t rows, int64_t cols, int64_t ld, in
     else launch_variant<SNIP_FMT_BF16, SNIP_BLOCK_BLK_128x128, false>(a, false, true, want_rows, grid, st);
     SNIP_CUDA_TRY(cudaGetLastError());
     if (want_stats) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1);
-        cfg.blockDim = dim3(1024);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const ReduceSets sets = {{a.partials, nullptr}, {stats, nullptr}};
-        SNIP_CUDA_TRY(cudaLaunchKernelEx(&cfg, stats_reduce_kernel, sets, nparts));
+        rc = launch_reduce(ReduceSets{{a.partials, nullptr}, {stats, nullptr}}, 1, nparts, link, st);
+        if (rc) return rc;
     }
     if (want_rows) {
         row_stats_reduce_kernel<<<(unsigned)ceil_div(rows, 256), 256, 0, st>>>(a.row_partials, rows, tc, row_stats);
@@ -1190,7 +1220,7 @@ static void launch_dual32(const DualArgs &d, bool stats, dim3 grid, cudaStream_t
 
 // kind: SNIP_DUAL_ROW_COLT, SNIP_DUAL_BLK_BLKT or SNIP_DUAL_ROW32_COL32T (power-of-two scales only).
 int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int kind, int pow2, const DualOut &oa, const DualOut &ob,
-                       void *ws, size_t ws_bytes, cudaStream_t st)
+                       void *ws, size_t ws_bytes, cudaStream_t st, const ChainLink &link)
 {
     if (!x) return SNIP_ERR_ARG;
     const bool blk = kind == SNIP_DUAL_BLK_BLKT, sub32 = kind == SNIP_DUAL_ROW32_COL32T;
@@ -1226,6 +1256,8 @@ int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, in
         q.pow2 = pow2;
         q.seed = o[i]->seed;
         q.sf = static_cast<uint32_t *>(o[i]->sf);
+        q.tensor_amax = nullptr;
+        q.chain = link.role; q.zero = link.zero; q.zero_words = link.zero_words;
         q.tiles_r = (int32_t)tr; q.tiles_c = (int32_t)tc; q.ntiles = tr * tc;
     }
     const int64_t nparts = persistent_ctas(tr * tc, kDualCtasPerSm);
@@ -1259,17 +1291,8 @@ int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, in
     else launch_dual<SNIP_FMT_FP4_E2M1, SNIP_FMT_FP4_E2M1>(d, blk, stats, grid, st);
     SNIP_CUDA_TRY(cudaGetLastError());
     if (stats) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2);
-        cfg.blockDim = dim3(1024);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const ReduceSets sets = {{d.a.partials, d.b.partials}, {oa.stats, ob.stats}};
-        SNIP_CUDA_TRY(cudaLaunchKernelEx(&cfg, stats_reduce_kernel, sets, nparts));
+        rc = launch_reduce(ReduceSets{{d.a.partials, d.b.partials}, {oa.stats, ob.stats}}, 2, nparts, link, st);
+        if (rc) return rc;
     }
     return SNIP_OK;
 }
@@ -1277,7 +1300,7 @@ int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, in
 // Two-level option (see include/snip.h): both copies of a tensor from one read.
 int quantize_nvfp4_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, const float *tensor_amax, void *codes_a, void *sf_a,
                              snip_stats_t *stats_a, void *codes_b, void *sf_b, snip_stats_t *stats_b, int rounding, uint64_t seed, void *ws,
-                             size_t ws_bytes, cudaStream_t st)
+                             size_t ws_bytes, cudaStream_t st, const ChainLink &link)
 {
     if (rounding != SNIP_ROUND_NEAREST_EVEN && rounding != SNIP_ROUND_STOCHASTIC) return SNIP_ERR_ARG;
     const bool sr = rounding == SNIP_ROUND_STOCHASTIC;
@@ -1308,6 +1331,7 @@ int quantize_nvfp4_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t 
         q.seed = seed;
         q.sf = static_cast<uint32_t *>(sf[i]);
         q.tensor_amax = tensor_amax;
+        q.chain = link.role; q.zero = link.zero; q.zero_words = link.zero_words;
         q.tiles_r = (int32_t)tr; q.tiles_c = (int32_t)tc; q.ntiles = tr * tc;
     }
     const int64_t nparts = persistent_ctas(tr * tc, kDualCtasPerSm);
@@ -1318,17 +1342,8 @@ int quantize_nvfp4_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t 
     else launch_persistent(quantize_nvfp4_dual_kernel<false, false>, d, grid, st, kSmemBytes32);
     SNIP_CUDA_TRY(cudaGetLastError());
     if (stats) {
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(2);
-        cfg.blockDim = dim3(1024);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const ReduceSets sets = {{d.a.partials, d.b.partials}, {stats_a, stats_b}};
-        SNIP_CUDA_TRY(cudaLaunchKernelEx(&cfg, stats_reduce_kernel, sets, nparts));
+        rc = launch_reduce(ReduceSets{{d.a.partials, d.b.partials}, {stats_a, stats_b}}, 2, nparts, link, st);
+        if (rc) return rc;
     }
     return SNIP_OK;
 }
@@ -1350,7 +1365,7 @@ extern "C" int snip_quantize_nvfp4_dual(const void *x, int64_t rows, int64_t col
                                         snip_stats_t *stats_transposed, int rounding, uint64_t seed, void *ws, size_t ws_bytes, void *stream)
 {
     return snip::quantize_nvfp4_dual_impl(x, rows, cols, ld, tensor_amax, codes_stored, sf_stored, stats_stored, codes_transposed, sf_transposed,
-                                          stats_transposed, rounding, seed, ws, ws_bytes, static_cast<cudaStream_t>(stream));
+                                          stats_transposed, rounding, seed, ws, ws_bytes, static_cast<cudaStream_t>(stream), snip::ChainLink());
 }
 
 extern "C" int snip_quantize_sizes(int64_t rows, int64_t cols, int fmt, int block, uint32_t flags,
@@ -1488,7 +1503,7 @@ extern "C" int snip_quantize_dual(const void *x, int64_t rows, int64_t cols, int
     const DualOut oa = {as_stored->fmt, as_stored->codes, as_stored->scales, as_stored->sf, as_stored->stats, as_stored->rounding, as_stored->seed};
     const DualOut ob = {transposed->fmt, transposed->codes, transposed->scales, transposed->sf, transposed->stats, transposed->rounding, transposed->seed};
     return quantize_dual_impl(x, rows, cols, ld, kind, pow2_scale ? 1 : 0, oa, ob, ws, ws_bytes,
-                              static_cast<cudaStream_t>(stream));
+                              static_cast<cudaStream_t>(stream), ChainLink());
 }
 
 // ---- stochastic rounding (paper Sec. 6.1) ------------------------------------------------------

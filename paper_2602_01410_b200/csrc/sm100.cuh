@@ -21,6 +21,10 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
     return t;
 }
 
+// Programmatic dependent launch: wait until the kernels ahead have completed and their writes are visible; let the kernel behind start.
+__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
 // Move registers between warpgroups (all four warps of an aligned group must execute it).
 template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
