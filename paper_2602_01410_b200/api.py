@@ -289,7 +289,7 @@ def snip_gemm_quantized(op, a: QTensor, b: QTensor, out_shape, out_dtype=OUT_BF1
     if ws is None:
         M, N = out_shape
         g, _ = snip_workspace_size(op, *_mnk(op, a, b), a.fmt, b.fmt)
-        ws = torch.zeros(g, dtype=torch.uint8, device=out.device)
+        ws = torch.empty(g, dtype=torch.uint8, device=out.device)
     _check("snip_gemm_quantized", _lib.snip_gemm_quantized(op, ctypes.byref(a), ctypes.byref(b), _p(out), out_dtype,
                                                            int(accumulate), _p(ws), ws.numel(), _stream()))
     return out
@@ -298,7 +298,7 @@ def snip_gemm_quantized(op, a: QTensor, b: QTensor, out_shape, out_dtype=OUT_BF1
 def snip_gemm_mx(op, a: QTensor, sf_a, b: QTensor, sf_b, out_shape, out_dtype=OUT_BF16, *, out=None, ws=None, device="cuda"):
     out = _out(out_shape, out_dtype, device, out)
     if ws is None:
-        ws = torch.zeros(256, dtype=torch.uint8, device=out.device)
+        ws = torch.empty(256, dtype=torch.uint8, device=out.device)
     _check("snip_gemm_mx", _lib.snip_gemm_mx(op, ctypes.byref(a), _p(sf_a), ctypes.byref(b), _p(sf_b), _p(out), out_dtype, _p(ws),
                                              ws.numel(), _stream()))
     return out
@@ -334,7 +334,7 @@ def snip_quantize_nvfp4_dual(x: torch.Tensor, tensor_amax: torch.Tensor, *, want
 def snip_gemm_nvfp4(op, a: QTensor, sf_a, amax_a, b: QTensor, sf_b, amax_b, out_shape, out_dtype=OUT_BF16, *, out=None, ws=None, device="cuda"):
     out = _out(out_shape, out_dtype, device, out)
     if ws is None:
-        ws = torch.zeros(256, dtype=torch.uint8, device=out.device)
+        ws = torch.empty(256, dtype=torch.uint8, device=out.device)
     _check("snip_gemm_nvfp4", _lib.snip_gemm_nvfp4(op, ctypes.byref(a), _p(sf_a), _p(amax_a), ctypes.byref(b), _p(sf_b), _p(amax_b), _p(out), out_dtype,
                                                    _p(ws), ws.numel(), _stream()))
     return out
@@ -352,7 +352,7 @@ def _linear(fn_name, A, B, out_shape, M, N, K, fmt_a, fmt_b, out_dtype, op, out,
     out = _out(out_shape, out_dtype, A.device, out)
     if ws is None:
         _, l = snip_workspace_size(op, M, N, K, fmt_a, fmt_b)
-        ws = torch.zeros(l, dtype=torch.uint8, device=A.device)
+        ws = torch.empty(l, dtype=torch.uint8, device=A.device)
     sa = torch.empty(24, dtype=torch.uint8, device=A.device) if want_stats else None
     sb = torch.empty(24, dtype=torch.uint8, device=A.device) if want_stats else None
     fn = getattr(_lib, fn_name)
@@ -400,7 +400,7 @@ def snip_linear_mx(op, A, B, fmt_a, fmt_b, out_dtype=OUT_BF16, *, out=None, ws=N
         shape = (N, K)
     out = _out(shape, out_dtype, A.device, out)
     if ws is None:
-        ws = torch.zeros(snip_linear_mx_workspace(op, M, N, K, fmt_a, fmt_b), dtype=torch.uint8, device=A.device)
+        ws = torch.empty(snip_linear_mx_workspace(op, M, N, K, fmt_a, fmt_b), dtype=torch.uint8, device=A.device)
     sa = torch.empty(32, dtype=torch.uint8, device=A.device) if want_stats else None
     sb = torch.empty(32, dtype=torch.uint8, device=A.device) if want_stats else None
     _check("snip_linear_mx", _lib.snip_linear_mx(op, _p(A), _p(B), _p(out), M, N, K, fmt_a, fmt_b, out_dtype, _p(sa), _p(sb), _p(ws),
@@ -426,7 +426,7 @@ def snip_linear_fwd_bwd(x, w, dy, fmt_fwd, fmt_dgrad, fmt_wgrad, out_dtype=OUT_B
     if stats is None:
         stats = torch.zeros(6 * 24, dtype=torch.uint8, device=dev)
     if ws is None:
-        ws = torch.zeros(snip_linear_fwd_bwd_workspace(M, N, K, fmt_fwd, fmt_dgrad, fmt_wgrad, pow2_scale), dtype=torch.uint8, device=dev)
+        ws = torch.empty(snip_linear_fwd_bwd_workspace(M, N, K, fmt_fwd, fmt_dgrad, fmt_wgrad, pow2_scale), dtype=torch.uint8, device=dev)
     _check("snip_linear_fwd_bwd", _lib.snip_linear_fwd_bwd(_p(x), _p(w), _p(dy), _p(y), _p(dx), _p(dw), M, N, K, fmt_fwd, fmt_dgrad, fmt_wgrad,
                                                            out_dtype, int(pow2_scale), ROUND_NEAREST_EVEN if dy_sr_seed is None else ROUND_STOCHASTIC,
                                                            0 if dy_sr_seed is None else dy_sr_seed, _p(stats), _p(ws), ws.numel(), _stream()))
@@ -445,7 +445,7 @@ def snip_linear_fwd_bwd_nvfp4(x, w, dy, bounds3, out_dtype=OUT_BF16, *, dy_sr_se
     if ws is None:
         n = ctypes.c_size_t()
         _check("snip_linear_fwd_bwd_nvfp4_workspace", _lib.snip_linear_fwd_bwd_nvfp4_workspace(M, N, K, ctypes.byref(n)))
-        ws = torch.zeros(n.value, dtype=torch.uint8, device=dev)
+        ws = torch.empty(n.value, dtype=torch.uint8, device=dev)
     _check("snip_linear_fwd_bwd_nvfp4", _lib.snip_linear_fwd_bwd_nvfp4(_p(x), _p(w), _p(dy), _p(y), _p(dx), _p(dw), M, N, K, out_dtype, _p(bounds3),
                                                                        ROUND_NEAREST_EVEN if dy_sr_seed is None else ROUND_STOCHASTIC,
                                                                        0 if dy_sr_seed is None else dy_sr_seed, _p(stats), _p(ws), ws.numel(), _stream()))
