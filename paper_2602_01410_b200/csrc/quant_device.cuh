@@ -137,20 +137,28 @@ __device__ __forceinline__ void philox4x32_10(uint32_t c0, uint32_t c1, uint32_t
     out[0] = c0; out[1] = c1; out[2] = c2; out[3] = c3;
 }
 
-// Stochastically rounded E2M1 value of t for the 16-bit uniform u: with a = min(|t|, 6), g the grid step
-// at a (0.5 below 2, 1 below 4, else 2) and lo = floor(a/g)*g, the result is lo + g iff
-// (a - lo)/g > (u + 1/2)/2^16, else lo; the sign of t is kept.  Every operation below is exact in
-// binary32, so the decision equals the one taken in exact arithmetic.
-__device__ __forceinline__ float sr_e2m1_value(float t, uint32_t u)
+// The 16-bit uniforms of an element pair (first element low) in the form sr_e2m1_value takes: 64 (65535 - u) + 31.
+__device__ __forceinline__ void sr_addends(uint32_t u2, uint32_t &r0, uint32_t &r1)
+{
+    const uint32_t n = ~u2;
+    r0 = ((n << 6) & 0x3FFFC0u) | 31u;
+    r1 = ((n >> 10) & 0x3FFFC0u) | 31u;
+}
+
+// Stochastically rounded E2M1 value of t for the 16-bit uniform u: with a = min(|t|, 6), g the grid step at a (0.5 below 2, 1 below 4,
+// else 2) and lo = floor(a/g)*g, the result is lo + g iff (a - lo)/g > (u + 1/2)/2^16, else lo; the sign of t is kept.
+// On the bits: from 1 up, a grid point is a binary32 number whose low 22 significand bits are zero, and the rule asks whether these
+// bits of a, f, exceed 32 (2u + 1), i.e. whether f + 64 (65535 - u) + 31 (= r, see sr_addends) carries out of them: one integer addition
+// and a mask round the way the rule says, exponent included.  Below 1 the same holds for a + 1, added with upward rounding (a strict
+// comparison with a multiple of the sum's last place cannot tell f from f rounded up).  About seven operations; in floating point it
+// took sixteen and an integer conversion (quarter rate).
+__device__ __forceinline__ float sr_e2m1_value(float t, uint32_t r)
 {
     const float a = fminf(fabsf(t), 6.0f);
-    const float g = a < 2.0f ? 0.5f : (a < 4.0f ? 1.0f : 2.0f);
-    const float inv_g = a < 2.0f ? 2.0f : (a < 4.0f ? 1.0f : 0.5f);
-    const float y = a * inv_g;
-    const float k = floorf(y);
-    const float thr = (float)(2u * u + 1u) * (1.0f / 131072.0f);
-    const float v = (k + ((y - k) > thr ? 1.0f : 0.0f)) * g;
-    return copysignf(v, t);
+    float off;
+    asm("set.lt.f32.f32 %0, %1, 0f3F800000;" : "=f"(off) : "f"(a));   // 1 below 1, else 0
+    const uint32_t q = (__float_as_uint(__fadd_ru(a, off)) + r) & 0xFFC00000u;
+    return copysignf(__uint_as_float(q) - off, t);
 }
 
 }  // namespace snip

@@ -167,13 +167,13 @@ __device__ __forceinline__ uint32_t encode_pair(const float2 x, const float2 s, 
     return c;
 }
 
-// Stochastic-rounding form for FP4: u2 holds the two 16-bit uniforms of the pair (first element low).
+// Stochastic-rounding form for FP4: r0, r1 hold the pair's uniforms (sr_addends).
 // The rounded values are at hand in binary32, so the error term needs no decode.
 template <bool STATS>
-__device__ __forceinline__ uint32_t encode_pair_sr_fp4(const float2 x, const float2 s, const float2 n, uint32_t u2, float2 &se2)
+__device__ __forceinline__ uint32_t encode_pair_sr_fp4(const float2 x, const float2 s, const float2 n, uint32_t r0, uint32_t r1, float2 &se2)
 {
     const float2 t = __fmul2_rn(x, s);
-    const float2 v = make_float2(sr_e2m1_value(t.x, u2 & 0xFFFFu), sr_e2m1_value(t.y, u2 >> 16));
+    const float2 v = make_float2(sr_e2m1_value(t.x, r0), sr_e2m1_value(t.y, r1));
     if (STATS) {
         const float2 e = __ffma2_rn(v, n, x);
         se2 = __ffma2_rn(e, e, se2);
@@ -189,7 +189,7 @@ __device__ __forceinline__ void pack8(const uint32_t (&c)[4], uint32_t (&out)[2]
         out[0] = c[0] | (c[1] << 16);
         out[1] = c[2] | (c[3] << 16);
     } else {
-        out[0] = c[0] | (c[1] << 8) | (c[2] << 16) | (c[3] << 24);
+        out[0] = __byte_perm(__byte_perm(c[0], c[1], 0x0040), __byte_perm(c[2], c[3], 0x0040), 0x5410);
         out[1] = 0;
     }
 }
@@ -604,6 +604,9 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
     static_assert(!((kRow && kRow32) || (kCol && kCol32)), "one row-tiled and one column-tiled output per pass");
     static_assert(!(kRow16 && (kRow || kRow32)) && !(kCol16 && (kCol || kCol32)), "one row-tiled and one column-tiled output per pass");
     constexpr bool kBlk = (A::kQuant && A::BLOCK == SNIP_BLOCK_BLK_128x128) || (B::kQuant && B::BLOCK == SNIP_BLOCK_BLK_128x128);
+    // both copies of a weight in one format: the 128x128 blocks are the same, so are the codes (12288 x 4096 FP8 43.8 -> 38.8 us, FP4
+    // 43.1 -> 33.3 us)
+    constexpr bool kSame = A::kQuant && B::kQuant && A::FMT == B::FMT && A::BLOCK == SNIP_BLOCK_BLK_128x128 && B::BLOCK == SNIP_BLOCK_BLK_128x128 && !A::SR && !B::SR;
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & 15, ty = tid >> 4;
     const int64_t r0 = (int64_t)tl.r * kTile, c0 = (int64_t)tl.c * kTile;
@@ -696,19 +699,28 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
             // element index r * cols + c, eight consecutive columns per generator call
             const uint64_t blk = ((uint64_t)(rbase + p) * (uint64_t)qa.cols + (uint64_t)cbase) >> 3;
             if (A::SR) philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)qa.seed, (uint32_t)(qa.seed >> 32), ua);
-            if (B::SR) philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)qb.seed, (uint32_t)(qb.seed >> 32), ub);
+            if (B::SR) {
+                // both copies of a tensor usually share their seed, then also the generator's words
+                if (A::SR && qa.seed == qb.seed) { ub[0] = ua[0]; ub[1] = ua[1]; ub[2] = ua[2]; ub[3] = ua[3]; }
+                else philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)qb.seed, (uint32_t)(qb.seed >> 32), ub);
+            }
         }
         float2 px = make_float2(0.0f, 0.0f), pe = make_float2(0.0f, 0.0f);
 #pragma unroll
         for (int i = 0; i < 4; ++i) {
             const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
             if (STATS) { if (ROWSTATS) px = __ffma2_rn(x, x, px); else sx2 = __ffma2_rn(x, x, sx2); }
+            uint32_t ra0 = 0, ra1 = 0, rb0 = 0, rb1 = 0;
+            if (A::SR) sr_addends(ua[i], ra0, ra1);
+            if (B::SR) sr_addends(ub[i], rb0, rb1);
             if (A::kQuant) {
-                if (A::SR) ca[i] = encode_pair_sr_fp4<STATS>(x, scale_pair<A>(sa, p, i), ninv_pair<A>(sa, p, i), ua[i], ROWSTATS ? pe : sea2);
+                if (A::SR) ca[i] = encode_pair_sr_fp4<STATS>(x, scale_pair<A>(sa, p, i), ninv_pair<A>(sa, p, i), ra0, ra1, ROWSTATS ? pe : sea2);
                 else ca[i] = encode_pair<A::FMT, STATS>(x, scale_pair<A>(sa, p, i), ninv_pair<A>(sa, p, i), ROWSTATS ? pe : sea2);
             }
-            if (B::kQuant) {
-                if (B::SR) cb[i] = encode_pair_sr_fp4<STATS>(x, scale_pair<B>(sb, p, i), ninv_pair<B>(sb, p, i), ub[i], seb2);
+            if (kSame) {
+                cb[i] = ca[i];
+            } else if (B::kQuant) {
+                if (B::SR) cb[i] = encode_pair_sr_fp4<STATS>(x, scale_pair<B>(sb, p, i), ninv_pair<B>(sb, p, i), rb0, rb1, seb2);
                 else cb[i] = encode_pair<B::FMT, STATS>(x, scale_pair<B>(sb, p, i), ninv_pair<B>(sb, p, i), seb2);
             }
         }
@@ -734,7 +746,7 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
     if (STATS) {
         ts.x += (double)(sx2.x + sx2.y);
         if (A::kQuant) ts.ea += (double)(sea2.x + sea2.y);
-        if (B::kQuant) ts.eb += (double)(seb2.x + seb2.y);
+        if (B::kQuant) ts.eb += kSame ? (double)(sea2.x + sea2.y) : (double)(seb2.x + seb2.y);
     }
     if (ROWSTATS) {
         // per row: add the 16 lanes that share the row, lane tx == 0 writes {sum x^2, sum err^2}
