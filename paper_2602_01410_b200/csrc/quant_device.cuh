@@ -152,9 +152,12 @@ __device__ __forceinline__ void sr_addends(uint32_t u2, uint32_t &r0, uint32_t &
 // and a mask round the way the rule says, exponent included.  Below 1 the same holds for a + 1, added with upward rounding (a strict
 // comparison with a multiple of the sum's last place cannot tell f from f rounded up).  About seven operations; in floating point it
 // took sixteen and an integer conversion (quarter rate).
+// SAT = false: |t| is known to be at most 6 up to rounding (a tile scaled by its own maximum; a few units in the last place above 6
+// still round to 6, the largest addend leaves 33 units to the next grid point).
+template <bool SAT>
 __device__ __forceinline__ float sr_e2m1_value(float t, uint32_t r)
 {
-    const float a = fminf(fabsf(t), 6.0f);
+    const float a = SAT ? fminf(fabsf(t), 6.0f) : fabsf(t);
     float off;
     asm("set.lt.f32.f32 %0, %1, 0f3F800000;" : "=f"(off) : "f"(a));   // 1 below 1, else 0
     const uint32_t q = (__float_as_uint(__fadd_ru(a, off)) + r) & 0xFFC00000u;

@@ -123,15 +123,17 @@ __device__ __forceinline__ void prefetch_commit() { asm volatile("cp.async.commi
 template <int N>
 __device__ __forceinline__ void prefetch_wait() { asm volatile("cp.async.wait_group %0;" ::"n"(N) : "memory"); }
 // Compile-time description of one output of a tile pass.
-template <int FMT_, int BLOCK_, bool TRANSPOSED_, bool CODES_, bool SR_ = false>
+// SR: stochastic rounding (FP4 only), with the output's own generator (1) or with the uniforms of the pass's first output (2).
+template <int FMT_, int BLOCK_, bool TRANSPOSED_, bool CODES_, int SR_ = 0>
 struct Out {
-    static constexpr int FMT = FMT_, BLOCK = BLOCK_;
-    static constexpr bool TRANSPOSED = TRANSPOSED_, CODES = CODES_, kQuant = (FMT_ != SNIP_FMT_BF16), SR = SR_;
+    static constexpr int FMT = FMT_, BLOCK = BLOCK_, SR = SR_;
+    static constexpr bool TRANSPOSED = TRANSPOSED_, CODES = CODES_, kQuant = (FMT_ != SNIP_FMT_BF16);
+    static constexpr bool kSat = BLOCK_ == SNIP_BLOCK_ROW_1x16 || BLOCK_ == SNIP_BLOCK_COL_16x1;   // rounded tile scales: products may exceed the format
     static_assert(!SR_ || FMT_ == SNIP_FMT_FP4_E2M1, "stochastic rounding is offered for FP4 E2M1 only");
 };
 struct NoOut {
-    static constexpr int FMT = SNIP_FMT_BF16, BLOCK = SNIP_BLOCK_BLK_128x128;
-    static constexpr bool TRANSPOSED = false, CODES = false, kQuant = false, SR = false;
+    static constexpr int FMT = SNIP_FMT_BF16, BLOCK = SNIP_BLOCK_BLK_128x128, SR = 0;
+    static constexpr bool TRANSPOSED = false, CODES = false, kQuant = false, kSat = false;
 };
 
 // Per-thread running sums over the tiles of a CTA (binary64: one add per tile and sum).
@@ -169,11 +171,11 @@ __device__ __forceinline__ uint32_t encode_pair(const float2 x, const float2 s, 
 
 // Stochastic-rounding form for FP4: r0, r1 hold the pair's uniforms (sr_addends).
 // The rounded values are at hand in binary32, so the error term needs no decode.
-template <bool STATS>
+template <bool STATS, bool SAT>
 __device__ __forceinline__ uint32_t encode_pair_sr_fp4(const float2 x, const float2 s, const float2 n, uint32_t r0, uint32_t r1, float2 &se2)
 {
     const float2 t = __fmul2_rn(x, s);
-    const float2 v = make_float2(sr_e2m1_value(t.x, r0), sr_e2m1_value(t.y, r1));
+    const float2 v = make_float2(sr_e2m1_value<SAT>(t.x, r0), sr_e2m1_value<SAT>(t.y, r1));
     if (STATS) {
         const float2 e = __ffma2_rn(v, n, x);
         se2 = __ffma2_rn(e, e, se2);
@@ -699,11 +701,7 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
             // element index r * cols + c, eight consecutive columns per generator call
             const uint64_t blk = ((uint64_t)(rbase + p) * (uint64_t)qa.cols + (uint64_t)cbase) >> 3;
             if (A::SR) philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)qa.seed, (uint32_t)(qa.seed >> 32), ua);
-            if (B::SR) {
-                // both copies of a tensor usually share their seed, then also the generator's words
-                if (A::SR && qa.seed == qb.seed) { ub[0] = ua[0]; ub[1] = ua[1]; ub[2] = ua[2]; ub[3] = ua[3]; }
-                else philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)qb.seed, (uint32_t)(qb.seed >> 32), ub);
-            }
+            if (B::SR == 1) philox4x32_10((uint32_t)blk, (uint32_t)(blk >> 32), (uint32_t)qb.seed, (uint32_t)(qb.seed >> 32), ub);
         }
         float2 px = make_float2(0.0f, 0.0f), pe = make_float2(0.0f, 0.0f);
 #pragma unroll
@@ -712,15 +710,16 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
             if (STATS) { if (ROWSTATS) px = __ffma2_rn(x, x, px); else sx2 = __ffma2_rn(x, x, sx2); }
             uint32_t ra0 = 0, ra1 = 0, rb0 = 0, rb1 = 0;
             if (A::SR) sr_addends(ua[i], ra0, ra1);
-            if (B::SR) sr_addends(ub[i], rb0, rb1);
+            if (B::SR == 1) sr_addends(ub[i], rb0, rb1);
+            if (B::SR == 2) { rb0 = ra0; rb1 = ra1; }
             if (A::kQuant) {
-                if (A::SR) ca[i] = encode_pair_sr_fp4<STATS>(x, scale_pair<A>(sa, p, i), ninv_pair<A>(sa, p, i), ra0, ra1, ROWSTATS ? pe : sea2);
+                if (A::SR) ca[i] = encode_pair_sr_fp4<STATS, A::kSat>(x, scale_pair<A>(sa, p, i), ninv_pair<A>(sa, p, i), ra0, ra1, ROWSTATS ? pe : sea2);
                 else ca[i] = encode_pair<A::FMT, STATS>(x, scale_pair<A>(sa, p, i), ninv_pair<A>(sa, p, i), ROWSTATS ? pe : sea2);
             }
             if (kSame) {
                 cb[i] = ca[i];
             } else if (B::kQuant) {
-                if (B::SR) cb[i] = encode_pair_sr_fp4<STATS>(x, scale_pair<B>(sb, p, i), ninv_pair<B>(sb, p, i), rb0, rb1, seb2);
+                if (B::SR) cb[i] = encode_pair_sr_fp4<STATS, B::kSat>(x, scale_pair<B>(sb, p, i), ninv_pair<B>(sb, p, i), rb0, rb1, seb2);
                 else cb[i] = encode_pair<B::FMT, STATS>(x, scale_pair<B>(sb, p, i), ninv_pair<B>(sb, p, i), seb2);
             }
         }
@@ -811,11 +810,9 @@ __device__ __forceinline__ void finish_stats(const ThreadStats &ts, QuantShared 
 
 // Dynamic shared memory of the kernels: the tile slot, then the QuantShared scratch.
 constexpr size_t kSmemBytes = (size_t)kStageBytes + sizeof(QuantShared);
-#ifndef SNIP_DUAL_CTAS
-#define SNIP_DUAL_CTAS 3
-#endif
 constexpr int kCtasPerSm = 4;
-constexpr int kDualCtasPerSm = SNIP_DUAL_CTAS;
+constexpr int kDualCtasPerSm = 3;     // four: 13 % slower (64 registers spill), two: 3 % slower
+constexpr int kDualCtasPerSmSr = 2;   // stochastic rounding: the generator's registers are worth more than the third CTA (3-5 %)
 
 // Walk of one CTA over its tiles without divisions in the loop.
 struct TileWalk {
@@ -865,8 +862,8 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_kernel(const Qu
 struct DualArgs {
     QuantArgs a, b;
 };
-template <int FMT_A, int FMT_B, bool BLK, bool STATS, bool SR_A = false, bool SR_B = false, bool SUB32 = false>
-__global__ void __launch_bounds__(kThreads, kDualCtasPerSm) quantize_dual_kernel(const DualArgs d)
+template <int FMT_A, int FMT_B, bool BLK, bool STATS, int SR_A = 0, int SR_B = 0, bool SUB32 = false>
+__global__ void __launch_bounds__(kThreads, SR_A || SR_B ? kDualCtasPerSmSr : kDualCtasPerSm) quantize_dual_kernel(const DualArgs d)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     QuantShared &sh = *reinterpret_cast<QuantShared *>(smem + kStageBytes);
@@ -895,7 +892,7 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSm) quantize_dual_kernel
 
 // Two-level option, both copies from one read: a = 1x16 tiles as stored, b = 16x1 tiles transposed, E2M1 codes.
 template <bool STATS, bool SR = false>
-__global__ void __launch_bounds__(kThreads, kDualCtasPerSm) quantize_nvfp4_dual_kernel(const DualArgs d)
+__global__ void __launch_bounds__(kThreads, SR ? kDualCtasPerSmSr : kDualCtasPerSm) quantize_nvfp4_dual_kernel(const DualArgs d)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     QuantShared &sh = *reinterpret_cast<QuantShared *>(smem + kStageBytes);
@@ -917,7 +914,7 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSm) quantize_nvfp4_dual_
         const Tile tl = {w.r, w.c, w.nr, w.nc};
         w.next();
         using A = Out<SNIP_FMT_FP4_E2M1, SNIP_BLOCK_ROW_1x16, false, true, SR>;
-        using B = Out<SNIP_FMT_FP4_E2M1, SNIP_BLOCK_COL_16x1, true, true, SR>;
+        using B = Out<SNIP_FMT_FP4_E2M1, SNIP_BLOCK_COL_16x1, true, true, SR ? 2 : 0>;
         process_tile<A, B, STATS, false>(d.a, d.b, tl, slot, sh, s32, ts, [&] {
             if (w.valid()) prefetch_tile(d.a, w.r, w.c, smem);
             prefetch_commit();
@@ -1207,7 +1204,7 @@ int quantize_impl_full(const void *x, int64_t rows, int64_t cols, int64_t ld, in
 // One read, two outputs.  blk = false: a = 1x128 tiles as stored, b = 128x1 tiles transposed;
 // blk = true: a = 128x128 blocks as stored, b = the same blocks transposed.
 // Two-output launch with stochastic rounding on the FP4 outputs that ask for it (row/column kinds only).
-template <int FMT_A, int FMT_B, bool SR_A, bool SR_B>
+template <int FMT_A, int FMT_B, int SR_A, int SR_B>
 static void launch_dual_sr(const DualArgs &d, bool stats, dim3 grid, cudaStream_t st)
 {
     if (stats) launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, true, SR_A, SR_B>, d, grid, st);
@@ -1223,7 +1220,7 @@ static void launch_dual(const DualArgs &d, bool blk, bool stats, dim3 grid, cuda
     else launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, false>, d, grid, st);
 }
 
-template <int FMT_A, int FMT_B, bool SR_A = false, bool SR_B = false>
+template <int FMT_A, int FMT_B, int SR_A = 0, int SR_B = 0>
 static void launch_dual32(const DualArgs &d, bool stats, dim3 grid, cudaStream_t st)
 {
     if (stats) launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, true, SR_A, SR_B, true>, d, grid, st, kSmemBytes32);
@@ -1272,17 +1269,18 @@ int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, in
         q.chain = link.role; q.zero = link.zero; q.zero_words = link.zero_words;
         q.tiles_r = (int32_t)tr; q.tiles_c = (int32_t)tc; q.ntiles = tr * tc;
     }
-    const int64_t nparts = persistent_ctas(tr * tc, kDualCtasPerSm);
+    const int64_t nparts = persistent_ctas(tr * tc, oa.sr || ob.sr ? kDualCtasPerSmSr : kDualCtasPerSm);
     dim3 grid((unsigned)nparts);
     const bool a8 = oa.fmt == SNIP_FMT_FP8_E4M3, b8 = ob.fmt == SNIP_FMT_FP8_E4M3;
     constexpr int F8 = SNIP_FMT_FP8_E4M3, F4 = SNIP_FMT_FP4_E2M1;
     if (sub32 && (oa.sr || ob.sr)) {
         if ((oa.sr && a8) || (ob.sr && b8)) return SNIP_ERR_UNSUPPORTED;   // stochastic rounding is offered for FP4 codes
-        if (oa.sr && ob.sr) launch_dual32<F4, F4, true, true>(d, stats, grid, st);
-        else if (oa.sr && b8) launch_dual32<F4, F8, true, false>(d, stats, grid, st);
-        else if (oa.sr) launch_dual32<F4, F4, true, false>(d, stats, grid, st);
-        else if (a8) launch_dual32<F8, F4, false, true>(d, stats, grid, st);
-        else launch_dual32<F4, F4, false, true>(d, stats, grid, st);
+        if (oa.sr && ob.sr && oa.seed == ob.seed) launch_dual32<F4, F4, 1, 2>(d, stats, grid, st);   // one generator call serves both copies
+        else if (oa.sr && ob.sr) launch_dual32<F4, F4, 1, 1>(d, stats, grid, st);
+        else if (oa.sr && b8) launch_dual32<F4, F8, 1, 0>(d, stats, grid, st);
+        else if (oa.sr) launch_dual32<F4, F4, 1, 0>(d, stats, grid, st);
+        else if (a8) launch_dual32<F8, F4, 0, 1>(d, stats, grid, st);
+        else launch_dual32<F4, F4, 0, 1>(d, stats, grid, st);
     } else if (sub32) {
         if (a8 && b8) launch_dual32<F8, F8>(d, stats, grid, st);
         else if (a8) launch_dual32<F8, F4>(d, stats, grid, st);
@@ -1291,11 +1289,12 @@ int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, in
     } else
     if (oa.sr || ob.sr) {
         if (blk || (oa.sr && a8) || (ob.sr && b8)) return SNIP_ERR_UNSUPPORTED;   // FP4 row / column tiles only
-        if (oa.sr && ob.sr) launch_dual_sr<F4, F4, true, true>(d, stats, grid, st);
-        else if (oa.sr && b8) launch_dual_sr<F4, F8, true, false>(d, stats, grid, st);
-        else if (oa.sr) launch_dual_sr<F4, F4, true, false>(d, stats, grid, st);
-        else if (a8) launch_dual_sr<F8, F4, false, true>(d, stats, grid, st);
-        else launch_dual_sr<F4, F4, false, true>(d, stats, grid, st);
+        if (oa.sr && ob.sr && oa.seed == ob.seed) launch_dual_sr<F4, F4, 1, 2>(d, stats, grid, st);   // one generator call serves both copies
+        else if (oa.sr && ob.sr) launch_dual_sr<F4, F4, 1, 1>(d, stats, grid, st);
+        else if (oa.sr && b8) launch_dual_sr<F4, F8, 1, 0>(d, stats, grid, st);
+        else if (oa.sr) launch_dual_sr<F4, F4, 1, 0>(d, stats, grid, st);
+        else if (a8) launch_dual_sr<F8, F4, 0, 1>(d, stats, grid, st);
+        else launch_dual_sr<F4, F4, 0, 1>(d, stats, grid, st);
     } else
     if (a8 && b8) launch_dual<SNIP_FMT_FP8_E4M3, SNIP_FMT_FP8_E4M3>(d, blk, stats, grid, st);
     else if (a8) launch_dual<SNIP_FMT_FP8_E4M3, SNIP_FMT_FP4_E2M1>(d, blk, stats, grid, st);
@@ -1346,7 +1345,7 @@ int quantize_nvfp4_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t 
         q.chain = link.role; q.zero = link.zero; q.zero_words = link.zero_words;
         q.tiles_r = (int32_t)tr; q.tiles_c = (int32_t)tc; q.ntiles = tr * tc;
     }
-    const int64_t nparts = persistent_ctas(tr * tc, kDualCtasPerSm);
+    const int64_t nparts = persistent_ctas(tr * tc, sr ? kDualCtasPerSmSr : kDualCtasPerSm);
     dim3 grid((unsigned)nparts);
     if (stats && sr) launch_persistent(quantize_nvfp4_dual_kernel<true, true>, d, grid, st, kSmemBytes32);
     else if (stats) launch_persistent(quantize_nvfp4_dual_kernel<true, false>, d, grid, st, kSmemBytes32);
