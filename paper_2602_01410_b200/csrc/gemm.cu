@@ -22,6 +22,7 @@
 #include "common.cuh"
 #include "quant_device.cuh"
 #include "sm100.cuh"
+#include "work_items.cuh"
 
 namespace snip {
 
@@ -32,13 +33,11 @@ namespace {
 constexpr int BM = 128;
 constexpr int kGemmThreads = 384;  // warps 0-3: producer, MMA issuer, 2 scale loaders (wgrad) or idle; warps 4-11: epilogue
 constexpr int kNumEpiWarps = 8;
-// Slicing of the weight-gradient product's last wave (see launch_gemm)
-constexpr int kMaxSlices = 4, kMinSliceStages = 8, kMaxSlicedItems = 160;
-constexpr size_t kSliceCountersOffset = 256, kSliceCountersBytes = 8192;   // counters: [sliced tile][epilogue warp], 32 bits each
-static_assert((size_t)kMaxSlicedItems / 2 * kNumEpiWarps * 4 <= kSliceCountersBytes, "counter area");
+static_assert(kNumEpiWarps == kSliceWarps, "slice counters");
+constexpr int kMinSliceStages = 8;   // shortest contraction slice of the weight-gradient product's last wave
 constexpr int kSfCols = 32;  // tensor-memory columns holding constant scale factors (kind::mxf4)
 
-enum ScaleMode { SCALE_NONE = 0, SCALE_BLOCK_B = 1, SCALE_VEC_B = 2 };
+enum ScaleMode { SCALE_BLOCK_B = 1, SCALE_VEC_B = 2 };
 
 struct GemmArgs {
     int32_t Mo, No, Kc;        // output rows / cols, contraction length in elements
@@ -53,43 +52,18 @@ struct GemmArgs {
     uint32_t stage_tx_bytes;   // bytes the two TMA loads of one stage report to the barrier
     uint64_t wait_limit_ns;    // bound of every device-side wait
     uint32_t *status;
-    // Work items: item w < split_first is tile w over the whole contraction; the tiles from split_first on (the last,
-    // partial wave of a persistent grid) are cut into nsplit contraction slices each, item split_first + r * nsplit + j
-    // being slice j of tile split_first + r.  nsplit == 1: no slicing, num_items == number of tiles.
-    int32_t split_first, nsplit, num_items;
+    WorkSplit work;
     float *partials;           // [tail tile r][slice j][epilogue warp][column quad][row lane][4]: FP32 sums of a slice
     uint32_t *counters;        // [tail tile r][epilogue warp]: slices that have delivered their sums (zero at launch)
     int32_t chain;             // ChainRole
     StatJobs stats;            // reductions left by the quantizers ahead
 };
 
-struct WorkItem {
-    int t, ks0, ks1;       // tile, stage range of the contraction
-    int tail, slice, nsl;  // index of a sliced tile among the sliced tiles, slice, number of slices (1: whole tile)
-};
-template <bool SLICED>   // false: every item is a whole tile (known at compile time)
-__device__ __forceinline__ WorkItem work_item(const GemmArgs &g, int w, int num_kstages)
-{
-    WorkItem wi;
-    if (!SLICED || w < g.split_first) {
-        wi.t = w; wi.ks0 = 0; wi.ks1 = num_kstages; wi.tail = 0; wi.slice = 0; wi.nsl = 1;
-    } else {
-        const int i = w - g.split_first;
-        wi.tail = i / g.nsplit;
-        wi.slice = i - wi.tail * g.nsplit;
-        wi.nsl = g.nsplit;
-        wi.t = g.split_first + wi.tail;
-        wi.ks0 = (int)((int64_t)wi.slice * num_kstages / g.nsplit);
-        wi.ks1 = (int)((int64_t)(wi.slice + 1) * num_kstages / g.nsplit);
-    }
-    return wi;
-}
-
 template <MmaKind KIND, int BN, int SCALE>
 struct Cfg {
-    static constexpr int kStageElemsX = (KIND == MmaKind::F16) ? 64 : 128;   // TMA x step per stage
+    static constexpr int kStageElemsX = 128;                                 // TMA x step per stage
     static constexpr int kChunkElems = 128;                                  // scale granularity
-    static constexpr int kStageK = (KIND == MmaKind::F16) ? 64 : (KIND == MmaKind::F8F6F4 ? 128 : 256);
+    static constexpr int kStageK = KIND == MmaKind::F8F6F4 ? 128 : 256;
     static constexpr int kABytes = BM * 128;
     static constexpr int kBBytes = BN * 128;
     static constexpr int kStageBytes = kABytes + kBBytes;
@@ -119,19 +93,6 @@ struct Cfg {
     static constexpr int kTmemCols = 512;
     static_assert(kAccCols + (KIND == MmaKind::MXF4 ? kSfCols : 0) <= 512, "tensor memory budget");
 };
-
-__device__ __forceinline__ void tile_coords(int t, int num_m, int num_n, int &m_idx, int &n_idx)
-{
-    // groups of 16 row-tiles share their B panels in L2 while they are resident together
-    constexpr int kGroupM = 16;
-    const int group_size = kGroupM * num_n;
-    const int g = t / group_size;
-    const int first_m = g * kGroupM;
-    const int gm = min(num_m - first_m, kGroupM);
-    const int r = t - g * group_size;
-    m_idx = first_m + r % gm;
-    n_idx = r / gm;
-}
 
 // Reciprocal from the special-function unit (one instruction, ~1 ulp; a subnormal result is flushed to zero,
 // which only affects products of scales beyond FP32's range).
@@ -303,8 +264,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            for (int w = blockIdx.x; w < g.num_items && ok; w += gridDim.x) {
-                const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g, w, num_kstages);
+            for (int w = blockIdx.x; w < g.work.num_items && ok; w += gridDim.x) {
+                const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
                 int m_idx, n_idx;
                 tile_coords(wi.t, num_m, num_n, m_idx, n_idx);
                 for (int ks = wi.ks0; ks < wi.ks1; ++ks, ++it) {
@@ -325,8 +286,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             uint32_t it = 0, cc = 0;
             bool ok = true;
             const uint32_t sfa = tmem_base + C::kSfCol0, sfb = tmem_base + C::kSfCol0 + 16;
-            for (int w = blockIdx.x; w < g.num_items && ok; w += gridDim.x) {
-                const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g, w, num_kstages);
+            for (int w = blockIdx.x; w < g.work.num_items && ok; w += gridDim.x) {
+                const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
                 for (int ks = wi.ks0; ks < wi.ks1 && ok; ++ks, ++it) {
                     const int s = it % S;
                     const uint32_t ph = (it / S) & 1u;
@@ -334,18 +295,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     tc_fence_after_sync();
                     const uint64_t adesc = make_smem_desc_k128(smem_a0 + s * C::kABytes);
                     const uint64_t bdesc = make_smem_desc_k128(smem_b0 + s * C::kBBytes);
-                    if (KIND == MmaKind::F16) {
-                        const uint32_t a = cc & 1u;
-                        if (ks == wi.ks0) {
-                            if (!mbar_wait(tempty_bar(a), ((cc >> 1) & 1u) ^ 1u, abort_flag, g.wait_limit_ns)) { ok = false; break; }
-                            tc_fence_after_sync();
-                        }
-#pragma unroll
-                        for (int k = 0; k < 4; ++k)
-                            mma_ss<KIND, false>(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc, (ks > wi.ks0 || k > 0) ? 1u : 0u, 0, 0);
-                        tc_commit<false>(empty_bar(s));
-                        if (ks == wi.ks1 - 1) { tc_commit<false>(tfull_bar(a)); ++cc; }
-                    } else if (KIND == MmaKind::F8F6F4) {
+                    if (KIND == MmaKind::F8F6F4) {
                         const uint32_t a = cc & 1u;
                         if (!mbar_wait(tempty_bar(a), ((cc >> 1) & 1u) ^ 1u, abort_flag, g.wait_limit_ns)) { ok = false; break; }
                         tc_fence_after_sync();
@@ -389,8 +339,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const bool rows_side = (warp == 2);
         constexpr int kChunksPerStage = C::kStageK / C::kChunkElems;
         uint32_t total = 0;            // chunks of all of this CTA's work items
-        for (int w = blockIdx.x; w < g.num_items; w += gridDim.x) {
-            const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g, w, num_kstages);
+        for (int w = blockIdx.x; w < g.work.num_items; w += gridDim.x) {
+            const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
             total += (uint32_t)(min(kChunksPerStage * wi.ks1, num_chunks) - kChunksPerStage * wi.ks0);
         }
         const uint32_t ring_u32 = smem_u32(scale_ring);
@@ -400,7 +350,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const float *src0 = nullptr, *src1 = nullptr;
         int64_t stride = 0;
         auto item_sources = [&]() {
-            const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g, pw < g.num_items ? pw : (int)blockIdx.x, num_kstages);
+            const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, pw < g.work.num_items ? pw : (int)blockIdx.x, num_kstages);
             int m_idx, n_idx;
             tile_coords(wi.t, num_m, num_n, m_idx, n_idx);
             const int c0 = kChunksPerStage * wi.ks0;
@@ -484,8 +434,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const uint32_t stage_u32 = out_stage0 + e * (C::kOutSlots * 2048);   // this warp's staging tiles: 32 rows x 64 bytes each
         uint32_t cc = 0;
         bool ok = true;
-        for (int w = blockIdx.x; w < g.num_items && ok; w += gridDim.x) {
-            const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g, w, num_kstages);
+        for (int w = blockIdx.x; w < g.work.num_items && ok; w += gridDim.x) {
+            const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
             int m_idx, n_idx;
             tile_coords(wi.t, num_m, num_n, m_idx, n_idx);
             const int row0 = m_idx * BM + q * 32;
@@ -493,7 +443,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             const int col0 = n_idx * BN + h * HALF;
             const bool row_ok = row < g.Mo;
             constexpr int kChunksPerStage = C::kStageK / C::kChunkElems;
-            const int nacc = (KIND == MmaKind::F16) ? 1 : min(kChunksPerStage * wi.ks1, num_chunks) - kChunksPerStage * wi.ks0;
+            const int nacc = min(kChunksPerStage * wi.ks1, num_chunks) - kChunksPerStage * wi.ks0;
             const int blk0 = col0 >> 7;
             const int blk_last = (g.No - 1) >> 7;
 
@@ -515,17 +465,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 cp_async_commit();
             };
 
-            float2 acc[SCALE == SCALE_NONE ? 1 : HALF / 2];
-            if (SCALE != SCALE_NONE) {
+            float2 acc[HALF / 2];
 #pragma unroll
-                for (int i = 0; i < HALF / 2; ++i) acc[i] = make_float2(0.0f, 0.0f);
-                if (SCALE == SCALE_BLOCK_B) {
-                    // out-of-range rows / columns read 1.0 (their products are zero anyway)
-                    for (int i = lane; i < C::kRingFloatsPerWarp; i += 32) ring[i] = 1.0f;
-                    __syncwarp();
-                    prefetch_group(0);
-                    prefetch_group(1);
-                }
+            for (int i = 0; i < HALF / 2; ++i) acc[i] = make_float2(0.0f, 0.0f);
+            if (SCALE == SCALE_BLOCK_B) {
+                // out-of-range rows / columns read 1.0 (their products are zero anyway)
+                for (int i = lane; i < C::kRingFloatsPerWarp; i += 32) ring[i] = 1.0f;
+                __syncwarp();
+                prefetch_group(0);
+                prefetch_group(1);
             }
             // Block mode: the reciprocal factors 1/(S_a*S_b) of the four chunks of group gn, from its slot (which must
             // have landed and been made visible to the warp), into a register queue that the chunk loop shifts.
@@ -592,18 +540,16 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 };
 #pragma unroll
                 for (int gi = 0; gi < D; ++gi) load_group(gi, v[gi]);
-                if (SCALE != SCALE_NONE) {
-                    // In the shadow of the first load.  Block mode: with the last chunk of a group of four the register
-                    // queue is empty; the next group's slot (requested four chunks ago) is turned into the next four
-                    // factors and the slot of the group just finished is refilled two groups ahead.  One warp barrier
-                    // per four chunks: between the copies of all lanes and the reads of all lanes.
-                    if (SCALE == SCALE_BLOCK_B) {
-                        if ((c & 3) == 3 && c + 1 < nacc) {
-                            cp_async_wait<0>();
-                            __syncwarp();
-                            load_factors((c >> 2) + 1);
-                            prefetch_group((c >> 2) + 2);
-                        }
+                // In the shadow of the first load.  Block mode: with the last chunk of a group of four the register
+                // queue is empty; the next group's slot (requested four chunks ago) is turned into the next four
+                // factors and the slot of the group just finished is refilled two groups ahead.  One warp barrier
+                // per four chunks: between the copies of all lanes and the reads of all lanes.
+                if (SCALE == SCALE_BLOCK_B) {
+                    if ((c & 3) == 3 && c + 1 < nacc) {
+                        cp_async_wait<0>();
+                        __syncwarp();
+                        load_factors((c >> 2) + 1);
+                        prefetch_group((c >> 2) + 2);
                     }
                 }
                 // all of this warp's reads of buffer `a` are done: hand it back to the MMA warp
@@ -613,12 +559,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     if (lane == 0) mbar_arrive(tempty_bar(a));
                 };
                 auto consume_group = [&](int gi, const uint32_t (&cur)[GC]) {
-                    if (SCALE == SCALE_NONE) {
-                        float o[32];
-#pragma unroll
-                        for (int i = 0; i < 32; ++i) o[i] = __uint_as_float(cur[i]);
-                        if (row_ok) store32<OUT_F32>(g, row, col0 + 32 * gi, o);
-                    } else if (SCALE == SCALE_BLOCK_B) {
+                    if (SCALE == SCALE_BLOCK_B) {
                         const float2 ff = make_float2(f[gi], f[gi]);
 #pragma unroll
                         for (int i = 0; i < GC / 2; ++i)
@@ -666,7 +607,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     if (lane == 0) mbar_arrive(vempty_bar(vd / C::kVecBlock));
                 }
             }
-            if (SCALE != SCALE_NONE) {
+            {
                 cp_async_wait<0>();
                 if (ok) {
                     if (C::kTmaOut && !g.accumulate) {
@@ -771,29 +712,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
 }
 
-// Simple bf16 transpose (used only for BF16-tagged dgrad / wgrad operands).
-__global__ void transpose_bf16_kernel(const uint16_t *__restrict__ in, uint16_t *__restrict__ out, int64_t rows, int64_t cols)
-{
-    __shared__ uint16_t tile[64][66];
-    const int64_t r0 = (int64_t)blockIdx.y * 64, c0 = (int64_t)blockIdx.x * 64;
-    for (int i = threadIdx.y; i < 64; i += blockDim.y) {
-        const int64_t r = r0 + i, c = c0 + threadIdx.x * 2;
-        if (r < rows && c < cols) {
-            const uint32_t v = *reinterpret_cast<const uint32_t *>(in + r * cols + c);
-            tile[i][threadIdx.x * 2] = (uint16_t)(v & 0xFFFFu);
-            tile[i][threadIdx.x * 2 + 1] = (uint16_t)(v >> 16);
-        }
-    }
-    __syncthreads();
-    for (int i = threadIdx.y; i < 64; i += blockDim.y) {
-        const int64_t c = c0 + i, r = r0 + threadIdx.x * 2;
-        if (c < cols && r < rows) {
-            const uint32_t v = (uint32_t)tile[threadIdx.x * 2][i] | ((uint32_t)tile[threadIdx.x * 2 + 1][i] << 16);
-            *reinterpret_cast<uint32_t *>(out + c * rows + r) = v;
-        }
-    }
-}
-
 // ---- host side ---------------------------------------------------------------------------
 
 typedef CUresult (*EncodeTiledFn)(CUtensorMap *, CUtensorMapDataType, cuuint32_t, void *, const cuuint64_t *, const cuuint64_t *,
@@ -852,21 +770,10 @@ int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
     const int num_tiles = (int)(ceil_div(g.Mo, BM) * ceil_div(g.No, BN));
     const int sms = sm_count();
     GemmArgs ga = g;
-    ga.split_first = num_tiles; ga.nsplit = 1; ga.num_items = num_tiles;
-    if (SCALE == SCALE_VEC_B && g.partials && sms > 0) {
-        // The tiles of the last, partial wave (all tiles, if there are fewer than SMs) are cut along the contraction into as
-        // many slices as there are SMs to take them: at most kMaxSlices, none shorter than kMinSliceStages stages.
-        const int full = (num_tiles / sms) * sms, rest = num_tiles - full;
-        const int num_kstages = (int)ceil_div(g.Kc, C::kStageK);
-        int ns = rest > 0 ? sms / rest : 1;
-        if (ns > kMaxSlices) ns = kMaxSlices;
-        while (ns > 1 && (num_kstages / ns < kMinSliceStages || rest * ns > kMaxSlicedItems)) --ns;
-        if (ns > 1) {
-            ga.split_first = full; ga.nsplit = ns; ga.num_items = full + rest * ns;
-            if (!cleared) SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)rest * kNumEpiWarps * sizeof(uint32_t), st));
-        }
-    }
-    const int grid = ga.num_items < sms ? ga.num_items : sms;
+    ga.work = plan_work(num_tiles, (int)ceil_div(g.Kc, C::kStageK), sms, kMinSliceStages, SCALE == SCALE_VEC_B && g.partials);
+    if (ga.work.nsplit > 1 && !cleared)
+        SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * sizeof(uint32_t), st));
+    const int grid = ga.work.num_items < sms ? ga.work.num_items : sms;
     return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, tmA, tmB, tmO, ga, idesc);
 }
 
@@ -888,6 +795,7 @@ size_t gemm_ws_bytes() { return 256; }
 // status word, arrival counters, one FP32 tile per slice.
 size_t gemm_ws_bytes_sliced() { return kSliceCountersOffset + kSliceCountersBytes + (size_t)kMaxSlicedItems * BM * 256 * sizeof(float); }
 
+// (gemm_bf16.cu slices the same way.)
 // The parts of a workspace of gemm_ws_bytes() or gemm_ws_bytes_sliced(), for one GEMM.
 GemmWs gemm_ws(void *ws, size_t ws_bytes)
 {
@@ -917,11 +825,15 @@ void gemm_debug_hooks(uint64_t *wait_limit_ns, int *tx_skew)
     *tx_skew = g_tx_skew.load();
 }
 
+bool gemm_slicing_enabled() { return g_slicing.load() != 0; }
+
 int gemm_pair_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, int64_t Mo, int64_t No, int64_t Kc, const float *sa,
                    int64_t sa_chunk_stride, const float *sb, int64_t sb_chunk_stride, int64_t sb_blk_stride, int scale_mode, void *out,
                    int out_dtype, int accumulate, uint32_t *status, uint64_t wait_limit_ns, int tx_skew, cudaStream_t st);
 
 int launch_stat_jobs(const StatJobs &jobs, cudaStream_t st);   // quantize.cu
+int gemm_bf16_impl(const void *a, bool a_mn, const void *b, bool b_mn, int64_t Mo, int64_t No, int64_t Kc, void *out, int out_dtype, int accumulate,
+                   const GemmWs &w, cudaStream_t st, const ChainLink &link);   // gemm_bf16.cu
 
 // Zeroes the status word of a GEMM workspace (enqueued; allocates nothing).
 int gemm_clear_status(void *ws, cudaStream_t st)
@@ -939,19 +851,12 @@ int make_tiled_map_2d(CUtensorMap *map, const void *ptr, int dtype, int64_t rows
 }
 int gemm_sm_count() { return sm_count(); }
 
-int transpose_bf16(const void *in, void *out, int64_t rows, int64_t cols, cudaStream_t st)
-{
-    dim3 grid((unsigned)ceil_div(cols, 64), (unsigned)ceil_div(rows, 64)), block(32, 8);
-    transpose_bf16_kernel<<<grid, block, 0, st>>>(static_cast<const uint16_t *>(in), static_cast<uint16_t *>(out), rows, cols);
-    SNIP_CUDA_TRY(cudaGetLastError());
-    return SNIP_OK;
-}
-
 // Core GEMM over stored operands.  a_codes: [Mo][Kc] and b_codes: [No][Kc], contraction-major.
-// scale_mode: SCALE_NONE for BF16, SCALE_BLOCK_B (fwd / dgrad), SCALE_VEC_B (wgrad).
+// scale_mode: SCALE_BLOCK_B (fwd / dgrad) or SCALE_VEC_B (wgrad); unused for BF16.  mn: BF16 operands stored [Kc][lines] instead (bit 0: A,
+// bit 1: B).
 int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, int64_t Mo, int64_t No, int64_t Kc, const float *sa,
               int64_t sa_chunk_stride, const float *sb, int64_t sb_chunk_stride, int64_t sb_blk_stride, int scale_mode, void *out,
-              int out_dtype, int accumulate, const GemmWs &w, cudaStream_t st, const ChainLink &link)
+              int out_dtype, int accumulate, const GemmWs &w, cudaStream_t st, const ChainLink &link, int mn)
 {
     if (!a_codes || !b_codes || !out) return SNIP_ERR_ARG;
     if (!valid_dim(Mo) || !valid_dim(No) || !valid_dim(Kc) || Mo > INT32_MAX || No > INT32_MAX || Kc > INT32_MAX) return SNIP_ERR_SHAPE;
@@ -968,6 +873,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // The status word starts at zero for this call unless the caller runs several GEMMs against one word
     // and has cleared it itself (an earlier GEMM's timeout must survive the later ones).
     if (!w.cleared) { rc = gemm_clear_status(w.status, st); if (rc) return rc; }
+    if (a16) return gemm_bf16_impl(a_codes, mn & 1, b_codes, mn & 2, Mo, No, Kc, out, out_dtype, accumulate, w, st, link);
 
     GemmArgs g;
     g.Mo = (int32_t)Mo; g.No = (int32_t)No; g.Kc = (int32_t)Kc;
@@ -977,9 +883,8 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     g.status = w.status;
     g.chain = link.role;
     if (link.jobs) g.stats = *link.jobs;
-    g.split_first = 0; g.nsplit = 1; g.num_items = 0;   // set per launch
     g.partials = nullptr; g.counters = nullptr;
-    if (!a16 && scale_mode == SCALE_VEC_B && w.partials && g_slicing.load()) {
+    if (scale_mode == SCALE_VEC_B && w.partials && g_slicing.load()) {
         g.counters = w.counters;
         g.partials = w.partials;
     }
@@ -991,7 +896,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // The CTA-pair kernels (gemm_pair.cu) are an alternative form of the same product, kept for comparison: they
     // run only when asked for through snip_debug_set (on the 7B shapes they are slower than the kernels below).
     const int choice = g_kernel_choice.load();
-    if (!a16 && choice == 2) {
+    if (choice == 2) {
         rc = launch_stat_jobs(g.stats, st);   // these kernels do not reduce statistics
         if (rc) return rc;
         return gemm_pair_impl(fmt_a, fmt_b, a_codes, b_codes, Mo, No, Kc, sa, sa_chunk_stride, sb, sb_chunk_stride, sb_blk_stride, scale_mode,
@@ -1003,16 +908,6 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     rc = f32 ? make_operand_map(&tmO, out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, Mo, No, No * 4, 16, 32, CU_TENSOR_MAP_SWIZZLE_64B)
              : make_operand_map(&tmO, out, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Mo, No, No * 2, 32, 32, CU_TENSOR_MAP_SWIZZLE_64B);
     if (rc) return rc;
-    if (a16) {
-        rc = make_operand_map(&tmA, a_codes, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, Mo, Kc, Kc * 2, 64, BM);
-        if (rc) return rc;
-        rc = make_operand_map(&tmB, b_codes, CU_TENSOR_MAP_DATA_TYPE_BFLOAT16, No, Kc, Kc * 2, 64, 256);
-        if (rc) return rc;
-        const uint32_t idesc = make_idesc(1, 1, BM, 256);
-        g.stage_tx_bytes = (BM + 256) * 128 + tx_skew;
-        return f32 ? launch_gemm<MmaKind::F16, 256, SCALE_NONE, true>(tmA, tmB, tmO, g, idesc, w.cleared, st)
-                   : launch_gemm<MmaKind::F16, 256, SCALE_NONE, false>(tmA, tmB, tmO, g, idesc, w.cleared, st);
-    }
     if (fmt_a == SNIP_FMT_FP4_E2M1 && fmt_b == SNIP_FMT_FP4_E2M1 && (scale_mode == SCALE_BLOCK_B || (Kc % 128) != 0)) {
         // Packed FP4 on both sides, forward / input gradient, or a contraction length ending in a 64-wide tile: kind::mxf4 on the
         // packed bytes (fetched as plain u8, exact extents).  Its 128x192 tile (what tensor memory allows next to the scale
@@ -1085,10 +980,9 @@ extern "C" int snip_gemm_quantized(int op, const snip_qtensor_t *a, const snip_q
         Mo = a->cols; No = b->cols; Kc = a->rows;
         sa_cs = Mo; sb_cs = No; sb_bs = 0; mode = SCALE_VEC_B;
     }
-    if (!q) mode = SCALE_NONE;
     if (!ws || ws_bytes < gemm_ws_bytes()) return SNIP_ERR_WORKSPACE;
     return gemm_impl(a->fmt, b->fmt, a->codes, b->codes, Mo, No, Kc, sa, sa_cs, sb, sb_cs, sb_bs, mode, out, out_dtype, accumulate,
-                     gemm_ws(ws, ws_bytes), static_cast<cudaStream_t>(stream), ChainLink());
+                     gemm_ws(ws, ws_bytes), static_cast<cudaStream_t>(stream), ChainLink(), 0);
 }
 
 extern "C" int snip_debug_set(int key, long long value)

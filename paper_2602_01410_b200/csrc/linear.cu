@@ -5,11 +5,9 @@
 
 namespace snip {
 
-int quantize_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags, void *codes,
-                  float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st);
 int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, int64_t Mo, int64_t No, int64_t Kc, const float *sa,
               int64_t sa_chunk_stride, const float *sb, int64_t sb_chunk_stride, int64_t sb_blk_stride, int scale_mode, void *out,
-              int out_dtype, int accumulate, const GemmWs &w, cudaStream_t st, const ChainLink &link);
+              int out_dtype, int accumulate, const GemmWs &w, cudaStream_t st, const ChainLink &link, int mn);
 GemmWs gemm_ws(void *ws, size_t ws_bytes);
 int32_t gemm_ws_zero_words();
 int quantize_impl_ex(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags, int pow2, void *sf,
@@ -17,7 +15,6 @@ int quantize_impl_ex(const void *x, int64_t rows, int64_t cols, int64_t ld, int 
                      const ChainLink &link);
 int gemm_mx_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, const void *sfa, const void *sfb, int64_t Mo, int64_t No,
                  int64_t Kc, void *out, int out_dtype, const GemmWs &w, cudaStream_t st, const ChainLink &link);
-int transpose_bf16(const void *in, void *out, int64_t rows, int64_t cols, cudaStream_t st);
 size_t gemm_ws_bytes();
 size_t gemm_ws_bytes_sliced();   // with room for the weight-gradient product's contraction slices
 int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int kind, int pow2, const DualOut &oa, const DualOut &ob,
@@ -30,13 +27,12 @@ int gemm_nvfp4_impl(const void *a_codes, const void *b_codes, const void *sfa, c
 
 namespace {
 
-enum { SCALE_NONE = 0, SCALE_BLOCK_B = 1, SCALE_VEC_B = 2 };
+enum { SCALE_BLOCK_B = 1, SCALE_VEC_B = 2 };
 
 size_t code_bytes(int fmt, int64_t rows, int64_t cols)
 {
     if (fmt == SNIP_FMT_FP8_E4M3) return (size_t)(rows * cols);
-    if (fmt == SNIP_FMT_FP4_E2M1) return (size_t)(rows * cols / 2) + 64;  // + tail slack, see snip_quantize_sizes
-    return (size_t)(rows * cols * 2);  // bf16 transposed copy
+    return (size_t)(rows * cols / 2) + 64;  // FP4: + tail slack, see snip_quantize_sizes
 }
 size_t scale_bytes(int block, int64_t rows, int64_t cols)
 {
@@ -95,7 +91,7 @@ size_t linear_ws_bytes(int op, int64_t M, int64_t N, int64_t K, int fmt_a, int f
     const LinearPlan p = plan_for(op, M, N, K);
     Carve c(nullptr, 0);
     c.take(gemm_ws_bytes_sliced());
-    const bool need_a = fmt_a != SNIP_FMT_BF16 || p.tr_a, need_b = fmt_b != SNIP_FMT_BF16 || p.tr_b;
+    const bool need_a = fmt_a != SNIP_FMT_BF16, need_b = fmt_b != SNIP_FMT_BF16;   // BF16 operands are read in place
     if (need_a) { c.take(code_bytes(fmt_a, p.rows_a, p.cols_a)); c.take(scale_bytes(p.block_a, p.rows_a, p.cols_a)); }
     if (need_b) { c.take(code_bytes(fmt_b, p.rows_b, p.cols_b)); c.take(scale_bytes(p.block_b, p.rows_b, p.cols_b)); }
     c.take(stats_bytes(p.rows_a, p.cols_a));
@@ -118,11 +114,10 @@ int linear_impl(int op, const void *A, const void *B, void *out, int64_t M, int6
     Carve c(ws, ws_bytes);
     void *gws = c.take(gemm_ws_bytes_sliced());
     const bool q = fmt_a != SNIP_FMT_BF16;
-    const bool need_a = q || p.tr_a, need_b = q || p.tr_b;
     void *codes_a = nullptr, *codes_b = nullptr;
     float *scales_a = nullptr, *scales_b = nullptr;
-    if (need_a) { codes_a = c.take(code_bytes(fmt_a, p.rows_a, p.cols_a)); scales_a = static_cast<float *>(c.take(scale_bytes(p.block_a, p.rows_a, p.cols_a))); }
-    if (need_b) { codes_b = c.take(code_bytes(fmt_b, p.rows_b, p.cols_b)); scales_b = static_cast<float *>(c.take(scale_bytes(p.block_b, p.rows_b, p.cols_b))); }
+    if (q) { codes_a = c.take(code_bytes(fmt_a, p.rows_a, p.cols_a)); scales_a = static_cast<float *>(c.take(scale_bytes(p.block_a, p.rows_a, p.cols_a))); }
+    if (q) { codes_b = c.take(code_bytes(fmt_b, p.rows_b, p.cols_b)); scales_b = static_cast<float *>(c.take(scale_bytes(p.block_b, p.rows_b, p.cols_b))); }
     const size_t sws_a_bytes = stats_bytes(p.rows_a, p.cols_a), sws_b_bytes = stats_bytes(p.rows_b, p.cols_b);
     void *sws_a = c.take(sws_a_bytes), *sws_b = c.take(sws_b_bytes);
     void *sf_a = nullptr, *sf_b = nullptr;
@@ -148,18 +143,30 @@ int linear_impl(int op, const void *A, const void *B, void *out, int64_t M, int6
         ga = codes_a; gb = codes_b;
         if (mx) return gemm_mx_impl(fmt_a, fmt_b, ga, gb, sf_a, sf_b, p.Mo, p.No, p.Kc, out, out_dtype, gw, st, after);
     } else {
-        // BF16 tag: identity quantization; only operands whose contraction index is not contiguous are copied
-        if (p.tr_a) { rc = transpose_bf16(A, codes_a, p.rows_a, p.cols_a, st); if (rc) return rc; ga = codes_a; }
-        if (p.tr_b) { rc = transpose_bf16(B, codes_b, p.rows_b, p.cols_b, st); if (rc) return rc; gb = codes_b; }
-        if (stats_a) { rc = quantize_impl(A, p.rows_a, p.cols_a, p.cols_a, SNIP_FMT_BF16, SNIP_BLOCK_BLK_128x128, SNIP_Q_STATS, nullptr, nullptr, stats_a, nullptr, sws_a, sws_a_bytes, st); if (rc) return rc; }
-        if (stats_b) { rc = quantize_impl(B, p.rows_b, p.cols_b, p.cols_b, SNIP_FMT_BF16, SNIP_BLOCK_BLK_128x128, SNIP_Q_STATS, nullptr, nullptr, stats_b, nullptr, sws_b, sws_b_bytes, st); if (rc) return rc; }
+        // BF16 tag: identity quantization; both operands are read as they lie, in the operand order their contraction calls for
+        const ChainLink *next = &first;
+        if (stats_a) {
+            rc = quantize_impl_ex(A, p.rows_a, p.cols_a, p.cols_a, SNIP_FMT_BF16, SNIP_BLOCK_BLK_128x128, SNIP_Q_STATS, 0, nullptr, nullptr, nullptr, stats_a, nullptr,
+                                  sws_a, sws_a_bytes, st, *next);
+            if (rc) return rc;
+            next = &beside;
+        }
+        if (stats_b) {
+            rc = quantize_impl_ex(B, p.rows_b, p.cols_b, p.cols_b, SNIP_FMT_BF16, SNIP_BLOCK_BLK_128x128, SNIP_Q_STATS, 0, nullptr, nullptr, nullptr, stats_b, nullptr,
+                                  sws_b, sws_b_bytes, st, *next);
+            if (rc) return rc;
+            next = &beside;
+        }
+        gw.cleared = next != &first;
+        return gemm_impl(fmt_a, fmt_b, A, B, p.Mo, p.No, p.Kc, nullptr, 0, nullptr, 0, 0, 0, out, out_dtype, accumulate, gw, st,
+                         gw.cleared ? after : ChainLink(), (p.tr_a ? 1 : 0) | (p.tr_b ? 2 : 0));
     }
     int64_t sa_cs = p.Mo, sb_cs, sb_bs;
     if (op == SNIP_OP_FWD) { sb_bs = ceil_div(K, 128); sb_cs = 1; }
     else if (op == SNIP_OP_DGRAD) { sb_bs = 1; sb_cs = ceil_div(K, 128); }
     else { sb_bs = 0; sb_cs = p.No; }
-    return gemm_impl(fmt_a, fmt_b, ga, gb, p.Mo, p.No, p.Kc, scales_a, sa_cs, scales_b, sb_cs, sb_bs, q ? p.scale_mode : SCALE_NONE, out,
-                     out_dtype, accumulate, gw, st, q ? after : ChainLink());
+    return gemm_impl(fmt_a, fmt_b, ga, gb, p.Mo, p.No, p.Kc, scales_a, sa_cs, scales_b, sb_cs, sb_bs, p.scale_mode, out,
+                     out_dtype, accumulate, gw, st, after, 0);
 }
 
 
@@ -319,7 +326,7 @@ extern "C" int snip_linear_fwd_bwd(const void *X, const void *W, const void *dY,
         else if (op == SNIP_OP_DGRAD) { sb_bs = 1; sb_cs = ceil_div(K, 128); }
         else { sb_bs = 0; sb_cs = p.No; }
         return gemm_impl(fmt[ia], fmt[ib], f.codes[ia], f.codes[ib], p.Mo, p.No, p.Kc, f.scales[ia], p.Mo, f.scales[ib], sb_cs, sb_bs, p.scale_mode, out,
-                         out_dtype, 0, gw, st, link);
+                         out_dtype, 0, gw, st, link, 0);
     };
     rc = quantize_dual_impl(X, M, K, K, kind_xdy, mx, out_of(0), out_of(1), f.stats_ws[0], f.stats_ws_bytes[0], st, quant[0]);
     if (rc) return rc;

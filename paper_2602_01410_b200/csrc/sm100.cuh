@@ -342,6 +342,20 @@ __device__ __forceinline__ uint64_t make_smem_desc_k128(uint32_t smem_addr)
     return d;
 }
 
+// Shared-memory matrix descriptor for an MN-major 16-bit operand tile: boxes of 64 lines (128 bytes, contiguous) x contraction rows,
+// 128-byte swizzle, rows 128 B apart (so 8 rows of the contraction are 1024 B), boxes box_bytes apart along the lines.  Base
+// 1024-byte aligned; 16 rows of the contraction are a step of 2048 bytes.
+__device__ __forceinline__ uint64_t make_smem_desc_mn128(uint32_t smem_addr, uint32_t box_bytes)
+{
+    uint64_t d = 0;
+    d |= (uint64_t)((smem_addr & 0x3FFFFu) >> 4);
+    d |= (uint64_t)(box_bytes >> 4) << 16;           // leading byte offset: to the next 64 lines
+    d |= (uint64_t)(1024 >> 4) << 32;                // stride byte offset: to the next 8 rows of the contraction
+    d |= (uint64_t)1 << 46;
+    d |= (uint64_t)2 << 61;
+    return d;
+}
+
 // Instruction descriptor for kind::f16 / kind::f8f6f4, FP32 accumulate, K-major A and B.
 //   a_fmt / b_fmt: kind::f16: 0 = f16, 1 = bf16;  kind::f8f6f4: 0 = e4m3, 1 = e5m2, 5 = e2m1
 __host__ __device__ constexpr uint32_t make_idesc(uint32_t a_fmt, uint32_t b_fmt, uint32_t M, uint32_t N)
