@@ -83,18 +83,26 @@ int require_sm100();
 // Launch with (pdl) or without the attribute that lets the kernel start beside the one ahead of it (griddepcontrol in the kernel
 // decides what waits).
 template <typename... KArgs, typename... Args>
-int launch_chained(void (*kern)(KArgs...), int grid, int threads, size_t smem_bytes, cudaStream_t st, bool pdl, const Args &...args)
+int launch_chained(void (*kern)(KArgs...), int grid, int threads, size_t smem_bytes, cudaStream_t st, bool pdl, int cluster, const Args &...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
     cfg.blockDim = dim3((unsigned)threads);
     cfg.dynamicSmemBytes = smem_bytes;
     cfg.stream = st;
-    cudaLaunchAttribute attr[1];
-    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = pdl ? 1 : 0;
+    cfg.numAttrs = 0;
+    if (pdl) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
+    }
+    if (cluster > 1) {
+        attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
+        attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;
+        attr[cfg.numAttrs].val.clusterDim.y = 1;
+        attr[cfg.numAttrs++].val.clusterDim.z = 1;
+    }
     SNIP_CUDA_TRY(cudaLaunchKernelEx(&cfg, kern, args...));
     return SNIP_OK;
 }

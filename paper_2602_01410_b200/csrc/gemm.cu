@@ -774,7 +774,7 @@ int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
     if (ga.work.nsplit > 1 && !cleared)
         SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * sizeof(uint32_t), st));
     const int grid = ga.work.num_items < sms ? ga.work.num_items : sms;
-    return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, tmA, tmB, tmO, ga, idesc);
+    return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, 1, tmA, tmB, tmO, ga, idesc);
 }
 
 template <MmaKind KIND, int BN>

@@ -323,7 +323,7 @@ int launch_mx(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap 
     SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
     const int num_tiles = (int)(ceil_div(g.Mo, BM) * ceil_div(g.No, BN));
     const int grid = num_tiles < sms ? num_tiles : sms;
-    return launch_chained(kern, grid, kThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, tmA, tmB, tmO, g, idesc);
+    return launch_chained(kern, grid, kThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, 1, tmA, tmB, tmO, g, idesc);
 }
 
 }  // namespace

@@ -20,14 +20,14 @@ struct WorkSplit {
 
 // The tiles of the last, partial wave (all tiles, if there are fewer than SMs) are cut along the contraction into as many slices as
 // there are SMs to take them: at most kMaxSlices, none shorter than min_stages pipeline stages.
-inline WorkSplit plan_work(int num_tiles, int num_stages, int sms, int min_stages, bool slice)
+inline WorkSplit plan_work(int num_tiles, int num_stages, int sms, int min_stages, bool slice, int max_items = kMaxSlicedItems)
 {
     WorkSplit s = {num_tiles, 1, num_tiles};
     if (!slice || sms <= 0) return s;
     const int full = (num_tiles / sms) * sms, rest = num_tiles - full;
     int ns = rest > 0 ? sms / rest : 1;
     if (ns > kMaxSlices) ns = kMaxSlices;
-    while (ns > 1 && (num_stages / ns < min_stages || rest * ns > kMaxSlicedItems)) --ns;
+    while (ns > 1 && (num_stages / ns < min_stages || rest * ns > max_items)) --ns;
     if (ns > 1) { s.split_first = full; s.nsplit = ns; s.num_items = full + rest * ns; }
     return s;
 }
