@@ -290,8 +290,8 @@ int snip_workspace_size(int op, int64_t M, int64_t N, int64_t K, int fmt_a, int 
  * only).  Operand formats: (BF16,BF16), (FP8,FP8), (FP4,FP4), (FP8,FP4), (FP4,FP8); pairs
  * that mix BF16 with a quantized operand return SNIP_ERR_UNSUPPORTED.
  * ws must hold at least 256 bytes (gemm_bytes of snip_workspace_size to allow slicing, see there);
- * its first word is the device status word read by snip_poll_status.  The call itself zeroes that word on the stream before the
- * kernel starts (a 4-byte memset node), so the workspace needs no initialisation by the caller.
+ * its first word is the device status word read by snip_poll_status.  The kernel itself clears that word when it starts, so the
+ * workspace needs no initialisation by the caller.
  */
 int snip_gemm_quantized(int op, const snip_qtensor_t *a_host, const snip_qtensor_t *b_host,
                         void *out, int out_dtype, int accumulate, void *ws, size_t ws_bytes,

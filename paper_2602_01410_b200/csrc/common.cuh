@@ -66,8 +66,11 @@ struct GemmWs {
     uint32_t *status = nullptr;
     uint32_t *counters = nullptr;
     float *partials = nullptr;
-    bool cleared = false;
+    bool cleared = false;   // false: the kernel clears the status word itself (status_begin)
 };
+
+// Non-zero mark of a launch that clears its status word itself; 0 where the word has been cleared.
+uint32_t status_mark(bool cleared);
 
 // What a chain passes along: the first quantizer clears `zero_words` words at `zero` (GEMM status word and slice counters).
 struct ChainLink {
@@ -80,10 +83,10 @@ struct ChainLink {
 // Fails with SNIP_ERR_UNSUPPORTED unless the current device is compute capability 10.x.
 int require_sm100();
 
-// Launch with (pdl) or without the attribute that lets the kernel start beside the one ahead of it (griddepcontrol in the kernel
-// decides what waits).
+// Launch of a GEMM with the attribute that lets it start beside the kernel ahead of it (griddepcontrol in the kernel decides what
+// waits: on its own, everything but the prologue).
 template <typename... KArgs, typename... Args>
-int launch_chained(void (*kern)(KArgs...), int grid, int threads, size_t smem_bytes, cudaStream_t st, bool pdl, int cluster, const Args &...args)
+int launch_chained(void (*kern)(KArgs...), int grid, int threads, size_t smem_bytes, cudaStream_t st, int cluster, const Args &...args)
 {
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)grid);
@@ -92,11 +95,9 @@ int launch_chained(void (*kern)(KArgs...), int grid, int threads, size_t smem_by
     cfg.stream = st;
     cudaLaunchAttribute attr[2];
     cfg.attrs = attr;
-    cfg.numAttrs = 0;
-    if (pdl) {
-        attr[cfg.numAttrs].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[cfg.numAttrs++].val.programmaticStreamSerializationAllowed = 1;
-    }
+    cfg.numAttrs = 1;
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
     if (cluster > 1) {
         attr[cfg.numAttrs].id = cudaLaunchAttributeClusterDimension;
         attr[cfg.numAttrs].val.clusterDim.x = (unsigned)cluster;

@@ -52,6 +52,7 @@ struct GemmArgs {
     uint32_t stage_tx_bytes;   // bytes the two TMA loads of one stage report to the barrier
     uint64_t wait_limit_ns;    // bound of every device-side wait
     uint32_t *status;
+    uint32_t status_mark;      // see status_begin
     WorkSplit work;
     float *partials;           // [tail tile r][slice j][epilogue warp][column quad][row lane][4]: FP32 sums of a slice
     uint32_t *counters;        // [tail tile r][epilogue warp]: slices that have delivered their sums (zero at launch)
@@ -244,6 +245,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // everything up to here touches nothing that a kernel ahead on the stream writes
     if (g.chain != CHAIN_BESIDE) pdl_wait();
     pdl_launch_dependents();
+    status_begin(g.status, g.status_mark);
 
     if (KIND == MmaKind::MXF4) {
         // constant scale factors 2^0 (UE8M0 byte 127) for every row of A and B
@@ -703,7 +705,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         // give copies and MMAs still in flight time to land before the CTA's resources go away
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
-        if (threadIdx.x == 0) atomicExch(g.status, (uint32_t)SNIP_ERR_TIMEOUT);
+        if (threadIdx.x == 0) status_report(g.status, g.status_mark, (uint32_t)SNIP_ERR_TIMEOUT, g.wait_limit_ns);
         __syncthreads();
     }
     if (warp == 1) {
@@ -774,7 +776,7 @@ int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
     if (ga.work.nsplit > 1 && !cleared)
         SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * sizeof(uint32_t), st));
     const int grid = ga.work.num_items < sms ? ga.work.num_items : sms;
-    return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, 1, tmA, tmB, tmO, ga, idesc);
+    return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, 1, tmA, tmB, tmO, ga, idesc);
 }
 
 template <MmaKind KIND, int BN>
@@ -835,11 +837,12 @@ int launch_stat_jobs(const StatJobs &jobs, cudaStream_t st);   // quantize.cu
 int gemm_bf16_impl(const void *a, bool a_mn, const void *b, bool b_mn, int64_t Mo, int64_t No, int64_t Kc, void *out, int out_dtype, int accumulate,
                    const GemmWs &w, cudaStream_t st, const ChainLink &link);   // gemm_bf16.cu
 
-// Zeroes the status word of a GEMM workspace (enqueued; allocates nothing).
-int gemm_clear_status(void *ws, cudaStream_t st)
+uint32_t status_mark(bool cleared)
 {
-    SNIP_CUDA_TRY(cudaMemsetAsync(ws, 0, sizeof(uint32_t), st));
-    return SNIP_OK;
+    static std::atomic<uint32_t> next{1};
+    if (cleared) return 0;
+    const uint32_t m = next.fetch_add(1);
+    return m ? m : next.fetch_add(1);
 }
 
 // Shared with the power-of-two-scale GEMMs: 2-D tiled tensor map over a row-major matrix.
@@ -870,9 +873,6 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     if (!a16 && (!aligned16(sa) || !aligned16(sb))) return SNIP_ERR_ALIGN;   // scale factors are fetched 16 bytes at a time
     int rc = require_sm100();
     if (rc != SNIP_OK) return rc;
-    // The status word starts at zero for this call unless the caller runs several GEMMs against one word
-    // and has cleared it itself (an earlier GEMM's timeout must survive the later ones).
-    if (!w.cleared) { rc = gemm_clear_status(w.status, st); if (rc) return rc; }
     if (a16) return gemm_bf16_impl(a_codes, mn & 1, b_codes, mn & 2, Mo, No, Kc, out, out_dtype, accumulate, w, st, link);
 
     GemmArgs g;
@@ -881,6 +881,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     g.sb = sb; g.sb_chunk_stride = sb_chunk_stride; g.sb_blk_stride = sb_blk_stride;
     g.out = out; g.ldo = No; g.accumulate = accumulate;
     g.status = w.status;
+    g.status_mark = status_mark(w.cleared);
     g.chain = link.role;
     if (link.jobs) g.stats = *link.jobs;
     g.partials = nullptr; g.counters = nullptr;
@@ -897,8 +898,9 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // run only when asked for through snip_debug_set (on the 7B shapes they are slower than the kernels below).
     const int choice = g_kernel_choice.load();
     if (choice == 2) {
-        rc = launch_stat_jobs(g.stats, st);   // these kernels do not reduce statistics
+        rc = launch_stat_jobs(g.stats, st);   // these kernels neither reduce statistics nor clear the status word
         if (rc) return rc;
+        if (!w.cleared) SNIP_CUDA_TRY(cudaMemsetAsync(g.status, 0, sizeof(uint32_t), st));
         return gemm_pair_impl(fmt_a, fmt_b, a_codes, b_codes, Mo, No, Kc, sa, sa_chunk_stride, sb, sb_chunk_stride, sb_blk_stride, scale_mode,
                               out, out_dtype, accumulate, g.status, g.wait_limit_ns, tx_skew, st);
     }

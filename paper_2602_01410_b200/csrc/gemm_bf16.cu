@@ -47,6 +47,7 @@ struct Bf16Args {
     uint32_t stage_tx_bytes;
     uint64_t wait_limit_ns;
     uint32_t *status;
+    uint32_t status_mark;      // see status_begin
     WorkSplit work;
     float *partials;           // see gemm.cu
     uint32_t *counters;
@@ -109,6 +110,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     // everything up to here touches nothing that a kernel ahead on the stream writes
     if (g.chain != CHAIN_BESIDE) pdl_wait();
     pdl_launch_dependents();
+    status_begin(g.status, g.status_mark);
 
     // a whole converged warp waits, with one answer for all its lanes; a failed wait raises the abort flag of both CTAs
     auto wait_all = [&](uint32_t bar, uint32_t parity) {
@@ -307,7 +309,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     if (*abort_flag) {
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
-        if (threadIdx.x == 0) atomicExch(g.status, (uint32_t)SNIP_ERR_TIMEOUT);
+        if (threadIdx.x == 0) status_report(g.status, g.status_mark, (uint32_t)SNIP_ERR_TIMEOUT, g.wait_limit_ns);
         __syncthreads();
     }
     if (warp == 1) {
@@ -321,7 +323,7 @@ int launch_bf16(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
 {
     auto kern = gemm_bf16_kernel<PAIR, A_MN, B_MN, OUT_F32>;
     SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, Cfg<PAIR>::kSmemBytes));
-    return launch_chained(kern, grid, kThreads, Cfg<PAIR>::kSmemBytes, st, g.chain != CHAIN_NONE, PAIR ? 2 : 1, tmA, tmB, tmO, g, idesc);
+    return launch_chained(kern, grid, kThreads, Cfg<PAIR>::kSmemBytes, st, PAIR ? 2 : 1, tmA, tmB, tmO, g, idesc);
 }
 template <bool PAIR>
 int launch_bf16_order(bool a_mn, bool b_mn, bool f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const Bf16Args &g,
@@ -337,7 +339,6 @@ int launch_bf16_order(bool a_mn, bool b_mn, bool f32, const CUtensorMap &tmA, co
 
 int make_tiled_map_2d(CUtensorMap *map, const void *ptr, int dtype, int64_t rows, int64_t inner_elems, int64_t row_bytes, int box_x_elems,
                       int box_rows, int swizzle);
-int gemm_clear_status(void *ws, cudaStream_t st);
 int gemm_sm_count();
 void gemm_debug_hooks(uint64_t *wait_limit_ns, int *tx_skew);
 bool gemm_slicing_enabled();
@@ -351,6 +352,7 @@ int gemm_bf16_impl(const void *a, bool a_mn, const void *b, bool b_mn, int64_t M
     g.Mo = (int32_t)Mo; g.No = (int32_t)No; g.Kc = (int32_t)Kc;
     g.out_acc = accumulate ? static_cast<float *>(out) : nullptr;
     g.status = w.status;
+    g.status_mark = status_mark(w.cleared);
     g.counters = w.counters; g.partials = w.partials;
     g.chain = link.role;
     if (link.jobs) g.stats = *link.jobs;

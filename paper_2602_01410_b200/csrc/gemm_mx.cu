@@ -47,6 +47,7 @@ struct MxArgs {
     int32_t n_atoms_b;         // ceil(No/128)
     uint32_t stage_tx_bytes;   // bytes reported to a stage's barrier (operands + scale-factor atoms)
     uint32_t *status;
+    uint32_t status_mark;      // see status_begin
     const float *amax_a, *amax_b;   // two-level option: the tensors' magnitude bounds (device); else null
     uint64_t wait_limit_ns;    // bound of every device-side wait
     int32_t chain;             // ChainRole
@@ -139,6 +140,7 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     // everything up to here touches nothing that a kernel ahead on the stream writes
     if (g.chain != CHAIN_BESIDE) pdl_wait();
     pdl_launch_dependents();
+    status_begin(g.status, g.status_mark);
 
     if (warp == 0) {
         // ================= producer: operand tiles and scale-factor atoms =================
@@ -304,7 +306,7 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     if (*abort_flag) {
         const uint64_t t0 = globaltimer_ns();
         while (globaltimer_ns() - t0 < 2000000ull) __nanosleep(1000);
-        if (threadIdx.x == 0) atomicExch(g.status, (uint32_t)SNIP_ERR_TIMEOUT);
+        if (threadIdx.x == 0) status_report(g.status, g.status_mark, (uint32_t)SNIP_ERR_TIMEOUT, g.wait_limit_ns);
         __syncthreads();
     }
     if (warp == 1) {
@@ -323,14 +325,13 @@ int launch_mx(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap 
     SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
     const int num_tiles = (int)(ceil_div(g.Mo, BM) * ceil_div(g.No, BN));
     const int grid = num_tiles < sms ? num_tiles : sms;
-    return launch_chained(kern, grid, kThreads, C::kSmemBytes, st, g.chain != CHAIN_NONE, 1, tmA, tmB, tmO, g, idesc);
+    return launch_chained(kern, grid, kThreads, C::kSmemBytes, st, 1, tmA, tmB, tmO, g, idesc);
 }
 
 }  // namespace
 
 int make_tiled_map_2d(CUtensorMap *map, const void *ptr, int dtype, int64_t rows, int64_t inner_elems, int64_t row_bytes, int box_x_elems,
                       int box_rows, int swizzle);
-int gemm_clear_status(void *ws, cudaStream_t st);
 GemmWs gemm_ws(void *ws, size_t ws_bytes);
 int gemm_sm_count();
 void gemm_debug_hooks(uint64_t *wait_limit_ns, int *tx_skew);   // testing hooks of snip_debug_set (gemm.cu)
@@ -347,7 +348,6 @@ int gemm_mx_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes,
     if (!aligned16(a_codes) || !aligned16(b_codes) || !aligned16(sfa) || !aligned16(sfb) || !aligned16(out) || !aligned16(w.status)) return SNIP_ERR_ALIGN;
     int rc = require_sm100();
     if (rc != SNIP_OK) return rc;
-    if (!w.cleared) { rc = gemm_clear_status(w.status, st); if (rc) return rc; }   // see gemm_impl
     const bool f32 = out_dtype == SNIP_OUT_FP32;
     const bool a4 = fmt_a == SNIP_FMT_FP4_E2M1, b4 = fmt_b == SNIP_FMT_FP4_E2M1;
 
@@ -357,6 +357,7 @@ int gemm_mx_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes,
     g.sfb = static_cast<const uint8_t *>(sfb);
     g.n_atoms_b = (int32_t)ceil_div(No, 128);
     g.status = w.status;
+    g.status_mark = status_mark(w.cleared);
     g.chain = link.role;
     if (link.jobs) g.stats = *link.jobs;
     int tx_skew = 0;
@@ -403,7 +404,6 @@ int gemm_nvfp4_impl(const void *a_codes, const void *b_codes, const void *sfa, c
     if ((reinterpret_cast<uintptr_t>(amax_a) & 3u) || (reinterpret_cast<uintptr_t>(amax_b) & 3u)) return SNIP_ERR_ALIGN;
     int rc = require_sm100();
     if (rc != SNIP_OK) return rc;
-    if (!w.cleared) { rc = gemm_clear_status(w.status, st); if (rc) return rc; }
     const bool f32 = out_dtype == SNIP_OUT_FP32;
     MxArgs g;
     g.Mo = (int32_t)Mo; g.No = (int32_t)No; g.Kc = (int32_t)Kc;
@@ -411,6 +411,7 @@ int gemm_nvfp4_impl(const void *a_codes, const void *b_codes, const void *sfa, c
     g.sfb = static_cast<const uint8_t *>(sfb);
     g.n_atoms_b = (int32_t)ceil_div(No, 128);
     g.status = w.status;
+    g.status_mark = status_mark(w.cleared);
     g.chain = link.role;
     if (link.jobs) g.stats = *link.jobs;
     int tx_skew = 0;

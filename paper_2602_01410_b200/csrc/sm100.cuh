@@ -25,6 +25,24 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 __device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
 __device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
+// Status word of a GEMM (word[0]) cleared by the launch itself, in place of a memset ahead of it (which cost the kernel a 4 us gap):
+// CTA 0 clears it and leaves the launch's mark in word[1]; a CTA that gives up later reports only once that mark is there, so that the
+// clearing cannot erase the report (bounded: a CTA 0 that never came to run would hold it up for `limit_ns` at most).
+__device__ __forceinline__ void status_begin(uint32_t *word, uint32_t mark)
+{
+    if (mark != 0 && blockIdx.x == 0 && threadIdx.x == 0) {
+        atomicExch(word, 0u);
+        __threadfence();
+        atomicExch(word + 1, mark);
+    }
+}
+__device__ __forceinline__ void status_report(uint32_t *word, uint32_t mark, uint32_t value, uint64_t limit_ns)
+{
+    const uint64_t t0 = globaltimer_ns();
+    while (mark != 0 && atomicAdd(word + 1, 0u) != mark && globaltimer_ns() - t0 < limit_ns) __nanosleep(1000);
+    atomicExch(word, value);
+}
+
 // Move registers between warpgroups (all four warps of an aligned group must execute it).
 template <int N> __device__ __forceinline__ void reg_alloc() { asm volatile("setmaxnreg.inc.sync.aligned.u32 %0;" ::"n"(N)); }
 template <int N> __device__ __forceinline__ void reg_dealloc() { asm volatile("setmaxnreg.dec.sync.aligned.u32 %0;" ::"n"(N)); }
