@@ -80,6 +80,26 @@ struct ChainLink {
     StatJobs *jobs = nullptr;   // quantizers append, the next GEMM takes them
 };
 
+// One tensor of the two-output quantizer (quantize.cu: quantize_dual_impl, quantize_xwd_impl).
+constexpr int kDualTwoLevel = 16;   // kind beyond snip_dual_kind_t: 1x16 / 16x1 tiles of the two-level option
+struct DualTask {
+    const void *x;
+    int64_t rows, cols, ld;
+    int kind;                  // snip_dual_kind_t or kDualTwoLevel
+    int pow2;
+    const float *tensor_amax;  // two-level option only
+    DualOut a, b;
+    void *ws;                  // statistics scratch
+    size_t ws_bytes;
+};
+inline DualTask two_level_task(const void *x, int64_t rows, int64_t cols, int64_t ld, const float *amax, void *codes_a, void *sf_a, snip_stats_t *stats_a,
+                               void *codes_b, void *sf_b, snip_stats_t *stats_b, int rounding, uint64_t seed, void *ws, size_t ws_bytes)
+{
+    const int sr = rounding == SNIP_ROUND_STOCHASTIC ? 1 : 0;
+    return {x, rows, cols, ld, kDualTwoLevel, 0, amax, DualOut{SNIP_FMT_FP4_E2M1, codes_a, nullptr, sf_a, stats_a, sr, seed},
+            DualOut{SNIP_FMT_FP4_E2M1, codes_b, nullptr, sf_b, stats_b, sr, seed}, ws, ws_bytes};
+}
+
 // Fails with SNIP_ERR_UNSUPPORTED unless the current device is compute capability 10.x.
 int require_sm100();
 

@@ -245,7 +245,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // everything up to here touches nothing that a kernel ahead on the stream writes
     if (g.chain != CHAIN_BESIDE) pdl_wait();
     pdl_launch_dependents();
-    status_begin(g.status, g.status_mark);
 
     if (KIND == MmaKind::MXF4) {
         // constant scale factors 2^0 (UE8M0 byte 127) for every row of A and B
@@ -263,6 +262,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
       reg_dealloc<40>();  // frees (168-40)*128 = 16384 registers
       if (warp == 0) {
         // ================= TMA producer =================
+        status_begin(g.status, g.status_mark);
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;

@@ -17,11 +17,7 @@ int gemm_mx_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes,
                  int64_t Kc, void *out, int out_dtype, const GemmWs &w, cudaStream_t st, const ChainLink &link);
 size_t gemm_ws_bytes();
 size_t gemm_ws_bytes_sliced();   // with room for the weight-gradient product's contraction slices
-int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int kind, int pow2, const DualOut &oa, const DualOut &ob,
-                       void *ws, size_t ws_bytes, cudaStream_t st, const ChainLink &link);
-int quantize_nvfp4_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, const float *tensor_amax, void *codes_a, void *sf_a,
-                             snip_stats_t *stats_a, void *codes_b, void *sf_b, snip_stats_t *stats_b, int rounding, uint64_t seed, void *ws,
-                             size_t ws_bytes, cudaStream_t st, const ChainLink &link);
+int quantize_xwd_impl(const DualTask (&t)[3], cudaStream_t st, const ChainLink &link);
 int gemm_nvfp4_impl(const void *a_codes, const void *b_codes, const void *sfa, const void *sfb, const float *amax_a, const float *amax_b,
                     int64_t Mo, int64_t No, int64_t Kc, void *out, int out_dtype, const GemmWs &w, cudaStream_t st, const ChainLink &link);
 
@@ -302,18 +298,16 @@ extern "C" int snip_linear_fwd_bwd(const void *X, const void *W, const void *dY,
         const int sr = (i >= 4 && dy_rounding == SNIP_ROUND_STOCHASTIC && fmt[i] == SNIP_FMT_FP4_E2M1) ? 1 : 0;
         return DualOut{fmt[i], f.codes[i], f.scales[i], f.sf[i], stats6 ? stats6 + i : nullptr, sr, dy_seed};
     };
-    // One chain: the three quantizers side by side (each tensor is read once and leaves both of its copies), then the three GEMMs, which
-    // are independent of one another: the next one takes the SMs that the last wave of the one ahead leaves idle.  The first quantizer
+    // One chain: the three tensors through the quantizer (each is read once and leaves both of its copies), then the three GEMMs, which
+    // are independent of one another: the next one takes the SMs that the last wave of the one ahead leaves idle.  The quantizer
     // clears the status word (one for the three GEMMs) and the slice counters, the first GEMM reduces the statistics.
     StatJobs jobs;
-    ChainLink quant[3], mult[3];
-    for (int i = 0; i < 3; ++i) {
-        quant[i].role = i ? CHAIN_BESIDE : CHAIN_FIRST;
-        quant[i].jobs = &jobs;
-        mult[i].role = i ? CHAIN_BESIDE : CHAIN_AFTER;
-    }
-    quant[0].zero = static_cast<uint32_t *>(f.gws);
-    quant[0].zero_words = gemm_ws_zero_words();
+    ChainLink quant, mult[3];
+    quant.role = CHAIN_FIRST;
+    quant.jobs = &jobs;
+    quant.zero = static_cast<uint32_t *>(f.gws);
+    quant.zero_words = gemm_ws_zero_words();
+    for (int i = 0; i < 3; ++i) mult[i].role = i ? CHAIN_BESIDE : CHAIN_AFTER;
     mult[0].jobs = &jobs;
     GemmWs gw = gemm_ws(f.gws, gemm_ws_bytes_sliced());
     gw.cleared = true;
@@ -328,11 +322,10 @@ extern "C" int snip_linear_fwd_bwd(const void *X, const void *W, const void *dY,
         return gemm_impl(fmt[ia], fmt[ib], f.codes[ia], f.codes[ib], p.Mo, p.No, p.Kc, f.scales[ia], p.Mo, f.scales[ib], sb_cs, sb_bs, p.scale_mode, out,
                          out_dtype, 0, gw, st, link, 0);
     };
-    rc = quantize_dual_impl(X, M, K, K, kind_xdy, mx, out_of(0), out_of(1), f.stats_ws[0], f.stats_ws_bytes[0], st, quant[0]);
-    if (rc) return rc;
-    rc = quantize_dual_impl(W, N, K, K, kind_w, mx, out_of(2), out_of(3), f.stats_ws[1], f.stats_ws_bytes[1], st, quant[1]);
-    if (rc) return rc;
-    rc = quantize_dual_impl(dY, M, N, N, kind_xdy, mx, out_of(4), out_of(5), f.stats_ws[2], f.stats_ws_bytes[2], st, quant[2]);
+    const DualTask tensors[3] = {{X, M, K, K, kind_xdy, mx, nullptr, out_of(0), out_of(1), f.stats_ws[0], f.stats_ws_bytes[0]},
+                                 {W, N, K, K, kind_w, mx, nullptr, out_of(2), out_of(3), f.stats_ws[1], f.stats_ws_bytes[1]},
+                                 {dY, M, N, N, kind_xdy, mx, nullptr, out_of(4), out_of(5), f.stats_ws[2], f.stats_ws_bytes[2]}};
+    rc = quantize_xwd_impl(tensors, st, quant);
     if (rc) return rc;
     rc = gemm(SNIP_OP_FWD, 0, 2, Y);
     if (rc) return rc;
@@ -399,27 +392,24 @@ extern "C" int snip_linear_fwd_bwd_nvfp4(const void *X, const void *W, const voi
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const float *bx = bounds3, *bw = bounds3 + 1, *bdy = bounds3 + 2;
     auto stat = [&](int i) { return stats6 ? stats6 + i : nullptr; };
-    // the chain of snip_linear_fwd_bwd: three quantizers side by side, three GEMMs behind them
+    // the chain of snip_linear_fwd_bwd
     StatJobs jobs;
-    ChainLink quant[3], mult[3];
-    for (int i = 0; i < 3; ++i) {
-        quant[i].role = i ? CHAIN_BESIDE : CHAIN_FIRST;
-        quant[i].jobs = &jobs;
-        mult[i].role = i ? CHAIN_BESIDE : CHAIN_AFTER;
-    }
-    quant[0].zero = static_cast<uint32_t *>(f.gws);
-    quant[0].zero_words = 1;
+    ChainLink quant, mult[3];
+    quant.role = CHAIN_FIRST;
+    quant.jobs = &jobs;
+    quant.zero = static_cast<uint32_t *>(f.gws);
+    quant.zero_words = 1;
+    for (int i = 0; i < 3; ++i) mult[i].role = i ? CHAIN_BESIDE : CHAIN_AFTER;
     mult[0].jobs = &jobs;
     GemmWs gw = gemm_ws(f.gws, gemm_ws_bytes());
     gw.cleared = true;
-    int rc = quantize_nvfp4_dual_impl(X, M, K, K, bx, f.codes[0], f.sf[0], stat(0), f.codes[1], f.sf[1], stat(1), SNIP_ROUND_NEAREST_EVEN, 0,
-                                      f.stats_ws[0], f.stats_ws_bytes[0], st, quant[0]);
-    if (rc) return rc;
-    rc = quantize_nvfp4_dual_impl(W, N, K, K, bw, f.codes[2], f.sf[2], stat(2), f.codes[3], f.sf[3], stat(3), SNIP_ROUND_NEAREST_EVEN, 0, f.stats_ws[1],
-                                  f.stats_ws_bytes[1], st, quant[1]);
-    if (rc) return rc;
-    rc = quantize_nvfp4_dual_impl(dY, M, N, N, bdy, f.codes[4], f.sf[4], stat(4), f.codes[5], f.sf[5], stat(5), dy_rounding, dy_seed, f.stats_ws[2],
-                                  f.stats_ws_bytes[2], st, quant[2]);
+    const DualTask tensors[3] = {two_level_task(X, M, K, K, bx, f.codes[0], f.sf[0], stat(0), f.codes[1], f.sf[1], stat(1), SNIP_ROUND_NEAREST_EVEN, 0,
+                                                f.stats_ws[0], f.stats_ws_bytes[0]),
+                                 two_level_task(W, N, K, K, bw, f.codes[2], f.sf[2], stat(2), f.codes[3], f.sf[3], stat(3), SNIP_ROUND_NEAREST_EVEN, 0,
+                                                f.stats_ws[1], f.stats_ws_bytes[1]),
+                                 two_level_task(dY, M, N, N, bdy, f.codes[4], f.sf[4], stat(4), f.codes[5], f.sf[5], stat(5), dy_rounding, dy_seed,
+                                                f.stats_ws[2], f.stats_ws_bytes[2])};
+    int rc = quantize_xwd_impl(tensors, st, quant);
     if (rc) return rc;
     rc = gemm_nvfp4_impl(f.codes[0], f.codes[2], f.sf[0], f.sf[2], bx, bw, M, N, K, Y, out_dtype, gw, st, mult[0]);
     if (rc) return rc;

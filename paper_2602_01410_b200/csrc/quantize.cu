@@ -21,6 +21,8 @@
 #include <cuda_bf16.h>
 #include <float.h>
 
+#include <type_traits>
+
 #include "common.cuh"
 #include "quant_device.cuh"
 
@@ -47,6 +49,10 @@ struct QuantArgs {
     uint32_t *sf;         // optional: UE8M0 bytes of 1/S in 512-byte atoms for hardware block scaling; null if unused
                           // (two-level option: the E4M3 scale bytes, two atoms per 128x128 tile)
     const float *tensor_amax;   // two-level option: bound of the tensor's magnitudes (device); else unused
+};
+
+// What a launch does for the chain it belongs to.
+struct ChainArgs {
     int chain;            // ChainRole
     uint32_t *zero;       // words this launch clears for the kernels behind it
     int32_t zero_words;
@@ -54,13 +60,13 @@ struct QuantArgs {
 
 // Start of every quantizer: wait for the kernel ahead on the stream (unless independent of it), let the one behind be scheduled
 // (it waits for this grid where it has to), clear what the chain asks for.
-__device__ __forceinline__ void chain_begin(const QuantArgs &a)
+__device__ __forceinline__ void chain_begin(const ChainArgs &a)
 {
     if (a.chain != CHAIN_BESIDE) asm volatile("griddepcontrol.wait;" ::: "memory");
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.zero_words; i += gridDim.x * blockDim.x) a.zero[i] = 0u;
 }
-__device__ __forceinline__ void chain_end(const QuantArgs &a)
+__device__ __forceinline__ void chain_end(const ChainArgs &a)
 {
     if (a.chain == CHAIN_BESIDE) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -780,7 +786,7 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
 
 // End of a CTA's walk: its threads' sums -> one CtaPartial per output (warp shuffles, then warp order).
 template <bool HAS_B>
-__device__ __forceinline__ void finish_stats(const ThreadStats &ts, QuantShared &sh, CtaPartial *pa, CtaPartial *pb)
+__device__ __forceinline__ void finish_stats(const ThreadStats &ts, QuantShared &sh, int slot, CtaPartial *pa, CtaPartial *pb)
 {
     double x = ts.x, ea = ts.ea, eb = ts.eb;
     float am = ts.amax;
@@ -799,10 +805,10 @@ __device__ __forceinline__ void finish_stats(const ThreadStats &ts, QuantShared 
         double tx_ = 0.0, ta = 0.0, tb = 0.0, tm = 0.0;
 #pragma unroll
         for (int w = 0; w < 8; ++w) { tx_ += sh.red_d[w][0]; ta += sh.red_d[w][1]; tb += sh.red_d[w][2]; tm = fmax(tm, sh.red_d[w][3]); }
-        CtaPartial *d = pa + blockIdx.x;
+        CtaPartial *d = pa + slot;
         d->sumsq_x = tx_; d->sumsq_err = ta; d->amax = (float)tm;
         if (HAS_B) {
-            d = pb + blockIdx.x;
+            d = pb + slot;
             d->sumsq_x = tx_; d->sumsq_err = tb; d->amax = (float)tm;
         }
     }
@@ -817,9 +823,9 @@ constexpr int kDualCtasPerSmSr = 2;   // stochastic rounding: the generator's re
 // Walk of one CTA over its tiles without divisions in the loop.
 struct TileWalk {
     int r, c, step_r, step_c, nr, nc;
-    __device__ __forceinline__ TileWalk(int nr_, int nc_) : nr(nr_), nc(nc_)
+    __device__ __forceinline__ TileWalk(int first, int nr_, int nc_) : nr(nr_), nc(nc_)
     {
-        r = (int)blockIdx.x / nc_; c = (int)blockIdx.x % nc_;
+        r = first / nc_; c = first % nc_;
         step_r = (int)gridDim.x / nc_; step_c = (int)gridDim.x % nc_;
     }
     __device__ __forceinline__ bool valid() const { return r < nr; }
@@ -831,15 +837,15 @@ struct TileWalk {
 };
 
 template <int FMT, int BLOCK, bool TRANSPOSED, bool CODES, bool STATS, bool ROWSTATS, bool SR = false>
-__global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_kernel(const QuantArgs a)
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_kernel(const QuantArgs a, const ChainArgs chain)
 {
     extern __shared__ __align__(128) uint8_t smem[];
     QuantShared &sh = *reinterpret_cast<QuantShared *>(smem + kStageBytes);
     QuantShared32 *s32 = reinterpret_cast<QuantShared32 *>(smem + kSmemBytes);   // present only for the 32-long tile kinds
     const uint4 *slot = reinterpret_cast<const uint4 *>(smem) + threadIdx.x;
-    chain_begin(a);
+    chain_begin(chain);
     ThreadStats ts;
-    TileWalk w((int)a.tiles_r, (int)a.tiles_c);
+    TileWalk w((int)blockIdx.x, (int)a.tiles_r, (int)a.tiles_c);
     if (w.valid()) prefetch_tile(a, w.r, w.c, smem);
     prefetch_commit();
     while (w.valid()) {
@@ -852,77 +858,139 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_kernel(const Qu
         });
         __syncthreads();  // the scratch arrays are reused by the next tile
     }
-    if (STATS) finish_stats<false>(ts, sh, a.partials, nullptr);
-    chain_end(a);
+    if (STATS) finish_stats<false>(ts, sh, (int)blockIdx.x, a.partials, nullptr);
+    chain_end(chain);
 }
 
-// Two outputs from one read (the tile kinds a tensor is consumed with, paper Fig. 5): `a` as stored
-// (1x128 tiles along the columns, or 128x128 blocks) and `b` transposed (128x1 tiles along the rows, or
-// the same 128x128 blocks), each with its own format, scales and statistics.
-struct DualArgs {
+// Two outputs from one read (the tile kinds a tensor is consumed with, paper Fig. 5): `a` as stored and `b` transposed, each with its
+// own format, scales and statistics:
+//   FAM_128: 1x128 tiles along the columns and 128x1 tiles along the rows (activations, gradients), or the same 128x128 blocks (weights)
+//   FAM_32 : 1x32 and 32x1 tiles, power-of-two scales;   FAM_NV: 1x16 and 16x1 tiles of the two-level option, E2M1 codes
+enum Family { FAM_128 = 0, FAM_32 = 1, FAM_NV = 2 };
+
+struct DualJob {
     QuantArgs a, b;
+    int32_t first;      // position of its first tile in the launch's sequence (quantize_small_kernel)
+    int32_t variant;    // formats and rounding (dual_variant), + kBlkVariant for 128x128 blocks
 };
-template <int FMT_A, int FMT_B, bool BLK, bool STATS, int SR_A = 0, int SR_B = 0, bool SUB32 = false>
-__global__ void __launch_bounds__(kThreads, SR_A || SR_B ? kDualCtasPerSmSr : kDualCtasPerSm) quantize_dual_kernel(const DualArgs d)
-{
-    extern __shared__ __align__(128) uint8_t smem[];
-    QuantShared &sh = *reinterpret_cast<QuantShared *>(smem + kStageBytes);
-    QuantShared32 *s32 = reinterpret_cast<QuantShared32 *>(smem + kSmemBytes);   // present only with SUB32
-    const uint4 *slot = reinterpret_cast<const uint4 *>(smem) + threadIdx.x;
-    chain_begin(d.a);
-    ThreadStats ts;
-    TileWalk w((int)d.a.tiles_r, (int)d.a.tiles_c);
-    if (w.valid()) prefetch_tile(d.a, w.r, w.c, smem);
-    prefetch_commit();
-    while (w.valid()) {
-        prefetch_wait<0>();
-        const Tile tl = {w.r, w.c, w.nr, w.nc};
-        w.next();
-        using A = Out<FMT_A, SUB32 ? SNIP_BLOCK_ROW_1x32 : BLK ? SNIP_BLOCK_BLK_128x128 : SNIP_BLOCK_ROW_1x128, false, true, SR_A>;
-        using B = Out<FMT_B, SUB32 ? SNIP_BLOCK_COL_32x1 : BLK ? SNIP_BLOCK_BLK_128x128 : SNIP_BLOCK_COL_128x1, true, true, SR_B>;
-        process_tile<A, B, STATS, false>(d.a, d.b, tl, slot, sh, s32, ts, [&] {
-            if (w.valid()) prefetch_tile(d.a, w.r, w.c, smem);
-            prefetch_commit();
-        });
-        __syncthreads();
-    }
-    if (STATS) finish_stats<true>(ts, sh, d.a.partials, d.b.partials);
-    chain_end(d.a);
-}
+constexpr int kBlkVariant = 64;
+__host__ __device__ constexpr int dual_variant(bool a4, bool b4, int sr_a, int sr_b) { return (a4 ? 1 : 0) | (b4 ? 2 : 0) | (sr_a << 2) | (sr_b << 3); }
 
-// Two-level option, both copies from one read: a = 1x16 tiles as stored, b = 16x1 tiles transposed, E2M1 codes.
-template <bool STATS, bool SR = false>
-__global__ void __launch_bounds__(kThreads, SR ? kDualCtasPerSmSr : kDualCtasPerSm) quantize_nvfp4_dual_kernel(const DualArgs d)
+struct DualScratch {
+    uint8_t *smem;
+    const uint4 *slot;
+    QuantShared *sh;
+    QuantShared32 *s32;   // present only for the 32- and 16-long tile kinds (which use it as QuantShared16)
+};
+
+template <class A, class B, bool STATS>
+__device__ __forceinline__ void run_job(const DualJob &d, int first, const DualScratch &m, const TwoLevel &tw)
 {
-    extern __shared__ __align__(128) uint8_t smem[];
-    QuantShared &sh = *reinterpret_cast<QuantShared *>(smem + kStageBytes);
-    QuantShared32 *s32 = reinterpret_cast<QuantShared32 *>(smem + kSmemBytes);   // holds this kernel's QuantShared16
-    const uint4 *slot = reinterpret_cast<const uint4 *>(smem) + threadIdx.x;
-    chain_begin(d.a);
-    TwoLevel tw;
-    {
-        const float bound = *d.a.tensor_amax;
-        tw.enc = bound == 0.0f ? 1.0f : fminf(__fdiv_rn(2688.0f, bound), FLT_MAX);
-        tw.inv_enc = __fdiv_rn(1.0f, tw.enc);
-    }
     ThreadStats ts;
-    TileWalk w((int)d.a.tiles_r, (int)d.a.tiles_c);
-    if (w.valid()) prefetch_tile(d.a, w.r, w.c, smem);
+    TileWalk w(first, (int)d.a.tiles_r, (int)d.a.tiles_c);
+    if (w.valid()) prefetch_tile(d.a, w.r, w.c, m.smem);
     prefetch_commit();
     while (w.valid()) {
         prefetch_wait<0>();
         const Tile tl = {w.r, w.c, w.nr, w.nc};
         w.next();
-        using A = Out<SNIP_FMT_FP4_E2M1, SNIP_BLOCK_ROW_1x16, false, true, SR>;
-        using B = Out<SNIP_FMT_FP4_E2M1, SNIP_BLOCK_COL_16x1, true, true, SR ? 2 : 0>;
-        process_tile<A, B, STATS, false>(d.a, d.b, tl, slot, sh, s32, ts, [&] {
-            if (w.valid()) prefetch_tile(d.a, w.r, w.c, smem);
+        process_tile<A, B, STATS, false>(d.a, d.b, tl, m.slot, *m.sh, m.s32, ts, [&] {
+            if (w.valid()) prefetch_tile(d.a, w.r, w.c, m.smem);
             prefetch_commit();
         }, tw);
         __syncthreads();
     }
-    if (STATS) finish_stats<true>(ts, sh, d.a.partials, d.b.partials);
-    chain_end(d.a);
+    if (STATS) finish_stats<true>(ts, *m.sh, first, d.a.partials, d.b.partials);
+}
+
+template <int FAM, int V, bool STATS>
+__device__ __forceinline__ void run_variant(const DualJob &d, int first, const DualScratch &m)
+{
+    constexpr bool BLK = (V & kBlkVariant) != 0;
+    constexpr int ROW = BLK ? SNIP_BLOCK_BLK_128x128 : FAM == FAM_128 ? SNIP_BLOCK_ROW_1x128 : FAM == FAM_32 ? SNIP_BLOCK_ROW_1x32 : SNIP_BLOCK_ROW_1x16;
+    constexpr int COL = BLK ? SNIP_BLOCK_BLK_128x128 : FAM == FAM_128 ? SNIP_BLOCK_COL_128x1 : FAM == FAM_32 ? SNIP_BLOCK_COL_32x1 : SNIP_BLOCK_COL_16x1;
+    constexpr int FA = (V & 1) ? SNIP_FMT_FP4_E2M1 : SNIP_FMT_FP8_E4M3, FB = (V & 2) ? SNIP_FMT_FP4_E2M1 : SNIP_FMT_FP8_E4M3;
+    constexpr int SRA = (V >> 2) & 1, SRB = (V >> 3) & 3;   // SRB: 1 own generator, 2 the first output's uniforms
+    TwoLevel tw;
+    if (FAM == FAM_NV) {
+        const float bound = *d.a.tensor_amax;
+        tw.enc = bound == 0.0f ? 1.0f : fminf(__fdiv_rn(2688.0f, bound), FLT_MAX);
+        tw.inv_enc = __fdiv_rn(1.0f, tw.enc);
+    }
+    run_job<Out<FA, ROW, false, true, SRA>, Out<FB, COL, true, true, SRB>, STATS>(d, first, m, tw);
+}
+
+__device__ __forceinline__ DualScratch dual_scratch(uint8_t *smem)
+{
+    return {smem, reinterpret_cast<const uint4 *>(smem) + threadIdx.x, reinterpret_cast<QuantShared *>(smem + kStageBytes),
+            reinterpret_cast<QuantShared32 *>(smem + kSmemBytes)};
+}
+
+template <int FAM, int V, bool STATS>
+__global__ void __launch_bounds__(kThreads, (V & 28) ? kDualCtasPerSmSr : kDualCtasPerSm) quantize_dual_kernel(const DualJob d, const ChainArgs chain)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    chain_begin(chain);
+    run_variant<FAM, V, STATS>(d, (int)blockIdx.x, dual_scratch(smem));
+    chain_end(chain);
+}
+
+// The combinations of formats and roundings that exist, as F(variant).
+#define SNIP_NV_VARIANTS(F) F(dual_variant(true, true, 0, 0)) F(dual_variant(true, true, 1, 2))
+#define SNIP_ROWCOL_VARIANTS(F)                                                                                                    \
+    SNIP_NV_VARIANTS(F)                                                                                                            \
+    F(dual_variant(false, false, 0, 0)) F(dual_variant(false, true, 0, 0)) F(dual_variant(true, false, 0, 0))                      \
+    F(dual_variant(true, true, 1, 1)) F(dual_variant(true, true, 1, 0)) F(dual_variant(true, true, 0, 1))                          \
+    F(dual_variant(true, false, 1, 0)) F(dual_variant(false, true, 0, 1))
+#define SNIP_BLK_VARIANTS(F)                                                                                                       \
+    F(kBlkVariant + dual_variant(false, false, 0, 0)) F(kBlkVariant + dual_variant(false, true, 0, 0))                             \
+    F(kBlkVariant + dual_variant(true, false, 0, 0)) F(kBlkVariant + dual_variant(true, true, 0, 0))
+
+// Small tensors: X, W and dY of a linear layer in one launch (2.8 us of the host and a place in the chain each), their tiles one
+// sequence dealt to the CTAs, a tile or two each.  The variant is chosen at run time; that keeps the arguments out of the
+// instructions and costs 10 % on large tensors, which therefore have launches of their own (see quantize_xwd_impl).
+constexpr int kMaxJobs = 3;
+struct DualGroup {
+    DualJob job[kMaxJobs];
+    ChainArgs chain;
+};
+template <int FAM, bool STATS>
+__global__ void __launch_bounds__(kThreads, kDualCtasPerSmSr) quantize_small_kernel(const __grid_constant__ DualGroup g)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    const DualScratch m = dual_scratch(smem);
+    chain_begin(g.chain);
+#pragma unroll 1
+    for (int j = 0; j < kMaxJobs; ++j) {
+        const DualJob &d = g.job[j];
+        int first = ((int)blockIdx.x - d.first) % (int)gridDim.x;
+        if (first < 0) first += (int)gridDim.x;
+        if (first >= (int)d.a.ntiles) continue;
+#define SNIP_RUN(V) case V: run_variant<FAM, V, STATS>(d, first, m); break;
+        switch (d.variant) {
+            SNIP_NV_VARIANTS(SNIP_RUN)
+            default: break;
+        }
+#undef SNIP_RUN
+        if constexpr (FAM != FAM_NV) {
+#define SNIP_RUN(V) case V: if constexpr (V != dual_variant(true, true, 0, 0) && V != dual_variant(true, true, 1, 2)) run_variant<FAM, V, STATS>(d, first, m); break;
+            switch (d.variant) {
+                SNIP_ROWCOL_VARIANTS(SNIP_RUN)
+                default: break;
+            }
+#undef SNIP_RUN
+        }
+        if constexpr (FAM == FAM_128) {
+#define SNIP_RUN(V) case V: run_variant<FAM, V, STATS>(d, first, m); break;
+            switch (d.variant) {
+                SNIP_BLK_VARIANTS(SNIP_RUN)
+                default: break;
+            }
+#undef SNIP_RUN
+        }
+        __syncthreads();   // the scratch is free for the next tensor
+    }
+    chain_end(g.chain);
 }
 
 // Fixed-order reduction of the per-CTA partials into one snip_stats_t (deterministic: every thread
@@ -989,7 +1057,7 @@ __global__ void row_stats_reduce_kernel(const float2 *row_partials, int64_t rows
 // Launch of a persistent kernel: its dynamic shared memory exceeds the default limit, so the limit is
 // raised first (a per-function, per-device attribute; setting it again is cheap).
 template <typename Kernel, typename Args>
-void launch_persistent(Kernel kernel, const Args &args, dim3 grid, cudaStream_t st, size_t smem_bytes = kSmemBytes)
+void launch_persistent(Kernel kernel, const Args &args, const ChainArgs &chain, dim3 grid, cudaStream_t st, size_t smem_bytes = kSmemBytes)
 {
     if (cudaFuncSetAttribute(kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem_bytes) != cudaSuccess) return;  // left in cudaGetLastError
     // Programmatic stream serialization: when the kernel before it on the stream signals its dependents early (the
@@ -1005,31 +1073,32 @@ void launch_persistent(Kernel kernel, const Args &args, dim3 grid, cudaStream_t 
     attr[0].val.programmaticStreamSerializationAllowed = 1;
     cfg.attrs = attr;
     cfg.numAttrs = 1;
-    cudaLaunchKernelEx(&cfg, kernel, args);   // an error stays in cudaGetLastError for the caller
+    if constexpr (std::is_same_v<Args, DualGroup>) cudaLaunchKernelEx(&cfg, kernel, args);   // an error stays in cudaGetLastError for the caller
+    else cudaLaunchKernelEx(&cfg, kernel, args, chain);
 }
 
 template <int FMT, int BLOCK, bool TRANSPOSED>
-void launch_variant(const QuantArgs &a, bool codes, bool stats, bool rowstats, dim3 grid, cudaStream_t st)
+void launch_variant(const QuantArgs &a, const ChainArgs &ch, bool codes, bool stats, bool rowstats, dim3 grid, cudaStream_t st)
 {
-    if (codes && stats && rowstats) launch_persistent(quantize_kernel<FMT, BLOCK, TRANSPOSED, true, true, true>, a, grid, st);
-    else if (codes && stats) launch_persistent(quantize_kernel<FMT, BLOCK, TRANSPOSED, true, true, false>, a, grid, st);
-    else if (codes) launch_persistent(quantize_kernel<FMT, BLOCK, TRANSPOSED, true, false, false>, a, grid, st);
-    else if (rowstats) launch_persistent(quantize_kernel<FMT, BLOCK, false, false, true, true>, a, grid, st);
-    else launch_persistent(quantize_kernel<FMT, BLOCK, false, false, true, false>, a, grid, st);
+    if (codes && stats && rowstats) launch_persistent(quantize_kernel<FMT, BLOCK, TRANSPOSED, true, true, true>, a, ch, grid, st);
+    else if (codes && stats) launch_persistent(quantize_kernel<FMT, BLOCK, TRANSPOSED, true, true, false>, a, ch, grid, st);
+    else if (codes) launch_persistent(quantize_kernel<FMT, BLOCK, TRANSPOSED, true, false, false>, a, ch, grid, st);
+    else if (rowstats) launch_persistent(quantize_kernel<FMT, BLOCK, false, false, true, true>, a, ch, grid, st);
+    else launch_persistent(quantize_kernel<FMT, BLOCK, false, false, true, false>, a, ch, grid, st);
 }
 
 template <int FMT>
-void launch_fmt(const QuantArgs &a, int block, bool transposed, bool codes, bool stats, bool rowstats, dim3 grid, cudaStream_t st)
+void launch_fmt(const QuantArgs &a, const ChainArgs &ch, int block, bool transposed, bool codes, bool stats, bool rowstats, dim3 grid, cudaStream_t st)
 {
     if (block == SNIP_BLOCK_ROW_1x128) {
-        if (transposed) launch_variant<FMT, SNIP_BLOCK_ROW_1x128, true>(a, codes, stats, rowstats, grid, st);
-        else launch_variant<FMT, SNIP_BLOCK_ROW_1x128, false>(a, codes, stats, rowstats, grid, st);
+        if (transposed) launch_variant<FMT, SNIP_BLOCK_ROW_1x128, true>(a, ch, codes, stats, rowstats, grid, st);
+        else launch_variant<FMT, SNIP_BLOCK_ROW_1x128, false>(a, ch, codes, stats, rowstats, grid, st);
     } else if (block == SNIP_BLOCK_COL_128x1) {
-        if (transposed) launch_variant<FMT, SNIP_BLOCK_COL_128x1, true>(a, codes, stats, rowstats, grid, st);
-        else launch_variant<FMT, SNIP_BLOCK_COL_128x1, false>(a, codes, stats, rowstats, grid, st);
+        if (transposed) launch_variant<FMT, SNIP_BLOCK_COL_128x1, true>(a, ch, codes, stats, rowstats, grid, st);
+        else launch_variant<FMT, SNIP_BLOCK_COL_128x1, false>(a, ch, codes, stats, rowstats, grid, st);
     } else {
-        if (transposed) launch_variant<FMT, SNIP_BLOCK_BLK_128x128, true>(a, codes, stats, rowstats, grid, st);
-        else launch_variant<FMT, SNIP_BLOCK_BLK_128x128, false>(a, codes, stats, rowstats, grid, st);
+        if (transposed) launch_variant<FMT, SNIP_BLOCK_BLK_128x128, true>(a, ch, codes, stats, rowstats, grid, st);
+        else launch_variant<FMT, SNIP_BLOCK_BLK_128x128, false>(a, ch, codes, stats, rowstats, grid, st);
     }
 }
 
@@ -1038,16 +1107,16 @@ constexpr int kCtasPerSm32 = 3;   // what the larger shared-memory footprint all
 
 // 32-long tile kinds: 1x32 tiles as stored, 32x1 tiles transposed.
 template <int FMT>
-void launch_fmt32(const QuantArgs &a, int block, bool codes, bool stats, dim3 grid, cudaStream_t st)
+void launch_fmt32(const QuantArgs &a, const ChainArgs &ch, int block, bool codes, bool stats, dim3 grid, cudaStream_t st)
 {
     if (block == SNIP_BLOCK_ROW_1x32) {
-        if (codes && stats) launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_ROW_1x32, false, true, true, false>, a, grid, st, kSmemBytes32);
-        else if (codes) launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_ROW_1x32, false, true, false, false>, a, grid, st, kSmemBytes32);
-        else launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_ROW_1x32, false, false, true, false>, a, grid, st, kSmemBytes32);
+        if (codes && stats) launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_ROW_1x32, false, true, true, false>, a, ch, grid, st, kSmemBytes32);
+        else if (codes) launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_ROW_1x32, false, true, false, false>, a, ch, grid, st, kSmemBytes32);
+        else launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_ROW_1x32, false, false, true, false>, a, ch, grid, st, kSmemBytes32);
     } else {
-        if (codes && stats) launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_COL_32x1, true, true, true, false>, a, grid, st, kSmemBytes32);
-        else if (codes) launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_COL_32x1, true, true, false, false>, a, grid, st, kSmemBytes32);
-        else launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_COL_32x1, false, false, true, false>, a, grid, st, kSmemBytes32);
+        if (codes && stats) launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_COL_32x1, true, true, true, false>, a, ch, grid, st, kSmemBytes32);
+        else if (codes) launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_COL_32x1, true, true, false, false>, a, ch, grid, st, kSmemBytes32);
+        else launch_persistent(quantize_kernel<FMT, SNIP_BLOCK_COL_32x1, false, false, true, false>, a, ch, grid, st, kSmemBytes32);
     }
 }
 
@@ -1165,7 +1234,7 @@ int quantize_impl_full(const void *x, int64_t rows, int64_t cols, int64_t ld, in
     a.pow2 = pow2; a.sf = static_cast<uint32_t *>(sf);
     a.seed = seed;
     a.tensor_amax = nullptr;
-    a.chain = link.role; a.zero = link.zero; a.zero_words = link.zero_words;
+    const ChainArgs ch = {link.role, link.zero, link.zero_words};
     a.codes = want_codes ? static_cast<uint8_t *>(codes) : nullptr;
     a.scales = want_codes ? scales : nullptr;
     a.partials = any_stats ? static_cast<CtaPartial *>(ws) : nullptr;
@@ -1174,21 +1243,21 @@ int quantize_impl_full(const void *x, int64_t rows, int64_t cols, int64_t ld, in
     const int64_t nparts = persistent_ctas(tr * tc, b32 ? kCtasPerSm32 : kCtasPerSm);
     dim3 grid((unsigned)nparts);
     if (b32) {
-        if (fmt == SNIP_FMT_FP8_E4M3) launch_fmt32<SNIP_FMT_FP8_E4M3>(a, block, want_codes, any_stats, grid, st);
-        else launch_fmt32<SNIP_FMT_FP4_E2M1>(a, block, want_codes, any_stats, grid, st);
+        if (fmt == SNIP_FMT_FP8_E4M3) launch_fmt32<SNIP_FMT_FP8_E4M3>(a, ch, block, want_codes, any_stats, grid, st);
+        else launch_fmt32<SNIP_FMT_FP4_E2M1>(a, ch, block, want_codes, any_stats, grid, st);
     } else
     if (sr) {
         const bool row = block == SNIP_BLOCK_ROW_1x128 && !transposed, colt = block == SNIP_BLOCK_COL_128x1 && transposed;
         if (fmt != SNIP_FMT_FP4_E2M1 || !want_codes || want_rows || !(row || colt)) return SNIP_ERR_UNSUPPORTED;
         constexpr int F4 = SNIP_FMT_FP4_E2M1;
-        if (row && any_stats) launch_persistent(quantize_kernel<F4, SNIP_BLOCK_ROW_1x128, false, true, true, false, true>, a, grid, st);
-        else if (row) launch_persistent(quantize_kernel<F4, SNIP_BLOCK_ROW_1x128, false, true, false, false, true>, a, grid, st);
-        else if (any_stats) launch_persistent(quantize_kernel<F4, SNIP_BLOCK_COL_128x1, true, true, true, false, true>, a, grid, st);
-        else launch_persistent(quantize_kernel<F4, SNIP_BLOCK_COL_128x1, true, true, false, false, true>, a, grid, st);
+        if (row && any_stats) launch_persistent(quantize_kernel<F4, SNIP_BLOCK_ROW_1x128, false, true, true, false, true>, a, ch, grid, st);
+        else if (row) launch_persistent(quantize_kernel<F4, SNIP_BLOCK_ROW_1x128, false, true, false, false, true>, a, ch, grid, st);
+        else if (any_stats) launch_persistent(quantize_kernel<F4, SNIP_BLOCK_COL_128x1, true, true, true, false, true>, a, ch, grid, st);
+        else launch_persistent(quantize_kernel<F4, SNIP_BLOCK_COL_128x1, true, true, false, false, true>, a, ch, grid, st);
     } else
-    if (fmt == SNIP_FMT_FP8_E4M3) launch_fmt<SNIP_FMT_FP8_E4M3>(a, block, transposed, want_codes, any_stats, want_rows, grid, st);
-    else if (fmt == SNIP_FMT_FP4_E2M1) launch_fmt<SNIP_FMT_FP4_E2M1>(a, block, transposed, want_codes, any_stats, want_rows, grid, st);
-    else launch_variant<SNIP_FMT_BF16, SNIP_BLOCK_BLK_128x128, false>(a, false, true, want_rows, grid, st);
+    if (fmt == SNIP_FMT_FP8_E4M3) launch_fmt<SNIP_FMT_FP8_E4M3>(a, ch, block, transposed, want_codes, any_stats, want_rows, grid, st);
+    else if (fmt == SNIP_FMT_FP4_E2M1) launch_fmt<SNIP_FMT_FP4_E2M1>(a, ch, block, transposed, want_codes, any_stats, want_rows, grid, st);
+    else launch_variant<SNIP_FMT_BF16, SNIP_BLOCK_BLK_128x128, false>(a, ch, false, true, want_rows, grid, st);
     SNIP_CUDA_TRY(cudaGetLastError());
     if (want_stats) {
         rc = launch_reduce(ReduceSets{{a.partials, nullptr}, {stats, nullptr}}, 1, nparts, link, st);
@@ -1201,159 +1270,144 @@ int quantize_impl_full(const void *x, int64_t rows, int64_t cols, int64_t ld, in
     return SNIP_OK;
 }
 
-// One read, two outputs.  blk = false: a = 1x128 tiles as stored, b = 128x1 tiles transposed;
-// blk = true: a = 128x128 blocks as stored, b = the same blocks transposed.
-// Two-output launch with stochastic rounding on the FP4 outputs that ask for it (row/column kinds only).
-template <int FMT_A, int FMT_B, int SR_A, int SR_B>
-static void launch_dual_sr(const DualArgs &d, bool stats, dim3 grid, cudaStream_t st)
-{
-    if (stats) launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, true, SR_A, SR_B>, d, grid, st);
-    else launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, false, SR_A, SR_B>, d, grid, st);
-}
+namespace {
 
-template <int FMT_A, int FMT_B>
-static void launch_dual(const DualArgs &d, bool blk, bool stats, dim3 grid, cudaStream_t st)
+// Checks one tensor and fills its job.
+int fill_job(const DualTask &t, DualJob &d, int &family)
 {
-    if (blk && stats) launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, true, true>, d, grid, st);
-    else if (blk) launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, true, false>, d, grid, st);
-    else if (stats) launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, true>, d, grid, st);
-    else launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, false>, d, grid, st);
-}
-
-template <int FMT_A, int FMT_B, int SR_A = 0, int SR_B = 0>
-static void launch_dual32(const DualArgs &d, bool stats, dim3 grid, cudaStream_t st)
-{
-    if (stats) launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, true, SR_A, SR_B, true>, d, grid, st, kSmemBytes32);
-    else launch_persistent(quantize_dual_kernel<FMT_A, FMT_B, false, false, SR_A, SR_B, true>, d, grid, st, kSmemBytes32);
-}
-
-// kind: SNIP_DUAL_ROW_COLT, SNIP_DUAL_BLK_BLKT or SNIP_DUAL_ROW32_COL32T (power-of-two scales only).
-int quantize_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, int kind, int pow2, const DualOut &oa, const DualOut &ob,
-                       void *ws, size_t ws_bytes, cudaStream_t st, const ChainLink &link)
-{
-    if (!x) return SNIP_ERR_ARG;
-    const bool blk = kind == SNIP_DUAL_BLK_BLKT, sub32 = kind == SNIP_DUAL_ROW32_COL32T;
-    if (sub32 && !pow2) return SNIP_ERR_UNSUPPORTED;
-    if (!valid_dim(rows) || !valid_dim(cols) || ld < cols || (ld % 8) != 0 || rows > INT32_MAX || ld > INT32_MAX) return SNIP_ERR_SHAPE;
-    const DualOut *o[2] = {&oa, &ob};
+    const DualOut *o[2] = {&t.a, &t.b};
+    const bool nv = t.kind == kDualTwoLevel, blk = t.kind == SNIP_DUAL_BLK_BLKT, sub32 = t.kind == SNIP_DUAL_ROW32_COL32T;
+    if (!t.x || (nv && !t.tensor_amax)) return SNIP_ERR_ARG;
+    if (sub32 && !t.pow2) return SNIP_ERR_UNSUPPORTED;
+    if (!valid_dim(t.rows) || !valid_dim(t.cols) || t.ld < t.cols || (t.ld % 8) != 0 || t.rows > INT32_MAX || t.ld > INT32_MAX) return SNIP_ERR_SHAPE;
     for (int i = 0; i < 2; ++i) {
         if (o[i]->fmt != SNIP_FMT_FP8_E4M3 && o[i]->fmt != SNIP_FMT_FP4_E2M1) return SNIP_ERR_UNSUPPORTED;
-        if (!o[i]->codes || !o[i]->scales) return SNIP_ERR_ARG;
-        if (o[i]->sf && !pow2) return SNIP_ERR_UNSUPPORTED;
+        if (!o[i]->codes || (nv ? !o[i]->sf : !o[i]->scales)) return SNIP_ERR_ARG;
+        if (o[i]->sf && !t.pow2 && !nv) return SNIP_ERR_UNSUPPORTED;
         if (!aligned16(o[i]->codes) || !aligned16(o[i]->scales) || (o[i]->sf && !aligned16(o[i]->sf)) ||
             (o[i]->stats && (reinterpret_cast<uintptr_t>(o[i]->stats) & 7u)))
             return SNIP_ERR_ALIGN;
+        if (o[i]->sr && (blk || o[i]->fmt != SNIP_FMT_FP4_E2M1)) return SNIP_ERR_UNSUPPORTED;   // FP4 row / column tiles only
     }
-    if ((oa.stats == nullptr) != (ob.stats == nullptr)) return SNIP_ERR_ARG;
-    if (!aligned16(x)) return SNIP_ERR_ALIGN;
-    const bool stats = oa.stats != nullptr;
-    const size_t one = stats_ws_bytes(rows, cols, false);
-    if (stats && (!ws || ws_bytes < 2 * one)) return SNIP_ERR_WORKSPACE;
-    if (stats && !aligned16(ws)) return SNIP_ERR_ALIGN;
-    int rc = require_sm100();
-    if (rc != SNIP_OK) return rc;
-    const int64_t tr = ceil_div(rows, kTile), tc = ceil_div(cols, kTile);
-    DualArgs d;
+    if ((t.a.stats == nullptr) != (t.b.stats == nullptr)) return SNIP_ERR_ARG;
+    if (!aligned16(t.x) || (reinterpret_cast<uintptr_t>(t.tensor_amax) & 3u)) return SNIP_ERR_ALIGN;
+    const bool stats = t.a.stats != nullptr;
+    const size_t one = stats_ws_bytes(t.rows, t.cols, false);
+    if (stats && (!t.ws || t.ws_bytes < 2 * one)) return SNIP_ERR_WORKSPACE;
+    if (stats && !aligned16(t.ws)) return SNIP_ERR_ALIGN;
+    const int64_t tr = ceil_div(t.rows, kTile), tc = ceil_div(t.cols, kTile);
     for (int i = 0; i < 2; ++i) {
         QuantArgs &q = i ? d.b : d.a;
-        q.x = static_cast<const uint16_t *>(x);
-        q.rows = (int32_t)rows; q.cols = (int32_t)cols; q.ld = (int32_t)ld;
+        q.x = static_cast<const uint16_t *>(t.x);
+        q.rows = (int32_t)t.rows; q.cols = (int32_t)t.cols; q.ld = (int32_t)t.ld;
         q.codes = static_cast<uint8_t *>(o[i]->codes);
         q.scales = o[i]->scales;
-        q.partials = stats ? reinterpret_cast<CtaPartial *>(static_cast<uint8_t *>(ws) + i * one) : nullptr;
+        q.partials = stats ? reinterpret_cast<CtaPartial *>(static_cast<uint8_t *>(t.ws) + i * one) : nullptr;
         q.row_partials = nullptr;
-        q.pow2 = pow2;
+        q.pow2 = t.pow2;
         q.seed = o[i]->seed;
         q.sf = static_cast<uint32_t *>(o[i]->sf);
-        q.tensor_amax = nullptr;
-        q.chain = link.role; q.zero = link.zero; q.zero_words = link.zero_words;
+        q.tensor_amax = t.tensor_amax;
         q.tiles_r = (int32_t)tr; q.tiles_c = (int32_t)tc; q.ntiles = tr * tc;
     }
-    const int64_t nparts = persistent_ctas(tr * tc, oa.sr || ob.sr ? kDualCtasPerSmSr : kDualCtasPerSm);
-    dim3 grid((unsigned)nparts);
-    const bool a8 = oa.fmt == SNIP_FMT_FP8_E4M3, b8 = ob.fmt == SNIP_FMT_FP8_E4M3;
-    constexpr int F8 = SNIP_FMT_FP8_E4M3, F4 = SNIP_FMT_FP4_E2M1;
-    if (sub32 && (oa.sr || ob.sr)) {
-        if ((oa.sr && a8) || (ob.sr && b8)) return SNIP_ERR_UNSUPPORTED;   // stochastic rounding is offered for FP4 codes
-        if (oa.sr && ob.sr && oa.seed == ob.seed) launch_dual32<F4, F4, 1, 2>(d, stats, grid, st);   // one generator call serves both copies
-        else if (oa.sr && ob.sr) launch_dual32<F4, F4, 1, 1>(d, stats, grid, st);
-        else if (oa.sr && b8) launch_dual32<F4, F8, 1, 0>(d, stats, grid, st);
-        else if (oa.sr) launch_dual32<F4, F4, 1, 0>(d, stats, grid, st);
-        else if (a8) launch_dual32<F8, F4, 0, 1>(d, stats, grid, st);
-        else launch_dual32<F4, F4, 0, 1>(d, stats, grid, st);
-    } else if (sub32) {
-        if (a8 && b8) launch_dual32<F8, F8>(d, stats, grid, st);
-        else if (a8) launch_dual32<F8, F4>(d, stats, grid, st);
-        else if (b8) launch_dual32<F4, F8>(d, stats, grid, st);
-        else launch_dual32<F4, F4>(d, stats, grid, st);
-    } else
-    if (oa.sr || ob.sr) {
-        if (blk || (oa.sr && a8) || (ob.sr && b8)) return SNIP_ERR_UNSUPPORTED;   // FP4 row / column tiles only
-        if (oa.sr && ob.sr && oa.seed == ob.seed) launch_dual_sr<F4, F4, 1, 2>(d, stats, grid, st);   // one generator call serves both copies
-        else if (oa.sr && ob.sr) launch_dual_sr<F4, F4, 1, 1>(d, stats, grid, st);
-        else if (oa.sr && b8) launch_dual_sr<F4, F8, 1, 0>(d, stats, grid, st);
-        else if (oa.sr) launch_dual_sr<F4, F4, 1, 0>(d, stats, grid, st);
-        else if (a8) launch_dual_sr<F8, F4, 0, 1>(d, stats, grid, st);
-        else launch_dual_sr<F4, F4, 0, 1>(d, stats, grid, st);
-    } else
-    if (a8 && b8) launch_dual<SNIP_FMT_FP8_E4M3, SNIP_FMT_FP8_E4M3>(d, blk, stats, grid, st);
-    else if (a8) launch_dual<SNIP_FMT_FP8_E4M3, SNIP_FMT_FP4_E2M1>(d, blk, stats, grid, st);
-    else if (b8) launch_dual<SNIP_FMT_FP4_E2M1, SNIP_FMT_FP8_E4M3>(d, blk, stats, grid, st);
-    else launch_dual<SNIP_FMT_FP4_E2M1, SNIP_FMT_FP4_E2M1>(d, blk, stats, grid, st);
-    SNIP_CUDA_TRY(cudaGetLastError());
-    if (stats) {
-        rc = launch_reduce(ReduceSets{{d.a.partials, d.b.partials}, {oa.stats, ob.stats}}, 2, nparts, link, st);
-        if (rc) return rc;
-    }
+    // one generator call serves both copies when they share their seed
+    const int sr_b = !t.b.sr ? 0 : (t.a.sr && t.a.seed == t.b.seed) ? 2 : 1;
+    d.variant = (blk ? kBlkVariant : 0) + dual_variant(t.a.fmt == SNIP_FMT_FP4_E2M1, t.b.fmt == SNIP_FMT_FP4_E2M1, t.a.sr, sr_b);
+    family = nv ? FAM_NV : sub32 ? FAM_32 : FAM_128;
     return SNIP_OK;
 }
 
-// Two-level option (see include/snip.h): both copies of a tensor from one read.
-int quantize_nvfp4_dual_impl(const void *x, int64_t rows, int64_t cols, int64_t ld, const float *tensor_amax, void *codes_a, void *sf_a,
-                             snip_stats_t *stats_a, void *codes_b, void *sf_b, snip_stats_t *stats_b, int rounding, uint64_t seed, void *ws,
-                             size_t ws_bytes, cudaStream_t st, const ChainLink &link)
+int64_t dual_ctas(const DualJob &d) { return persistent_ctas(d.a.ntiles, (d.variant & 28) ? kDualCtasPerSmSr : kDualCtasPerSm); }
+
+template <int FAM, int V>
+void launch_dual(const DualJob &d, const ChainArgs &ch, bool stats, cudaStream_t st)
 {
-    if (rounding != SNIP_ROUND_NEAREST_EVEN && rounding != SNIP_ROUND_STOCHASTIC) return SNIP_ERR_ARG;
-    const bool sr = rounding == SNIP_ROUND_STOCHASTIC;
-    if (!x || !tensor_amax || !codes_a || !sf_a || !codes_b || !sf_b) return SNIP_ERR_ARG;
-    if (!valid_dim(rows) || !valid_dim(cols) || ld < cols || (ld % 8) != 0 || rows > INT32_MAX || ld > INT32_MAX) return SNIP_ERR_SHAPE;
-    if ((stats_a == nullptr) != (stats_b == nullptr)) return SNIP_ERR_ARG;
-    if (!aligned16(x) || !aligned16(codes_a) || !aligned16(sf_a) || !aligned16(codes_b) || !aligned16(sf_b) ||
-        (reinterpret_cast<uintptr_t>(tensor_amax) & 3u) || (stats_a && ((reinterpret_cast<uintptr_t>(stats_a) | reinterpret_cast<uintptr_t>(stats_b)) & 7u)))
-        return SNIP_ERR_ALIGN;
-    const bool stats = stats_a != nullptr;
-    const size_t one = stats_ws_bytes(rows, cols, false);
-    if (stats && (!ws || ws_bytes < 2 * one)) return SNIP_ERR_WORKSPACE;
-    if (stats && !aligned16(ws)) return SNIP_ERR_ALIGN;
+    constexpr size_t smem = FAM == FAM_128 ? kSmemBytes : kSmemBytes32;
+    const dim3 grid((unsigned)dual_ctas(d));
+    if (stats) launch_persistent(quantize_dual_kernel<FAM, V, true>, d, ch, grid, st, smem);
+    else launch_persistent(quantize_dual_kernel<FAM, V, false>, d, ch, grid, st, smem);
+}
+
+template <int FAM>
+void launch_small(const DualGroup &g, bool stats, dim3 grid, cudaStream_t st)
+{
+    constexpr size_t smem = FAM == FAM_128 ? kSmemBytes : kSmemBytes32;
+    if (stats) launch_persistent(quantize_small_kernel<FAM, true>, g, g.chain, grid, st, smem);
+    else launch_persistent(quantize_small_kernel<FAM, false>, g, g.chain, grid, st, smem);
+}
+
+int launch_dual_reduce(const DualTask &t, const DualJob &d, int64_t ctas, const ChainLink &link, cudaStream_t st)
+{
+    if (!t.a.stats) return SNIP_OK;
+    return launch_reduce(ReduceSets{{d.a.partials, d.b.partials}, {t.a.stats, t.b.stats}}, 2, d.a.ntiles < ctas ? d.a.ntiles : ctas, link, st);
+}
+
+}  // namespace
+
+// Both copies of one tensor.
+int quantize_dual_impl(const DualTask &t, cudaStream_t st, const ChainLink &link)
+{
+    DualJob d;
+    int family = 0;
+    int rc = fill_job(t, d, family);
+    if (rc) return rc;
+    rc = require_sm100();
+    if (rc != SNIP_OK) return rc;
+    d.first = 0;
+    const ChainArgs ch = {link.role, link.zero, link.zero_words};
+    const bool stats = t.a.stats != nullptr;
+    if (family == FAM_NV) {
+#define SNIP_LAUNCH(V) case V: launch_dual<FAM_NV, V>(d, ch, stats, st); break;
+        switch (d.variant) { SNIP_NV_VARIANTS(SNIP_LAUNCH) default: return SNIP_ERR_UNSUPPORTED; }
+#undef SNIP_LAUNCH
+    } else if (family == FAM_32) {
+#define SNIP_LAUNCH(V) case V: launch_dual<FAM_32, V>(d, ch, stats, st); break;
+        switch (d.variant) { SNIP_ROWCOL_VARIANTS(SNIP_LAUNCH) default: return SNIP_ERR_UNSUPPORTED; }
+#undef SNIP_LAUNCH
+    } else {
+#define SNIP_LAUNCH(V) case V: launch_dual<FAM_128, V>(d, ch, stats, st); break;
+        switch (d.variant) { SNIP_ROWCOL_VARIANTS(SNIP_LAUNCH) SNIP_BLK_VARIANTS(SNIP_LAUNCH) default: return SNIP_ERR_UNSUPPORTED; }
+#undef SNIP_LAUNCH
+    }
+    SNIP_CUDA_TRY(cudaGetLastError());
+    return launch_dual_reduce(t, d, dual_ctas(d), link, st);
+}
+
+// The quantizers of a linear layer's X, W and dY (`link`: the first member of the chain): one launch where the three fit one wave
+// of small kernels, else one each.
+int quantize_xwd_impl(const DualTask (&t)[3], cudaStream_t st, const ChainLink &link)
+{
+    DualGroup g;
+    int family[3];
+    int64_t total = 0;
+    for (int i = 0; i < 3; ++i) {
+        const int rc = fill_job(t[i], g.job[i], family[i]);
+        if (rc) return rc;
+        g.job[i].first = (int32_t)(total < INT32_MAX ? total : 0);
+        total += g.job[i].a.ntiles;
+    }
     int rc = require_sm100();
     if (rc != SNIP_OK) return rc;
-    const int64_t tr = ceil_div(rows, kTile), tc = ceil_div(cols, kTile);
-    DualArgs d;
-    void *codes[2] = {codes_a, codes_b}, *sf[2] = {sf_a, sf_b};
-    for (int i = 0; i < 2; ++i) {
-        QuantArgs &q = i ? d.b : d.a;
-        q.x = static_cast<const uint16_t *>(x);
-        q.rows = (int32_t)rows; q.cols = (int32_t)cols; q.ld = (int32_t)ld;
-        q.codes = static_cast<uint8_t *>(codes[i]);
-        q.scales = nullptr;
-        q.partials = stats ? reinterpret_cast<CtaPartial *>(static_cast<uint8_t *>(ws) + i * one) : nullptr;
-        q.row_partials = nullptr;
-        q.pow2 = 0;
-        q.seed = seed;
-        q.sf = static_cast<uint32_t *>(sf[i]);
-        q.tensor_amax = tensor_amax;
-        q.chain = link.role; q.zero = link.zero; q.zero_words = link.zero_words;
-        q.tiles_r = (int32_t)tr; q.tiles_c = (int32_t)tc; q.ntiles = tr * tc;
+    const bool stats = t[0].a.stats != nullptr;
+    const bool alike = family[0] == family[1] && family[0] == family[2] && (t[1].a.stats != nullptr) == stats && (t[2].a.stats != nullptr) == stats;
+    if (!alike || total > kDualCtasPerSmSr * (int64_t)gemm_sm_count()) {
+        ChainLink beside;
+        beside.role = CHAIN_BESIDE;
+        beside.jobs = link.jobs;
+        for (int i = 0; i < 3; ++i) {
+            rc = quantize_dual_impl(t[i], st, i ? beside : link);
+            if (rc) return rc;
+        }
+        return SNIP_OK;
     }
-    const int64_t nparts = persistent_ctas(tr * tc, sr ? kDualCtasPerSmSr : kDualCtasPerSm);
-    dim3 grid((unsigned)nparts);
-    if (stats && sr) launch_persistent(quantize_nvfp4_dual_kernel<true, true>, d, grid, st, kSmemBytes32);
-    else if (stats) launch_persistent(quantize_nvfp4_dual_kernel<true, false>, d, grid, st, kSmemBytes32);
-    else if (sr) launch_persistent(quantize_nvfp4_dual_kernel<false, true>, d, grid, st, kSmemBytes32);
-    else launch_persistent(quantize_nvfp4_dual_kernel<false, false>, d, grid, st, kSmemBytes32);
+    g.chain = {link.role, link.zero, link.zero_words};
+    const dim3 grid((unsigned)total);
+    if (family[0] == FAM_128) launch_small<FAM_128>(g, stats, grid, st);
+    else if (family[0] == FAM_32) launch_small<FAM_32>(g, stats, grid, st);
+    else launch_small<FAM_NV>(g, stats, grid, st);
     SNIP_CUDA_TRY(cudaGetLastError());
-    if (stats) {
-        rc = launch_reduce(ReduceSets{{d.a.partials, d.b.partials}, {stats_a, stats_b}}, 2, nparts, link, st);
+    for (int i = 0; i < 3; ++i) {
+        rc = launch_dual_reduce(t[i], g.job[i], total, link, st);
         if (rc) return rc;
     }
     return SNIP_OK;
@@ -1375,8 +1429,11 @@ extern "C" int snip_quantize_nvfp4_dual(const void *x, int64_t rows, int64_t col
                                         void *sf_stored, snip_stats_t *stats_stored, void *codes_transposed, void *sf_transposed,
                                         snip_stats_t *stats_transposed, int rounding, uint64_t seed, void *ws, size_t ws_bytes, void *stream)
 {
-    return snip::quantize_nvfp4_dual_impl(x, rows, cols, ld, tensor_amax, codes_stored, sf_stored, stats_stored, codes_transposed, sf_transposed,
-                                          stats_transposed, rounding, seed, ws, ws_bytes, static_cast<cudaStream_t>(stream), snip::ChainLink());
+    using namespace snip;
+    if (rounding != SNIP_ROUND_NEAREST_EVEN && rounding != SNIP_ROUND_STOCHASTIC) return SNIP_ERR_ARG;
+    const DualTask t = two_level_task(x, rows, cols, ld, tensor_amax, codes_stored, sf_stored, stats_stored, codes_transposed, sf_transposed, stats_transposed,
+                                      rounding, seed, ws, ws_bytes);
+    return quantize_dual_impl(t, static_cast<cudaStream_t>(stream), ChainLink());
 }
 
 extern "C" int snip_quantize_sizes(int64_t rows, int64_t cols, int fmt, int block, uint32_t flags,
@@ -1513,8 +1570,8 @@ extern "C" int snip_quantize_dual(const void *x, int64_t rows, int64_t cols, int
     if ((as_stored->rounding & ~1) || (transposed->rounding & ~1)) return SNIP_ERR_ARG;
     const DualOut oa = {as_stored->fmt, as_stored->codes, as_stored->scales, as_stored->sf, as_stored->stats, as_stored->rounding, as_stored->seed};
     const DualOut ob = {transposed->fmt, transposed->codes, transposed->scales, transposed->sf, transposed->stats, transposed->rounding, transposed->seed};
-    return quantize_dual_impl(x, rows, cols, ld, kind, pow2_scale ? 1 : 0, oa, ob, ws, ws_bytes,
-                              static_cast<cudaStream_t>(stream), ChainLink());
+    const DualTask t = {x, rows, cols, ld, kind, pow2_scale ? 1 : 0, nullptr, oa, ob, ws, ws_bytes};
+    return quantize_dual_impl(t, static_cast<cudaStream_t>(stream), ChainLink());
 }
 
 // ---- stochastic rounding (paper Sec. 6.1) ------------------------------------------------------
