@@ -5,20 +5,26 @@
 // registers.  The scheme-generation step needs the error of every option (Sec. 4.4), not only of
 // the format currently in use.
 //
-// One CTA owns a 128x128 tile, each thread an 8x8 sub-block (the quantizer's load pattern).  The
-// arithmetic per option is the quantizer's: S = FPX_MAX/amax (binary32 quotient), code =
-// RNE_fmt(fl32(x*S)), error term x - value(code)/S.  HBM-bound on the read (2 bytes per element)
-// only when one option is selected; with all four options of X / dY the conversions make it
-// ALU-bound at roughly 1.5x the read time, still far below four separate passes.
+// One persistent launch for all six tensors, three CTAs of 256 threads per SM; a CTA takes 128x128 tiles, each thread an 8x8 sub-block
+// that it fetches itself (cp.async into a private slot, one tile ahead).  The arithmetic per option is the quantizer's: S =
+// FPX_MAX/amax (binary32 quotient, one division per tile and format, shared through shared memory), code = RNE_fmt(fl32(x*S)), error
+// term x - value(code)/S.  X and dY with four options are bound by instruction issue (about 17 per element), Y, dX and dW by HBM:
+// every CTA walks both kinds of tensor side by side, in proportion, so that the two overlap.  A reduction of the CTAs' sums follows.
+// Six tensors of an 8192 x 3200 x 9600 linear: 250 us as twelve launches of one tile per CTA, with the divisions repeated by every
+// thread and the elements unpacked once per option.
 #include "common.cuh"
 #include "quant_device.cuh"
 
 namespace snip {
 
+int gemm_sm_count();  // gemm.cu
+
 namespace {
 
 constexpr int kTile = 128;
 constexpr int kThreads = 256;
+constexpr int kCtas = 3;             // per SM
+constexpr int kSlotBytes = kTile * kTile * 2;
 
 enum { MODE_PLAIN = 0, MODE_BLK = 1, MODE_ROWCOL = 2 };
 
@@ -28,29 +34,29 @@ struct StatsPartial {
     double v[8];
 };
 
-struct LayerStatsArgs {
+struct StatsTensor {
     const uint16_t *x;
-    int64_t rows, cols;
-    StatsPartial *partials;
+    int32_t rows, cols, tiles_c, ntiles;
+    int32_t mode, out;               // out: index of the tensor in the result
+    StatsPartial *partials;          // one per CTA that has tiles of it
+};
+// Tensors with error sums (heavy) and without (light), each list one sequence of tiles dealt to the CTAs in turn.
+struct LayerStatsArgs {
+    StatsTensor t[6];
+    int32_t nheavy, nlight;          // t[0 .. nheavy), t[nheavy .. nheavy + nlight)
 };
 
-// Adds, for the 8 elements of one 128-bit load, the squared error under format FMT with the scale
-// pairs s2 / negated reciprocal pairs n2 (element pair i uses s2[i], n2[i]).
-template <int FMT>
-__device__ __forceinline__ void err8(const uint4 &v, const float2 (&s2)[4], const float2 (&n2)[4], float2 &se2)
-{
-    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-    for (int i = 0; i < 4; ++i) {
-        const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
-        const float2 t = __fmul2_rn(x, s2[i]);
-        float2 d;
-        if (FMT == SNIP_FMT_FP8_E4M3) d = dec_e4m3x2(cvt_e4m3x2(t.x, t.y));
-        else d = dec_e2m1x2(cvt_e2m1x2(t.x, t.y));
-        const float2 e = __ffma2_rn(d, n2[i], x);
-        se2 = __ffma2_rn(e, e, se2);
-    }
-}
+struct Scales {                      // of one tile line: scale and negated reciprocal for both formats
+    float s8, n8, s4, n4;
+};
+struct Shared {
+    __align__(16) uint8_t slot[kSlotBytes];
+    uint32_t col_amax[8][kTile / 2];  // packed bf16 pairs, one row per warp
+    __align__(16) Scales row[kTile];
+    __align__(16) Scales col[kTile];
+    uint32_t blk_amax[2][8];
+    double red[8][5];
+};
 
 template <int FMT>
 __device__ __forceinline__ float ninv_of(float amax)
@@ -58,203 +64,346 @@ __device__ __forceinline__ float ninv_of(float amax)
     constexpr float kMax = (FMT == SNIP_FMT_FP8_E4M3) ? 448.0f : 6.0f;
     return -amax * (1.0f / kMax);
 }
-
-// One format's error sums for this thread's 8x8 sub-block.  row_am[p]: amax of the 1x128 tile of
-// row p; col_am[j]: amax of the 128x1 tile of column j; blk_am: amax of the 128x128 block.
-template <int FMT, int MODE>
-__device__ __forceinline__ void format_errors(const uint4 (&v)[8], const float (&row_am)[8], const float (&col_am)[8], float blk_am,
-                                              float &err_a, float &err_b)
+template <bool F8, bool F4>
+__device__ __forceinline__ Scales scales_of(float am)
 {
-    float2 ea = make_float2(0.0f, 0.0f), eb = make_float2(0.0f, 0.0f);
-    if (MODE == MODE_BLK) {
-        const float s = tile_scale<FMT>(blk_am, 0), n = ninv_of<FMT>(blk_am);
-        float2 s2[4], n2[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) { s2[i] = make_float2(s, s); n2[i] = make_float2(n, n); }
-#pragma unroll
-        for (int p = 0; p < 8; ++p) err8<FMT>(v[p], s2, n2, ea);
-    } else {
-        float2 cs2[4], cn2[4];
-#pragma unroll
-        for (int i = 0; i < 4; ++i) {
-            cs2[i] = make_float2(tile_scale<FMT>(col_am[2 * i], 0), tile_scale<FMT>(col_am[2 * i + 1], 0));
-            cn2[i] = make_float2(ninv_of<FMT>(col_am[2 * i]), ninv_of<FMT>(col_am[2 * i + 1]));
-        }
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {
-            const float s = tile_scale<FMT>(row_am[p], 0), n = ninv_of<FMT>(row_am[p]);
-            float2 rs2[4], rn2[4];
-#pragma unroll
-            for (int i = 0; i < 4; ++i) { rs2[i] = make_float2(s, s); rn2[i] = make_float2(n, n); }
-            err8<FMT>(v[p], rs2, rn2, ea);
-            err8<FMT>(v[p], cs2, cn2, eb);
-        }
-    }
-    err_a = ea.x + ea.y;
-    err_b = eb.x + eb.y;
+    Scales s = {0.0f, 0.0f, 0.0f, 0.0f};
+    if (F8) { s.s8 = tile_scale<SNIP_FMT_FP8_E4M3>(am, 0); s.n8 = ninv_of<SNIP_FMT_FP8_E4M3>(am); }
+    if (F4) { s.s4 = tile_scale<SNIP_FMT_FP4_E2M1>(am, 0); s.n4 = ninv_of<SNIP_FMT_FP4_E2M1>(am); }
+    return s;
 }
 
-template <int MODE, bool F8, bool F4>
-__global__ void __launch_bounds__(kThreads) layer_stats_kernel(const LayerStatsArgs a)
+// Adds the squared error of an element pair under format FMT.
+template <int FMT>
+__device__ __forceinline__ void err_pair(const float2 x, const float2 s, const float2 n, float2 &se2)
 {
-    __shared__ uint32_t col_amax[8][kTile / 2];  // packed bf16 pairs, one row per warp
-    __shared__ float col_amax_f[kTile];
-    __shared__ float red[8][5];
-    __shared__ float red_m[8];
+    const float2 t = __fmul2_rn(x, s);
+    const float2 d = (FMT == SNIP_FMT_FP8_E4M3) ? dec_e4m3x2(cvt_e4m3x2(t.x, t.y)) : dec_e2m1x2(cvt_e2m1x2(t.x, t.y));
+    const float2 e = __ffma2_rn(d, n, x);
+    se2 = __ffma2_rn(e, e, se2);
+}
 
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
-    const int tx = tid & 15, ty = tid >> 4;
-    const int64_t r0 = (int64_t)blockIdx.y * kTile, c0 = (int64_t)blockIdx.x * kTile;
-    const int64_t rbase = r0 + 8 * ty, cbase = c0 + 8 * tx;
-
-    uint4 v[8];
+// A CTA's walk over one list: tile `tile` of tensor `j`, in steps of the grid.
+struct Walk {
+    int j, end, tile, left;          // left: items of the whole walk that have not been taken
+    __device__ __forceinline__ void start(const LayerStatsArgs &a, int first, int count)
     {
-        const uint16_t *xb = a.x + rbase * a.cols + cbase;
-        const bool ok = rbase < a.rows && cbase < a.cols;  // dims are multiples of 64: all 64 elements or none
-        const uint32_t ld32 = (uint32_t)a.cols;
-#pragma unroll
-        for (int p = 0; p < 8; ++p) v[p] = ok ? __ldg(reinterpret_cast<const uint4 *>(xb + p * ld32)) : make_uint4(0, 0, 0, 0);
+        j = first; end = first + count; left = 0;
+        int base = 0;
+        for (int i = first; i < end; ++i) {
+            const int rel = offset(base);
+            if (rel < a.t[i].ntiles) left += (a.t[i].ntiles - rel + (int)gridDim.x - 1) / (int)gridDim.x;
+            base = (base + a.t[i].ntiles) % (int)gridDim.x;
+        }
+        seq = 0;
+        tile = offset(0);
+        skip(a);
     }
-
-    float row_am[8], col_am[8], blk_am = 0.0f;
-#pragma unroll
-    for (int p = 0; p < 8; ++p) { row_am[p] = 0.0f; col_am[p] = 0.0f; }
-    if (MODE == MODE_ROWCOL) {
-        // rows: fold the 8 columns of this thread, pack two rows per register, reduce over the 16 lanes of a row
-        uint32_t pk[4];
-#pragma unroll
-        for (int q = 0; q < 4; ++q) {
-            uint32_t m0 = absmax2(absmax2(absmax2(absmax2(0u, v[2 * q].x), v[2 * q].y), v[2 * q].z), v[2 * q].w);
-            uint32_t m1 = absmax2(absmax2(absmax2(absmax2(0u, v[2 * q + 1].x), v[2 * q + 1].y), v[2 * q + 1].z), v[2 * q + 1].w);
-            m0 = max2(m0, m0 >> 16);
-            m1 = max2(m1, m1 << 16);
-            pk[q] = (m0 & 0xFFFFu) | (m1 & 0xFFFF0000u);
-        }
-#pragma unroll
-        for (int off = 1; off < 16; off <<= 1)
-#pragma unroll
-            for (int q = 0; q < 4; ++q) pk[q] = max2(pk[q], __shfl_xor_sync(0xFFFFFFFFu, pk[q], off));
-#pragma unroll
-        for (int q = 0; q < 4; ++q) { row_am[2 * q] = bf16lo(pk[q]); row_am[2 * q + 1] = bf16hi(pk[q]); }
-        // columns: this thread's 8 rows, the two row groups of the warp, then the 8 warps through shared memory
-        uint32_t cm[4] = {0, 0, 0, 0};
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {
-            cm[0] = absmax2(cm[0], v[p].x);
-            cm[1] = absmax2(cm[1], v[p].y);
-            cm[2] = absmax2(cm[2], v[p].z);
-            cm[3] = absmax2(cm[3], v[p].w);
-        }
-#pragma unroll
-        for (int q = 0; q < 4; ++q) cm[q] = max2(cm[q], __shfl_xor_sync(0xFFFFFFFFu, cm[q], 16));
-        if (lane < 16) *reinterpret_cast<uint4 *>(&col_amax[warp][4 * tx]) = make_uint4(cm[0], cm[1], cm[2], cm[3]);
-        __syncthreads();
-        if (tid < kTile) {
-            const uint16_t *h = reinterpret_cast<const uint16_t *>(&col_amax[0][0]);
-            uint32_t m = 0;
-#pragma unroll
-            for (int w = 0; w < 8; ++w) m = max(m, (uint32_t)h[w * kTile + tid]);  // non-negative bf16: integer order
-            col_amax_f[tid] = __uint_as_float(m << 16);
-        }
-        __syncthreads();
-        const float4 c0v = *reinterpret_cast<const float4 *>(&col_amax_f[8 * tx]);
-        const float4 c1v = *reinterpret_cast<const float4 *>(&col_amax_f[8 * tx + 4]);
-        col_am[0] = c0v.x; col_am[1] = c0v.y; col_am[2] = c0v.z; col_am[3] = c0v.w;
-        col_am[4] = c1v.x; col_am[5] = c1v.y; col_am[6] = c1v.z; col_am[7] = c1v.w;
-    } else if (MODE == MODE_BLK) {
-        uint32_t m = 0;
-#pragma unroll
-        for (int p = 0; p < 8; ++p) m = absmax2(absmax2(absmax2(absmax2(m, v[p].x), v[p].y), v[p].z), v[p].w);
-#pragma unroll
-        for (int off = 1; off < 32; off <<= 1) m = max2(m, __shfl_xor_sync(0xFFFFFFFFu, m, off));
-        if (lane == 0) red_m[warp] = fmaxf(bf16lo(m), bf16hi(m));
-        __syncthreads();
-        blk_am = red_m[0];
-#pragma unroll
-        for (int w = 1; w < 8; ++w) blk_am = fmaxf(blk_am, red_m[w]);
-    }
-
-    float acc[5] = {0.0f, 0.0f, 0.0f, 0.0f, 0.0f};
+    __device__ __forceinline__ void next(const LayerStatsArgs &a)
     {
-        float2 sx2 = make_float2(0.0f, 0.0f);
-#pragma unroll
-        for (int p = 0; p < 8; ++p) {
-            const uint32_t w[4] = {v[p].x, v[p].y, v[p].z, v[p].w};
-#pragma unroll
-            for (int i = 0; i < 4; ++i) {
-                const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
-                sx2 = __ffma2_rn(x, x, sx2);
-            }
+        --left;
+        tile += (int)gridDim.x;
+        skip(a);
+    }
+private:
+    int seq;                         // position of tensor j's first tile in the sequence, modulo the grid
+    __device__ __forceinline__ int offset(int base) const
+    {
+        const int r = (int)blockIdx.x - base;
+        return r < 0 ? r + (int)gridDim.x : r;
+    }
+    __device__ __forceinline__ void skip(const LayerStatsArgs &a)
+    {
+        while (j < end && tile >= a.t[j].ntiles) {
+            seq = (seq + a.t[j].ntiles) % (int)gridDim.x;
+            tile = offset(seq);
+            ++j;
         }
-        acc[0] = sx2.x + sx2.y;
     }
-    if (MODE != MODE_PLAIN) {
-        if (F8) format_errors<SNIP_FMT_FP8_E4M3, MODE>(v, row_am, col_am, blk_am, acc[1], acc[2]);
-        if (F4) format_errors<SNIP_FMT_FP4_E2M1, MODE>(v, row_am, col_am, blk_am, acc[3], acc[4]);
-    }
+};
 
+struct Item {
+    int j, tile;                     // j < 0: none
+};
+
+__device__ __forceinline__ void fetch(const LayerStatsArgs &a, const Item it, uint8_t *slot)
+{
+    if (it.j >= 0) {
+        const StatsTensor &t = a.t[it.j];
+        const int tid = threadIdx.x, tr = it.tile / t.tiles_c, tc = it.tile - tr * t.tiles_c;
+        const int r = tr * kTile + 8 * (tid >> 4), c = tc * kTile + 8 * (tid & 15);
+        const bool ok = r < t.rows && c < t.cols;    // dims are multiples of 64: all 64 elements or none
+        const uint16_t *src = t.x + (ok ? (int64_t)r * t.cols + c : 0);
+        const uint32_t step = ok ? (uint32_t)t.cols : 0u, dst = (uint32_t)__cvta_generic_to_shared(slot) + tid * 16;
+        const int nbytes = ok ? 16 : 0;              // 0: the slot is zero-filled, nothing is read
+#pragma unroll
+        for (int p = 0; p < 8; ++p)
+            asm volatile("cp.async.cg.shared.global [%0], [%1], 16, %2;" ::"r"(dst + p * (kThreads * 16)), "l"(src + p * step), "r"(nbytes) : "memory");
+    }
+    asm volatile("cp.async.commit_group;" ::: "memory");
+}
+
+// The CTA's sums of one tensor -> its partial (block reduction in a fixed order); the sums start again at zero.
+__device__ __forceinline__ void flush(const StatsTensor &t, int slot, Shared &sh, double (&acc)[5])
+{
+    const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
 #pragma unroll
     for (int k = 0; k < 5; ++k) {
 #pragma unroll
         for (int off = 16; off > 0; off >>= 1) acc[k] += __shfl_xor_sync(0xFFFFFFFFu, acc[k], off);
     }
+    __syncthreads();
     if (lane == 0) {
 #pragma unroll
-        for (int k = 0; k < 5; ++k) red[warp][k] = acc[k];
+        for (int k = 0; k < 5; ++k) sh.red[warp][k] = acc[k];
     }
     __syncthreads();
-    if (tid < 5) {
+    if (threadIdx.x < 5) {
         double d = 0.0;
 #pragma unroll
-        for (int w = 0; w < 8; ++w) d += (double)red[w][tid];
-        a.partials[(int64_t)blockIdx.y * gridDim.x + blockIdx.x].v[tid] = d;
+        for (int w = 0; w < 8; ++w) d += sh.red[w][threadIdx.x];
+        t.partials[slot].v[threadIdx.x] = d;
     }
+#pragma unroll
+    for (int k = 0; k < 5; ++k) acc[k] = 0.0;
 }
 
-// Fixed-order sum of the per-CTA partials; dst[k] (null = skip) receives column k.
-struct ReduceDst {
-    double *p[5];
-};
-__global__ void __launch_bounds__(1024) layer_stats_reduce_kernel(const StatsPartial *partials, int64_t n, const ReduceDst dst)
+__device__ __forceinline__ int first_tile(const LayerStatsArgs &a, int list, int j)
 {
-    __shared__ double sh[32][5];
-    asm volatile("griddepcontrol.wait;" ::: "memory");
-    double d[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
-    for (int64_t i = threadIdx.x; i < n; i += 1024) {
+    int base = 0;
+    for (int i = list; i < j; ++i) base = (base + a.t[i].ntiles) % (int)gridDim.x;
+    const int r = (int)blockIdx.x - base;
+    return r < 0 ? r + (int)gridDim.x : r;
+}
+
+template <bool F8, bool F4>
+__global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __grid_constant__ LayerStatsArgs a)
+{
+    extern __shared__ __align__(128) uint8_t smem[];
+    Shared &sh = *reinterpret_cast<Shared *>(smem);
+    const uint4 *slot = reinterpret_cast<const uint4 *>(sh.slot) + threadIdx.x;
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
+    const int tx = tid & 15, ty = tid >> 4;
+
+    Walk heavy, light;
+    heavy.start(a, 0, a.nheavy);
+    light.start(a, a.nheavy, a.nlight);
+    const int nh = heavy.left, nl = light.left;
+    // next item: the list of which the smaller share has been taken
+    auto take = [&]() -> Item {
+        if (heavy.left == 0 && light.left == 0) return {-1, 0};
+        const bool h = light.left == 0 || (heavy.left > 0 && (int64_t)heavy.left * nl >= (int64_t)light.left * nh);
+        Walk &w = h ? heavy : light;
+        const Item it = {w.j, w.tile};
+        w.next(a);
+        return it;
+    };
+    double hacc[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, lacc = 0.0;
+    int hj = -1, lj = -1, parity = 0;
+    auto flush_heavy = [&]() { if (hj >= 0) flush(a.t[hj], first_tile(a, 0, hj), sh, hacc); };
+    auto flush_light = [&]() {
+        if (lj < 0) return;
+        double t[5] = {lacc, 0.0, 0.0, 0.0, 0.0};
+        flush(a.t[lj], first_tile(a, a.nheavy, lj), sh, t);
+        lacc = 0.0;
+    };
+
+    Item cur = take();
+    fetch(a, cur, sh.slot);
+    while (cur.j >= 0) {
+        const Item nxt = take();
+        asm volatile("cp.async.wait_group 0;" ::: "memory");
+        const int mode = a.t[cur.j].mode;
+        float2 sx2 = make_float2(0.0f, 0.0f);
+        if (mode == MODE_PLAIN) {
+            if (cur.j != lj) { flush_light(); lj = cur.j; }
 #pragma unroll
-        for (int k = 0; k < 5; ++k) d[k] += partials[i].v[k];
+            for (int p = 0; p < 8; ++p) {
+                const uint4 v = slot[p * kThreads];
+                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
+                    sx2 = __ffma2_rn(x, x, sx2);
+                }
+            }
+            fetch(a, nxt, sh.slot);
+            lacc += (double)(sx2.x + sx2.y);
+        } else {
+            if (cur.j != hj) { flush_heavy(); hj = cur.j; }
+            const bool rowcol = mode == MODE_ROWCOL;
+            float2 e8a = make_float2(0.0f, 0.0f), e8b = e8a, e4a = e8a, e4b = e8a;
+            // maxima (signs are garbage until masked: max.xorsign.abs keeps magnitudes only)
+            uint32_t rmax[8], cm[4] = {0, 0, 0, 0};
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                const uint4 v = slot[p * kThreads];
+                rmax[p] = absmax2x(absmax2x(v.x, v.y), absmax2x(v.z, v.w));
+                cm[0] = absmax2x(cm[0], v.x);
+                cm[1] = absmax2x(cm[1], v.y);
+                cm[2] = absmax2x(cm[2], v.z);
+                cm[3] = absmax2x(cm[3], v.w);
+            }
+            if (rowcol) {
+                // rows: exchange-halving butterfly over the 16 lanes of a row group; lane tx ends up with rows 4 bit3 + 2 bit2 + {0, 1}
+                // and derives the scales of the one its bit 0 names
+                uint32_t pk[4];
+#pragma unroll
+                for (int q = 0; q < 4; ++q)
+                    pk[q] = max2(__byte_perm(rmax[2 * q], rmax[2 * q + 1], 0x5410) & 0x7FFF7FFFu, __byte_perm(rmax[2 * q], rmax[2 * q + 1], 0x7632) & 0x7FFF7FFFu);
+                const bool b3 = (tx & 8) != 0, b2 = (tx & 4) != 0;
+                uint32_t k0 = b3 ? pk[2] : pk[0], k1 = b3 ? pk[3] : pk[1];
+                const uint32_t g0 = b3 ? pk[0] : pk[2], g1 = b3 ? pk[1] : pk[3];
+                k0 = max2(k0, __shfl_xor_sync(0xFFFFFFFFu, g0, 8));
+                k1 = max2(k1, __shfl_xor_sync(0xFFFFFFFFu, g1, 8));
+                uint32_t k = b2 ? k1 : k0;
+                const uint32_t g = b2 ? k0 : k1;
+                k = max2(k, __shfl_xor_sync(0xFFFFFFFFu, g, 4));
+                k = max2(k, __shfl_xor_sync(0xFFFFFFFFu, k, 2));
+                k = max2(k, __shfl_xor_sync(0xFFFFFFFFu, k, 1));
+                const float am = (tx & 1) ? bf16hi(k) : bf16lo(k);
+                const Scales rs = scales_of<F8, F4>(am);
+                if (!(tx & 2)) sh.row[8 * ty + ((tx >> 3) & 1) * 4 + ((tx >> 2) & 1) * 2 + (tx & 1)] = rs;
+                // columns: the two row groups of a warp, then the 8 warps through shared memory
+#pragma unroll
+                for (int q = 0; q < 4; ++q) cm[q] = absmax2x(cm[q], __shfl_xor_sync(0xFFFFFFFFu, cm[q], 16));
+                if (lane < 16) *reinterpret_cast<uint4 *>(&sh.col_amax[warp][4 * tx]) = make_uint4(cm[0], cm[1], cm[2], cm[3]);
+                __syncthreads();
+                if (tid < kTile) {
+                    const uint16_t *h = reinterpret_cast<const uint16_t *>(&sh.col_amax[0][0]);
+                    uint32_t m = 0;
+#pragma unroll
+                    for (int w = 0; w < 8; ++w) m = max(m, (uint32_t)h[w * kTile + tid] & 0x7FFFu);   // non-negative bf16: integer order
+                    sh.col[tid] = scales_of<F8, F4>(__uint_as_float(m << 16));
+                }
+                __syncthreads();
+                float2 cs8[4], cn8[4], cs4[4], cn4[4];
+#pragma unroll
+                for (int i = 0; i < 4; ++i) {
+                    const float4 c0 = *reinterpret_cast<const float4 *>(&sh.col[8 * tx + 2 * i]), c1 = *reinterpret_cast<const float4 *>(&sh.col[8 * tx + 2 * i + 1]);
+                    cs8[i] = make_float2(c0.x, c1.x); cn8[i] = make_float2(c0.y, c1.y);
+                    cs4[i] = make_float2(c0.z, c1.z); cn4[i] = make_float2(c0.w, c1.w);
+                }
+#pragma unroll
+                for (int p = 0; p < 8; ++p) {
+                    const uint4 v = slot[p * kThreads];
+                    const float4 r = *reinterpret_cast<const float4 *>(&sh.row[8 * ty + p]);
+                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
+                        sx2 = __ffma2_rn(x, x, sx2);
+                        if (F8) {
+                            err_pair<SNIP_FMT_FP8_E4M3>(x, make_float2(r.x, r.x), make_float2(r.y, r.y), e8a);
+                            err_pair<SNIP_FMT_FP8_E4M3>(x, cs8[i], cn8[i], e8b);
+                        }
+                        if (F4) {
+                            err_pair<SNIP_FMT_FP4_E2M1>(x, make_float2(r.z, r.z), make_float2(r.w, r.w), e4a);
+                            err_pair<SNIP_FMT_FP4_E2M1>(x, cs4[i], cn4[i], e4b);
+                        }
+                    }
+                }
+            } else {
+                uint32_t m = absmax2x(absmax2x(cm[0], cm[1]), absmax2x(cm[2], cm[3])) & 0x7FFF7FFFu;
+                m = __reduce_max_sync(0xFFFFFFFFu, max(m & 0xFFFFu, m >> 16));
+                parity ^= 1;   // the other half may still be read by warps that are behind
+                if (lane == 0) sh.blk_amax[parity][warp] = m;
+                __syncthreads();
+                uint32_t bm = sh.blk_amax[parity][0];
+#pragma unroll
+                for (int w = 1; w < 8; ++w) bm = max(bm, sh.blk_amax[parity][w]);
+                const Scales s = scales_of<F8, F4>(__uint_as_float(bm << 16));
+                const float2 s8 = make_float2(s.s8, s.s8), n8 = make_float2(s.n8, s.n8), s4 = make_float2(s.s4, s.s4), n4 = make_float2(s.n4, s.n4);
+#pragma unroll
+                for (int p = 0; p < 8; ++p) {
+                    const uint4 v = slot[p * kThreads];
+                    const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
+                        sx2 = __ffma2_rn(x, x, sx2);
+                        if (F8) err_pair<SNIP_FMT_FP8_E4M3>(x, s8, n8, e8a);
+                        if (F4) err_pair<SNIP_FMT_FP4_E2M1>(x, s4, n4, e4a);
+                    }
+                }
+            }
+            fetch(a, nxt, sh.slot);
+            hacc[0] += (double)(sx2.x + sx2.y);
+            if (F8) { hacc[1] += (double)(e8a.x + e8a.y); hacc[2] += (double)(e8b.x + e8b.y); }
+            if (F4) { hacc[3] += (double)(e4a.x + e4a.y); hacc[4] += (double)(e4b.x + e4b.y); }
+        }
+        cur = nxt;
+    }
+    flush_heavy();
+    flush_light();
+}
+
+// Fixed-order sums of the CTAs' partials, one block per tensor of the result; every value of the result is written (0 for what was not
+// asked for).
+struct ReduceArgs {
+    const StatsPartial *partials[6];   // null: tensor not given
+    int32_t n[6];
+    uint32_t fmt_mask;
+    snip_layer_stats_t *out;
+};
+__global__ void __launch_bounds__(256) layer_stats_reduce_kernel(const ReduceArgs a)
+{
+    __shared__ double sh[8][5];
+    asm volatile("griddepcontrol.wait;" ::: "memory");
+    const int i = blockIdx.x;
+    double d[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+    if (a.partials[i]) {
+        for (int k = threadIdx.x; k < a.n[i]; k += 256) {
+#pragma unroll
+            for (int c = 0; c < 5; ++c) d[c] += a.partials[i][k].v[c];
+        }
     }
 #pragma unroll
-    for (int k = 0; k < 5; ++k) {
+    for (int c = 0; c < 5; ++c) {
 #pragma unroll
-        for (int off = 16; off > 0; off >>= 1) d[k] += __shfl_xor_sync(0xFFFFFFFFu, d[k], off);
+        for (int off = 16; off > 0; off >>= 1) d[c] += __shfl_xor_sync(0xFFFFFFFFu, d[c], off);
     }
     const int lane = threadIdx.x & 31, warp = threadIdx.x >> 5;
     if (lane == 0) {
 #pragma unroll
-        for (int k = 0; k < 5; ++k) sh[warp][k] = d[k];
+        for (int c = 0; c < 5; ++c) sh[warp][c] = d[c];
     }
     __syncthreads();
-    if (threadIdx.x < 5 && dst.p[threadIdx.x]) {
-        double t = 0.0;
-        for (int w = 0; w < 32; ++w) t += sh[w][threadIdx.x];
-        *dst.p[threadIdx.x] = t;
+    if (threadIdx.x == 0) {
+        double t[5];
+#pragma unroll
+        for (int c = 0; c < 5; ++c) {
+            t[c] = 0.0;
+            for (int w = 0; w < 8; ++w) t[c] += sh[w][c];
+        }
+        a.out->sumsq[i] = t[0];
+        const int q = i == 0 ? 0 : i == 1 ? 1 : i == 3 ? 2 : -1;   // X, W, dY have error sums
+        if (q >= 0) {
+#pragma unroll
+            for (int f = 0; f < 2; ++f) {
+                const bool on = (a.fmt_mask & (2u << f)) != 0;
+                a.out->sumsq_err[q][f][SNIP_BLOCK_ROW_1x128] = on && q != 1 ? t[1 + 2 * f] : 0.0;
+                a.out->sumsq_err[q][f][SNIP_BLOCK_COL_128x1] = on && q != 1 ? t[2 + 2 * f] : 0.0;
+                a.out->sumsq_err[q][f][SNIP_BLOCK_BLK_128x128] = on && q == 1 ? t[1 + 2 * f] : 0.0;
+            }
+        }
     }
-}
-
-template <int MODE>
-void launch_mode(const LayerStatsArgs &a, uint32_t fmt_mask, dim3 grid, cudaStream_t st)
-{
-    const bool f8 = (fmt_mask & 2u) != 0, f4 = (fmt_mask & 4u) != 0;
-    if (f8 && f4) layer_stats_kernel<MODE, true, true><<<grid, kThreads, 0, st>>>(a);
-    else if (f8) layer_stats_kernel<MODE, true, false><<<grid, kThreads, 0, st>>>(a);
-    else layer_stats_kernel<MODE, false, true><<<grid, kThreads, 0, st>>>(a);
 }
 
 size_t tensor_ws_bytes(int64_t rows, int64_t cols)
 {
     return align_up((size_t)(ceil_div(rows, kTile) * ceil_div(cols, kTile)) * sizeof(StatsPartial), 256);
+}
+
+template <bool F8, bool F4>
+int launch_stats(const LayerStatsArgs &a, int grid, cudaStream_t st)
+{
+    auto kern = layer_stats_kernel<F8, F4>;
+    SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared)));
+    kern<<<grid, kThreads, sizeof(Shared), st>>>(a);
+    SNIP_CUDA_TRY(cudaGetLastError());
+    return SNIP_OK;
 }
 
 }  // namespace
@@ -265,7 +414,6 @@ extern "C" int snip_layer_stats_workspace(int64_t M, int64_t N, int64_t K, size_
     using namespace snip;
     if (!ws_bytes) return SNIP_ERR_ARG;
     if (!valid_dim(M) || !valid_dim(N) || !valid_dim(K)) return SNIP_ERR_SHAPE;
-    // one scratch region per tensor, so that the six passes need no ordering among themselves
     *ws_bytes = 2 * (tensor_ws_bytes(M, K) + tensor_ws_bytes(N, K) + tensor_ws_bytes(M, N));
     return SNIP_OK;
 }
@@ -285,53 +433,58 @@ extern "C" int snip_layer_stats(const snip_layer_tensors_t *t, uint32_t fmt_mask
     if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int64_t M = t->M, N = t->N, K = t->K;
-    struct T { const void *p; int64_t r, c; int qidx; } tens[6] = {
-        {t->X, M, K, 0}, {t->W, N, K, 1}, {t->Y, M, N, -1}, {t->dY, M, N, 2}, {t->dX, M, K, -1}, {t->dW, N, K, -1}};
+    struct T { const void *p; int64_t r, c; int mode; } tens[6] = {
+        {t->X, M, K, MODE_ROWCOL}, {t->W, N, K, MODE_BLK}, {t->Y, M, N, MODE_PLAIN}, {t->dY, M, N, MODE_ROWCOL}, {t->dX, M, K, MODE_PLAIN}, {t->dW, N, K, MODE_PLAIN}};
     // every argument is checked before anything is enqueued
+    LayerStatsArgs a = {};
+    ReduceArgs red = {};
+    red.fmt_mask = fmt_mask;
+    red.out = out;
+    int64_t total = 0;
+    uint8_t *cursor = static_cast<uint8_t *>(ws);
+    StatsPartial *parts[6];
     for (int i = 0; i < 6; ++i) {
+        parts[i] = reinterpret_cast<StatsPartial *>(cursor);
+        cursor += tensor_ws_bytes(tens[i].r, tens[i].c);
         if (!tens[i].p) continue;
         if (!aligned16(tens[i].p)) return SNIP_ERR_ALIGN;
         if (ceil_div(tens[i].r, kTile) > 65535) return SNIP_ERR_SHAPE;
+        const int64_t n = ceil_div(tens[i].r, kTile) * ceil_div(tens[i].c, kTile);
+        if (n > INT32_MAX || tens[i].c > INT32_MAX) return SNIP_ERR_SHAPE;
+        total += n;
     }
-    SNIP_CUDA_TRY(cudaMemsetAsync(out, 0, sizeof(snip_layer_stats_t), st));
-    uint8_t *cursor = static_cast<uint8_t *>(ws);
-    for (int i = 0; i < 6; ++i) {
-        const size_t region = tensor_ws_bytes(tens[i].r, tens[i].c);
-        StatsPartial *parts = reinterpret_cast<StatsPartial *>(cursor);
-        cursor += region;
-        if (!tens[i].p) continue;
-        const int64_t tr = ceil_div(tens[i].r, kTile), tc = ceil_div(tens[i].c, kTile);
-        LayerStatsArgs a;
-        a.x = static_cast<const uint16_t *>(tens[i].p);
-        a.rows = tens[i].r; a.cols = tens[i].c;
-        a.partials = parts;
-        dim3 grid((unsigned)tc, (unsigned)tr);
-        const int q = tens[i].qidx;
-        ReduceDst dst = {{&out->sumsq[i], nullptr, nullptr, nullptr, nullptr}};
-        if (q < 0 || !(fmt_mask & 6u)) {
-            layer_stats_kernel<MODE_PLAIN, false, false><<<grid, kThreads, 0, st>>>(a);
-        } else if (q == 1) {
-            launch_mode<MODE_BLK>(a, fmt_mask, grid, st);
-            if (fmt_mask & 2u) dst.p[1] = &out->sumsq_err[q][0][SNIP_BLOCK_BLK_128x128];
-            if (fmt_mask & 4u) dst.p[3] = &out->sumsq_err[q][1][SNIP_BLOCK_BLK_128x128];
-        } else {
-            launch_mode<MODE_ROWCOL>(a, fmt_mask, grid, st);
-            if (fmt_mask & 2u) { dst.p[1] = &out->sumsq_err[q][0][SNIP_BLOCK_ROW_1x128]; dst.p[2] = &out->sumsq_err[q][0][SNIP_BLOCK_COL_128x1]; }
-            if (fmt_mask & 4u) { dst.p[3] = &out->sumsq_err[q][1][SNIP_BLOCK_ROW_1x128]; dst.p[4] = &out->sumsq_err[q][1][SNIP_BLOCK_COL_128x1]; }
+    const int64_t cap = kCtas * (int64_t)gemm_sm_count();
+    const int grid = (int)(total < cap ? total : cap);
+    for (int heavy = 1; heavy >= 0; --heavy) {
+        for (int i = 0; i < 6; ++i) {
+            const int mode = fmt_mask ? tens[i].mode : MODE_PLAIN;
+            if (!tens[i].p || (mode != MODE_PLAIN) != (heavy == 1)) continue;
+            StatsTensor &s = a.t[a.nheavy + a.nlight];
+            s.x = static_cast<const uint16_t *>(tens[i].p);
+            s.rows = (int32_t)tens[i].r; s.cols = (int32_t)tens[i].c;
+            s.tiles_c = (int32_t)ceil_div(tens[i].c, kTile);
+            s.ntiles = (int32_t)(ceil_div(tens[i].r, kTile) * s.tiles_c);
+            s.mode = mode; s.out = i;
+            s.partials = parts[i];
+            red.partials[i] = parts[i];
+            red.n[i] = s.ntiles < grid ? s.ntiles : grid;
+            if (heavy) ++a.nheavy; else ++a.nlight;
         }
-        SNIP_CUDA_TRY(cudaGetLastError());
-        cudaLaunchConfig_t cfg = {};
-        cfg.gridDim = dim3(1);
-        cfg.blockDim = dim3(1024);
-        cfg.stream = st;
-        cudaLaunchAttribute attr[1];
-        attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
-        attr[0].val.programmaticStreamSerializationAllowed = 1;
-        cfg.attrs = attr;
-        cfg.numAttrs = 1;
-        const StatsPartial *cparts = parts;
-        const int64_t nparts = tr * tc;
-        SNIP_CUDA_TRY(cudaLaunchKernelEx(&cfg, layer_stats_reduce_kernel, cparts, nparts, dst));
     }
+    if (grid > 0) {
+        const bool f8 = (fmt_mask & 2u) != 0, f4 = (fmt_mask & 4u) != 0;
+        rc = f8 && f4 ? launch_stats<true, true>(a, grid, st) : f8 ? launch_stats<true, false>(a, grid, st) : launch_stats<false, true>(a, grid, st);
+        if (rc) return rc;
+    }
+    cudaLaunchConfig_t cfg = {};
+    cfg.gridDim = dim3(6);
+    cfg.blockDim = dim3(256);
+    cfg.stream = st;
+    cudaLaunchAttribute attr[1];
+    attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    attr[0].val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = attr;
+    cfg.numAttrs = 1;
+    SNIP_CUDA_TRY(cudaLaunchKernelEx(&cfg, layer_stats_reduce_kernel, red));
     return SNIP_OK;
 }
