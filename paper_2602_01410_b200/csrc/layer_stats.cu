@@ -5,13 +5,16 @@
 // registers.  The scheme-generation step needs the error of every option (Sec. 4.4), not only of
 // the format currently in use.
 //
-// One persistent launch for all six tensors, three CTAs of 256 threads per SM; a CTA takes 128x128 tiles, each thread an 8x8 sub-block
-// that it fetches itself (cp.async into a private slot, one tile ahead).  The arithmetic per option is the quantizer's: S =
+// One persistent launch for all six tensors, three CTAs of 256 threads per SM.  X, W and dY are bound by instruction issue and the FP32
+// pipe (three operations and a conversion per element and option), Y, dX and dW, of which only the norm is wanted, by HBM; so every SM
+// works on both kinds at once, some CTAs on tiles of the first, some streaming the second.  Tiles are 128x128, each thread an 8x8
+// sub-block that it fetches itself (cp.async into a private slot, one tile ahead).  The arithmetic per option is the quantizer's: S =
 // FPX_MAX/amax (binary32 quotient, one division per tile and format, shared through shared memory), code = RNE_fmt(fl32(x*S)), error
-// term x - value(code)/S.  X and dY with four options are bound by instruction issue (about 17 per element), Y, dX and dW by HBM:
-// every CTA walks both kinds of tensor side by side, in proportion, so that the two overlap.  A reduction of the CTAs' sums follows.
-// Six tensors of an 8192 x 3200 x 9600 linear: 250 us as twelve launches of one tile per CTA, with the divisions repeated by every
-// thread and the elements unpacked once per option.
+// term x - value(code)/S.  A reduction of the CTAs' sums follows.
+// Six tensors of an 8192 x 3200 x 9600 linear: 250 -> 147 us, X with four options 16384 x 4096: 98 -> 72 us (before: thirteen launches of one
+// tile per CTA, every thread dividing for all of its rows and columns).
+#include <stddef.h>
+
 #include "common.cuh"
 #include "quant_device.cuh"
 
@@ -27,6 +30,7 @@ constexpr int kCtas = 3;             // per SM
 constexpr int kSlotBytes = kTile * kTile * 2;
 
 enum { MODE_PLAIN = 0, MODE_BLK = 1, MODE_ROWCOL = 2 };
+constexpr int kChunk = kThreads * 64;   // elements a CTA takes at a time of a tensor without error sums
 
 // per CTA: [0] sum x^2; [1] FP8 kind A; [2] FP8 kind B; [3] FP4 kind A; [4] FP4 kind B
 // (ROWCOL: A = ROW, B = COL; BLK: A = BLK, B unused)
@@ -36,26 +40,28 @@ struct StatsPartial {
 
 struct StatsTensor {
     const uint16_t *x;
-    int32_t rows, cols, tiles_c, ntiles;
-    int32_t mode, out;               // out: index of the tensor in the result
-    StatsPartial *partials;          // one per CTA that has tiles of it
+    int32_t rows, cols, tiles_c;
+    int32_t nitems;                  // tiles, or chunks (MODE_PLAIN)
+    int32_t mode;
+    StatsPartial *partials;          // one per CTA that has items of it
 };
-// Tensors with error sums (heavy) and without (light), each list one sequence of tiles dealt to the CTAs in turn.
+// Tensors with error sums (heavy) and without (light); each list is one sequence of items dealt in turn to the CTAs that work on it.
 struct LayerStatsArgs {
     StatsTensor t[6];
     int32_t nheavy, nlight;          // t[0 .. nheavy), t[nheavy .. nheavy + nlight)
+    int32_t light_ctas;              // the first CTAs stream the light tensors, the others take tiles
 };
 
 struct Scales {                      // of one tile line: scale and negated reciprocal for both formats
     float s8, n8, s4, n4;
 };
 struct Shared {
-    __align__(16) uint8_t slot[kSlotBytes];
     uint32_t col_amax[8][kTile / 2];  // packed bf16 pairs, one row per warp
     __align__(16) Scales row[kTile];
-    __align__(16) Scales col[kTile];
+    __align__(16) float col[4][kTile];   // the four values apart: a thread reads eight consecutive columns (interleaved, 8-way bank conflicts)
     uint32_t blk_amax[2][8];
     double red[8][5];
+    __align__(16) uint8_t slot[2][kSlotBytes];   // the tile at hand and the next one; not there in a launch without heavy tensors
 };
 
 template <int FMT>
@@ -83,54 +89,10 @@ __device__ __forceinline__ void err_pair(const float2 x, const float2 s, const f
     se2 = __ffma2_rn(e, e, se2);
 }
 
-// A CTA's walk over one list: tile `tile` of tensor `j`, in steps of the grid.
-struct Walk {
-    int j, end, tile, left;          // left: items of the whole walk that have not been taken
-    __device__ __forceinline__ void start(const LayerStatsArgs &a, int first, int count)
-    {
-        j = first; end = first + count; left = 0;
-        int base = 0;
-        for (int i = first; i < end; ++i) {
-            const int rel = offset(base);
-            if (rel < a.t[i].ntiles) left += (a.t[i].ntiles - rel + (int)gridDim.x - 1) / (int)gridDim.x;
-            base = (base + a.t[i].ntiles) % (int)gridDim.x;
-        }
-        seq = 0;
-        tile = offset(0);
-        skip(a);
-    }
-    __device__ __forceinline__ void next(const LayerStatsArgs &a)
-    {
-        --left;
-        tile += (int)gridDim.x;
-        skip(a);
-    }
-private:
-    int seq;                         // position of tensor j's first tile in the sequence, modulo the grid
-    __device__ __forceinline__ int offset(int base) const
-    {
-        const int r = (int)blockIdx.x - base;
-        return r < 0 ? r + (int)gridDim.x : r;
-    }
-    __device__ __forceinline__ void skip(const LayerStatsArgs &a)
-    {
-        while (j < end && tile >= a.t[j].ntiles) {
-            seq = (seq + a.t[j].ntiles) % (int)gridDim.x;
-            tile = offset(seq);
-            ++j;
-        }
-    }
-};
-
-struct Item {
-    int j, tile;                     // j < 0: none
-};
-
-__device__ __forceinline__ void fetch(const LayerStatsArgs &a, const Item it, uint8_t *slot)
+__device__ __forceinline__ void fetch(const StatsTensor &t, int tile, uint8_t *slot)
 {
-    if (it.j >= 0) {
-        const StatsTensor &t = a.t[it.j];
-        const int tid = threadIdx.x, tr = it.tile / t.tiles_c, tc = it.tile - tr * t.tiles_c;
+    if (tile < t.nitems) {
+        const int tid = threadIdx.x, tr = tile / t.tiles_c, tc = tile - tr * t.tiles_c;
         const int r = tr * kTile + 8 * (tid >> 4), c = tc * kTile + 8 * (tid & 15);
         const bool ok = r < t.rows && c < t.cols;    // dims are multiples of 64: all 64 elements or none
         const uint16_t *src = t.x + (ok ? (int64_t)r * t.cols + c : 0);
@@ -168,12 +130,44 @@ __device__ __forceinline__ void flush(const StatsTensor &t, int slot, Shared &sh
     for (int k = 0; k < 5; ++k) acc[k] = 0.0;
 }
 
-__device__ __forceinline__ int first_tile(const LayerStatsArgs &a, int list, int j)
+// Sum of squares of 64 elements per thread (eight 16-byte pieces).
+__device__ __forceinline__ float sumsq64(const uint4 (&v)[8])
 {
-    int base = 0;
-    for (int i = list; i < j; ++i) base = (base + a.t[i].ntiles) % (int)gridDim.x;
-    const int r = (int)blockIdx.x - base;
-    return r < 0 ? r + (int)gridDim.x : r;
+    float2 s = make_float2(0.0f, 0.0f);
+#pragma unroll
+    for (int p = 0; p < 8; ++p) {
+        const uint32_t w[4] = {v[p].x, v[p].y, v[p].z, v[p].w};
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
+            s = __ffma2_rn(x, x, s);
+        }
+    }
+    return s.x + s.y;
+}
+
+// The light tensors: contiguous arrays, streamed.
+__device__ __forceinline__ void run_light(const LayerStatsArgs &a, int cta, int ctas, Shared &sh)
+{
+    int first = cta;
+    for (int j = a.nheavy; j < a.nheavy + a.nlight; ++j) {
+        const StatsTensor &t = a.t[j];
+        const int64_t n = (int64_t)t.rows * t.cols;
+        double acc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        int c = first;
+        for (; c < t.nitems; c += ctas) {
+            const int64_t base = (int64_t)c * kChunk + threadIdx.x * 8;
+            uint4 v[8];
+#pragma unroll
+            for (int p = 0; p < 8; ++p) {
+                const int64_t at = base + p * (kThreads * 8);
+                v[p] = at < n ? __ldg(reinterpret_cast<const uint4 *>(t.x + at)) : make_uint4(0, 0, 0, 0);
+            }
+            acc[0] += (double)sumsq64(v);
+        }
+        if (first < t.nitems) flush(t, first, sh, acc);
+        first = c - t.nitems;   // the deal goes on where this tensor ended
+    }
 }
 
 template <bool F8, bool F4>
@@ -186,53 +180,23 @@ __global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __gr
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & 15, ty = tid >> 4;
 
-    Walk heavy, light;
-    heavy.start(a, 0, a.nheavy);
-    light.start(a, a.nheavy, a.nlight);
-    const int nh = heavy.left, nl = light.left;
-    // next item: the list of which the smaller share has been taken
-    auto take = [&]() -> Item {
-        if (heavy.left == 0 && light.left == 0) return {-1, 0};
-        const bool h = light.left == 0 || (heavy.left > 0 && (int64_t)heavy.left * nl >= (int64_t)light.left * nh);
-        Walk &w = h ? heavy : light;
-        const Item it = {w.j, w.tile};
-        w.next(a);
-        return it;
-    };
-    double hacc[5] = {0.0, 0.0, 0.0, 0.0, 0.0}, lacc = 0.0;
-    int hj = -1, lj = -1, parity = 0;
-    auto flush_heavy = [&]() { if (hj >= 0) flush(a.t[hj], first_tile(a, 0, hj), sh, hacc); };
-    auto flush_light = [&]() {
-        if (lj < 0) return;
-        double t[5] = {lacc, 0.0, 0.0, 0.0, 0.0};
-        flush(a.t[lj], first_tile(a, a.nheavy, lj), sh, t);
-        lacc = 0.0;
-    };
-
-    Item cur = take();
-    fetch(a, cur, sh.slot);
-    while (cur.j >= 0) {
-        const Item nxt = take();
-        asm volatile("cp.async.wait_group 0;" ::: "memory");
-        const int mode = a.t[cur.j].mode;
-        float2 sx2 = make_float2(0.0f, 0.0f);
-        if (mode == MODE_PLAIN) {
-            if (cur.j != lj) { flush_light(); lj = cur.j; }
-#pragma unroll
-            for (int p = 0; p < 8; ++p) {
-                const uint4 v = slot[p * kThreads];
-                const uint32_t w[4] = {v.x, v.y, v.z, v.w};
-#pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
-                    sx2 = __ffma2_rn(x, x, sx2);
-                }
-            }
-            fetch(a, nxt, sh.slot);
-            lacc += (double)(sx2.x + sx2.y);
-        } else {
-            if (cur.j != hj) { flush_heavy(); hj = cur.j; }
-            const bool rowcol = mode == MODE_ROWCOL;
+    if ((int)blockIdx.x < a.light_ctas) { run_light(a, (int)blockIdx.x, a.light_ctas, sh); return; }
+    const int ctas = (int)gridDim.x - a.light_ctas;
+    int first = (int)blockIdx.x - a.light_ctas, parity = 0;
+    for (int j = 0; j < a.nheavy; ++j) {
+        const StatsTensor &t = a.t[j];
+        if (first >= t.nitems) { first -= t.nitems; continue; }
+        const bool rowcol = t.mode == MODE_ROWCOL;
+        double hacc[5] = {0.0, 0.0, 0.0, 0.0, 0.0};
+        int tile = first;
+        int buf = 0;
+        fetch(t, tile, sh.slot[0]);
+        for (; tile < t.nitems; tile += ctas) {
+            fetch(t, tile + ctas, sh.slot[buf ^ 1]);
+            asm volatile("cp.async.wait_group 1;" ::: "memory");
+            const uint4 *slot = reinterpret_cast<const uint4 *>(sh.slot[buf]) + threadIdx.x;
+            buf ^= 1;
+            float2 sx2 = make_float2(0.0f, 0.0f);
             float2 e8a = make_float2(0.0f, 0.0f), e8b = e8a, e4a = e8a, e4b = e8a;
             // maxima (signs are garbage until masked: max.xorsign.abs keeps magnitudes only)
             uint32_t rmax[8], cm[4] = {0, 0, 0, 0};
@@ -275,15 +239,20 @@ __global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __gr
                     uint32_t m = 0;
 #pragma unroll
                     for (int w = 0; w < 8; ++w) m = max(m, (uint32_t)h[w * kTile + tid] & 0x7FFFu);   // non-negative bf16: integer order
-                    sh.col[tid] = scales_of<F8, F4>(__uint_as_float(m << 16));
+                    const Scales cs = scales_of<F8, F4>(__uint_as_float(m << 16));
+                    sh.col[0][tid] = cs.s8; sh.col[1][tid] = cs.n8; sh.col[2][tid] = cs.s4; sh.col[3][tid] = cs.n4;
                 }
                 __syncthreads();
                 float2 cs8[4], cn8[4], cs4[4], cn4[4];
 #pragma unroll
-                for (int i = 0; i < 4; ++i) {
-                    const float4 c0 = *reinterpret_cast<const float4 *>(&sh.col[8 * tx + 2 * i]), c1 = *reinterpret_cast<const float4 *>(&sh.col[8 * tx + 2 * i + 1]);
-                    cs8[i] = make_float2(c0.x, c1.x); cn8[i] = make_float2(c0.y, c1.y);
-                    cs4[i] = make_float2(c0.z, c1.z); cn4[i] = make_float2(c0.w, c1.w);
+                for (int i = 0; i < 2; ++i) {
+                    auto get = [&](int k, float2 (&d)[4]) {
+                        const float4 c = *reinterpret_cast<const float4 *>(&sh.col[k][8 * tx + 4 * i]);
+                        d[2 * i] = make_float2(c.x, c.y);
+                        d[2 * i + 1] = make_float2(c.z, c.w);
+                    };
+                    if (F8) { get(0, cs8); get(1, cn8); }
+                    if (F4) { get(2, cs4); get(3, cn4); }
                 }
 #pragma unroll
                 for (int p = 0; p < 8; ++p) {
@@ -328,15 +297,13 @@ __global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __gr
                     }
                 }
             }
-            fetch(a, nxt, sh.slot);
             hacc[0] += (double)(sx2.x + sx2.y);
             if (F8) { hacc[1] += (double)(e8a.x + e8a.y); hacc[2] += (double)(e8b.x + e8b.y); }
             if (F4) { hacc[3] += (double)(e4a.x + e4a.y); hacc[4] += (double)(e4b.x + e4b.y); }
         }
-        cur = nxt;
+        flush(t, first, sh, hacc);
+        first = tile - t.nitems;
     }
-    flush_heavy();
-    flush_light();
 }
 
 // Fixed-order sums of the CTAs' partials, one block per tensor of the result; every value of the result is written (0 for what was not
@@ -399,9 +366,10 @@ size_t tensor_ws_bytes(int64_t rows, int64_t cols)
 template <bool F8, bool F4>
 int launch_stats(const LayerStatsArgs &a, int grid, cudaStream_t st)
 {
+    const size_t smem = a.nheavy ? sizeof(Shared) : offsetof(Shared, slot);
     auto kern = layer_stats_kernel<F8, F4>;
     SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(Shared)));
-    kern<<<grid, kThreads, sizeof(Shared), st>>>(a);
+    kern<<<grid, kThreads, smem, st>>>(a);
     SNIP_CUDA_TRY(cudaGetLastError());
     return SNIP_OK;
 }
@@ -463,13 +431,29 @@ extern "C" int snip_layer_stats(const snip_layer_tensors_t *t, uint32_t fmt_mask
             s.x = static_cast<const uint16_t *>(tens[i].p);
             s.rows = (int32_t)tens[i].r; s.cols = (int32_t)tens[i].c;
             s.tiles_c = (int32_t)ceil_div(tens[i].c, kTile);
-            s.ntiles = (int32_t)(ceil_div(tens[i].r, kTile) * s.tiles_c);
-            s.mode = mode; s.out = i;
+            s.nitems = heavy ? (int32_t)(ceil_div(tens[i].r, kTile) * s.tiles_c) : (int32_t)ceil_div(tens[i].r * tens[i].c, (int64_t)kChunk);
+            s.mode = mode;
             s.partials = parts[i];
             red.partials[i] = parts[i];
-            red.n[i] = s.ntiles < grid ? s.ntiles : grid;
             if (heavy) ++a.nheavy; else ++a.nlight;
         }
+    }
+    // CTAs of each kind by their cost per 128x128 elements, measured: about 5 (1x128 and 128x1 tiles), 3 (128x128) and 1 (norm only)
+    int64_t cost[2] = {0, 0};
+    for (int i = 0; i < a.nheavy + a.nlight; ++i)
+        cost[i < a.nheavy ? 0 : 1] += (int64_t)a.t[i].nitems * (a.t[i].mode == MODE_ROWCOL ? 5 : a.t[i].mode == MODE_BLK ? 3 : 1);
+    a.light_ctas = a.nheavy == 0 ? grid : 0;
+    if (a.nheavy && a.nlight) {
+        a.light_ctas = (int32_t)(grid * cost[1] / (cost[0] + cost[1]));
+        if (a.light_ctas < 1) a.light_ctas = 1;
+        if (a.light_ctas > grid - 1) a.light_ctas = grid - 1;
+    }
+    for (int i = 0, h = 0; i < 6; ++i) {
+        if (!tens[i].p) continue;
+        h = 0;
+        while (a.t[h].partials != parts[i]) ++h;
+        const int ctas = h < a.nheavy ? grid - a.light_ctas : a.light_ctas;
+        red.n[i] = a.t[h].nitems < ctas ? a.t[h].nitems : ctas;
     }
     if (grid > 0) {
         const bool f8 = (fmt_mask & 2u) != 0, f4 = (fmt_mask & 4u) != 0;
