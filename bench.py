@@ -622,7 +622,7 @@ def run_profile_case(name):
         return run_layer_stats_case(api, torch, device, parts[2] if len(parts) > 2 else "x")
     mx = parts[1].startswith("mx")
     if parts[1].startswith("pair"):
-        # the CTA-pair form of the paper-rule GEMM (an alternative kept for comparison; see include/snip.h, snip_debug_set)
+        # the CTA-pair form of the paper-rule GEMM whatever the shape (see include/snip.h, snip_debug_set)
         api.snip_debug_set(api.DEBUG_GEMM_KERNEL, api.GEMM_KERNEL_PAIR)
         parts[1] = parts[1][4:]
     fmt = {"bf16": FMT_BF16, "fp8": FMT_FP8, "fp4": FMT_FP4, "mxfp8": FMT_FP8, "mxfp4": FMT_FP4}[parts[1]]

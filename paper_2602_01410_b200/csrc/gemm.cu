@@ -30,7 +30,7 @@ using namespace sm100;
 
 namespace {
 
-constexpr int BM = 128;
+constexpr int CM = 128;   // output rows of a CTA
 constexpr int kGemmThreads = 384;  // warps 0-3: producer, MMA issuer, 2 scale loaders (wgrad) or idle; warps 4-11: epilogue
 constexpr int kNumEpiWarps = 8;
 static_assert(kNumEpiWarps == kSliceWarps, "slice counters");
@@ -60,15 +60,18 @@ struct GemmArgs {
     StatJobs stats;            // reductions left by the quantizers ahead
 };
 
-template <MmaKind KIND, int BN, int SCALE>
+template <MmaKind KIND, int BN, int SCALE, bool PAIR>
 struct Cfg {
+    static constexpr int kCtas = PAIR ? 2 : 1;
+    static constexpr int BM = CM * kCtas;                                    // rows of a tile
+    static constexpr int kBLines = BN / kCtas;                               // B lines fetched by a CTA
     static constexpr int kStageElemsX = 128;                                 // TMA x step per stage
     static constexpr int kChunkElems = 128;                                  // scale granularity
     static constexpr int kStageK = KIND == MmaKind::F8F6F4 ? 128 : 256;
-    static constexpr int kABytes = BM * 128;
-    static constexpr int kBBytes = BN * 128;
+    static constexpr int kABytes = CM * 128;
+    static constexpr int kBBytes = kBLines * 128;
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = (BN >= 256 || SCALE == 1) ? 4 : 5;
+    static constexpr int kStages = PAIR ? 6 : (BN >= 256 || SCALE == 1) ? 4 : 5;
     // block mode (fwd / dgrad) fetches four chunks of scale factors per instruction into two alternating group slots:
     // [4 chunks][32 rows] S_a, then [2 blocks][4 chunks] S_b
     static constexpr int kGroupFloats = 144;
@@ -184,13 +187,13 @@ __device__ __forceinline__ void store_frag(const GemmArgs &g, int64_t row, int c
     }
 }
 
-template <MmaKind KIND, int BN, int SCALE, bool OUT_F32>
+template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmO,
             const GemmArgs g, const uint32_t idesc)
 {
-    using C = Cfg<KIND, BN, SCALE>;
-    constexpr int S = C::kStages;
+    using C = Cfg<KIND, BN, SCALE, PAIR>;
+    constexpr int S = C::kStages, BM = C::BM;
     constexpr int HALF = BN / 2;     // columns handled by one epilogue warp
     // registers per tensor-memory load: 16 in vector mode (wgrad: 16 rows x 32 columns as a fragment), 32 otherwise (32 rows x
     // 32 columns; fwd / dgrad: 2.5 % faster than 16)
@@ -221,13 +224,15 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     volatile uint32_t *abort_flag = tmem_slot + 1;
 
     const int warp = threadIdx.x >> 5, lane = threadIdx.x & 31;
+    const uint32_t rank = PAIR ? cluster_ctarank() : 0u;   // 0 = leader: its barriers and its MMA warp serve the pair
+    const int unit = (int)blockIdx.x / C::kCtas, units = (int)gridDim.x / C::kCtas;
     const int num_m = (g.Mo + BM - 1) / BM, num_n = (g.No + BN - 1) / BN;
     const int num_chunks = (g.Kc + C::kChunkElems - 1) / C::kChunkElems;
     const int num_kstages = (g.Kc + C::kStageK - 1) / C::kStageK;
 
     if (threadIdx.x == 0) {
         for (int s = 0; s < S; ++s) { mbar_init(full_bar(s), 1); mbar_init(empty_bar(s), 1); }
-        for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), kNumEpiWarps); }
+        for (int a = 0; a < 2; ++a) { mbar_init(tfull_bar(a), 1); mbar_init(tempty_bar(a), kNumEpiWarps * C::kCtas); }
         for (int k = 0; k < kVBlocks; ++k) { mbar_init(vfull_bar(k), 2); mbar_init(vempty_bar(k), kNumEpiWarps); }
         *abort_flag = 0u;
         fence_barrier_init();
@@ -235,8 +240,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         prefetch_tensormap(&tmB);
     }
     if (warp == 1) {
-        tmem_alloc<false>(smem_u32(tmem_slot), C::kTmemCols);
-        tmem_relinquish<false>();
+        tmem_alloc<PAIR>(smem_u32(tmem_slot), C::kTmemCols);
+        tmem_relinquish<PAIR>();
     }
     tc_fence_before_sync();
     __syncthreads();
@@ -258,25 +263,44 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         tc_fence_after_sync();
     }
 
+    if (PAIR) {   // both CTAs' barriers and tensor memory (constant scale factors included) are ready before anyone signals across the pair
+        tc_fence_before_sync();
+        cluster_sync();
+        tc_fence_after_sync();
+    }
+    // Bounded wait; a failed one raises the abort flag of both CTAs.
+    auto wait1 = [&](uint32_t bar, uint32_t parity) {
+        const bool got = mbar_wait(bar, parity, abort_flag, g.wait_limit_ns);
+        if (PAIR && !got) st_cluster_u32(mapa(smem_u32(const_cast<uint32_t *>(abort_flag)), rank ^ 1u), 1u);
+        return got;
+    };
+
     if (warp < 4) {
       reg_dealloc<40>();  // frees (168-40)*128 = 16384 registers
       if (warp == 0) {
         // ================= TMA producer =================
         status_begin(g.status, g.status_mark);
+        const uint32_t lead_full0 = PAIR ? mapa(full_bar(0), 0) : 0u;
         if (lane == 0) {
             uint32_t it = 0;
             bool ok = true;
-            for (int w = blockIdx.x; w < g.work.num_items && ok; w += gridDim.x) {
+            for (int w = unit; w < g.work.num_items && ok; w += units) {
                 const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
                 int m_idx, n_idx;
                 tile_coords(wi.t, num_m, num_n, m_idx, n_idx);
                 for (int ks = wi.ks0; ks < wi.ks1; ++ks, ++it) {
                     const int s = it % S;
                     const uint32_t ph = (it / S) & 1u;
-                    if (!mbar_wait(empty_bar(s), ph ^ 1u, abort_flag, g.wait_limit_ns)) { ok = false; break; }
-                    mbar_arrive_expect_tx(full_bar(s), g.stage_tx_bytes);
-                    tma_load_2d(smem_a0 + s * C::kABytes, &tmA, full_bar(s), ks * C::kStageElemsX, m_idx * BM);
-                    tma_load_2d(smem_b0 + s * C::kBBytes, &tmB, full_bar(s), ks * C::kStageElemsX, n_idx * BN);
+                    if (!wait1(empty_bar(s), ph ^ 1u)) { ok = false; break; }
+                    if (rank == 0) mbar_arrive_expect_tx(full_bar(s), C::kCtas * g.stage_tx_bytes);
+                    const int row = m_idx * BM + (int)rank * CM, col = n_idx * BN + (int)rank * C::kBLines;
+                    if (PAIR) {   // each CTA fetches its own share (no multicast); the leader's barrier counts the bytes of both
+                        tma_load_2d_pair(smem_a0 + s * C::kABytes, &tmA, lead_full0 + 8u * s, ks * C::kStageElemsX, row);
+                        tma_load_2d_pair(smem_b0 + s * C::kBBytes, &tmB, lead_full0 + 8u * s, ks * C::kStageElemsX, col);
+                    } else {
+                        tma_load_2d(smem_a0 + s * C::kABytes, &tmA, full_bar(s), ks * C::kStageElemsX, row);
+                        tma_load_2d(smem_b0 + s * C::kBBytes, &tmB, full_bar(s), ks * C::kStageElemsX, col);
+                    }
                 }
             }
         }
@@ -284,46 +308,50 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         // ================= MMA issuer =================
         // Block mode: an elected lane, under which the operands of the tcgen05 instructions stay in uniform registers (issue of a chunk
         // 204 -> 55 cycles, 2-4 % of the FP4 kernels); in vector mode it costs the promotion warps registers and gains nothing.
-        if (SCALE == SCALE_BLOCK_B ? elect_one() : lane == 0) {
+        if (rank == 0 && (SCALE == SCALE_BLOCK_B ? elect_one() : lane == 0)) {
+            const uint32_t peer0 = PAIR ? mapa(bar0, 1) : 0u;
             uint32_t it = 0, cc = 0;
             bool ok = true;
             const uint32_t sfa = tmem_base + C::kSfCol0, sfb = tmem_base + C::kSfCol0 + 16;
-            for (int w = blockIdx.x; w < g.work.num_items && ok; w += gridDim.x) {
+            for (int w = unit; w < g.work.num_items && ok; w += units) {
                 const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
                 for (int ks = wi.ks0; ks < wi.ks1 && ok; ++ks, ++it) {
                     const int s = it % S;
                     const uint32_t ph = (it / S) & 1u;
-                    if (!mbar_wait(full_bar(s), ph, abort_flag, g.wait_limit_ns)) { ok = false; break; }
+                    if (!wait1(full_bar(s), ph)) { ok = false; break; }
                     tc_fence_after_sync();
                     const uint64_t adesc = make_smem_desc_k128(smem_a0 + s * C::kABytes);
                     const uint64_t bdesc = make_smem_desc_k128(smem_b0 + s * C::kBBytes);
                     if (KIND == MmaKind::F8F6F4) {
                         const uint32_t a = cc & 1u;
-                        if (!mbar_wait(tempty_bar(a), ((cc >> 1) & 1u) ^ 1u, abort_flag, g.wait_limit_ns)) { ok = false; break; }
+                        if (!wait1(tempty_bar(a), ((cc >> 1) & 1u) ^ 1u)) { ok = false; break; }
                         tc_fence_after_sync();
 #pragma unroll
                         for (int k = 0; k < 4; ++k)
-                            mma_ss<KIND, false>(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc, k > 0 ? 1u : 0u, 0, 0);
+                            mma_ss<KIND, PAIR>(tmem_base + a * BN, adesc + 2 * k, bdesc + 2 * k, idesc, k > 0 ? 1u : 0u, 0, 0);
                         // one commit serves both hand-offs (a stage is one chunk here): the producer takes it as
                         // "stage s is free", the epilogue warps as "the chunk's partial sums are complete"
-                        tc_commit<false>(empty_bar(s));
+                        tc_commit<PAIR>(empty_bar(s));
+                        if (PAIR) tc_commit<PAIR>(peer0 + 8u * (S + s));
                         ++cc;
                     } else {
 #pragma unroll
                         for (int h = 0; h < 2; ++h) {
                             if (2 * ks + h < num_chunks) {
                                 const uint32_t a = cc & 1u;
-                                if (!mbar_wait(tempty_bar(a), ((cc >> 1) & 1u) ^ 1u, abort_flag, g.wait_limit_ns)) { ok = false; break; }
+                                if (!wait1(tempty_bar(a), ((cc >> 1) & 1u) ^ 1u)) { ok = false; break; }
                                 tc_fence_after_sync();
 #pragma unroll
                                 for (int k = 0; k < 2; ++k)
-                                    mma_ss<KIND, false>(tmem_base + a * BN, adesc + 2 * (2 * h + k), bdesc + 2 * (2 * h + k), idesc,
+                                    mma_ss<KIND, PAIR>(tmem_base + a * BN, adesc + 2 * (2 * h + k), bdesc + 2 * (2 * h + k), idesc,
                                                  k > 0 ? 1u : 0u, sfa, sfb);
-                                tc_commit<false>(tfull_bar(a));
+                                tc_commit<PAIR>(tfull_bar(a));
+                                if (PAIR) tc_commit<PAIR>(peer0 + 8u * (2 * S + a));
                                 ++cc;
                             }
                         }
-                        tc_commit<false>(empty_bar(s));
+                        tc_commit<PAIR>(empty_bar(s));
+                        if (PAIR) tc_commit<PAIR>(peer0 + 8u * (S + s));
                     }
                 }
             }
@@ -341,18 +369,18 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const bool rows_side = (warp == 2);
         constexpr int kChunksPerStage = C::kStageK / C::kChunkElems;
         uint32_t total = 0;            // chunks of all of this CTA's work items
-        for (int w = blockIdx.x; w < g.work.num_items; w += gridDim.x) {
+        for (int w = unit; w < g.work.num_items; w += units) {
             const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
             total += (uint32_t)(min(kChunksPerStage * wi.ks1, num_chunks) - kChunksPerStage * wi.ks0);
         }
         const uint32_t ring_u32 = smem_u32(scale_ring);
-        int pw = blockIdx.x, pj = 0, pn = 0;   // work item and chunk of the next request, chunks of that item
+        int pw = unit, pj = 0, pn = 0;   // work item and chunk of the next request, chunks of that item
         uint32_t pc = 0;               // its position in the sequence of this CTA's chunks
         bool ok = true;
         const float *src0 = nullptr, *src1 = nullptr;
         int64_t stride = 0;
         auto item_sources = [&]() {
-            const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, pw < g.work.num_items ? pw : (int)blockIdx.x, num_kstages);
+            const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, pw < g.work.num_items ? pw : unit, num_kstages);
             int m_idx, n_idx;
             tile_coords(wi.t, num_m, num_n, m_idx, n_idx);
             const int c0 = kChunksPerStage * wi.ks0;
@@ -360,7 +388,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             // rows / columns outside the matrix repeat the last four factors (their sums are never stored)
             if (rows_side) {
                 stride = g.sa_chunk_stride;
-                src0 = g.sa + c0 * stride + min(m_idx * BM + 4 * lane, g.Mo - 4);
+                src0 = g.sa + c0 * stride + min(m_idx * BM + (int)rank * CM + 4 * lane, g.Mo - 4);
             } else {
                 stride = g.sb_chunk_stride;
                 src0 = g.sb + c0 * stride + min(n_idx * BN + 4 * lane, g.No - 4);
@@ -371,7 +399,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         auto request = [&]() {
             if (pc < total && ok) {
                 const uint32_t d = pc % C::kVecDepth;
-                if ((pc % C::kVecBlock) == 0 && !__all_sync(0xFFFFFFFFu, mbar_wait(vempty_bar(d / C::kVecBlock), ((pc / C::kVecDepth) & 1u) ^ 1u, abort_flag, g.wait_limit_ns))) ok = false;
+                if ((pc % C::kVecBlock) == 0 && !__all_sync(0xFFFFFFFFu, wait1(vempty_bar(d / C::kVecBlock), ((pc / C::kVecDepth) & 1u) ^ 1u))) ok = false;
                 else {
                     const uint32_t slot = ring_u32 + d * (C::kVecSlotFloats * 4);
                     if (rows_side) {
@@ -382,7 +410,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     }
                     src0 += stride;
                     src1 += stride;
-                    if (++pj == pn) { pj = 0; pw += gridDim.x; item_sources(); }
+                    if (++pj == pn) { pj = 0; pw += units; item_sources(); }
                 }
             }
             ++pc;
@@ -424,6 +452,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     } else {
         reg_alloc<232>();    // needs (232-168)*256 = 16384 <= 16384 (an unsatisfiable request would block forever)
         // ================= promotion / epilogue warps =================
+        const uint32_t lead_tempty0 = PAIR ? mapa(tempty_bar(0), 0) : 0u;
         const int e = warp - 4;          // 0..7
         const int q = warp & 3;          // tensor-memory lane quarter this warp may access
         const int h = e >> 2;            // column half
@@ -436,11 +465,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         const uint32_t stage_u32 = out_stage0 + e * (C::kOutSlots * 2048);   // this warp's staging tiles: 32 rows x 64 bytes each
         uint32_t cc = 0;
         bool ok = true;
-        for (int w = blockIdx.x; w < g.work.num_items && ok; w += gridDim.x) {
+        for (int w = unit; w < g.work.num_items && ok; w += units) {
             const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
             int m_idx, n_idx;
             tile_coords(wi.t, num_m, num_n, m_idx, n_idx);
-            const int row0 = m_idx * BM + q * 32;
+            const int row0 = m_idx * BM + (int)rank * CM + q * 32;
             const int row = row0 + lane;
             const int col0 = n_idx * BN + h * HALF;
             const bool row_ok = row < g.Mo;
@@ -507,7 +536,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const uint32_t vd = cc % C::kVecDepth;
                 const float *vslot = scale_ring + vd * C::kVecSlotFloats;
                 if (SCALE == SCALE_VEC_B && (cc % C::kVecBlock) == 0) {
-                    const bool got = mbar_wait(vfull_bar(vd / C::kVecBlock), (cc / C::kVecDepth) & 1u, abort_flag, g.wait_limit_ns);
+                    const bool got = wait1(vfull_bar(vd / C::kVecBlock), (cc / C::kVecDepth) & 1u);
                     if (!__all_sync(0xFFFFFFFFu, got)) { ok = false; break; }
                 }
                 float4 rf = make_float4(0.0f, 0.0f, 0.0f, 0.0f), cf[2][2];   // row factors; column factors of two 32-column blocks
@@ -529,7 +558,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const uint32_t done_bar = (KIND == MmaKind::F8F6F4) ? empty_bar(cc % S) : tfull_bar(a);
                 const uint32_t done_par = (KIND == MmaKind::F8F6F4) ? ((cc / S) & 1u) : ((cc >> 1) & 1u);
                 {
-                    const bool got = mbar_wait(done_bar, done_par, abort_flag, g.wait_limit_ns);
+                    const bool got = wait1(done_bar, done_par);
                     if (!__all_sync(0xFFFFFFFFu, got)) { ok = false; break; }
                 }
                 tc_fence_after_sync();
@@ -558,7 +587,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 auto release_buffer = [&]() {
                     tc_fence_before_sync();
                     __syncwarp();
-                    if (lane == 0) mbar_arrive(tempty_bar(a));
+                    if (lane == 0) {
+                        if (PAIR) mbar_arrive_cluster_relaxed(lead_tempty0 + 8u * a);
+                        else mbar_arrive(tempty_bar(a));
+                    }
                 };
                 auto consume_group = [&](int gi, const uint32_t (&cur)[GC]) {
                     if (SCALE == SCALE_BLOCK_B) {
@@ -646,15 +678,17 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                             // order, whoever came last, so the result does not depend on the order of arrival.
                             float *av = reinterpret_cast<float *>(acc);
                             constexpr size_t kWarpFloats = 32 * HALF;
-                            float *first = g.partials + (size_t)(wi.tail * wi.nsl) * kNumEpiWarps * kWarpFloats + e * kWarpFloats + lane * 4;
-                            float *mine = first + (size_t)wi.slice * kNumEpiWarps * kWarpFloats;
+                            constexpr int kWarps = kNumEpiWarps * C::kCtas;   // promotion warps of a tile
+                            const int ew = (int)rank * kNumEpiWarps + e;
+                            float *first = g.partials + (size_t)(wi.tail * wi.nsl) * kWarps * kWarpFloats + ew * kWarpFloats + lane * 4;
+                            float *mine = first + (size_t)wi.slice * kWarps * kWarpFloats;
 #pragma unroll
                             for (int j4 = 0; j4 < HALF / 4; ++j4)
                                 __stcg(reinterpret_cast<float4 *>(mine + j4 * 128), make_float4(av[4 * j4], av[4 * j4 + 1], av[4 * j4 + 2], av[4 * j4 + 3]));
                             __threadfence();
                             __syncwarp();
                             uint32_t old = 0;
-                            if (lane == 0) old = atomicAdd(g.counters + wi.tail * kNumEpiWarps + e, 1u);
+                            if (lane == 0) old = atomicAdd(g.counters + wi.tail * kWarps + ew, 1u);
                             old = __shfl_sync(0xFFFFFFFFu, old, 0);
                             write_out = (old == (uint32_t)wi.nsl - 1u);
                             if (write_out) {
@@ -664,7 +698,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 #pragma unroll
                                 for (int b0 = 0; b0 < HALF / 4; b0 += HALF / 8) {
                                     for (int sl = 0; sl < wi.nsl; ++sl) {
-                                        const float *src = first + (size_t)sl * kNumEpiWarps * kWarpFloats + b0 * 128;
+                                        const float *src = first + (size_t)sl * kWarps * kWarpFloats + b0 * 128;
                                         float4 u[HALF / 8];
 #pragma unroll
                                         for (int j = 0; j < HALF / 8; ++j) u[j] = __ldcg(reinterpret_cast<const float4 *>(src + j * 128));
@@ -701,6 +735,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     if (g.chain == CHAIN_BESIDE) pdl_wait();
     tc_fence_before_sync();
     __syncthreads();
+    if (PAIR) cluster_sync();   // no more arrivals from the other CTA, and the pair's MMAs read no more of this CTA's memory
     if (*abort_flag) {
         // give copies and MMAs still in flight time to land before the CTA's resources go away
         const uint64_t t0 = globaltimer_ns();
@@ -710,7 +745,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     }
     if (warp == 1) {
         tc_fence_after_sync();
-        tmem_dealloc<false>(tmem_base, C::kTmemCols);
+        tmem_dealloc<PAIR>(tmem_base, C::kTmemCols);
     }
 }
 
@@ -762,32 +797,39 @@ int sm_count()
     return n;
 }
 
-template <MmaKind KIND, int BN, int SCALE, bool OUT_F32>
+template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32>
 int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc, bool cleared, cudaStream_t st)
 {
-    using C = Cfg<KIND, BN, SCALE>;
-    auto kern = gemm_kernel<KIND, BN, SCALE, OUT_F32>;
+    using C = Cfg<KIND, BN, SCALE, PAIR>;
+    auto kern = gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32>;
     // a per-function, per-device attribute; setting it on every launch is cheap and correct on any device
     SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
-    const int num_tiles = (int)(ceil_div(g.Mo, BM) * ceil_div(g.No, BN));
-    const int sms = sm_count();
+    const int num_tiles = (int)(ceil_div(g.Mo, C::BM) * ceil_div(g.No, BN));
+    const int units = sm_count() / C::kCtas;
     GemmArgs ga = g;
-    ga.work = plan_work(num_tiles, (int)ceil_div(g.Kc, C::kStageK), sms, kMinSliceStages, SCALE == SCALE_VEC_B && g.partials);
+    ga.work = plan_work(num_tiles, (int)ceil_div(g.Kc, C::kStageK), units, kMinSliceStages, SCALE == SCALE_VEC_B && g.partials, kMaxSlicedItems / C::kCtas);
     if (ga.work.nsplit > 1 && !cleared)
-        SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * sizeof(uint32_t), st));
-    const int grid = ga.work.num_items < sms ? ga.work.num_items : sms;
-    return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, 1, tmA, tmB, tmO, ga, idesc);
+        SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * C::kCtas * sizeof(uint32_t), st));
+    const int grid = (ga.work.num_items < units ? ga.work.num_items : units) * C::kCtas;
+    return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, C::kCtas, tmA, tmB, tmO, ga, idesc);
 }
 
+template <MmaKind KIND, int BN, int SCALE>
+int launch_gemm_form(bool pair, bool out_f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc,
+                     bool cleared, cudaStream_t st)
+{
+    if (pair)
+        return out_f32 ? launch_gemm<KIND, BN, SCALE, true, true>(tmA, tmB, tmO, g, idesc, cleared, st)
+                       : launch_gemm<KIND, BN, SCALE, true, false>(tmA, tmB, tmO, g, idesc, cleared, st);
+    return out_f32 ? launch_gemm<KIND, BN, SCALE, false, true>(tmA, tmB, tmO, g, idesc, cleared, st)
+                   : launch_gemm<KIND, BN, SCALE, false, false>(tmA, tmB, tmO, g, idesc, cleared, st);
+}
 template <MmaKind KIND, int BN>
-int launch_gemm_scale(int scale, bool out_f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g,
+int launch_gemm_scale(int scale, bool pair, bool out_f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g,
                       uint32_t idesc, bool cleared, cudaStream_t st)
 {
-    if (scale == SCALE_BLOCK_B)
-        return out_f32 ? launch_gemm<KIND, BN, SCALE_BLOCK_B, true>(tmA, tmB, tmO, g, idesc, cleared, st)
-                       : launch_gemm<KIND, BN, SCALE_BLOCK_B, false>(tmA, tmB, tmO, g, idesc, cleared, st);
-    return out_f32 ? launch_gemm<KIND, BN, SCALE_VEC_B, true>(tmA, tmB, tmO, g, idesc, cleared, st)
-                   : launch_gemm<KIND, BN, SCALE_VEC_B, false>(tmA, tmB, tmO, g, idesc, cleared, st);
+    return scale == SCALE_BLOCK_B ? launch_gemm_form<KIND, BN, SCALE_BLOCK_B>(pair, out_f32, tmA, tmB, tmO, g, idesc, cleared, st)
+                                  : launch_gemm_form<KIND, BN, SCALE_VEC_B>(pair, out_f32, tmA, tmB, tmO, g, idesc, cleared, st);
 }
 
 }  // namespace
@@ -795,7 +837,7 @@ int launch_gemm_scale(int scale, bool out_f32, const CUtensorMap &tmA, const CUt
 size_t gemm_ws_bytes() { return 256; }
 // Workspace with which the weight-gradient product may slice the tiles of its last wave along the contraction:
 // status word, arrival counters, one FP32 tile per slice.
-size_t gemm_ws_bytes_sliced() { return kSliceCountersOffset + kSliceCountersBytes + (size_t)kMaxSlicedItems * BM * 256 * sizeof(float); }
+size_t gemm_ws_bytes_sliced() { return kSliceCountersOffset + kSliceCountersBytes + (size_t)kMaxSlicedItems * CM * 256 * sizeof(float); }
 
 // (gemm_bf16.cu slices the same way.)
 // The parts of a workspace of gemm_ws_bytes() or gemm_ws_bytes_sliced(), for one GEMM.
@@ -817,7 +859,7 @@ namespace {
 std::atomic<long long> g_wait_limit_ns{2000000000ll};   // bound of every device-side wait of the GEMM kernels
 std::atomic<int> g_tx_skew{0};                           // bytes added to what a stage's barrier expects (a wait that cannot complete)
 std::atomic<int> g_slicing{1};                           // 0: the weight-gradient product never slices its last wave
-std::atomic<int> g_kernel_choice{0};                     // 0, 1 = single-CTA kernels, 2 = CTA-pair kernels for quantized operands
+std::atomic<int> g_kernel_choice{0};                     // 0 = by shape, 1 = single-CTA form, 2 = CTA-pair form (paper-rule kernels)
 }  // namespace
 
 // The hooks' current values, for the other GEMM families (gemm_mx.cu).
@@ -829,11 +871,6 @@ void gemm_debug_hooks(uint64_t *wait_limit_ns, int *tx_skew)
 
 bool gemm_slicing_enabled() { return g_slicing.load() != 0; }
 
-int gemm_pair_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, int64_t Mo, int64_t No, int64_t Kc, const float *sa,
-                   int64_t sa_chunk_stride, const float *sb, int64_t sb_chunk_stride, int64_t sb_blk_stride, int scale_mode, void *out,
-                   int out_dtype, int accumulate, uint32_t *status, uint64_t wait_limit_ns, int tx_skew, cudaStream_t st);
-
-int launch_stat_jobs(const StatJobs &jobs, cudaStream_t st);   // quantize.cu
 int gemm_bf16_impl(const void *a, bool a_mn, const void *b, bool b_mn, int64_t Mo, int64_t No, int64_t Kc, void *out, int out_dtype, int accumulate,
                    const GemmWs &w, cudaStream_t st, const ChainLink &link);   // gemm_bf16.cu
 
@@ -894,16 +931,14 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     const int tx_skew = g_tx_skew.load();
     const bool f32 = out_dtype == SNIP_OUT_FP32;
 
-    // The CTA-pair kernels (gemm_pair.cu) are an alternative form of the same product, kept for comparison: they
-    // run only when asked for through snip_debug_set (on the 7B shapes they are slower than the kernels below).
+    // Pairs of CTAs on 256-row tiles halve a CTA's share of B and keep six stages instead of four: forward and input gradient 2-4 % faster
+    // (FP8 16384x12288x4096 837 -> 808 us, 8192x8640x3200 248 -> 239 us, FP4 655 -> 635 us).  The weight gradient, whose promotion sets the pace,
+    // gains nothing (FP8 1062 / 1059 us, FP4 950 / 956 us) and neither do shapes with fewer such tiles than pairs of SMs.
     const int choice = g_kernel_choice.load();
-    if (choice == 2) {
-        rc = launch_stat_jobs(g.stats, st);   // these kernels neither reduce statistics nor clear the status word
-        if (rc) return rc;
-        if (!w.cleared) SNIP_CUDA_TRY(cudaMemsetAsync(g.status, 0, sizeof(uint32_t), st));
-        return gemm_pair_impl(fmt_a, fmt_b, a_codes, b_codes, Mo, No, Kc, sa, sa_chunk_stride, sb, sb_chunk_stride, sb_blk_stride, scale_mode,
-                              out, out_dtype, accumulate, g.status, g.wait_limit_ns, tx_skew, st);
-    }
+    auto use_pair = [&](int tile_n) {
+        if (choice != 0) return choice == 2;
+        return scale_mode == SCALE_BLOCK_B && ceil_div(Mo, 256) * ceil_div(No, tile_n) >= sm_count() / 2;
+    };
 
     CUtensorMap tmA, tmB, tmO;
     // output boxes of 32 rows x 64 bytes for the TMA stores of the block-mode epilogue
@@ -918,17 +953,21 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         // cap: 16384x12288x4096 755 -> 673 us, 8192x3200x8640 215 -> 193 us, 8192x2048x256 16.4 -> 14.5 us.  The weight gradient over
         // whole chunks takes the path below: with two operations per element the wider tile is as fast or faster.
         constexpr int BN = 192;
-        rc = make_operand_map(&tmA, a_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, Mo, Kc / 2, Kc / 2, 128, BM);
+        const bool pair = use_pair(BN);
+        const int ctas = pair ? 2 : 1;
+        rc = make_operand_map(&tmA, a_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, Mo, Kc / 2, Kc / 2, 128, CM);
         if (rc) return rc;
-        rc = make_operand_map(&tmB, b_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, No, Kc / 2, Kc / 2, 128, BN);
+        rc = make_operand_map(&tmB, b_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, No, Kc / 2, Kc / 2, 128, BN / ctas);
         if (rc) return rc;
-        const uint32_t idesc = make_idesc_block_scaled(1, 1, BM, BN);
-        g.stage_tx_bytes = (BM + BN) * 128 + tx_skew;
-        return launch_gemm_scale<MmaKind::MXF4, BN>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
+        const uint32_t idesc = make_idesc_block_scaled(1, 1, CM * ctas, BN);
+        g.stage_tx_bytes = (CM + BN / ctas) * 128 + tx_skew;
+        return launch_gemm_scale<MmaKind::MXF4, BN>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
     }
     // FP8 x FP8, the mixed pairs and the FP4 x FP4 weight gradient over whole chunks: kind::f8f6f4; FP4 operands are expanded by
     // the TMA unit to one 16-byte-aligned group per 16 elements, which is the layout this MMA kind reads
     constexpr int BN = 256;
+    const bool pair = use_pair(BN);
+    const int ctas = pair ? 2 : 1;
     const bool a4 = fmt_a == SNIP_FMT_FP4_E2M1, b4 = fmt_b == SNIP_FMT_FP4_E2M1;
     // The expanding 4-bit tensor-map type only accepts an inner extent that is a multiple of 128
     // elements.  A contraction length ending in a 64-wide tile is therefore declared rounded up: the
@@ -938,16 +977,16 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // length never get here: both maps would be padded.)
     const int64_t kpad = ceil_div(Kc, 128) * 128;
     rc = make_operand_map(&tmA, a_codes, a4 ? CU_TENSOR_MAP_DATA_TYPE_16U4_ALIGN16B : CU_TENSOR_MAP_DATA_TYPE_UINT8, Mo, a4 ? kpad : Kc,
-                          a4 ? Kc / 2 : Kc, 128, BM);
+                          a4 ? Kc / 2 : Kc, 128, CM);
     if (rc) return rc;
     rc = make_operand_map(&tmB, b_codes, b4 ? CU_TENSOR_MAP_DATA_TYPE_16U4_ALIGN16B : CU_TENSOR_MAP_DATA_TYPE_UINT8, No, b4 ? kpad : Kc,
-                          b4 ? Kc / 2 : Kc, 128, BN);
+                          b4 ? Kc / 2 : Kc, 128, BN / ctas);
     if (rc) return rc;
-    const uint32_t idesc = make_idesc(a4 ? 5 : 0, b4 ? 5 : 0, BM, BN);
+    const uint32_t idesc = make_idesc(a4 ? 5 : 0, b4 ? 5 : 0, CM * ctas, BN);
     // an FP4 operand expanded by the TMA unit occupies 128 B per row in shared memory but reports
     // only its 64 packed source bytes to the barrier
-    g.stage_tx_bytes = BM * (a4 ? 64 : 128) + BN * (b4 ? 64 : 128) + tx_skew;
-    return launch_gemm_scale<MmaKind::F8F6F4, BN>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
+    g.stage_tx_bytes = CM * (a4 ? 64 : 128) + BN / ctas * (b4 ? 64 : 128) + tx_skew;
+    return launch_gemm_scale<MmaKind::F8F6F4, BN>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
 }
 
 }  // namespace snip

@@ -1158,18 +1158,6 @@ size_t stats_ws_bytes(int64_t rows, int64_t cols, bool rowstats)
 
 }  // namespace
 
-namespace {
-__global__ void stat_jobs_kernel(const StatJobs jobs) { reduce_stats_warp(jobs.job[blockIdx.x], threadIdx.x); }
-}  // namespace
-// The reductions of a chain as a launch of their own.
-int launch_stat_jobs(const StatJobs &jobs, cudaStream_t st)
-{
-    if (jobs.count == 0) return SNIP_OK;
-    stat_jobs_kernel<<<jobs.count, 32, 0, st>>>(jobs);
-    SNIP_CUDA_TRY(cudaGetLastError());
-    return SNIP_OK;
-}
-
 // Internal entry used by snip_quantize and by the linear-layer calls.
 int quantize_impl_ex(const void *x, int64_t rows, int64_t cols, int64_t ld, int fmt, int block, uint32_t flags, int pow2, void *sf,
                      void *codes, float *scales, snip_stats_t *stats, double *row_stats, void *ws, size_t ws_bytes, cudaStream_t st, const ChainLink &link = ChainLink());
