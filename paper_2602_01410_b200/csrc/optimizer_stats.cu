@@ -14,7 +14,11 @@ int gemm_sm_count();
 namespace {
 
 constexpr int kThreads = 256;
-constexpr int kCtasPerSm = 8;
+// Every CTA of the grid resident, two groups in flight per thread (120 KB per SM).  Eight CTAs per SM at 40 registers were launched before,
+// six fitted: 11008 x 4096 with bf16 gradients 76.4 -> 70.8 us = 6.37 TB/s, 97 % of the copy rate.  Three groups on five CTAs or four on
+// four: 72.1 / 71.7 us, and 14.5 instead of 12.5 us on 2048 x 2048.
+constexpr int kCtasPerSm = 6;
+constexpr int kGroups = 2;
 
 __device__ __forceinline__ float sens_term_sq(float m, float v, float g, float omb1, float omb2, float eps)
 {
@@ -30,7 +34,7 @@ __device__ __forceinline__ float sens_term_sq(float m, float v, float g, float o
 }
 
 template <bool G_BF16>
-__global__ void __launch_bounds__(kThreads) adamw_sensitivity_kernel(const float *__restrict__ m, const float *__restrict__ v, const void *__restrict__ g,
+__global__ void __launch_bounds__(kThreads, kCtasPerSm) adamw_sensitivity_kernel(const float *__restrict__ m, const float *__restrict__ v, const void *__restrict__ g,
                                                                      int64_t n4, float omb1, float omb2, float eps, double *partials)
 {
     __shared__ double red[kThreads / 32];
@@ -49,15 +53,23 @@ __global__ void __launch_bounds__(kThreads) adamw_sensitivity_kernel(const float
         return (sens_term_sq(mm.x, vv.x, gg.x, omb1, omb2, eps) + sens_term_sq(mm.y, vv.y, gg.y, omb1, omb2, eps)) +
                (sens_term_sq(mm.z, vv.z, gg.z, omb1, omb2, eps) + sens_term_sq(mm.w, vv.w, gg.w, omb1, omb2, eps));
     };
-    // two groups of four elements per iteration: 80 (bf16 g) or 96 bytes in flight per thread
+    // kGroups groups of four elements per iteration, all loads first
     const int64_t stride = (int64_t)gridDim.x * kThreads;
     int64_t i = (int64_t)blockIdx.x * kThreads + threadIdx.x;
-    for (; i + stride < n4; i += 2 * stride) {
-        const float4 m0 = __ldg(m4 + i), v0 = __ldg(v4 + i), m1 = __ldg(m4 + i + stride), v1 = __ldg(v4 + i + stride);
-        const float4 g0 = load_g(i), g1 = load_g(i + stride);
-        acc += (double)(four(m0, v0, g0) + four(m1, v1, g1));
+    for (; i + (kGroups - 1) * stride < n4; i += kGroups * stride) {
+        float4 mm[kGroups], vv[kGroups], gg[kGroups];
+#pragma unroll
+        for (int u = 0; u < kGroups; ++u) {
+            mm[u] = __ldg(m4 + i + u * stride);
+            vv[u] = __ldg(v4 + i + u * stride);
+            gg[u] = load_g(i + u * stride);
+        }
+        float t = 0.0f;
+#pragma unroll
+        for (int u = 0; u < kGroups; ++u) t += four(mm[u], vv[u], gg[u]);
+        acc += (double)t;
     }
-    if (i < n4) acc += (double)four(__ldg(m4 + i), __ldg(v4 + i), load_g(i));
+    for (; i < n4; i += stride) acc += (double)four(__ldg(m4 + i), __ldg(v4 + i), load_g(i));
 #pragma unroll
     for (int off = 16; off > 0; off >>= 1) acc += __shfl_xor_sync(0xFFFFFFFFu, acc, off);
     if ((threadIdx.x & 31) == 0) red[threadIdx.x >> 5] = acc;
