@@ -492,8 +492,8 @@ int snip_select_scheme(int m, int n, const double *q, const int64_t *w, int64_t 
  *                              leaves on its own and snip_poll_status reports SNIP_ERR_TIMEOUT.
  *                              Nothing traps or faults; used with a short wait limit by the tests.
  *   SNIP_DEBUG_GEMM_KERNEL   : 0 (default) = the library chooses by shape, 1 = one CTA per tile, 2 = a pair of
- *                              CTAs per tile, for every quantized GEMM under the paper's rule (the two forms of
- *                              the same kernels; for A/B comparisons and tests).
+ *                              CTAs per tile, 3 = one CTA per tile of 128 columns, for every quantized GEMM under
+ *                              the paper's rule (forms of the same kernels; for A/B comparisons and tests).
  *   SNIP_DEBUG_GEMM_SLICING  : 1 (default) = the weight-gradient product may slice its last wave
  *                              when its workspace has room (snip_workspace_size), 0 = never.
  * Returns SNIP_ERR_ARG for an unknown key or a value out of range.

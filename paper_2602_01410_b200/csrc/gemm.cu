@@ -34,7 +34,9 @@ constexpr int CM = 128;   // output rows of a CTA
 constexpr int kGemmThreads = 384;  // warps 0-3: producer, MMA issuer, 2 scale loaders (wgrad) or idle; warps 4-11: epilogue
 constexpr int kNumEpiWarps = 8;
 static_assert(kNumEpiWarps == kSliceWarps, "slice counters");
-constexpr int kMinSliceStages = 8;   // shortest contraction slice of the weight-gradient product's last wave
+// Contraction slices of the weight-gradient product's last wave: no shorter than kMinSliceStages, and only where they shorten the CTAs' sequence
+// of stages by what the exchange of the partial sums takes (8-13 us; 2048 tokens x 256 x 2048: 15.6 us whole, 20.6 us in two slices).
+constexpr int kMinSliceStages = 8, kMinSavedStages = 20;
 constexpr int kSfCols = 32;  // tensor-memory columns holding constant scale factors (kind::mxf4)
 
 enum ScaleMode { SCALE_BLOCK_B = 1, SCALE_VEC_B = 2 };
@@ -71,7 +73,7 @@ struct Cfg {
     static constexpr int kABytes = CM * 128;
     static constexpr int kBBytes = kBLines * 128;
     static constexpr int kStageBytes = kABytes + kBBytes;
-    static constexpr int kStages = PAIR ? 6 : (BN >= 256 || SCALE == 1) ? 4 : 5;
+    static constexpr int kStages = PAIR ? 6 : BN <= 128 ? (SCALE == 1 ? 5 : 6) : (BN >= 256 || SCALE == 1) ? 4 : 5;
     // block mode (fwd / dgrad) fetches four chunks of scale factors per instruction into two alternating group slots:
     // [4 chunks][32 rows] S_a, then [2 blocks][4 chunks] S_b
     static constexpr int kGroupFloats = 144;
@@ -87,7 +89,7 @@ struct Cfg {
     // block mode (fwd / dgrad) writes its output through kOutSlots 2 KB staging tiles per warp and TMA stores; where shared
     // memory has room for a warp's whole bf16 tile no store is waited for before the next tile's sums
     static constexpr bool kTmaOut = (SCALE == 1);
-    static constexpr int kOutSlots = (BN == 192) ? 3 : 1;
+    static constexpr int kOutSlots = (BN == 192) ? 3 : (BN == 128) ? 2 : 1;
     static constexpr int kOutStageBytes = kTmaOut ? kNumEpiWarps * kOutSlots * 2048 : 0;
     static constexpr int kSmemBytes = kStages * kStageBytes + kSbInvBytes + kOutStageBytes + 256 + 1024;  // + barriers + alignment slack
     static_assert(kSmemBytes <= 232448, "shared memory budget");
@@ -199,8 +201,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // 32 columns; fwd / dgrad: 2.5 % faster than 16)
     constexpr int GC = (SCALE == SCALE_VEC_B) ? 16 : 32;
     constexpr int G = HALF / GC;     // groups handled by one epilogue warp per chunk
-    constexpr int D = (SCALE == SCALE_VEC_B) ? (G < 6 ? G : 4) : (BN == 192) ? G : 2;   // groups of staging registers next to the accumulators
-    // (192-wide tiles: 96 accumulators leave room for the whole chunk, so the buffer goes back before any multiplication)
+    constexpr int D = (SCALE == SCALE_VEC_B) ? (G < 6 ? G : 4) : (BN <= 192) ? G : 2;   // groups of staging registers next to the accumulators
+    // (tiles of up to 192 columns: at most 96 accumulators leave room for the whole chunk, so the buffer goes back before any multiplication)
 
     extern __shared__ uint8_t smem_raw[];
     // operand tiles need 1024-byte alignment for the 128-byte swizzle
@@ -483,7 +485,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
             // outside the matrix together: row counts are multiples of 64); lanes 0..3 (0..7 with two blocks)
             // fetch S_b of one chunk each.  Group gn lands in slot gn % 2; groups are requested in order, so the source pointers
             // only step (64-bit index products and bounds per request: 3-6 % of the FP4 kernels).
-            constexpr int kBlocksPerWarp = ((HALF % 128) == 0) ? 1 : 2;
+            constexpr int kBlocksPerWarp = ((HALF % 128) == 0 || (128 % HALF) == 0) ? 1 : 2;
             const float *pa = g.sa + (int64_t)(lane >> 3) * g.sa_chunk_stride + row0 + (lane & 7) * 4;
             const float *pb = g.sb + (int64_t)min(blk0 + (lane >> 2), blk_last) * g.sb_blk_stride + (int64_t)(lane & 3) * g.sb_chunk_stride;
             const int64_t pa_step = 4 * g.sa_chunk_stride, pb_step = 4 * g.sb_chunk_stride;
@@ -693,20 +695,46 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                             write_out = (old == (uint32_t)wi.nsl - 1u);
                             if (write_out) {
                                 __threadfence();
-                                // half a warp's share at a time, all its loads of a slice in flight together: 2 L2 round trips per
-                                // slice (one per 16 bytes before: 25 us at the end of every sliced launch)
+                                // The loads of half a warp's share of a slice are in flight together: 2 L2 round trips per slice (one per 16
+                                // bytes: 25 us at the end of every sliced launch).  Narrow tiles have registers for half a share of all slices
+                                // (22.5 -> 20.6 us for 8192 tokens x 256 x 2048; with 128 sums per thread it would spill).
+                                if constexpr (HALF <= 64) {
+                                    constexpr int kBatch = HALF / 8;
 #pragma unroll
-                                for (int b0 = 0; b0 < HALF / 4; b0 += HALF / 8) {
-                                    for (int sl = 0; sl < wi.nsl; ++sl) {
-                                        const float *src = first + (size_t)sl * kWarps * kWarpFloats + b0 * 128;
-                                        float4 u[HALF / 8];
+                                    for (int b0 = 0; b0 < HALF / 4; b0 += kBatch) {
+                                        float4 u[kMaxSlices][kBatch];
 #pragma unroll
-                                        for (int j = 0; j < HALF / 8; ++j) u[j] = __ldcg(reinterpret_cast<const float4 *>(src + j * 128));
+                                        for (int sl = 0; sl < kMaxSlices; ++sl) {
+                                            const float *src = first + (size_t)sl * kWarps * kWarpFloats + b0 * 128;
+                                            if (sl < wi.nsl) {
 #pragma unroll
-                                        for (int j = 0; j < HALF / 8; ++j) {
+                                                for (int j = 0; j < kBatch; ++j) u[sl][j] = __ldcg(reinterpret_cast<const float4 *>(src + j * 128));
+                                            }
+                                        }
+#pragma unroll
+                                        for (int j = 0; j < kBatch; ++j) {
+                                            float4 t = u[0][j];
+#pragma unroll
+                                            for (int sl = 1; sl < kMaxSlices; ++sl)
+                                                if (sl < wi.nsl) { t.x += u[sl][j].x; t.y += u[sl][j].y; t.z += u[sl][j].z; t.w += u[sl][j].w; }
                                             float *d = av + 4 * (b0 + j);
-                                            if (sl == 0) { d[0] = u[j].x; d[1] = u[j].y; d[2] = u[j].z; d[3] = u[j].w; }
-                                            else { d[0] += u[j].x; d[1] += u[j].y; d[2] += u[j].z; d[3] += u[j].w; }
+                                            d[0] = t.x; d[1] = t.y; d[2] = t.z; d[3] = t.w;
+                                        }
+                                    }
+                                } else {
+#pragma unroll
+                                    for (int b0 = 0; b0 < HALF / 4; b0 += HALF / 8) {
+                                        for (int sl = 0; sl < wi.nsl; ++sl) {
+                                            const float *src = first + (size_t)sl * kWarps * kWarpFloats + b0 * 128;
+                                            float4 u[HALF / 8];
+#pragma unroll
+                                            for (int j = 0; j < HALF / 8; ++j) u[j] = __ldcg(reinterpret_cast<const float4 *>(src + j * 128));
+#pragma unroll
+                                            for (int j = 0; j < HALF / 8; ++j) {
+                                                float *d = av + 4 * (b0 + j);
+                                                if (sl == 0) { d[0] = u[j].x; d[1] = u[j].y; d[2] = u[j].z; d[3] = u[j].w; }
+                                                else { d[0] += u[j].x; d[1] += u[j].y; d[2] += u[j].z; d[3] += u[j].w; }
+                                            }
                                         }
                                     }
                                 }
@@ -807,7 +835,8 @@ int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
     const int num_tiles = (int)(ceil_div(g.Mo, C::BM) * ceil_div(g.No, BN));
     const int units = sm_count() / C::kCtas;
     GemmArgs ga = g;
-    ga.work = plan_work(num_tiles, (int)ceil_div(g.Kc, C::kStageK), units, kMinSliceStages, SCALE == SCALE_VEC_B && g.partials, kMaxSlicedItems / C::kCtas);
+    ga.work = plan_work(num_tiles, (int)ceil_div(g.Kc, C::kStageK), units, kMinSliceStages, kMinSavedStages, SCALE == SCALE_VEC_B && g.partials,
+                        kMaxSlicedItems / C::kCtas);
     if (ga.work.nsplit > 1 && !cleared)
         SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * C::kCtas * sizeof(uint32_t), st));
     const int grid = (ga.work.num_items < units ? ga.work.num_items : units) * C::kCtas;
@@ -830,6 +859,18 @@ int launch_gemm_scale(int scale, bool pair, bool out_f32, const CUtensorMap &tmA
 {
     return scale == SCALE_BLOCK_B ? launch_gemm_form<KIND, BN, SCALE_BLOCK_B>(pair, out_f32, tmA, tmB, tmO, g, idesc, cleared, st)
                                   : launch_gemm_form<KIND, BN, SCALE_VEC_B>(pair, out_f32, tmA, tmB, tmO, g, idesc, cleared, st);
+}
+
+// 128-wide tiles, one CTA each.
+template <MmaKind KIND>
+int launch_gemm_narrow(int scale, bool out_f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc,
+                       bool cleared, cudaStream_t st)
+{
+    if (scale == SCALE_BLOCK_B)
+        return out_f32 ? launch_gemm<KIND, 128, SCALE_BLOCK_B, false, true>(tmA, tmB, tmO, g, idesc, cleared, st)
+                       : launch_gemm<KIND, 128, SCALE_BLOCK_B, false, false>(tmA, tmB, tmO, g, idesc, cleared, st);
+    return out_f32 ? launch_gemm<KIND, 128, SCALE_VEC_B, false, true>(tmA, tmB, tmO, g, idesc, cleared, st)
+                   : launch_gemm<KIND, 128, SCALE_VEC_B, false, false>(tmA, tmB, tmO, g, idesc, cleared, st);
 }
 
 }  // namespace
@@ -859,7 +900,7 @@ namespace {
 std::atomic<long long> g_wait_limit_ns{2000000000ll};   // bound of every device-side wait of the GEMM kernels
 std::atomic<int> g_tx_skew{0};                           // bytes added to what a stage's barrier expects (a wait that cannot complete)
 std::atomic<int> g_slicing{1};                           // 0: the weight-gradient product never slices its last wave
-std::atomic<int> g_kernel_choice{0};                     // 0 = by shape, 1 = single-CTA form, 2 = CTA-pair form (paper-rule kernels)
+std::atomic<int> g_kernel_choice{0};                     // 0 = by shape, 1 = single-CTA form, 2 = CTA-pair form, 3 = 128-wide tiles (paper-rule kernels)
 }  // namespace
 
 // The hooks' current values, for the other GEMM families (gemm_mx.cu).
@@ -940,6 +981,22 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         return scale_mode == SCALE_BLOCK_B && ceil_div(Mo, 256) * ceil_div(No, tile_n) >= sm_count() / 2;
     };
 
+    // Tiles 128 columns wide, one CTA each, where they shorten the launch: as a rule where the wider tiles leave more than half of the SMs idle,
+    // so that twice the tiles still are one wave (forward FP8 1024x2048x4096 18.0 -> 12.5 us, 8192x256x2048 11.2 -> 8.3 us, 512x512x512 6.6 -> 5.2
+    // us; FP4 1024x4096x4096, two waves either way, 24.8 -> 18.6 us; weight gradient 8192x256x2048 28.6 -> 20.6 us).  A launch lasts as long as
+    // the pipeline stages that its SMs run one after the other (kMinSavedStages more where its last wave is sliced) times what a stage of a narrow
+    // tile takes next to a wide one's: measured 0.64-0.68 forward and input gradient (0.72 against 192 columns), 0.69-0.79 weight gradient.
+    auto use_narrow = [&](int tile_n, int stage_k, float ratio) {
+        if (choice != 0) return choice == 3;
+        auto stages = [&](int bn) {
+            const int sms = sm_count(), tiles = (int)(ceil_div(Mo, CM) * ceil_div(No, bn)), per_tile = (int)ceil_div(Kc, stage_k);
+            const WorkSplit sp = plan_work(tiles, per_tile, sms, kMinSliceStages, kMinSavedStages, scale_mode == SCALE_VEC_B && g.partials);
+            if (sp.nsplit > 1) return (float)(sp.split_first / sms) * per_tile + (float)per_tile / sp.nsplit + kMinSavedStages;
+            return (float)ceil_div(tiles, sms) * per_tile;
+        };
+        return stages(128) * ratio < stages(tile_n);
+    };
+
     CUtensorMap tmA, tmB, tmO;
     // output boxes of 32 rows x 64 bytes for the TMA stores of the block-mode epilogue
     rc = f32 ? make_operand_map(&tmO, out, CU_TENSOR_MAP_DATA_TYPE_FLOAT32, Mo, No, No * 4, 16, 32, CU_TENSOR_MAP_SWIZZLE_64B)
@@ -952,8 +1009,9 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         // warps' registers at once, and with half the operand bytes and a quarter of the tensor time it stays below the power
         // cap: 16384x12288x4096 755 -> 673 us, 8192x3200x8640 215 -> 193 us, 8192x2048x256 16.4 -> 14.5 us.  The weight gradient over
         // whole chunks takes the path below: with two operations per element the wider tile is as fast or faster.
-        constexpr int BN = 192;
-        const bool pair = use_pair(BN);
+        const bool narrow = use_narrow(192, 256, 0.72f);
+        const int BN = narrow ? 128 : 192;
+        const bool pair = !narrow && use_pair(BN);
         const int ctas = pair ? 2 : 1;
         rc = make_operand_map(&tmA, a_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, Mo, Kc / 2, Kc / 2, 128, CM);
         if (rc) return rc;
@@ -961,12 +1019,14 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         if (rc) return rc;
         const uint32_t idesc = make_idesc_block_scaled(1, 1, CM * ctas, BN);
         g.stage_tx_bytes = (CM + BN / ctas) * 128 + tx_skew;
-        return launch_gemm_scale<MmaKind::MXF4, BN>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
+        if (narrow) return launch_gemm_narrow<MmaKind::MXF4>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
+        return launch_gemm_scale<MmaKind::MXF4, 192>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
     }
     // FP8 x FP8, the mixed pairs and the FP4 x FP4 weight gradient over whole chunks: kind::f8f6f4; FP4 operands are expanded by
     // the TMA unit to one 16-byte-aligned group per 16 elements, which is the layout this MMA kind reads
-    constexpr int BN = 256;
-    const bool pair = use_pair(BN);
+    const bool narrow = use_narrow(256, 128, scale_mode == SCALE_BLOCK_B ? 0.68f : 0.75f);
+    const int BN = narrow ? 128 : 256;
+    const bool pair = !narrow && use_pair(BN);
     const int ctas = pair ? 2 : 1;
     const bool a4 = fmt_a == SNIP_FMT_FP4_E2M1, b4 = fmt_b == SNIP_FMT_FP4_E2M1;
     // The expanding 4-bit tensor-map type only accepts an inner extent that is a multiple of 128
@@ -986,7 +1046,8 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // an FP4 operand expanded by the TMA unit occupies 128 B per row in shared memory but reports
     // only its 64 packed source bytes to the barrier
     g.stage_tx_bytes = CM * (a4 ? 64 : 128) + BN / ctas * (b4 ? 64 : 128) + tx_skew;
-    return launch_gemm_scale<MmaKind::F8F6F4, BN>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
+    if (narrow) return launch_gemm_narrow<MmaKind::F8F6F4>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
+    return launch_gemm_scale<MmaKind::F8F6F4, 256>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
 }
 
 }  // namespace snip
@@ -1032,7 +1093,7 @@ extern "C" int snip_debug_set(int key, long long value)
     switch (key) {
         case SNIP_DEBUG_WAIT_LIMIT_NS: if (value <= 0) return SNIP_ERR_ARG; g_wait_limit_ns.store(value); return SNIP_OK;
         case SNIP_DEBUG_TX_SKEW_BYTES: if (value < 0 || value > 4096 || (value % 16) != 0) return SNIP_ERR_ARG; g_tx_skew.store((int)value); return SNIP_OK;
-        case SNIP_DEBUG_GEMM_KERNEL: if (value < 0 || value > 2) return SNIP_ERR_ARG; g_kernel_choice.store((int)value); return SNIP_OK;
+        case SNIP_DEBUG_GEMM_KERNEL: if (value < 0 || value > 3) return SNIP_ERR_ARG; g_kernel_choice.store((int)value); return SNIP_OK;
         case SNIP_DEBUG_GEMM_SLICING: if (value < 0 || value > 1) return SNIP_ERR_ARG; g_slicing.store((int)value); return SNIP_OK;
         default: return SNIP_ERR_ARG;
     }

@@ -39,7 +39,8 @@ struct Cfg {
     static constexpr int kSmemBytes = kStages * kStageBytes + kOutStageBytes + 256 + 1024;
     static_assert(kSmemBytes <= 232448, "shared memory budget");
 };
-constexpr int kMinSliceStages = 16;              // 1024 elements, as in the other kernels
+// Contraction slices: see gemm.cu (0.30 us a stage; 4096 x 1024 x 2048 weight gradient 23.9 us whole, 26.6 us in two slices that save 32 stages)
+constexpr int kMinSliceStages = 16, kMinSavedStages = 40;
 
 struct Bf16Args {
     int32_t Mo, No, Kc;
@@ -378,7 +379,7 @@ int gemm_bf16_impl(const void *a, bool a_mn, const void *b, bool b_mn, int64_t M
     g.stage_tx_bytes = (pair ? Cfg<true>::kStageBytes : Cfg<false>::kStageBytes) + tx_skew;
     const uint32_t idesc = make_idesc(1, 1, tile_m, BN) | (a_mn ? 1u << 15 : 0u) | (b_mn ? 1u << 16 : 0u);
     const int num_tiles = (int)(ceil_div(Mo, tile_m) * ceil_div(No, BN));
-    g.work = plan_work(num_tiles, (int)(Kc / kStageK), sms / ctas, kMinSliceStages, w.partials != nullptr && gemm_slicing_enabled(), kMaxSlicedItems / ctas);
+    g.work = plan_work(num_tiles, (int)(Kc / kStageK), sms / ctas, kMinSliceStages, kMinSavedStages, w.partials != nullptr && gemm_slicing_enabled(), kMaxSlicedItems / ctas);
     if (g.work.nsplit > 1 && !w.cleared)
         SNIP_CUDA_TRY(cudaMemsetAsync(w.counters, 0, (size_t)(num_tiles - g.work.split_first) * kNumEpiWarps * ctas * sizeof(uint32_t), st));
     const int units = sms / ctas, grid = (g.work.num_items < units ? g.work.num_items : units) * ctas;

@@ -19,8 +19,9 @@ struct WorkSplit {
 };
 
 // The tiles of the last, partial wave (all tiles, if there are fewer than SMs) are cut along the contraction into as many slices as
-// there are SMs to take them: at most kMaxSlices, none shorter than min_stages pipeline stages.
-inline WorkSplit plan_work(int num_tiles, int num_stages, int sms, int min_stages, bool slice, int max_items = kMaxSlicedItems)
+// there are SMs to take them: at most kMaxSlices, none shorter than min_stages pipeline stages.  Whole if that saves fewer than
+// min_saved stages, which the exchange of the slices' sums costs.
+inline WorkSplit plan_work(int num_tiles, int num_stages, int sms, int min_stages, int min_saved, bool slice, int max_items = kMaxSlicedItems)
 {
     WorkSplit s = {num_tiles, 1, num_tiles};
     if (!slice || sms <= 0) return s;
@@ -28,6 +29,7 @@ inline WorkSplit plan_work(int num_tiles, int num_stages, int sms, int min_stage
     int ns = rest > 0 ? sms / rest : 1;
     if (ns > kMaxSlices) ns = kMaxSlices;
     while (ns > 1 && (num_stages / ns < min_stages || rest * ns > max_items)) --ns;
+    if (num_stages - num_stages / ns < min_saved) return s;
     if (ns > 1) { s.split_first = full; s.nsplit = ns; s.num_items = full + rest * ns; }
     return s;
 }
