@@ -996,15 +996,17 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSmSr) quantize_small_ker
 // Fixed-order reduction of the per-CTA partials into one snip_stats_t (deterministic: every thread
 // owns a fixed strided subset, warps combine with shuffles, warp results are added in warp order).
 // Launched with programmatic stream serialization: it may start while the quantizer still runs and
-// blocks in griddepcontrol.wait until that grid has completed and its writes are visible.
+// blocks in griddepcontrol.wait until that grid has completed and its writes are visible.  A few warps: they find room beside the quantizer's
+// last CTAs, and there are few sums to add one after the other (1024 threads: 0.3 us more between a quantizer and the GEMM behind it).
 struct ReduceSets {
     const CtaPartial *partials[2];
     snip_stats_t *out[2];
 };
-__global__ void __launch_bounds__(1024) stats_reduce_kernel(const ReduceSets sets, int64_t n)
+constexpr int kReduceWarps = 8;
+__global__ void __launch_bounds__(32 * kReduceWarps) stats_reduce_kernel(const ReduceSets sets, int64_t n)
 {
-    __shared__ double sh_x[32], sh_e[32];
-    __shared__ float sh_m[32];
+    __shared__ double sh_x[kReduceWarps], sh_e[kReduceWarps];
+    __shared__ float sh_m[kReduceWarps];
     const CtaPartial *partials = sets.partials[blockIdx.x];
     snip_stats_t *out = sets.out[blockIdx.x];
     // a quantizer launched behind this reduction may take the SMs the previous quantizer is leaving; it waits
@@ -1013,7 +1015,8 @@ __global__ void __launch_bounds__(1024) stats_reduce_kernel(const ReduceSets set
     asm volatile("griddepcontrol.wait;" ::: "memory");
     double dx = 0.0, de = 0.0;
     float am = 0.0f;
-    for (int64_t i = threadIdx.x; i < n; i += 1024) {
+#pragma unroll 4
+    for (int64_t i = threadIdx.x; i < n; i += 32 * kReduceWarps) {
         const double2 p = *reinterpret_cast<const double2 *>(&partials[i]);
         dx += p.x;
         de += p.y;
@@ -1031,7 +1034,8 @@ __global__ void __launch_bounds__(1024) stats_reduce_kernel(const ReduceSets set
     if (threadIdx.x == 0) {
         double tx = 0.0, te = 0.0;
         float tm = 0.0f;
-        for (int w = 0; w < 32; ++w) { tx += sh_x[w]; te += sh_e[w]; tm = fmaxf(tm, sh_m[w]); }
+#pragma unroll
+        for (int w = 0; w < kReduceWarps; ++w) { tx += sh_x[w]; te += sh_e[w]; tm = fmaxf(tm, sh_m[w]); }
         out->sumsq_x = tx;
         out->sumsq_err = te;
         out->amax = tm;
@@ -1129,7 +1133,7 @@ int launch_reduce(const ReduceSets &sets, int nsets, int64_t nparts, const Chain
     }
     cudaLaunchConfig_t cfg = {};
     cfg.gridDim = dim3((unsigned)nsets);
-    cfg.blockDim = dim3(1024);
+    cfg.blockDim = dim3(32 * kReduceWarps);
     cfg.stream = st;
     cudaLaunchAttribute attr[1];
     attr[0].id = cudaLaunchAttributeProgrammaticStreamSerialization;
