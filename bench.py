@@ -693,7 +693,7 @@ def run_layer_stats_case(api, torch, device, which, rows=16384, cols=4096, copie
         if i >= 2:
             times.append(e0.elapsed_time(e1))
     by = 2.0 * rows * cols
-    print(f"layer_stats_{which}: {min(times) * 1e3:.1f} us best of {len(times)} (memset + kernel + reduction), "
+    print(f"layer_stats_{which}: {min(times) * 1e3:.1f} us best of {len(times)} (kernel + reduction), "
           f"{by / (min(times) * 1e-3) / 1e9:.0f} GB/s of tensor read")
 
 

@@ -7,11 +7,14 @@
 //   warp 0      : TMA producer - streams 128-byte-wide operand tiles into a shared-memory ring
 //   warp 1      : MMA issuer   - one thread issues tcgen05.mma; owns the tensor-memory allocation
 //   warps 2..3  : weight-gradient product: loaders of the per-row / per-column scale factors (one ring of ready
-//                 reciprocals for the CTA); otherwise idle (they only give their registers to the epilogue warps)
+//                 reciprocals for the CTA); warp 2 also adds up the statistics of quantizers ahead.  They give their
+//                 registers to the epilogue warps
 //   warps 4..11 : promotion / epilogue - pull each chunk's partial sums out of tensor memory,
 //                 multiply by 1/(S_a*S_b) of that chunk and add into FP32 register accumulators
 //                 (so the scaling overlaps the next chunk's MMAs, which write the other
 //                 tensor-memory buffer), then round and store the tile.
+// Three forms, chosen by shape in gemm_impl: 128-row tiles of 256 (192) or of 128 columns on one CTA, 256-row tiles on a
+// pair of CTAs (tcgen05.mma.cta_group::2; the leader's MMA warp and barriers serve both).
 // All hand-offs use mbarriers with bounded waits; on a timeout the CTA raises a status word and
 // leaves cleanly (tensor memory is always released).
 #include <cuda.h>

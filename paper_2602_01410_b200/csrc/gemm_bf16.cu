@@ -5,10 +5,11 @@
 // and X[M,K] contracted over M) need no transposed copies.
 //
 // One CTA per SM, persistent, 384 threads; tiles of 256 x 256 shared by a pair of CTAs (tcgen05.mma.cta_group::2: each CTA holds 128
-// rows of A and of the accumulator and half of B's lines), or 128 x 256 on one CTA where there are few tiles.  Warp 0 streams 64-long stages of both operands (TMA, 128-byte swizzle),
-// warp 1 (of the pair's leader) issues the MMAs (one elected lane) into one of two 256-column accumulators, warp 2 reduces statistics left by the
-// quantizers ahead, warps 4-11 drain the other accumulator, round and store through the TMA unit.  The tiles of the last wave are
-// cut into contraction slices (work_items.cuh) where the workspace has room.  Every wait is bounded, as in gemm.cu.
+// rows of A and of the accumulator and half of B's lines), or 128 x 256 on one CTA where there are few tiles.  Warp 0 streams 64-long
+// stages of both operands (TMA, 128-byte swizzle), warp 1 (of the pair's leader) issues the MMAs (one elected lane) into one of two
+// 256-column accumulators, warp 2 reduces statistics left by the quantizers ahead, warps 4-11 drain the other accumulator, round and
+// store through the TMA unit.  The tiles of the last wave are cut into contraction slices (work_items.cuh) where the workspace has
+// room.  Every wait is bounded, as in gemm.cu.
 #include <cuda.h>
 #include <cuda_bf16.h>
 

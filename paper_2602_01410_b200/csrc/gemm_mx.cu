@@ -5,9 +5,10 @@
 // (Power-of-two block scales are the MX-format convention the paper cites in Sec. 2.3; the paper's own
 // rule FPX_MAX/amax needs the per-chunk FP32 promotion of gemm.cu.)
 //
-// One CTA per SM, persistent, 384 threads: warp 0 streams operand tiles (TMA) and 512-byte
-// scale-factor atoms (bulk copies) into a shared-memory ring; warp 1 copies each stage's atoms into
-// tensor memory (tcgen05.cp) and issues the MMAs; warps 4-11 drain the 128x256 FP32 accumulator
+// One CTA per SM, persistent, 384 threads; tiles of 256x256 shared by a pair of CTAs (tcgen05.mma.cta_group::2: each holds 128
+// rows and fetches half of B's lines), or 128x256 on one CTA where there are few.  Warp 0 streams operand tiles and 512-byte
+// scale-factor atoms into a shared-memory ring (both through tensor maps, so that a CTA can report them to its leader's
+// barrier); warp 1 copies each stage's atoms into tensor memory (tcgen05.cp) and issues the MMAs; warps 4-11 drain the FP32 accumulator
 // (one buffer: 256 columns, next to 12 or 24 scale-factor columns), round, and store through the TMA unit.
 // Warps 0 and 1 walk their loops as whole warps and one elected lane issues.  Every wait is bounded, as in gemm.cu.
 //

@@ -1,6 +1,6 @@
 // The three GEMMs of one linear layer under a precision choice (paper Fig. 5): quantize the two
 // operands with the tile kind their contraction calls for, then run the block-scaled GEMM.
-// Host-side composition only; all arithmetic is in the kernels of quantize.cu, gemm.cu and gemm_mx.cu.
+// Host-side composition only; all arithmetic is in the kernels of quantize.cu, gemm.cu, gemm_bf16.cu and gemm_mx.cu.
 #include "common.cuh"
 
 namespace snip {

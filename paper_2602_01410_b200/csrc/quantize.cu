@@ -16,7 +16,7 @@
 // Added options (paper Sec. 3.2 lets further quantization methods join the per-layer choices): the power-of-two scale
 // rule on the same tiles or on 32-long tiles (ROW_1x32 / COL_32x1: the maxima are combined over 4 lanes / 2 warps
 // instead of 16 lanes / 8 warps), with the scale exponents also written as the 512-byte atoms the block-scaled MMA
-// reads; and the two-level form in the style of NVFP4 (quantize_nvfp4_dual_kernel: 16-long tiles = two neighbouring
+// reads; and the two-level form in the style of NVFP4 (the two-output kernel's FAM_NV family: 16-long tiles = two neighbouring
 // lanes / the two row groups of a warp, an E4M3 scale byte per tile, a per-tensor factor from a caller-supplied bound).
 #include <cuda_bf16.h>
 #include <float.h>
