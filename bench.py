@@ -388,10 +388,10 @@ class TaggedStep:
                 for gi in range(3):
                     f = int(self.tags[l, j, gi])
                     self.flops_by_fmt[f] = self.flops_by_fmt.get(f, 0.0) + 2.0 * M * L.N * L.K
-        # a linear through snip_linear_fwd_bwd: 3 two-output quantizers + 3 reductions + 3 GEMMs; through the three separate calls, per GEMM:
-        # 2 quantizers (BF16 tags: statistics kernels, transposes) + 2 reductions + 1 GEMM
+        # a linear through snip_linear_fwd_bwd: 3 two-output quantizers + 3 GEMMs, which add up the statistics; through the three separate
+        # calls, per GEMM: 2 quantizers (BF16 tags: statistics only) + 1 GEMM
         n_fused = sum(1 for l in range(layers) for j in range(len(cfg.linears)) if FMT_BF16 not in [int(t) for t in self.tags[l, j]])
-        self.launches_per_step = n_fused * 9 + (layers * len(cfg.linears) - n_fused) * 15
+        self.launches_per_step = n_fused * 6 + (layers * len(cfg.linears) - n_fused) * 9
 
     def run(self, events=None, inputs=None, before=None):
         api, torch = self.api, self.torch
