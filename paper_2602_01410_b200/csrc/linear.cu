@@ -80,6 +80,23 @@ LinearPlan plan_for(int op, int64_t M, int64_t N, int64_t K)
     return p;
 }
 
+// What the members of a chain would refuse one by one is refused here, before the first of them is enqueued: a chain is enqueued whole
+// (CUDA's own errors aside) or not at all.  The dual quantizers check their three tensors and the statistics themselves, ahead of the
+// first launch.
+int check_outputs(int out_dtype, int accumulate, const void *o0, const void *o1 = nullptr, const void *o2 = nullptr)
+{
+    if (out_dtype != SNIP_OUT_BF16 && out_dtype != SNIP_OUT_FP32) return SNIP_ERR_ARG;
+    if (accumulate && out_dtype != SNIP_OUT_FP32) return SNIP_ERR_UNSUPPORTED;
+    return aligned16(o0) && aligned16(o1) && aligned16(o2) ? SNIP_OK : SNIP_ERR_ALIGN;
+}
+// Dimensions are 32-bit in the kernels, and so are the indices of scale-factor atoms.
+int check_dims(int64_t M, int64_t N, int64_t K, bool atoms)
+{
+    if (!valid_dim(M) || !valid_dim(N) || !valid_dim(K) || M > INT32_MAX || N > INT32_MAX || K > INT32_MAX) return SNIP_ERR_SHAPE;
+    const int64_t m = ceil_div(M, 128), n = ceil_div(N, 128), k = ceil_div(K, 128);
+    return atoms && (m * k > INT32_MAX || n * k > INT32_MAX || m * n > INT32_MAX) ? SNIP_ERR_SHAPE : SNIP_OK;
+}
+
 size_t sf_bytes(int64_t rows, int64_t cols) { return (size_t)(ceil_div(rows, 128) * ceil_div(cols, 128)) * 512; }
 
 size_t linear_ws_bytes(int op, int64_t M, int64_t N, int64_t K, int fmt_a, int fmt_b, bool mx = false)
@@ -102,10 +119,13 @@ int linear_impl(int op, const void *A, const void *B, void *out, int64_t M, int6
     if (mx && (fmt_a == SNIP_FMT_BF16 || fmt_b == SNIP_FMT_BF16 || accumulate)) return SNIP_ERR_UNSUPPORTED;
     if (!A || !B || !out) return SNIP_ERR_ARG;
     if (!valid_fmt(fmt_a) || !valid_fmt(fmt_b)) return SNIP_ERR_ARG;
-    if (!valid_dim(M) || !valid_dim(N) || !valid_dim(K)) return SNIP_ERR_SHAPE;
+    int rc = check_dims(M, N, K, mx);
+    if (rc) return rc;
     if ((fmt_a == SNIP_FMT_BF16) != (fmt_b == SNIP_FMT_BF16)) return SNIP_ERR_UNSUPPORTED;
     if (!ws || ws_bytes < linear_ws_bytes(op, M, N, K, fmt_a, fmt_b, mx)) return SNIP_ERR_WORKSPACE;
-    if (!aligned16(ws)) return SNIP_ERR_ALIGN;
+    if (!aligned16(ws) || !aligned16(A) || !aligned16(B) || !aligned16(stats_a) || !aligned16(stats_b)) return SNIP_ERR_ALIGN;
+    rc = check_outputs(out_dtype, accumulate, out);
+    if (rc) return rc;
     const LinearPlan p = plan_for(op, M, N, K);
     Carve c(ws, ws_bytes);
     void *gws = c.take(gemm_ws_bytes_sliced());
@@ -119,7 +139,6 @@ int linear_impl(int op, const void *A, const void *B, void *out, int64_t M, int6
     void *sf_a = nullptr, *sf_b = nullptr;
     if (mx) { sf_a = c.take(sf_bytes(p.rows_a, p.cols_a)); sf_b = c.take(sf_bytes(p.rows_b, p.cols_b)); }
 
-    int rc;
     const void *ga = A, *gb = B;
     // quantizers and GEMM form a chain: no statistics or clearing launches of their own, no gaps
     StatJobs jobs;
@@ -286,13 +305,16 @@ extern "C" int snip_linear_fwd_bwd(const void *X, const void *W, const void *dY,
     if (rc) return rc;
     if (!ws || ws_bytes < need) return SNIP_ERR_WORKSPACE;
     if (!aligned16(ws) || (stats6 && (reinterpret_cast<uintptr_t>(stats6) & 7u))) return SNIP_ERR_ALIGN;
-    cudaStream_t st = static_cast<cudaStream_t>(stream);
+    if (dy_rounding != SNIP_ROUND_NEAREST_EVEN && dy_rounding != SNIP_ROUND_STOCHASTIC) return SNIP_ERR_ARG;
     const bool mx = pow2_scale != 0;
+    rc = check_dims(M, N, K, mx);
+    if (!rc) rc = check_outputs(out_dtype, 0, Y, dX, dW);
+    if (rc) return rc;
+    cudaStream_t st = static_cast<cudaStream_t>(stream);
     const int fmt[6] = {fmt_fwd, fmt_wgrad, fmt_fwd, fmt_dgrad, fmt_dgrad, fmt_wgrad};
     const FwdBwdCarve f = carve_fwd_bwd(ws, M, N, K, fmt, pow2_scale);
     const int kind_xdy = pow2_scale == 2 ? SNIP_DUAL_ROW32_COL32T : SNIP_DUAL_ROW_COLT;
     const int kind_w = pow2_scale == 2 ? SNIP_DUAL_ROW32_COL32T : SNIP_DUAL_BLK_BLKT;
-    if (dy_rounding != SNIP_ROUND_NEAREST_EVEN && dy_rounding != SNIP_ROUND_STOCHASTIC) return SNIP_ERR_ARG;
     // stochastic rounding applies to the FP4 copies of dY (indices 4 and 5); an FP8 copy keeps nearest-even
     auto out_of = [&](int i) {
         const int sr = (i >= 4 && dy_rounding == SNIP_ROUND_STOCHASTIC && fmt[i] == SNIP_FMT_FP4_E2M1) ? 1 : 0;
@@ -389,6 +411,9 @@ extern "C" int snip_linear_fwd_bwd_nvfp4(const void *X, const void *W, const voi
     const NvCarve f = carve_nvfp4(ws, M, N, K);
     if (!ws || ws_bytes < f.total) return SNIP_ERR_WORKSPACE;
     if (!aligned16(ws) || (stats6 && (reinterpret_cast<uintptr_t>(stats6) & 7u))) return SNIP_ERR_ALIGN;
+    int rc = check_dims(M, N, K, true);
+    if (!rc) rc = check_outputs(out_dtype, 0, Y, dX, dW);
+    if (rc) return rc;
     cudaStream_t st = static_cast<cudaStream_t>(stream);
     const float *bx = bounds3, *bw = bounds3 + 1, *bdy = bounds3 + 2;
     auto stat = [&](int i) { return stats6 ? stats6 + i : nullptr; };
@@ -409,7 +434,7 @@ extern "C" int snip_linear_fwd_bwd_nvfp4(const void *X, const void *W, const voi
                                                 f.stats_ws[1], f.stats_ws_bytes[1]),
                                  two_level_task(dY, M, N, N, bdy, f.codes[4], f.sf[4], stat(4), f.codes[5], f.sf[5], stat(5), dy_rounding, dy_seed,
                                                 f.stats_ws[2], f.stats_ws_bytes[2])};
-    int rc = quantize_xwd_impl(tensors, st, quant);
+    rc = quantize_xwd_impl(tensors, st, quant);
     if (rc) return rc;
     rc = gemm_nvfp4_impl(f.codes[0], f.codes[2], f.sf[0], f.sf[2], bx, bw, M, N, K, Y, out_dtype, gw, st, mult[0]);
     if (rc) return rc;

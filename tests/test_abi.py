@@ -112,3 +112,39 @@ def test_host_side_checks_of_the_added_options(lib):
     assert lib.snip_linear_fwd_bwd_nvfp4_workspace(512, 512, 512, wb) == 0 and wb.value > 6 * 512 * 512 // 2
     lib.snip_linear_fwd_bwd_nvfp4.argtypes = [vp, vp, vp, vp, vp, vp, i64, i64, i64, i32, vp, i32, ctypes.c_uint64, vp, vp, sz, vp]
     assert lib.snip_linear_fwd_bwd_nvfp4(0x1000, 0x2000, 0x3000, 0x4000, 0x5000, 0x6000, 512, 512, 512, 0, 0x100, 0, 0, None, 0x7000, 64, None) == 5
+
+
+def test_linear_calls_refuse_before_anything_is_enqueued(lib):
+    # What only the products check (alignment and type of the outputs) and what only the second quantizer checks (alignment of the
+    # second operand and of its statistics) is refused ahead of the first launch: with no device, and with none asked for.
+    vp, i64, sz, i32 = ctypes.c_void_p, ctypes.c_int64, ctypes.c_size_t, ctypes.c_int
+    P, big = 0x10000, 1 << 40
+    lib.snip_linear_fwd_bwd.argtypes = [vp] * 6 + [i64] * 3 + [i32] * 6 + [ctypes.c_uint64, vp, vp, sz, vp]
+    lib.snip_linear_fwd_bwd_nvfp4.argtypes = [vp] * 6 + [i64] * 3 + [i32, vp, i32, ctypes.c_uint64, vp, vp, sz, vp]
+    lib.snip_linear_wgrad.argtypes = [vp, vp, vp, i64, i64, i64, i32, i32, i32, i32, vp, vp, vp, sz, vp]
+    lib.snip_linear_mx.argtypes = [i32, vp, vp, vp, i64, i64, i64, i32, i32, i32, vp, vp, vp, sz, vp]
+
+    def fwd_bwd(y=P, dx=P, dw=P, out=0, dims=(128, 128, 128), pow2=0, rounding=0):
+        return lib.snip_linear_fwd_bwd(P, P, P, y, dx, dw, *dims, 1, 1, 2, out, pow2, rounding, 0, P, P, big, None)
+
+    def nvfp4(y=P, dx=P, dw=P, out=0):
+        return lib.snip_linear_fwd_bwd_nvfp4(P, P, P, y, dx, dw, 128, 128, 128, out, P, 0, 0, P, P, big, None)
+
+    for call in (fwd_bwd, nvfp4, lambda **kw: fwd_bwd(pow2=1, **kw), lambda **kw: fwd_bwd(pow2=2, **kw)):
+        for name in ("y", "dx", "dw"):
+            assert call(**{name: P + 8}) == 3, name
+        assert call(out=2) == 1
+    assert fwd_bwd(rounding=2) == 1
+    assert fwd_bwd(dims=(1 << 31, 128, 128)) == 2
+
+    def wgrad(a=P, b=P, out=P, fmt=1, dtype=0, acc=0, sa=P, sb=P):
+        return lib.snip_linear_wgrad(a, b, out, 128, 128, 128, fmt, fmt, dtype, acc, sa, sb, P, big, None)
+
+    def mx(a=P, b=P, out=P, dtype=0, sa=P, sb=P):
+        return lib.snip_linear_mx(0, a, b, out, 128, 128, 128, 1, 1, dtype, sa, sb, P, big, None)
+
+    for call in (wgrad, lambda **kw: wgrad(fmt=0, **kw), mx):   # fmt 0: BF16 tags, statistics only ahead of the product
+        for name in ("a", "b", "out", "sa", "sb"):
+            assert call(**{name: P + 8}) == 3, name
+        assert call(dtype=2) == 1
+    assert wgrad(acc=1) == 4 and wgrad(fmt=0, acc=1) == 4
