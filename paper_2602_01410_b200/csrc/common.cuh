@@ -1,4 +1,4 @@
-// Shared host-side helpers of the SNIP library: status handling and argument checks.
+// Shared by all sources of the SNIP library: status handling, argument checks, chains of dependent launches.
 #pragma once
 #include <cuda_runtime.h>
 #include <stdint.h>
@@ -43,10 +43,35 @@ struct DualOut {
 //   CHAIN_NONE  : a call of its own (starts after the kernel ahead of it on the stream; a quantizer launches its own statistics
 //                 reduction)
 //   CHAIN_FIRST : starts after the kernel ahead of it has completed, then lets the next one start beside it
-//   CHAIN_BESIDE: independent of the members ahead of it: starts at once and waits for the one ahead only before it ends, so that
-//                 "the last member has completed" keeps meaning "all of them have"
+//   CHAIN_BESIDE: reads nothing that the member directly ahead of it writes: starts beside it and waits for it only before it ends,
+//                 so that "the last member has completed" keeps meaning "all of them have"
 //   CHAIN_AFTER : its prologue runs beside the members ahead of it, its work after they have completed
+// What a CHAIN_BESIDE member does read was written further ahead: the second and third quantizer read tensors made before the call, the
+// second and third GEMM read what the quantizers left.  That is complete when the member starts, because a grid is scheduled only when
+// every CTA of the one ahead has let it be, and a FIRST or AFTER member does so after its own wait (chain_start).  Hence the order of a
+// chain: FIRST, then BESIDE for further quantizers, AFTER for the first GEMM, BESIDE for the others.  The waits made those writes visible
+// to the grids that waited, not to the one that starts beside them: its SM's L1 may still hold an earlier call's values.  The quantizers
+// read past L1 (cp.async.cg, __ldcg); the GEMMs, which read scale factors and bounds through it, begin with an acquire (chain_acquire).
 enum ChainRole { CHAIN_NONE = 0, CHAIN_FIRST = 1, CHAIN_BESIDE = 2, CHAIN_AFTER = 3 };
+
+// First thing in a GEMM, ahead of the CTA's first barrier, which passes it on to all threads: nothing stale is read from L1, and the TMA
+// unit's reads of the operands are ordered behind the acquire too.  By a thread of a warp that has nothing to set up: the fence takes
+// about as long as tensor memory's allocation beside it (by every thread behind that, it was 0.3 us of each such GEMM).
+__device__ __forceinline__ void chain_acquire(int role)
+{
+    if (role == CHAIN_BESIDE && threadIdx.x == 96) asm volatile("fence.acq_rel.gpu;\n\tfence.proxy.async.global;" ::: "memory");
+}
+// Start of every kernel that may be a member of a chain, by all threads, before they touch memory that a kernel ahead writes.
+__device__ __forceinline__ void chain_start(int role)
+{
+    if (role != CHAIN_BESIDE) asm volatile("griddepcontrol.wait;" ::: "memory");
+    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+}
+// End of it.
+__device__ __forceinline__ void chain_finish(int role)
+{
+    if (role == CHAIN_BESIDE) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
 
 // Statistics partials left by the quantizers of a chain; the GEMM behind them reduces them in warps it has to spare (otherwise a
 // launch per quantizer, in the way of everything behind it).

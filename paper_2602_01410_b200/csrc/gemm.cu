@@ -208,6 +208,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // (tiles of up to 192 columns: at most 96 accumulators leave room for the whole chunk, so the buffer goes back before any multiplication)
 
     extern __shared__ uint8_t smem_raw[];
+    chain_acquire(g.chain);
     // operand tiles need 1024-byte alignment for the 128-byte swizzle
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
@@ -253,8 +254,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
     // everything up to here touches nothing that a kernel ahead on the stream writes
-    if (g.chain != CHAIN_BESIDE) pdl_wait();
-    pdl_launch_dependents();
+    chain_start(g.chain);
 
     if (KIND == MmaKind::MXF4) {
         // constant scale factors 2^0 (UE8M0 byte 127) for every row of A and B
@@ -763,7 +763,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
 
     // ---- teardown: every role ends here, tensor memory is always released ------------------
     __syncwarp();
-    if (g.chain == CHAIN_BESIDE) pdl_wait();
+    chain_finish(g.chain);
     tc_fence_before_sync();
     __syncthreads();
     if (PAIR) cluster_sync();   // no more arrivals from the other CTA, and the pair's MMAs read no more of this CTA's memory

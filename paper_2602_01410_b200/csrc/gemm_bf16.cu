@@ -71,6 +71,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     using C = Cfg<PAIR>;
     constexpr int S = C::kStages, kStageBytes = C::kStageBytes, kABytes = C::kABytes, BM = C::BM;
     extern __shared__ uint8_t smem_raw[];
+    chain_acquire(g.chain);
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     auto a_tile = [&](int s) { return smem_base + s * kStageBytes; };
@@ -110,8 +111,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
     // everything up to here touches nothing that a kernel ahead on the stream writes
-    if (g.chain != CHAIN_BESIDE) pdl_wait();
-    pdl_launch_dependents();
+    chain_start(g.chain);
     status_begin(g.status, g.status_mark);
 
     // a whole converged warp waits, with one answer for all its lanes; a failed wait raises the abort flag of both CTAs
@@ -304,7 +304,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
 
     // ---- teardown: every role ends here, tensor memory is always released ----
     __syncwarp();
-    if (g.chain == CHAIN_BESIDE) pdl_wait();
+    chain_finish(g.chain);
     tc_fence_before_sync();
     __syncthreads();
     if (PAIR) cluster_sync();   // no more arrivals from the other CTA, and the pair's MMAs read no more of this CTA's memory

@@ -94,6 +94,7 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     constexpr int HALF = BN / 2;
 
     extern __shared__ uint8_t smem_raw[];
+    chain_acquire(g.chain);
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     auto a_tile = [&](int s) { return smem_base + s * C::kStageBytes; };
@@ -138,8 +139,7 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
     tc_fence_after_sync();
     const uint32_t tmem_base = *tmem_slot;
     // everything up to here touches nothing that a kernel ahead on the stream writes
-    if (g.chain != CHAIN_BESIDE) pdl_wait();
-    pdl_launch_dependents();
+    chain_start(g.chain);
     status_begin(g.status, g.status_mark);
 
     // a whole converged warp waits, with one answer for all its lanes; a failed wait raises the abort flag of both CTAs
@@ -317,7 +317,7 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
 
     // ---- teardown ----
     __syncwarp();
-    if (g.chain == CHAIN_BESIDE) pdl_wait();
+    chain_finish(g.chain);
     tc_fence_before_sync();
     __syncthreads();
     if (PAIR) cluster_sync();   // no more arrivals from the other CTA, and the pair's MMAs read no more of this CTA's memory

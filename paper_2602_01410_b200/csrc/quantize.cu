@@ -58,17 +58,11 @@ struct ChainArgs {
     int32_t zero_words;
 };
 
-// Start of every quantizer: wait for the kernel ahead on the stream (unless independent of it), let the one behind be scheduled
-// (it waits for this grid where it has to), clear what the chain asks for.
+// Start of every quantizer: its place in the chain, then clear what the chain asks for.
 __device__ __forceinline__ void chain_begin(const ChainArgs &a)
 {
-    if (a.chain != CHAIN_BESIDE) asm volatile("griddepcontrol.wait;" ::: "memory");
-    asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+    chain_start(a.chain);
     for (int i = blockIdx.x * blockDim.x + threadIdx.x; i < a.zero_words; i += gridDim.x * blockDim.x) a.zero[i] = 0u;
-}
-__device__ __forceinline__ void chain_end(const ChainArgs &a)
-{
-    if (a.chain == CHAIN_BESIDE) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
 // Scratch shared memory of one CTA (next to the tile slot).
@@ -859,7 +853,7 @@ __global__ void __launch_bounds__(kThreads, kCtasPerSm) quantize_kernel(const Qu
         __syncthreads();  // the scratch arrays are reused by the next tile
     }
     if (STATS) finish_stats<false>(ts, sh, (int)blockIdx.x, a.partials, nullptr);
-    chain_end(chain);
+    chain_finish(chain.chain);
 }
 
 // Two outputs from one read (the tile kinds a tensor is consumed with, paper Fig. 5): `a` as stored and `b` transposed, each with its
@@ -913,7 +907,7 @@ __device__ __forceinline__ void run_variant(const DualJob &d, int first, const D
     constexpr int SRA = (V >> 2) & 1, SRB = (V >> 3) & 3;   // SRB: 1 own generator, 2 the first output's uniforms
     TwoLevel tw;
     if (FAM == FAM_NV) {
-        const float bound = *d.a.tensor_amax;
+        const float bound = __ldcg(d.a.tensor_amax);   // past L1, see ChainRole
         tw.enc = bound == 0.0f ? 1.0f : fminf(__fdiv_rn(2688.0f, bound), FLT_MAX);
         tw.inv_enc = __fdiv_rn(1.0f, tw.enc);
     }
@@ -932,7 +926,7 @@ __global__ void __launch_bounds__(kThreads, (V & 28) ? kDualCtasPerSmSr : kDualC
     extern __shared__ __align__(128) uint8_t smem[];
     chain_begin(chain);
     run_variant<FAM, V, STATS>(d, (int)blockIdx.x, dual_scratch(smem));
-    chain_end(chain);
+    chain_finish(chain.chain);
 }
 
 // The combinations of formats and roundings that exist, as F(variant).
@@ -990,7 +984,7 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSmSr) quantize_small_ker
         }
         __syncthreads();   // the scratch is free for the next tensor
     }
-    chain_end(g.chain);
+    chain_finish(g.chain.chain);
 }
 
 // Fixed-order reduction of the per-CTA partials into one snip_stats_t (deterministic: every thread

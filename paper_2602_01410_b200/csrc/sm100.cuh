@@ -21,10 +21,6 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
     return t;
 }
 
-// Programmatic dependent launch: wait until the kernels ahead have completed and their writes are visible; let the kernel behind start.
-__device__ __forceinline__ void pdl_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void pdl_launch_dependents() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
 // Status word of a GEMM (word[0]) cleared by the launch itself, in place of a memset ahead of it (which cost the kernel a 4 us gap):
 // CTA 0 clears it and leaves the launch's mark in word[1]; a CTA that gives up later reports only once that mark is there, so that the
 // clearing cannot erase the report (bounded: a CTA 0 that never came to run would hold it up for `limit_ns` at most).
