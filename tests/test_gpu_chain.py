@@ -111,3 +111,34 @@ def test_graph_replays_follow_replaced_inputs(api, kind, shape):
     for i, o in enumerate(got):
         for j, (g, ref) in enumerate(zip(o, want[i % 2])):
             assert torch.equal(g.view(torch.uint8), ref.view(torch.uint8)), (i, j)
+
+
+@pytest.mark.parametrize("kind", ["fp8", "pow2", "nvfp4", "separate", "tagged"])
+def test_a_refused_call_enqueues_nothing(api, kind):
+    # a misaligned output: the call returns an error and leaves workspace and statistics as they were
+    M, K, N = 256, 384, 192
+    x, w, dy, bounds = inputs(M, K, N, 51, 1.0)
+    ws, _ = layer(api, kind, M, K, N)
+    ws.fill_(0xA5)
+    stats = torch.full((6 * 24 + 16,), 0x5A, dtype=torch.uint8, device="cuda")
+    before = ws.clone(), stats.clone()
+    off = torch.empty(M * K + M * N + 64, dtype=torch.bfloat16, device="cuda")[4:]   # 8 bytes off
+    y, dx, dw = (torch.empty(s, dtype=torch.bfloat16, device="cuda") for s in ((M, N), (M, K), (N, K)))
+    p = lambda t: t.data_ptr()
+    stream = torch.cuda.current_stream().cuda_stream
+    for bad in range(3):
+        o = [p(off) if i == bad else p(t) for i, t in enumerate((y, dx, dw))]
+        if kind == "nvfp4":
+            rc = api._lib.snip_linear_fwd_bwd_nvfp4(p(x), p(w), p(dy), *o, M, N, K, api.OUT_BF16, p(bounds), 0, 0, p(stats), p(ws), ws.numel(), stream)
+        elif kind in ("fp8", "pow2"):
+            f = (FP8, FP8, FP8) if kind == "fp8" else (FP8, FP4, FP4)
+            rc = api._lib.snip_linear_fwd_bwd(p(x), p(w), p(dy), *o, M, N, K, *f, api.OUT_BF16, int(kind == "pow2"), 0, 0, p(stats), p(ws), ws.numel(), stream)
+        else:
+            f = (FP8, FP4, FP8)[bad] if kind == "separate" else BF16
+            fn = (api._lib.snip_linear_fwd, api._lib.snip_linear_dgrad, api._lib.snip_linear_wgrad)[bad]
+            a, b = ((x, w), (dy, w), (dy, x))[bad]
+            acc = (0,) if bad == 2 else ()
+            rc = fn(p(a), p(b), o[bad], M, N, K, f, f, api.OUT_BF16, *acc, p(stats), p(stats) + 32, p(ws), ws.numel(), stream)
+        assert rc == api.ERR_ALIGN, bad
+    torch.cuda.synchronize()
+    assert torch.equal(ws, before[0]) and torch.equal(stats, before[1])
