@@ -148,3 +148,17 @@ def test_linear_calls_refuse_before_anything_is_enqueued(lib):
             assert call(**{name: P + 8}) == 3, name
         assert call(dtype=2) == 1
     assert wgrad(acc=1) == 4 and wgrad(fmt=0, acc=1) == 4
+
+
+@pytest.mark.parametrize("missing", ["_cuda_getCurrentRawStream", "_cuda_getDevice"])
+def test_binding_does_not_depend_on_names_private_to_torch(lib, monkeypatch, missing):
+    import importlib.util
+    import types
+
+    import torch
+    monkeypatch.delattr(torch._C, missing, raising=False)
+    monkeypatch.setattr(torch.cuda, "current_stream", lambda *a: types.SimpleNamespace(cuda_stream=0x1230))
+    spec = importlib.util.spec_from_file_location("api_without_shortcut", os.path.join(ROOT, "paper_2602_01410_b200", "api.py"))
+    mod = importlib.util.module_from_spec(spec)
+    spec.loader.exec_module(mod)
+    assert mod._stream() == 0x1230
