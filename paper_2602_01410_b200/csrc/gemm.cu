@@ -572,7 +572,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 auto load_group = [&](int gi, uint32_t (&dst)[GC]) {
                     // vector mode: rows 16 * (gi % 2) .., columns 32 * (gi / 2) ..
                     if constexpr (SCALE == SCALE_VEC_B) tmem_ld_frag(taddr + ((uint32_t)(16 * (gi & 1)) << 16) + 32 * (gi >> 1), dst);
-                    else tmem_ld_cols(taddr + GC * gi, dst);
+                    else tmem_ld32(taddr + GC * gi, dst);
                 };
 #pragma unroll
                 for (int gi = 0; gi < D; ++gi) load_group(gi, v[gi]);

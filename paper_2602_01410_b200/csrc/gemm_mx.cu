@@ -19,8 +19,6 @@
 #include <cuda.h>
 #include <cuda_bf16.h>
 #include <float.h>
-#include <stdlib.h>
-#include <string.h>
 
 #include "common.cuh"
 #include "quant_device.cuh"

@@ -175,7 +175,6 @@ __global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __gr
 {
     extern __shared__ __align__(128) uint8_t smem[];
     Shared &sh = *reinterpret_cast<Shared *>(smem);
-    const uint4 *slot = reinterpret_cast<const uint4 *>(sh.slot) + threadIdx.x;
     asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
     const int tid = threadIdx.x, lane = tid & 31, warp = tid >> 5;
     const int tx = tid & 15, ty = tid >> 4;

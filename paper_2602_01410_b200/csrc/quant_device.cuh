@@ -42,16 +42,6 @@ __device__ __forceinline__ void reduce_stats_warp(const StatJob &job, int lane)
 __device__ __forceinline__ float bf16lo(uint32_t u) { return __uint_as_float(u << 16); }
 __device__ __forceinline__ float bf16hi(uint32_t u) { return __uint_as_float(u & 0xFFFF0000u); }
 
-__device__ __forceinline__ uint32_t absmax2(uint32_t acc, uint32_t v)
-{
-    // packed bf16 max of |v| against a non-negative accumulator
-    __nv_bfloat162 a = *reinterpret_cast<__nv_bfloat162 *>(&acc);
-    uint32_t av = v & 0x7FFF7FFFu;
-    __nv_bfloat162 b = *reinterpret_cast<__nv_bfloat162 *>(&av);
-    __nv_bfloat162 m = __hmax2(a, b);
-    return *reinterpret_cast<uint32_t *>(&m);
-}
-
 // packed bf16: magnitude of each half = max(|a|, |b|); the sign bits are meaningless (mask them at the end)
 __device__ __forceinline__ uint32_t absmax2x(uint32_t a, uint32_t b)
 {

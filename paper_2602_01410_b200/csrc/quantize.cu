@@ -931,17 +931,20 @@ __global__ void __launch_bounds__(kThreads, (V & 28) ? kDualCtasPerSmSr : kDualC
 
 // The combinations of formats and roundings that exist, as F(variant).
 #define SNIP_NV_VARIANTS(F) F(dual_variant(true, true, 0, 0)) F(dual_variant(true, true, 1, 2))
-#define SNIP_ROWCOL_VARIANTS(F)                                                                                                    \
+// Of row / column tiles: those of a linear layer (its stochastic copies share their seed), and the others of snip_quantize_dual.
+#define SNIP_LAYER_VARIANTS(F)                                                                                                     \
     SNIP_NV_VARIANTS(F)                                                                                                            \
     F(dual_variant(false, false, 0, 0)) F(dual_variant(false, true, 0, 0)) F(dual_variant(true, false, 0, 0))                      \
-    F(dual_variant(true, true, 1, 1)) F(dual_variant(true, true, 1, 0)) F(dual_variant(true, true, 0, 1))                          \
     F(dual_variant(true, false, 1, 0)) F(dual_variant(false, true, 0, 1))
+#define SNIP_ROWCOL_VARIANTS(F)                                                                                                    \
+    SNIP_LAYER_VARIANTS(F)                                                                                                         \
+    F(dual_variant(true, true, 1, 1)) F(dual_variant(true, true, 1, 0)) F(dual_variant(true, true, 0, 1))
 #define SNIP_BLK_VARIANTS(F)                                                                                                       \
     F(kBlkVariant + dual_variant(false, false, 0, 0)) F(kBlkVariant + dual_variant(false, true, 0, 0))                             \
     F(kBlkVariant + dual_variant(true, false, 0, 0)) F(kBlkVariant + dual_variant(true, true, 0, 0))
 
 // Small tensors: X, W and dY of a linear layer in one launch (2.8 us of the host and a place in the chain each), their tiles one
-// sequence dealt to the CTAs, a tile or two each.  The variant is chosen at run time; that keeps the arguments out of the
+// sequence dealt to the CTAs, a tile each.  The variant is chosen at run time; that keeps the arguments out of the
 // instructions and costs 10 % on large tensors, which therefore have launches of their own (see quantize_xwd_impl).
 constexpr int kMaxJobs = 3;
 struct DualGroup {
@@ -969,7 +972,7 @@ __global__ void __launch_bounds__(kThreads, kDualCtasPerSmSr) quantize_small_ker
         if constexpr (FAM != FAM_NV) {
 #define SNIP_RUN(V) case V: if constexpr (V != dual_variant(true, true, 0, 0) && V != dual_variant(true, true, 1, 2)) run_variant<FAM, V, STATS>(d, first, m); break;
             switch (d.variant) {
-                SNIP_ROWCOL_VARIANTS(SNIP_RUN)
+                SNIP_LAYER_VARIANTS(SNIP_RUN)
                 default: break;
             }
 #undef SNIP_RUN
@@ -1303,6 +1306,15 @@ int fill_job(const DualTask &t, DualJob &d, int &family)
     return SNIP_OK;
 }
 
+// Whether quantize_small_kernel has the variant of this job.
+bool in_small_kernel(const DualJob &d, int family)
+{
+#define SNIP_HAS(V) || d.variant == (V)
+    return (false SNIP_NV_VARIANTS(SNIP_HAS)) || (family != FAM_NV && (false SNIP_LAYER_VARIANTS(SNIP_HAS))) ||
+           (family == FAM_128 && (false SNIP_BLK_VARIANTS(SNIP_HAS)));
+#undef SNIP_HAS
+}
+
 int64_t dual_ctas(const DualJob &d) { return persistent_ctas(d.a.ntiles, (d.variant & 28) ? kDualCtasPerSmSr : kDualCtasPerSm); }
 
 template <int FAM, int V>
@@ -1376,7 +1388,9 @@ int quantize_xwd_impl(const DualTask (&t)[3], cudaStream_t st, const ChainLink &
     if (rc != SNIP_OK) return rc;
     const bool stats = t[0].a.stats != nullptr;
     const bool alike = family[0] == family[1] && family[0] == family[2] && (t[1].a.stats != nullptr) == stats && (t[2].a.stats != nullptr) == stats;
-    if (!alike || total > kDualCtasPerSmSr * (int64_t)gemm_sm_count()) {
+    bool small = alike && total <= kDualCtasPerSmSr * (int64_t)gemm_sm_count();
+    for (int i = 0; i < 3 && small; ++i) small = in_small_kernel(g.job[i], family[i]);
+    if (!small) {
         ChainLink beside;
         beside.role = CHAIN_BESIDE;
         beside.jobs = link.jobs;
