@@ -56,7 +56,8 @@ enum ChainRole { CHAIN_NONE = 0, CHAIN_FIRST = 1, CHAIN_BESIDE = 2, CHAIN_AFTER 
 
 // First thing in a GEMM, ahead of the CTA's first barrier, which passes it on to all threads: nothing stale is read from L1, and the TMA
 // unit's reads of the operands are ordered behind the acquire too.  By a thread of a warp that has nothing to set up: the fence takes
-// about as long as tensor memory's allocation beside it (by every thread behind that, it was 0.3 us of each such GEMM).
+// about as long as tensor memory's allocation beside it (a 512 x 512 x 512 layer 17.26 -> 17.38 us; by every thread behind the allocation
+// 17.54 us).
 __device__ __forceinline__ void chain_acquire(int role)
 {
     if (role == CHAIN_BESIDE && threadIdx.x == 96) asm volatile("fence.acq_rel.gpu;\n\tfence.proxy.async.global;" ::: "memory");

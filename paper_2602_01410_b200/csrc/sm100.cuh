@@ -24,6 +24,7 @@ __device__ __forceinline__ uint64_t globaltimer_ns()
 // Status word of a GEMM (word[0]) cleared by the launch itself, in place of a memset ahead of it (which cost the kernel a 4 us gap):
 // CTA 0 clears it and leaves the launch's mark in word[1]; a CTA that gives up later reports only once that mark is there, so that the
 // clearing cannot erase the report (bounded: a CTA 0 that never came to run would hold it up for `limit_ns` at most).
+// A replayed graph repeats the mark: there CTA 0, scheduled first, has the whole limit of the wait that ran out to clear the word in.
 __device__ __forceinline__ void status_begin(uint32_t *word, uint32_t mark)
 {
     if (mark != 0 && blockIdx.x == 0 && threadIdx.x == 0) {
