@@ -54,13 +54,16 @@ struct DualOut {
 // read past L1 (cp.async.cg, __ldcg); the GEMMs, which read scale factors and bounds through it, begin with an acquire (chain_acquire).
 enum ChainRole { CHAIN_NONE = 0, CHAIN_FIRST = 1, CHAIN_BESIDE = 2, CHAIN_AFTER = 3 };
 
-// First thing in a GEMM, ahead of the CTA's first barrier, which passes it on to all threads: nothing stale is read from L1, and the TMA
-// unit's reads of the operands are ordered behind the acquire too.  By a thread of a warp that has nothing to set up: the fence takes
-// about as long as tensor memory's allocation beside it (a 512 x 512 x 512 layer 17.26 -> 17.38 us; by every thread behind the allocation
-// 17.54 us).
-__device__ __forceinline__ void chain_acquire(int role)
+// First thing in a GEMM, ahead of the CTA's first barrier, which passes it on to all threads: an acquiring load of the status word (the
+// chain's first quantizer has cleared it), behind which nothing stale is read from L1, and a proxy fence that orders the TMA unit's reads of
+// the operands behind it too.  By a thread of a warp that has nothing to set up, beside the allocation of tensor memory.  A layer of 1152
+// tokens, 1216 -> 576: 26.43 us without it, 26.60 so, 26.96 with fence.acq_rel.gpu in its place (which waits for a full round of its own).
+__device__ __forceinline__ void chain_acquire(int role, const uint32_t *status)
 {
-    if (role == CHAIN_BESIDE && threadIdx.x == 96) asm volatile("fence.acq_rel.gpu;\n\tfence.proxy.async.global;" ::: "memory");
+    if (role == CHAIN_BESIDE && threadIdx.x == 96) {
+        uint32_t v;
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];\n\tfence.proxy.async.global;" : "=r"(v) : "l"(status) : "memory");
+    }
 }
 // Start of every kernel that may be a member of a chain, by all threads, before they touch memory that a kernel ahead writes.
 __device__ __forceinline__ void chain_start(int role)

@@ -208,7 +208,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     // (tiles of up to 192 columns: at most 96 accumulators leave room for the whole chunk, so the buffer goes back before any multiplication)
 
     extern __shared__ uint8_t smem_raw[];
-    chain_acquire(g.chain);
+    chain_acquire(g.chain, g.status);
     // operand tiles need 1024-byte alignment for the 128-byte swizzle
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));

@@ -71,7 +71,7 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     using C = Cfg<PAIR>;
     constexpr int S = C::kStages, kStageBytes = C::kStageBytes, kABytes = C::kABytes, BM = C::BM;
     extern __shared__ uint8_t smem_raw[];
-    chain_acquire(g.chain);
+    chain_acquire(g.chain, g.status);
     const uint32_t smem_base = (smem_u32(smem_raw) + 1023u) & ~1023u;
     uint8_t *smem_gen = smem_raw + (smem_base - smem_u32(smem_raw));
     auto a_tile = [&](int s) { return smem_base + s * kStageBytes; };
