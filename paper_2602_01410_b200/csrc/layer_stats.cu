@@ -64,30 +64,32 @@ struct Shared {
     __align__(16) uint8_t slot[2][kSlotBytes];   // the tile at hand and the next one; not there in a launch without heavy tensors
 };
 
-template <int FMT>
-__device__ __forceinline__ float ninv_of(float amax)
-{
-    constexpr float kMax = (FMT == SNIP_FMT_FP8_E4M3) ? 448.0f : 6.0f;
-    return -amax * (1.0f / kMax);
-}
+// (The reciprocal is the correctly rounded one of S itself: FP4's weighs whole sums, in which a bias like that of amax * fl(1/FPX_MAX)
+// would stay.)
 template <bool F8, bool F4>
 __device__ __forceinline__ Scales scales_of(float am)
 {
     Scales s = {0.0f, 0.0f, 0.0f, 0.0f};
-    if (F8) { s.s8 = tile_scale<SNIP_FMT_FP8_E4M3>(am, 0); s.n8 = ninv_of<SNIP_FMT_FP8_E4M3>(am); }
-    if (F4) { s.s4 = tile_scale<SNIP_FMT_FP4_E2M1>(am, 0); s.n4 = ninv_of<SNIP_FMT_FP4_E2M1>(am); }
+    if (F8) { s.s8 = tile_scale<SNIP_FMT_FP8_E4M3>(am, 0); s.n8 = -__frcp_rn(s.s8); }
+    if (F4) { s.s4 = tile_scale<SNIP_FMT_FP4_E2M1>(am, 0); s.n4 = -__frcp_rn(s.s4); }
     return s;
 }
 
-// Adds the squared error of an element pair under format FMT.
-template <int FMT>
-__device__ __forceinline__ void err_pair(const float2 x, const float2 s, const float2 n, float2 &se2)
+// Adds the squared error of an element pair under FP8; n = -1/S.
+__device__ __forceinline__ void err_pair_f8(const float2 x, const float2 s, const float2 n, float2 &se2)
 {
     const float2 t = __fmul2_rn(x, s);
-    const float2 d = (FMT == SNIP_FMT_FP8_E4M3) ? dec_e4m3x2(cvt_e4m3x2(t.x, t.y)) : dec_e2m1x2(cvt_e2m1x2(t.x, t.y));
-    const float2 e = __ffma2_rn(d, n, x);
+    const float2 e = __ffma2_rn(dec_e4m3x2(cvt_e4m3x2(t.x, t.y)), n, x);
     se2 = __ffma2_rn(e, e, se2);
 }
+// Under FP4, in units of 1/S^2 ...
+__device__ __forceinline__ void err_pair_f4(const float2 x, const float2 s, float2 &se2)
+{
+    const float2 e = fp4_scaled_rounding_err(__fmul2_rn(x, s));
+    se2 = __ffma2_rn(e, e, se2);
+}
+// ... and back to the units of x (two multiplications: 1/S^2 alone may leave binary32 where the product does not).
+__device__ __forceinline__ float unscale(const float2 se2, float n, float sum) { return fmaf((se2.x + se2.y) * n, n, sum); }
 
 __device__ __forceinline__ void fetch(const StatsTensor &t, int tile, uint8_t *slot)
 {
@@ -196,7 +198,8 @@ __global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __gr
             const uint4 *slot = reinterpret_cast<const uint4 *>(sh.slot[buf]) + threadIdx.x;
             buf ^= 1;
             float2 sx2 = make_float2(0.0f, 0.0f);
-            float2 e8a = make_float2(0.0f, 0.0f), e8b = e8a, e4a = e8a, e4b = e8a;
+            float2 e8a = make_float2(0.0f, 0.0f), e8b = e8a;
+            float e4a = 0.0f, e4b = 0.0f;
             // maxima (signs are garbage until masked: max.xorsign.abs keeps magnitudes only)
             uint32_t rmax[8], cm[4] = {0, 0, 0, 0};
 #pragma unroll
@@ -242,34 +245,48 @@ __global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __gr
                     sh.col[0][tid] = cs.s8; sh.col[1][tid] = cs.n8; sh.col[2][tid] = cs.s4; sh.col[3][tid] = cs.n4;
                 }
                 __syncthreads();
-                float2 cs8[4], cn8[4], cs4[4], cn4[4];
+                float2 cs8[4], cn8[4], cs4[4], c4[4];   // c4: FP4 errors squared of the column pairs, in units of their scales
+                auto get = [&](int k, float2 (&d)[4]) {
 #pragma unroll
-                for (int i = 0; i < 2; ++i) {
-                    auto get = [&](int k, float2 (&d)[4]) {
+                    for (int i = 0; i < 2; ++i) {
                         const float4 c = *reinterpret_cast<const float4 *>(&sh.col[k][8 * tx + 4 * i]);
                         d[2 * i] = make_float2(c.x, c.y);
                         d[2 * i + 1] = make_float2(c.z, c.w);
-                    };
-                    if (F8) { get(0, cs8); get(1, cn8); }
-                    if (F4) { get(2, cs4); get(3, cn4); }
-                }
+                    }
+                };
+                if (F8) { get(0, cs8); get(1, cn8); }
+                if (F4) get(2, cs4);
+#pragma unroll
+                for (int i = 0; i < 4; ++i) c4[i] = make_float2(0.0f, 0.0f);
 #pragma unroll
                 for (int p = 0; p < 8; ++p) {
                     const uint4 v = slot[p * kThreads];
                     const float4 r = *reinterpret_cast<const float4 *>(&sh.row[8 * ty + p]);
                     const uint32_t w[4] = {v.x, v.y, v.z, v.w};
+                    float2 r4 = make_float2(0.0f, 0.0f);   // of this row
 #pragma unroll
                     for (int i = 0; i < 4; ++i) {
                         const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
                         sx2 = __ffma2_rn(x, x, sx2);
                         if (F8) {
-                            err_pair<SNIP_FMT_FP8_E4M3>(x, make_float2(r.x, r.x), make_float2(r.y, r.y), e8a);
-                            err_pair<SNIP_FMT_FP8_E4M3>(x, cs8[i], cn8[i], e8b);
+                            err_pair_f8(x, make_float2(r.x, r.x), make_float2(r.y, r.y), e8a);
+                            err_pair_f8(x, cs8[i], cn8[i], e8b);
                         }
                         if (F4) {
-                            err_pair<SNIP_FMT_FP4_E2M1>(x, make_float2(r.z, r.z), make_float2(r.w, r.w), e4a);
-                            err_pair<SNIP_FMT_FP4_E2M1>(x, cs4[i], cn4[i], e4b);
+                            err_pair_f4(x, make_float2(r.z, r.z), r4);
+                            err_pair_f4(x, cs4[i], c4[i]);
                         }
+                    }
+                    if (F4) e4a = unscale(r4, r.w, e4a);
+                }
+                if (F4) {
+                    // (the column scales of this tile stay in place until every warp has passed the next tile's first barrier)
+                    float2 n[4];
+                    get(3, n);
+#pragma unroll
+                    for (int i = 0; i < 4; ++i) {
+                        e4b = fmaf(c4[i].x * n[i].x, n[i].x, e4b);
+                        e4b = fmaf(c4[i].y * n[i].y, n[i].y, e4b);
                     }
                 }
             } else {
@@ -282,7 +299,8 @@ __global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __gr
 #pragma unroll
                 for (int w = 1; w < 8; ++w) bm = max(bm, sh.blk_amax[parity][w]);
                 const Scales s = scales_of<F8, F4>(__uint_as_float(bm << 16));
-                const float2 s8 = make_float2(s.s8, s.s8), n8 = make_float2(s.n8, s.n8), s4 = make_float2(s.s4, s.s4), n4 = make_float2(s.n4, s.n4);
+                const float2 s8 = make_float2(s.s8, s.s8), n8 = make_float2(s.n8, s.n8), s4 = make_float2(s.s4, s.s4);
+                float2 b4 = make_float2(0.0f, 0.0f);
 #pragma unroll
                 for (int p = 0; p < 8; ++p) {
                     const uint4 v = slot[p * kThreads];
@@ -291,14 +309,15 @@ __global__ void __launch_bounds__(kThreads, kCtas) layer_stats_kernel(const __gr
                     for (int i = 0; i < 4; ++i) {
                         const float2 x = make_float2(bf16lo(w[i]), bf16hi(w[i]));
                         sx2 = __ffma2_rn(x, x, sx2);
-                        if (F8) err_pair<SNIP_FMT_FP8_E4M3>(x, s8, n8, e8a);
-                        if (F4) err_pair<SNIP_FMT_FP4_E2M1>(x, s4, n4, e4a);
+                        if (F8) err_pair_f8(x, s8, n8, e8a);
+                        if (F4) err_pair_f4(x, s4, b4);
                     }
                 }
+                e4a = unscale(b4, s.n4, e4a);
             }
             hacc[0] += (double)(sx2.x + sx2.y);
             if (F8) { hacc[1] += (double)(e8a.x + e8a.y); hacc[2] += (double)(e8b.x + e8b.y); }
-            if (F4) { hacc[3] += (double)(e4a.x + e4a.y); hacc[4] += (double)(e4b.x + e4b.y); }
+            if (F4) { hacc[3] += (double)e4a; hacc[4] += (double)e4b; }
         }
         flush(t, first, sh, hacc);
         first = tile - t.nitems;

@@ -111,6 +111,35 @@ __device__ __forceinline__ float2 dec_e2m1x2(uint32_t c)
     return __half22float2(*reinterpret_cast<__half2 *>(&h2));
 }
 
+// FP4 error term of an element pair in units of 1/S: value(code) - t, t the binary32 products that the codes were rounded from.  The f16
+// values of the codes (exact) enter the subtraction as they are; against decoding to binary32 and an FMA with -1/S it is a packed FMA and
+// two conversions less (12.4 -> 9.7 clocks per pair and scheduler, the whole term alone), at a factor S^-2 per tile line.  The
+// rounding of t stays in the term; next to FP4's coarse grid that is less than what a rounded 1/S left in it (the sums against 64 bits:
+// 5e-8 -> 1e-8 of the result).  FP8's grid is sixteen times finer, and there it is more (up to 1.4e-7), so FP8 keeps the exact product.
+__device__ __forceinline__ float2 fp4_scaled_err(uint32_t h2, const float2 t)
+{
+    float2 e;
+    asm("{\n\t.reg .f16 l, h;\n\tmov.b32 {l, h}, %2;\n\t"
+        "add.f32.f16 %0, l, %3;\n\t"
+        "add.f32.f16 %1, h, %4;\n\t}"
+        : "=f"(e.x), "=f"(e.y) : "r"(h2), "f"(-t.x), "f"(-t.y));
+    return e;
+}
+// ... of a code pair
+__device__ __forceinline__ float2 fp4_scaled_err_of_code(uint32_t c, const float2 t)
+{
+    uint32_t h2;
+    asm("{ .reg .b8 t, u; mov.b16 {t, u}, %1; cvt.rn.f16x2.e2m1x2 %0, t; }" : "=r"(h2) : "h"((uint16_t)c));
+    return fp4_scaled_err(h2, t);
+}
+// ... where the codes themselves are not wanted
+__device__ __forceinline__ float2 fp4_scaled_rounding_err(const float2 t)
+{
+    uint32_t h2;
+    asm("{ .reg .b8 c; cvt.rn.satfinite.e2m1x2.f32 c, %1, %2; cvt.rn.f16x2.e2m1x2 %0, c; }" : "=r"(h2) : "f"(t.y), "f"(t.x));
+    return fp4_scaled_err(h2, t);
+}
+
 // ---- stochastic rounding (paper Sec. 6.1: FP4 output gradients) ------------------------------------
 
 // Philox4x32 with 10 rounds (Salmon et al., SC'11): counter (c0, c1, 0, 0), key (k0, k1).
