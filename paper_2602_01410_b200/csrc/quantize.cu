@@ -142,12 +142,13 @@ struct ThreadStats {
     float amax = 0.0f;
 };
 
-// -1/S for the error term x - value(code)/S = x + value(code) * (-1/S).  Paper's rule: amax/FPX_MAX equals
-// 1/S to within one rounding, which the statistics (1e-4) do not see; power-of-two rule: exact, from the
-// exponent field.  For an empty tile the value is irrelevant (all codes are zero).
+// -1/S for the error term x - value(code)/S = x + value(code) * (-1/S).  Paper's rule: FP8: amax/FPX_MAX, which equals
+// 1/S to within one rounding; FP4, whose reciprocal weighs whole sums (kScaled below): the correctly rounded one of S.
+// Power-of-two rule: exact, from the exponent field.  For an empty tile the value is irrelevant (all codes are zero).
 template <int FMT>
 __device__ __forceinline__ float neg_inv(float amax, float s, int pow2)
 {
+    if (FMT == SNIP_FMT_FP4_E2M1 && !pow2) return -__frcp_rn(s);
     constexpr float kInvMax = (FMT == SNIP_FMT_FP8_E4M3) ? (1.0f / 448.0f) : (1.0f / 6.0f);
     return pow2 ? __uint_as_float(0x80000000u | ((254u << 23) - __float_as_uint(s))) : -amax * kInvMax;
 }
@@ -168,6 +169,18 @@ __device__ __forceinline__ uint32_t encode_pair(const float2 x, const float2 s, 
     }
     return c;
 }
+
+// FP4, nearest even, with the squared error in units of 1/S^2 (see fp4_scaled_err).
+__device__ __forceinline__ uint32_t encode_pair_fp4_scaled(const float2 x, const float2 s, float2 &se2)
+{
+    const float2 t = __fmul2_rn(x, s);
+    const uint32_t c = cvt_e2m1x2(t.x, t.y);
+    const float2 e = fp4_scaled_err_of_code(c, t);
+    se2 = __ffma2_rn(e, e, se2);
+    return c;
+}
+// Squared errors in units of 1/S^2 -> units of x^2 (two multiplications: 1/S^2 alone may leave binary32 where the product does not).
+__device__ __forceinline__ float unscale(float se, float n, float sum) { return fmaf(se * n, n, sum); }
 
 // Stochastic-rounding form for FP4: r0, r1 hold the pair's uniforms (sr_addends).
 // The rounded values are at hand in binary32, so the error term needs no decode.
@@ -308,6 +321,15 @@ __device__ __forceinline__ float2 scale_pair(const SubScales &sc, int p, int i)
     if (O::BLOCK == SNIP_BLOCK_COL_128x1 || O::BLOCK == SNIP_BLOCK_COL_32x1 || O::BLOCK == SNIP_BLOCK_COL_16x1) return make_float2(sc.s_col[2 * i], sc.s_col[2 * i + 1]);
     return make_float2(sc.s_blk, sc.s_blk);
 }
+// Outputs whose error terms are summed in units of 1/S^2 and weighed per tile line: FP4 rounded to nearest, except under the two-level rule
+// (there a tile's scale may be zero while its elements are not).
+template <class O>
+constexpr bool kScaledErr = O::kQuant && O::FMT == SNIP_FMT_FP4_E2M1 && !O::SR && !O::kSat;
+template <class O>
+constexpr bool kRowTiles = O::BLOCK == SNIP_BLOCK_ROW_1x128 || O::BLOCK == SNIP_BLOCK_ROW_1x32;
+template <class O>
+constexpr bool kColTiles = O::BLOCK == SNIP_BLOCK_COL_128x1 || O::BLOCK == SNIP_BLOCK_COL_32x1;
+
 template <class O>
 __device__ __forceinline__ float2 ninv_pair(const SubScales &sc, int p, int i)
 {
@@ -690,6 +712,10 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
     float2 sx2 = make_float2(0.0f, 0.0f), sea2 = make_float2(0.0f, 0.0f), seb2 = make_float2(0.0f, 0.0f);
     float rsx[8], rse[8];
     (void)rsx; (void)rse;
+    constexpr bool kSclA = STATS && !ROWSTATS && kScaledErr<A>, kSclB = STATS && !kSame && kScaledErr<B>;
+    float2 ua2[4], ub2[4];   // such errors: of the row at hand ([0]), of the four column pairs, of the block ([0])
+#pragma unroll
+    for (int i = 0; i < 4; ++i) ua2[i] = ub2[i] = make_float2(0.0f, 0.0f);
 #pragma unroll
     for (int p = 0; p < 8; ++p) {
         const uint4 vp = slot[p * kThreads];
@@ -714,15 +740,19 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
             if (B::SR == 2) { rb0 = ra0; rb1 = ra1; }
             if (A::kQuant) {
                 if (A::SR) ca[i] = encode_pair_sr_fp4<STATS, A::kSat>(x, scale_pair<A>(sa, p, i), ninv_pair<A>(sa, p, i), ra0, ra1, ROWSTATS ? pe : sea2);
+                else if (kSclA) ca[i] = encode_pair_fp4_scaled(x, scale_pair<A>(sa, p, i), ua2[kColTiles<A> ? i : 0]);
                 else ca[i] = encode_pair<A::FMT, STATS>(x, scale_pair<A>(sa, p, i), ninv_pair<A>(sa, p, i), ROWSTATS ? pe : sea2);
             }
             if (kSame) {
                 cb[i] = ca[i];
             } else if (B::kQuant) {
                 if (B::SR) cb[i] = encode_pair_sr_fp4<STATS, B::kSat>(x, scale_pair<B>(sb, p, i), ninv_pair<B>(sb, p, i), rb0, rb1, seb2);
+                else if (kSclB) cb[i] = encode_pair_fp4_scaled(x, scale_pair<B>(sb, p, i), ub2[kColTiles<B> ? i : 0]);
                 else cb[i] = encode_pair<B::FMT, STATS>(x, scale_pair<B>(sb, p, i), ninv_pair<B>(sb, p, i), seb2);
             }
         }
+        if (kSclA && kRowTiles<A>) { sea2.x = unscale(ua2[0].x + ua2[0].y, sa.n_row[p], sea2.x); ua2[0] = make_float2(0.0f, 0.0f); }
+        if (kSclB && kRowTiles<B>) { seb2.x = unscale(ub2[0].x + ub2[0].y, sb.n_row[p], seb2.x); ub2[0] = make_float2(0.0f, 0.0f); }
         if (ROWSTATS) {
             rsx[p] = px.x + px.y; rse[p] = pe.x + pe.y;
             sx2.x += rsx[p]; sea2.x += rse[p];
@@ -741,6 +771,21 @@ __device__ __forceinline__ void process_tile(const QuantArgs &qa, const QuantArg
         }
     }
     after_reads();
+
+    // column tiles: the reciprocals are read again here (128x1: they stay in place until every warp has passed the next tile's first barrier)
+    auto add_columns = [&](const float2 (&u)[4], const SubScales &sc, bool tiles32, float2 &se2) {
+#pragma unroll
+        for (int i = 0; i < 4; ++i) {
+            const float2 n = tiles32 ? make_float2(neg_inv_pow2(sc.s_col[2 * i]), neg_inv_pow2(sc.s_col[2 * i + 1]))
+                                     : *reinterpret_cast<const float2 *>(&sh.col_ninv[8 * tx + 2 * i]);
+            se2.x = unscale(u[i].x, n.x, se2.x);
+            se2.y = unscale(u[i].y, n.y, se2.y);
+        }
+    };
+    if (kSclA && kColTiles<A>) add_columns(ua2, sa, A::BLOCK == SNIP_BLOCK_COL_32x1, sea2);
+    if (kSclB && kColTiles<B>) add_columns(ub2, sb, B::BLOCK == SNIP_BLOCK_COL_32x1, seb2);
+    if (kSclA && A::BLOCK == SNIP_BLOCK_BLK_128x128) sea2.x = unscale(ua2[0].x + ua2[0].y, sa.n_blk, 0.0f);
+    if (kSclB && B::BLOCK == SNIP_BLOCK_BLK_128x128) seb2.x = unscale(ub2[0].x + ub2[0].y, sb.n_blk, 0.0f);
 
     if (STATS) {
         ts.x += (double)(sx2.x + sx2.y);
