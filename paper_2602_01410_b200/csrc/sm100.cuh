@@ -84,6 +84,16 @@ __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_add
 {
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
+// Arrivals by one lane of a converged warp, predicated by elect.sync: a `lane == 0` branch around the instruction, at the end of every
+// chunk of a GEMM, costs 2-6 % of its cycles.
+__device__ __forceinline__ void mbar_arrive_cluster_relaxed_elected(uint32_t cluster_addr)
+{
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\t@p mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];\n\t}" ::"r"(cluster_addr) : "memory");
+}
+__device__ __forceinline__ void mbar_arrive_elected(uint32_t bar)
+{
+    asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\t@p mbarrier.arrive.shared::cta.b64 _, [%0];\n\t}" ::"r"(bar) : "memory");
+}
 // Plain 32-bit store into the shared memory of a CTA of the cluster.
 __device__ __forceinline__ void st_cluster_u32(uint32_t cluster_addr, uint32_t v)
 {
