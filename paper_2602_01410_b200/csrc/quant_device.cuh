@@ -178,7 +178,10 @@ __device__ __forceinline__ float sr_e2m1_value(float t, uint32_t r)
 {
     const float a = SAT ? fminf(fabsf(t), 6.0f) : fabsf(t);
     float off;
-    asm("set.lt.f32.f32 %0, %1, 0f3F800000;" : "=f"(off) : "f"(a));   // 1 below 1, else 0
+    // 1 below 1, else 0: 2^120 - 2^120 a, which is 2^96 or more from the number next below 1 down (a set instruction would go to the
+    // integer pipe, the one this function is bound by: two-output quantizers of an 8192 x 8640 gradient 116.0 -> 114.3 us, two-level 135.8 ->
+    // 133.3 us)
+    asm("fma.rn.sat.f32 %0, %1, 0fFB800000, 0f7B800000;" : "=f"(off) : "f"(a));
     const uint32_t q = (__float_as_uint(__fadd_ru(a, off)) + r) & 0xFFC00000u;
     return copysignf(__uint_as_float(q) - off, t);
 }
