@@ -40,6 +40,10 @@ static_assert(kNumEpiWarps == kSliceWarps, "slice counters");
 // Contraction slices of the weight-gradient product's last wave: no shorter than kMinSliceStages, and only where they shorten the CTAs' sequence
 // of stages by what the exchange of the partial sums takes (8-13 us; 2048 tokens x 256 x 2048: 15.6 us whole, 20.6 us in two slices).
 constexpr int kMinSliceStages = 8, kMinSavedStages = 20;
+// Slices in a cluster exchange their sums through shared memory: about 3 us, ten stages of a 128-wide tile (2048 tokens x 256 x 2048, where
+// two slices save eight: 12.0 us whole, 12.6 us sliced).  256-wide tiles keep the exchange through L2: there are half as many of them as
+// narrow ones, and two slices of 64 such tiles come out level with 128 whole narrow ones (8192 x 1024 x 2048: 32.9 / 32.5 us).
+constexpr int kMinSavedStagesCluster = 12;
 constexpr int kSfCols = 32;  // tensor-memory columns holding constant scale factors (kind::mxf4)
 
 enum ScaleMode { SCALE_BLOCK_B = 1, SCALE_VEC_B = 2 };
@@ -97,6 +101,7 @@ struct Cfg {
     static constexpr int kSmemBytes = kStages * kStageBytes + kSbInvBytes + kOutStageBytes + 256 + 1024;  // + barriers + alignment slack
     static_assert(kSmemBytes <= 232448, "shared memory budget");
     static_assert(kStageBytes % 1024 == 0 && kSbInvBytes % 1024 == 0, "staging tiles must stay 1024-byte aligned");
+    static constexpr bool kClusterSlices = SCALE == 2 && BN == 128 && !PAIR;   // see plan_clusters
     static constexpr int kAccCols = 2 * BN;
     static constexpr int kSfCol0 = kAccCols;
     static constexpr int kTmemCols = 512;
@@ -192,7 +197,9 @@ __device__ __forceinline__ void store_frag(const GemmArgs &g, int64_t row, int c
     }
 }
 
-template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32>
+// CLUSTER: the CTAs of a cluster hold the slices of one tile, an item each (plan_clusters).  An instantiation of its own: with the cluster
+// barriers in the code of the others, unused, a 512 x 512 x 512 layer takes 17.0 instead of 16.0 us.
+template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32, bool CLUSTER>
 __global__ void __launch_bounds__(kGemmThreads, 1)
 gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUtensorMap tmB, const __grid_constant__ CUtensorMap tmO,
             const GemmArgs g, const uint32_t idesc)
@@ -205,6 +212,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
     constexpr int GC = (SCALE == SCALE_VEC_B) ? 16 : 32;
     constexpr int G = HALF / GC;     // groups handled by one epilogue warp per chunk
     constexpr int D = (SCALE == SCALE_VEC_B) ? (G < 6 ? G : 4) : (BN <= 192) ? G : 2;   // groups of staging registers next to the accumulators
+    static_assert(!CLUSTER || C::kClusterSlices, "slices in clusters: 128-wide tiles of the weight gradient");
     // (tiles of up to 192 columns: at most 96 accumulators leave room for the whole chunk, so the buffer goes back before any multiplication)
 
     extern __shared__ uint8_t smem_raw[];
@@ -462,6 +470,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         if (warp == 2)
             for (int i = blockIdx.x; i < g.stats.count; i += gridDim.x) reduce_stats_warp(g.stats.job[i], lane);
       }
+      if (CLUSTER) {   // the two barriers of the slices' exchange (below)
+          __syncwarp();
+          cluster_sync();
+          cluster_sync();
+      }
     } else {
         reg_alloc<232>();    // needs (232-168)*256 = 16384 <= 16384 (an unsatisfiable request would block forever)
         // ================= promotion / epilogue warps =================
@@ -648,7 +661,53 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     if (lane == 0) mbar_arrive(vempty_bar(vd / C::kVecBlock));
                 }
             }
-            {
+            if constexpr (CLUSTER) {
+                // A slice of a tile whose other slices are in this cluster (the CTA's only item).  The sums of fragment group gi belong to
+                // slice gi * nsl / G: every CTA writes the groups of the others into their stage memory, which no copy or MMA uses any
+                // more once all CTAs are here, and then adds its own groups in slice order and stores them.  Nothing is sent through L2
+                // and no CTA adds the whole tile: 8192 tokens x 256 x 2048 21.8 -> 17.6 us, 16384 x 512 x 1024 28.9 -> 24.1 us.  A CTA that gave
+                // up a wait takes part in both barriers all the same.
+                const int me = wi.slice, nsl = wi.nsl, per = (G + nsl - 1) / nsl;
+                float *av = reinterpret_cast<float *>(acc);
+                auto owner = [&](int gi) { return gi * nsl / G; };
+                auto slot = [&](int from, int gi) {   // of group gi, sent by slice `from`, in its owner's stage memory: [sender][warp][group][quad][lane]
+                    const int k = gi - (owner(gi) * G + nsl - 1) / nsl;
+                    return (uint32_t)((((from * kNumEpiWarps + e) * per + k) * 4) * 512 + lane * 16);
+                };
+                cluster_sync();
+                if (ok) {
+#pragma unroll
+                    for (int gi = 0; gi < G; ++gi) {
+                        if (owner(gi) != me) {
+                            const uint32_t dst = mapa(smem_base + slot(me, gi), (uint32_t)owner(gi));
+#pragma unroll
+                            for (int j = 0; j < 4; ++j)
+                                st_cluster_v4(dst + 512u * j, make_float4(av[16 * gi + 4 * j], av[16 * gi + 4 * j + 1], av[16 * gi + 4 * j + 2], av[16 * gi + 4 * j + 3]));
+                        }
+                    }
+                }
+                cluster_sync();
+                if (ok) {
+#pragma unroll
+                    for (int gi = 0; gi < G; ++gi) {
+                        if (owner(gi) == me) {
+                            float t[16];
+                            for (int sl = 0; sl < nsl; ++sl) {
+                                float u[16];
+#pragma unroll
+                                for (int j = 0; j < 4; ++j) {
+                                    const float4 x = sl == me ? make_float4(av[16 * gi + 4 * j], av[16 * gi + 4 * j + 1], av[16 * gi + 4 * j + 2], av[16 * gi + 4 * j + 3])
+                                                              : *reinterpret_cast<const float4 *>(smem_gen + slot(sl, gi) + 512 * j);
+                                    u[4 * j] = x.x; u[4 * j + 1] = x.y; u[4 * j + 2] = x.z; u[4 * j + 3] = x.w;
+                                }
+#pragma unroll
+                                for (int j = 0; j < 16; ++j) t[j] = sl == 0 ? u[j] : t[j] + u[j];
+                            }
+                            store_frag<OUT_F32>(g, row0 + 16 * (gi & 1) + (lane >> 2), col0 + 32 * (gi >> 1), t, lane);
+                        }
+                    }
+                }
+            } else {
                 cp_async_wait<0>();
                 if (ok) {
                     if (C::kTmaOut && !g.accumulate) {
@@ -830,22 +889,70 @@ int sm_count()
     return n;
 }
 
+// Clusters of `size` CTAs of the 128-wide weight-gradient kernel that the current device holds at a time (a cluster's CTAs share a GPC, so
+// this is less than SMs / size); 0 if it cannot be told.
+int max_clusters(int size)
+{
+    static thread_local int dev_cached = -1, n[kMaxSlices + 1];
+    int dev = 0;
+    cudaGetDevice(&dev);
+    if (dev != dev_cached) {
+        for (int c = 2; c <= kMaxSlices; ++c) {
+            using C = Cfg<MmaKind::F8F6F4, 128, SCALE_VEC_B, false>;
+            auto kern = gemm_kernel<MmaKind::F8F6F4, 128, SCALE_VEC_B, false, false, true>;
+            cudaLaunchAttribute attr[1];
+            attr[0].id = cudaLaunchAttributeClusterDimension;
+            attr[0].val.clusterDim.x = (unsigned)c; attr[0].val.clusterDim.y = 1; attr[0].val.clusterDim.z = 1;
+            cudaLaunchConfig_t cfg = {};
+            cfg.gridDim = dim3((unsigned)(c * (sm_count() / c)));
+            cfg.blockDim = dim3(kGemmThreads);
+            cfg.dynamicSmemBytes = C::kSmemBytes;
+            cfg.attrs = attr;
+            cfg.numAttrs = 1;
+            n[c] = 0;
+            if (cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes) != cudaSuccess ||
+                cudaOccupancyMaxActiveClusters(&n[c], kern, &cfg) != cudaSuccess) {
+                n[c] = 0;
+                cudaGetLastError();
+            }
+        }
+        dev_cached = dev;
+    }
+    return size >= 2 && size <= kMaxSlices ? n[size] : 0;
+}
+
+// All tiles in slices, the slices of a tile in a cluster, where all clusters run at the same time and slicing saves what the exchange costs;
+// nsplit == 1: not so.  128-wide tiles on one CTA each.
+WorkSplit plan_clusters(int num_tiles, int num_stages, bool slice)
+{
+    for (int ns = kMaxSlices; slice && ns > 1; --ns)
+        if (num_stages / ns >= kMinSliceStages && num_stages - num_stages / ns >= kMinSavedStagesCluster && num_tiles <= max_clusters(ns))
+            return {0, ns, num_tiles * ns};
+    return {num_tiles, 1, num_tiles};
+}
+
 template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32>
 int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc, bool cleared, cudaStream_t st)
 {
     using C = Cfg<KIND, BN, SCALE, PAIR>;
-    auto kern = gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32>;
-    // a per-function, per-device attribute; setting it on every launch is cheap and correct on any device
-    SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
-    const int num_tiles = (int)(ceil_div(g.Mo, C::BM) * ceil_div(g.No, BN));
+    const int num_tiles = (int)(ceil_div(g.Mo, C::BM) * ceil_div(g.No, BN)), num_stages = (int)ceil_div(g.Kc, C::kStageK);
     const int units = sm_count() / C::kCtas;
+    const bool slice = SCALE == SCALE_VEC_B && g.partials;
     GemmArgs ga = g;
-    ga.work = plan_work(num_tiles, (int)ceil_div(g.Kc, C::kStageK), units, kMinSliceStages, kMinSavedStages, SCALE == SCALE_VEC_B && g.partials,
-                        kMaxSlicedItems / C::kCtas);
+    auto launch = [&](auto kern, int cluster) -> int {
+        // a per-function, per-device attribute; setting it on every launch is cheap and correct on any device
+        SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
+        const int grid = (ga.work.num_items < units ? ga.work.num_items : units) * C::kCtas;
+        return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, cluster, tmA, tmB, tmO, ga, idesc);
+    };
+    if constexpr (C::kClusterSlices) {
+        ga.work = plan_clusters(num_tiles, num_stages, slice);
+        if (ga.work.nsplit > 1) return launch(gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32, true>, ga.work.nsplit);
+    }
+    ga.work = plan_work(num_tiles, num_stages, units, kMinSliceStages, kMinSavedStages, slice, kMaxSlicedItems / C::kCtas);
     if (ga.work.nsplit > 1 && !cleared)
         SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * C::kCtas * sizeof(uint32_t), st));
-    const int grid = (ga.work.num_items < units ? ga.work.num_items : units) * C::kCtas;
-    return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, C::kCtas, tmA, tmB, tmO, ga, idesc);
+    return launch(gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32, false>, C::kCtas);
 }
 
 template <MmaKind KIND, int BN, int SCALE>
@@ -996,7 +1103,10 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         if (choice != 0) return choice == 3;
         auto stages = [&](int bn) {
             const int sms = sm_count(), tiles = (int)(ceil_div(Mo, CM) * ceil_div(No, bn)), per_tile = (int)ceil_div(Kc, stage_k);
-            const WorkSplit sp = plan_work(tiles, per_tile, sms, kMinSliceStages, kMinSavedStages, scale_mode == SCALE_VEC_B && g.partials);
+            const bool slice = scale_mode == SCALE_VEC_B && g.partials;
+            const WorkSplit cl = plan_clusters(tiles, per_tile, slice && bn == 128);
+            if (cl.nsplit > 1) return (float)per_tile / cl.nsplit + kMinSavedStagesCluster;
+            const WorkSplit sp = plan_work(tiles, per_tile, sms, kMinSliceStages, kMinSavedStages, slice);
             if (sp.nsplit > 1) return (float)(sp.split_first / sms) * per_tile + (float)per_tile / sp.nsplit + kMinSavedStages;
             return (float)ceil_div(tiles, sms) * per_tile;
         };

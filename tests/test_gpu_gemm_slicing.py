@@ -97,3 +97,32 @@ def test_sliced_accumulate_garbage_workspace_and_minimum_workspace(api, slicing)
     torch.cuda.synchronize()
     assert api.snip_poll_status(small) == api.OK
     assert rel_fro(out3.cpu().numpy(), ref) <= 1e-5
+
+
+# Both ways of adding the slices, forced: 128-wide tiles (kernel choice 3) whose slices are the CTAs of a cluster - two, three and four
+# of them, ragged tiles on both sides, contractions ending in a 64-wide tile, one group of a tile more for a CTA than for another - and
+# 256- / 192-wide tiles (choice 1), which exchange through the workspace.
+@pytest.mark.parametrize("fa,fb", [(FP8, FP8), (FP4, FP4)])
+@pytest.mark.parametrize("choice,shape", [(3, (3584, 1024, 1024)), (3, (6208, 704, 448)), (3, (8256, 192, 64)), (3, (8192, 1024, 512)), (1, (8192, 448, 320)), (1, (8256, 512, 256))])
+def test_cluster_and_workspace_exchange(api, slicing, fa, fb, choice, shape):
+    M, K, N = shape
+    x, dy, a, b, keep = operands(api, M, K, N, fa, fb, 90 + choice + M + K + N)
+    start = torch.randn(N, K, device="cuda")
+    api.snip_debug_set(api.DEBUG_GEMM_KERNEL, choice)
+    try:
+        outs = {}
+        for mode in (0, 1, 1):
+            slicing(mode)
+            f32 = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32)
+            acc = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32, accumulate=True, out=start.clone())
+            b16 = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_BF16)
+            torch.cuda.synchronize()
+            assert torch.equal(acc, start + f32) and torch.equal(b16, f32.bfloat16())
+            if mode and mode in outs:
+                assert torch.equal(f32, outs[1])     # whatever the order of arrival
+            outs[mode] = f32.clone()
+    finally:
+        api.snip_debug_set(api.DEBUG_GEMM_KERNEL, api.GEMM_KERNEL_AUTO)
+    # they differ in the order of FP32 additions only: a few units in the last place of sums over at most 65 chunks
+    assert not torch.equal(outs[1], outs[0])
+    assert rel_fro(outs[1].cpu().numpy(), outs[0].cpu().numpy().astype(np.float64)) <= 1e-6

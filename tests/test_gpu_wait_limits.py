@@ -45,7 +45,7 @@ def check(api, hooks, ws, call):  # noqa: F811
 # 256 x 256: pairs, in all three products)
 @pytest.mark.parametrize("kind,choice,shape", [(k, c, (512, 384, 256)) for k in ("fp8", "fp4", "mixed") for c in (1, 2, 3)] +
                          [(k, 0, s) for k in ("pow2", "pow2-32", "nvfp4") for s in ((512, 384, 256), (2304, 2304, 2304))] +
-                         [("fp8", 0, (8192, 256, 320)), ("fp4", 0, (8192, 256, 320))])   # the last wave of the weight gradient sliced
+                         [(k, c, (8192, 256, 320)) for k in ("fp8", "fp4") for c in (0, 1)])   # the weight gradient sliced: in clusters, through the workspace
 def test_chained_layer(api, hooks, kind, choice, shape):  # noqa: F811
     t = inputs(*shape, 61, 1.0)
     ws, step = layer(api, kind, *shape)
