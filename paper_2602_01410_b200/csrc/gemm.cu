@@ -330,7 +330,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
         // Block mode: an elected lane, under which the operands of the tcgen05 instructions stay in uniform registers (issue of a chunk
         // 204 -> 55 cycles, 2-4 % of the FP4 kernels); in vector mode it costs the promotion warps registers and gains nothing.
         if (rank == 0 && (SCALE == SCALE_BLOCK_B ? elect_one() : lane == 0)) {
-            const uint32_t peer0 = PAIR ? mapa(bar0, 1) : 0u;
             uint32_t it = 0, cc = 0;
             bool ok = true;
             const uint32_t sfa = tmem_base + C::kSfCol0, sfb = tmem_base + C::kSfCol0 + 16;
@@ -353,7 +352,6 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                         // one commit serves both hand-offs (a stage is one chunk here): the producer takes it as
                         // "stage s is free", the epilogue warps as "the chunk's partial sums are complete"
                         tc_commit<PAIR>(empty_bar(s));
-                        if (PAIR) tc_commit<PAIR>(peer0 + 8u * (S + s));
                         ++cc;
                     } else {
 #pragma unroll
@@ -367,12 +365,10 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                                     mma_ss<KIND, PAIR>(tmem_base + a * BN, adesc + 2 * (2 * h + k), bdesc + 2 * (2 * h + k), idesc,
                                                  k > 0 ? 1u : 0u, sfa, sfb);
                                 tc_commit<PAIR>(tfull_bar(a));
-                                if (PAIR) tc_commit<PAIR>(peer0 + 8u * (2 * S + a));
                                 ++cc;
                             }
                         }
                         tc_commit<PAIR>(empty_bar(s));
-                        if (PAIR) tc_commit<PAIR>(peer0 + 8u * (S + s));
                     }
                 }
             }

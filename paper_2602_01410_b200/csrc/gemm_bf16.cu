@@ -159,7 +159,6 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
     } else if (warp == 1) {
       // ================= MMA issuer (leader; whole warp in the loop, one elected lane issues) =================
       if (rank == 0) {
-        const uint32_t peer0 = PAIR ? mapa(bar0, 1) : 0u;
         uint32_t it = 0, done = 0;
         bool ok = true;
         for (int w = unit; w < g.work.num_items && ok; w += units, ++done) {
@@ -180,10 +179,8 @@ gemm_bf16_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant_
                     for (int k = 0; k < 4; ++k)
                         mma_ss<MmaKind::F16, PAIR>(tmem_base + a * BN, adesc + kAStep * k, bdesc + kBStep * k, idesc, (ks > wi.ks0 || k > 0) ? 1u : 0u, 0, 0);
                     tc_commit<PAIR>(empty_bar(s));
-                    if (PAIR) tc_commit<PAIR>(peer0 + 8u * (S + s));
                     if (ks == wi.ks1 - 1) {
                         tc_commit<PAIR>(tfull_bar(a));
-                        if (PAIR) tc_commit<PAIR>(peer0 + 8u * (2 * S + a));
                     }
                 }
                 __syncwarp();

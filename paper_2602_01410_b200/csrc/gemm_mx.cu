@@ -192,7 +192,6 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
         // instructions stay in uniform registers, which makes each of them several times cheaper for the issuing thread than
         // under a `lane == 0` branch; with up to seventeen of them per stage that thread is what the tensor core waits for.
         if (rank == 0) {
-            const uint32_t peer0 = PAIR ? mapa(bar0, 1) : 0u;
             uint32_t it = 0, tiles_done = 0;
             bool ok = true;
             const uint32_t sfa = tmem_base + kSfaCol, sfb = tmem_base + (C::kNv ? kNvSfbCol : kSfbCol);
@@ -235,10 +234,8 @@ gemm_mx_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ 
                             }
                         }
                         tc_commit<PAIR>(empty_bar(s));
-                        if (PAIR) tc_commit<PAIR>(peer0 + 8u * (S + s));
                         if (ks == num_kstages - 1) {
                             tc_commit<PAIR>(tfull_bar);
-                            if (PAIR) tc_commit<PAIR>(peer0 + 8u * (2 * S));
                         }
                     }
                     __syncwarp();

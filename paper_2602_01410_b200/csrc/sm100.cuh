@@ -237,13 +237,14 @@ __device__ __forceinline__ void tmem_dealloc(uint32_t taddr, uint32_t ncols)
 __device__ __forceinline__ void tc_fence_before_sync() { asm volatile("tcgen05.fence::before_thread_sync;" ::: "memory"); }
 __device__ __forceinline__ void tc_fence_after_sync() { asm volatile("tcgen05.fence::after_thread_sync;" ::: "memory"); }
 
-// Make `bar` receive one arrival when all MMAs issued so far by this thread have completed.
-// With PAIR the MMAs tracked are those of the CTA pair and `bar` may be a shared::cluster address
-// (own or peer barrier).
+// Make `bar` receive one arrival when all MMAs issued so far by this thread have completed.  With PAIR the MMAs tracked are those of the
+// CTA pair, and the barrier at the same offset in both CTAs of the cluster of two receives one: one instruction for both, because the
+// second of two separate commits waits in the issuing thread behind the first (16384x12288x4096 FP4 forward 625 -> 619 us, 11008 x 4096 FP4
+// input gradient 548 -> 538 us; FP8 8192x8192x4096 231 -> 226 us).
 template <bool PAIR>
 __device__ __forceinline__ void tc_commit(uint32_t bar)
 {
-    if constexpr (PAIR) asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
+    if constexpr (PAIR) asm volatile("tcgen05.commit.cta_group::2.mbarrier::arrive::one.shared::cluster.multicast::cluster.b64 [%0], %1;" ::"r"(bar), "h"((uint16_t)3) : "memory");
     else asm volatile("tcgen05.commit.cta_group::1.mbarrier::arrive::one.shared::cluster.b64 [%0];" ::"r"(bar) : "memory");
 }
 
