@@ -605,8 +605,11 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 auto release_buffer = [&]() {
                     tc_fence_before_sync();
                     __syncwarp();
+                    // (one CTA on 256 columns hands back between two groups, where the branch is the cheaper one: 1024 x 4096 x 4096 FP8
+                    // 17.6 us elected, 17.4 us so)
                     if (PAIR) mbar_arrive_cluster_relaxed_elected(lead_tempty0 + 8u * a);
-                    else mbar_arrive_elected(tempty_bar(a));
+                    else if (SCALE == SCALE_VEC_B || G <= D) mbar_arrive_elected(tempty_bar(a));
+                    else if (lane == 0) mbar_arrive(tempty_bar(a));
                 };
                 auto consume_group = [&](int gi, const uint32_t (&cur)[GC]) {
                     if (SCALE == SCALE_BLOCK_B) {
