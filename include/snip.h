@@ -490,6 +490,8 @@ int snip_select_scheme(int m, int n, const double *q, const int64_t *w, int64_t 
  *                              expects.  Non-zero makes the first stage of every GEMM incomplete for
  *                              ever while every copy still lands: the kernel's waits run out, it
  *                              leaves on its own and snip_poll_status reports SNIP_ERR_TIMEOUT.
+ *                              (Where the slices of a tile are the CTAs of a cluster: the first
+ *                              slice's; the others have their sums and have to drop them.)
  *                              Nothing traps or faults; used with a short wait limit by the tests.
  *   SNIP_DEBUG_GEMM_KERNEL   : 0 (default) = the library chooses by shape, 1 = one CTA per tile, 2 = a pair of
  *                              CTAs per tile, 3 = one CTA per tile of 128 columns, for every quantized GEMM under

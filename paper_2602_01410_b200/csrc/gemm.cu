@@ -59,6 +59,7 @@ struct GemmArgs {
     int64_t ldo;
     int32_t accumulate;
     uint32_t stage_tx_bytes;   // bytes the two TMA loads of one stage report to the barrier
+    uint32_t tx_skew;          // testing hook, part of stage_tx_bytes: in a cluster of slices the first slice's only
     uint64_t wait_limit_ns;    // bound of every device-side wait
     uint32_t *status;
     uint32_t status_mark;      // see status_begin
@@ -309,11 +310,12 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 const WorkItem wi = work_item<SCALE == SCALE_VEC_B>(g.work, w, num_kstages);
                 int m_idx, n_idx;
                 tile_coords(wi.t, num_m, num_n, m_idx, n_idx);
+                const uint32_t tx_bytes = C::kCtas * g.stage_tx_bytes - (CLUSTER && wi.slice > 0 ? g.tx_skew : 0u);
                 for (int ks = wi.ks0; ks < wi.ks1; ++ks, ++it) {
                     const int s = it % S;
                     const uint32_t ph = (it / S) & 1u;
                     if (!wait1(empty_bar(s), ph ^ 1u)) { ok = false; break; }
-                    if (rank == 0) mbar_arrive_expect_tx(full_bar(s), C::kCtas * g.stage_tx_bytes);
+                    if (rank == 0) mbar_arrive_expect_tx(full_bar(s), tx_bytes);
                     const int row = m_idx * BM + (int)rank * CM, col = n_idx * BN + (int)rank * C::kBLines;
                     if (PAIR) {   // each CTA fetches its own share (no multicast); the leader's barrier counts the bytes of both
                         tma_load_2d_pair(smem_a0 + s * C::kABytes, &tmA, lead_full0 + 8u * s, ks * C::kStageElemsX, row);
@@ -665,7 +667,8 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 // slice gi * nsl / G: every CTA writes the groups of the others into their stage memory, which no copy or MMA uses any
                 // more once all CTAs are here, and then adds its own groups in slice order and stores them.  Nothing is sent through L2
                 // and no CTA adds the whole tile: 8192 tokens x 256 x 2048 21.8 -> 17.6 us, 16384 x 512 x 1024 28.9 -> 24.1 us.  A CTA that gave
-                // up a wait takes part in both barriers all the same.
+                // up a wait takes part in both barriers all the same; before the second one it raises the abort flag of every CTA here, because
+                // none of them has the tile's sums then.
                 const int me = wi.slice, nsl = wi.nsl, per = (G + nsl - 1) / nsl;
                 float *av = reinterpret_cast<float *>(acc);
                 auto owner = [&](int gi) { return gi * nsl / G; };
@@ -674,6 +677,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     return (uint32_t)((((from * kNumEpiWarps + e) * per + k) * 4) * 512 + lane * 16);
                 };
                 cluster_sync();
+                if (e == 0 && lane < nsl && *abort_flag) st_cluster_u32(mapa(smem_u32(const_cast<uint32_t *>(abort_flag)), (uint32_t)lane), 1u);
                 if (ok) {
 #pragma unroll
                     for (int gi = 0; gi < G; ++gi) {
@@ -686,6 +690,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                     }
                 }
                 cluster_sync();
+                ok = !*abort_flag;
                 if (ok) {
 #pragma unroll
                     for (int gi = 0; gi < G; ++gi) {
@@ -1079,8 +1084,8 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         g.partials = w.partials;
     }
     g.stage_tx_bytes = 0;
+    g.tx_skew = (uint32_t)g_tx_skew.load();
     g.wait_limit_ns = (uint64_t)g_wait_limit_ns.load();
-    const int tx_skew = g_tx_skew.load();
     const bool f32 = out_dtype == SNIP_OUT_FP32;
 
     // Pairs of CTAs on 256-row tiles halve a CTA's share of B and keep six stages instead of four: forward and input gradient 2-4 % faster
@@ -1133,7 +1138,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         rc = make_operand_map(&tmB, b_codes, CU_TENSOR_MAP_DATA_TYPE_UINT8, No, Kc / 2, Kc / 2, 128, BN / ctas);
         if (rc) return rc;
         const uint32_t idesc = make_idesc_block_scaled(1, 1, CM * ctas, BN);
-        g.stage_tx_bytes = (CM + BN / ctas) * 128 + tx_skew;
+        g.stage_tx_bytes = (CM + BN / ctas) * 128 + g.tx_skew;
         if (narrow) return launch_gemm_narrow<MmaKind::MXF4>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
         return launch_gemm_scale<MmaKind::MXF4, 192>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
     }
@@ -1160,7 +1165,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     const uint32_t idesc = make_idesc(a4 ? 5 : 0, b4 ? 5 : 0, CM * ctas, BN);
     // an FP4 operand expanded by the TMA unit occupies 128 B per row in shared memory but reports
     // only its 64 packed source bytes to the barrier
-    g.stage_tx_bytes = CM * (a4 ? 64 : 128) + BN / ctas * (b4 ? 64 : 128) + tx_skew;
+    g.stage_tx_bytes = CM * (a4 ? 64 : 128) + BN / ctas * (b4 ? 64 : 128) + g.tx_skew;
     if (narrow) return launch_gemm_narrow<MmaKind::F8F6F4>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
     return launch_gemm_scale<MmaKind::F8F6F4, 256>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
 }

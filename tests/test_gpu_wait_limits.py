@@ -88,3 +88,24 @@ def test_narrow_product_of_quantized_operands(api, hooks):  # noqa: F811
     ws = torch.full((256,), 0xFF, dtype=torch.uint8, device="cuda")
     api.snip_debug_set(api.DEBUG_GEMM_KERNEL, api.GEMM_KERNEL_NARROW)
     check(api, hooks, ws, lambda: [api.snip_gemm_quantized(api.OP_FWD, a, b, (M, N), api.OUT_FP32, ws=ws)])
+
+
+# A tile of the weight gradient whose slices are the CTAs of a cluster (128-wide tiles; 8192 tokens: four slices, 3072: three): the hook holds
+# up the first slice alone.  The others have their sums, but none of a cluster may store its share of a tile that one slice is missing from;
+# above all nothing may be added to a caller's gradient.
+@pytest.mark.parametrize("accumulate", [False, True])
+@pytest.mark.parametrize("fmt", [FP8, FP4])
+@pytest.mark.parametrize("M", [3072, 8192])
+def test_slices_of_a_tile_that_one_slice_is_missing_from(api, hooks, M, fmt, accumulate):  # noqa: F811
+    K, N = 320, 256
+    x, _, dy, _ = inputs(M, K, N, 65, 1.0)
+    (cd, sd, _, _), (cx, sx, _, _) = (api.snip_quantize(t, fmt, api.BLOCK_COL, api.Q_TRANSPOSED) for t in (dy, x))
+    a, b = api.make_qtensor(cd, sd, M, N, fmt, api.BLOCK_COL, True), api.make_qtensor(cx, sx, M, K, fmt, api.BLOCK_COL, True)
+    ws = torch.full((api.snip_workspace_size(api.OP_WGRAD, M, N, K, fmt, fmt)[0],), 0xFF, dtype=torch.uint8, device="cuda")
+    api.snip_debug_set(api.DEBUG_GEMM_KERNEL, api.GEMM_KERNEL_NARROW)
+    start = torch.randn(N, K, device="cuda")
+
+    def call():
+        return [api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32, accumulate=accumulate, out=start.clone(), ws=ws)]
+    _, during = check(api, hooks, ws, call)
+    assert torch.equal(during[0], start)
