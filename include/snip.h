@@ -507,6 +507,14 @@ int snip_select_scheme(int m, int n, const double *q, const int64_t *w, int64_t 
 int snip_debug_set(int key, long long value);
 
 /*
+ * How the calling thread's last quantized GEMM under the paper's rule was launched: plan_host[0] = columns of a tile,
+ * [1] = CTAs per tile (2: a pair), [2] = slices that tiles of the last wave (of a cluster launch: all tiles) are cut
+ * into along the contraction, [3] = CTAs of a cluster (1, a pair's 2, or the slices of a tile).  For the tests; zeros before
+ * the first such call.  Host-only.  (No counterpart in the paper.)
+ */
+int snip_debug_last_gemm(int plan_host[4]);
+
+/*
  * Read the device status word of a GEMM workspace.  Call after the stream has been
  * synchronized.  *status_host becomes SNIP_OK or SNIP_ERR_TIMEOUT (a bounded device-side wait
  * expired and the kernel returned early; outputs are then invalid).  Every GEMM entry point

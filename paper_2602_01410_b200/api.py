@@ -28,7 +28,7 @@ EXPORTS = (
     "snip_version", "snip_status_string", "snip_last_cuda_error", "snip_quantize_sizes",
     "snip_quantize", "snip_quantize_noalloc", "snip_quantize_mx_sizes", "snip_quantize_mx", "snip_quantize_dual_workspace", "snip_quantize_dual", "snip_quantize_sr", "snip_workspace_size", "snip_gemm_quantized", "snip_gemm_mx", "snip_quantize_nvfp4_sizes", "snip_quantize_nvfp4_dual", "snip_gemm_nvfp4", "snip_linear_fwd_bwd_nvfp4_workspace", "snip_linear_fwd_bwd_nvfp4", "snip_linear_fwd",
     "snip_linear_dgrad", "snip_linear_wgrad", "snip_linear_mx", "snip_linear_mx_workspace", "snip_linear_fwd_bwd_workspace", "snip_linear_fwd_bwd", "snip_layer_stats", "snip_layer_stats_workspace", "snip_adamw_sensitivity_workspace", "snip_adamw_sensitivity", "snip_loss_divergence", "snip_weight_divergence", "snip_select_scheme",
-    "snip_poll_status", "snip_debug_set",
+    "snip_poll_status", "snip_debug_set", "snip_debug_last_gemm",
 )
 
 
@@ -108,6 +108,7 @@ def _load():
     lib.snip_select_scheme.argtypes = [i32, i32, vp, vp, i64, i32, vp, vp, vp]
     lib.snip_poll_status.argtypes = [vp, ctypes.POINTER(i32)]
     lib.snip_debug_set.argtypes = [i32, ctypes.c_longlong]
+    lib.snip_debug_last_gemm.argtypes = [ctypes.POINTER(i32)]
     for name in EXPORTS:
         fn = getattr(lib, name)
         if fn.restype is ctypes.c_int and name not in ("snip_version",):
@@ -520,6 +521,13 @@ def snip_select_scheme(q, w, target: int, num_groups: int = 1):
 def snip_debug_set(key: int, value: int) -> None:
     """Testing hooks of the library (process-wide, off by default): see include/snip.h."""
     _check("snip_debug_set", _lib.snip_debug_set(key, value))
+
+
+def snip_debug_last_gemm() -> tuple:
+    """(columns of a tile, CTAs per tile, slices, CTAs of a cluster) of this thread's last quantized GEMM under the paper's rule."""
+    plan = (ctypes.c_int * 4)()
+    _check("snip_debug_last_gemm", _lib.snip_debug_last_gemm(plan))
+    return tuple(plan)
 
 
 def snip_poll_status(ws: torch.Tensor) -> int:

@@ -893,8 +893,12 @@ int sm_count()
     return n;
 }
 
-// Clusters of `size` CTAs of the 128-wide weight-gradient kernel that the current device holds at a time (a cluster's CTAs share a GPC, so
-// this is less than SMs / size); 0 if it cannot be told.
+// Clusters of `size` CTAs of the 128-wide weight-gradient kernel that find a place on the current device together (a cluster's CTAs share
+// a GPC, so this is less than SMs / size); 0 if it cannot be told.  The occupancy query answers for an idle device.  Clusters of two and
+// four fit up to that number also where they take over SMs one by one from the kernel ahead (74 and 33 of them, 60 runs each behind CTAs
+// that ended at random), but three CTAs are one and a half pairs of SMs: of 45 clusters up to four were left waiting for others to end,
+// 42 had one left in 1 run of 10, 41 none.  So odd sizes keep a tenth back.  4096 tokens, 45 tiles of 128 x 128, calls in a row: three
+// slices 27.2 us, two 16.0 us.
 int max_clusters(int size)
 {
     static thread_local int dev_cached = -1, n[kMaxSlices + 1];
@@ -919,6 +923,7 @@ int max_clusters(int size)
                 n[c] = 0;
                 cudaGetLastError();
             }
+            if (c & 1) n[c] -= n[c] / 10;
         }
         dev_cached = dev;
     }
@@ -935,6 +940,8 @@ WorkSplit plan_clusters(int num_tiles, int num_stages, bool slice)
     return {num_tiles, 1, num_tiles};
 }
 
+thread_local int last_gemm[4];   // see snip_debug_last_gemm
+
 template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32>
 int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc, bool cleared, cudaStream_t st)
 {
@@ -947,6 +954,7 @@ int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
         // a per-function, per-device attribute; setting it on every launch is cheap and correct on any device
         SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
         const int grid = (ga.work.num_items < units ? ga.work.num_items : units) * C::kCtas;
+        last_gemm[0] = BN; last_gemm[1] = C::kCtas; last_gemm[2] = ga.work.nsplit; last_gemm[3] = cluster;
         return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, cluster, tmA, tmB, tmO, ga, idesc);
     };
     if constexpr (C::kClusterSlices) {
@@ -1217,6 +1225,13 @@ extern "C" int snip_debug_set(int key, long long value)
         case SNIP_DEBUG_GEMM_SLICING: if (value < 0 || value > 1) return SNIP_ERR_ARG; g_slicing.store((int)value); return SNIP_OK;
         default: return SNIP_ERR_ARG;
     }
+}
+
+extern "C" int snip_debug_last_gemm(int plan_host[4])
+{
+    if (!plan_host) return SNIP_ERR_ARG;
+    for (int i = 0; i < 4; ++i) plan_host[i] = snip::last_gemm[i];
+    return SNIP_OK;
 }
 
 extern "C" int snip_poll_status(const void *ws, int *status_host)

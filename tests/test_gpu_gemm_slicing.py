@@ -126,3 +126,22 @@ def test_cluster_and_workspace_exchange(api, slicing, fa, fb, choice, shape):
     # they differ in the order of FP32 additions only: a few units in the last place of sums over at most 65 chunks
     assert not torch.equal(outs[1], outs[0])
     assert rel_fro(outs[1].cpu().numpy(), outs[0].cpu().numpy().astype(np.float64)) <= 1e-6
+
+
+# Clusters of three in numbers that only an idle device has room for (45 of 45): behind another kernel the last ones wait for a whole
+# tile's time.  4096 tokens are enough for four slices; from 34 tiles or so on there are three, and never more of them than nine tenths of
+# the SMs hold.
+@pytest.mark.parametrize("fmt", [FP8, FP4])
+def test_clusters_of_three_leave_room(api, fmt):
+    sms = torch.cuda.get_device_properties(0).multi_processor_count
+    M, K = 4096, 128
+    seen = set()
+    for tiles in range(30, 50):
+        x, dy, a, b, keep = operands(api, M, K, 128 * tiles, fmt, fmt, tiles)
+        api.snip_gemm_quantized(api.OP_WGRAD, a, b, (128 * tiles, K))
+        width, ctas, slices, cluster = api.snip_debug_last_gemm()
+        assert (width, ctas) == (128, 1) and cluster == slices
+        assert slices != 3 or 3 * tiles <= 0.9 * sms, tiles
+        seen.add(slices)
+    torch.cuda.synchronize()
+    assert seen == {2, 3, 4}
