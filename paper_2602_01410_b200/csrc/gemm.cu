@@ -1112,8 +1112,9 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // so that twice the tiles still are one wave (forward FP8 1024x2048x4096 18.0 -> 12.5 us, 8192x256x2048 11.2 -> 8.3 us, 512x512x512 6.6 -> 5.2
     // us; FP4 1024x4096x4096, two waves either way, 24.8 -> 18.6 us; weight gradient 8192x256x2048 28.6 -> 20.6 us).  A launch lasts as long as
     // the pipeline stages that its SMs run one after the other (kMinSavedStages more where its last wave is sliced) times what a stage of a narrow
-    // tile takes next to a wide one's: measured 0.64-0.68 forward and input gradient (0.76 against 192 columns: 473 and 621 cycles per
-    // chunk of a large product), 0.69-0.79 weight gradient.
+    // tile takes next to a wide one's: measured 0.64-0.68 forward and input gradient, 0.69-0.79 weight gradient.  FP4 against pairs 192 wide
+    // 0.70-0.72 (8192 x 1536 outputs over 4096 features, us narrow / wide: 2 waves to 2 18.3 / 24.9, 5 to 4 41 / 46, 4 to 3 33.4 / 35.6, 11 to 8 87 / 89,
+    // 7 to 5 55.9 / 56.8, 3 to 2 25.8 / 25.0).
     auto use_narrow = [&](int tile_n, int stage_k, float ratio) {
         if (choice != 0) return choice == 3;
         auto stages = [&](int bn) {
@@ -1140,7 +1141,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         // warps' registers at once, and with half the operand bytes and a quarter of the tensor time it stays below the power
         // cap: 16384x12288x4096 755 -> 673 us, 8192x3200x8640 215 -> 193 us, 8192x2048x256 16.4 -> 14.5 us.  The weight gradient over
         // whole chunks takes the path below: with two operations per element the wider tile is as fast or faster.
-        const bool narrow = use_narrow(192, 256, 0.76f);
+        const bool narrow = use_narrow(192, 256, 0.72f);
         const int BN = narrow ? 128 : 192;
         const bool pair = !narrow && use_pair(BN);
         const int ctas = pair ? 2 : 1;

@@ -75,3 +75,16 @@ def test_bf16_accumulates_into_fp32(api):
     out = api.snip_linear_wgrad(to_dev(dy), to_dev(x), BF16, BF16, api.OUT_FP32, accumulate=True, out=base)[0]
     torch.cuda.synchronize()
     assert rel_fro(out.cpu().numpy(), want) <= 1e-5
+
+
+# FP4 forward, where both widths take the same number of waves or the narrow ones a quarter or a third more: 128 columns; half as many
+# again: 192.  (Row tiles of an output of 1536 columns, i.e. 12 narrow or 8 wide tiles each; the counts are for 148 SMs.)
+@pytest.mark.parametrize("row_tiles,width", [(22, 128), (58, 128), (42, 128), (132, 128), (32, 192)])
+def test_width_of_fp4_tiles_by_waves(api, row_tiles, width):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("wave counts are for 148 SMs")
+    M, K, N = 128 * row_tiles, 128, 1536
+    X, W = torch.randn(M, K, device="cuda").bfloat16(), torch.randn(N, K, device="cuda").bfloat16()
+    api.snip_linear_fwd(X, W, FP4, FP4)
+    torch.cuda.synchronize()
+    assert api.snip_debug_last_gemm()[0] == width
