@@ -44,6 +44,8 @@ constexpr int kMinSliceStages = 8, kMinSavedStages = 20;
 // two slices save eight: 12.0 us whole, 12.6 us sliced).  256-wide tiles keep the exchange through L2: there are half as many of them as
 // narrow ones, and two slices of 64 such tiles come out level with 128 whole narrow ones (8192 x 1024 x 2048: 32.9 / 32.5 us).
 constexpr int kMinSavedStagesCluster = 12;
+// What the exchange through the workspace takes for 128-wide tiles, in the same measure: about 5 us more (see prefer_clusters).
+constexpr int kWorkspaceExchangeChunks = 24;
 constexpr int kSfCols = 32;  // tensor-memory columns holding constant scale factors (kind::mxf4)
 
 enum ScaleMode { SCALE_BLOCK_B = 1, SCALE_VEC_B = 2 };
@@ -945,6 +947,16 @@ WorkSplit plan_clusters(int num_tiles, int num_stages, bool slice)
 
 thread_local int last_gemm[4];   // see snip_debug_last_gemm
 
+// 128-wide tiles: slices in clusters, or fewer chunks each and the dearer exchange through the workspace?  Clusters fill the chip less well
+// (45 tiles: two slices each, 90 of 148 SMs, against three), so long contractions go through the workspace.  us, clusters / workspace: 45
+// tiles of 64 chunks 22.0 / 22.9, 76 24.6 / 24.6, 118 33.2 / 30.9, 256 61.5 / 50.4; 36 tiles (three against four) of 118 26.3 / 26.7, 160
+// 32.0 / 31.6, 256 44.7 / 41.6.
+bool prefer_clusters(const WorkSplit &clusters, const WorkSplit &workspace, int num_chunks)
+{
+    return clusters.nsplit > 1 && (float)num_chunks / clusters.nsplit + kMinSavedStagesCluster <=
+                                      (float)num_chunks / workspace.nsplit + (workspace.nsplit > 1 ? kWorkspaceExchangeChunks : 0);
+}
+
 template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32>
 int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc, bool cleared, cudaStream_t st)
 {
@@ -960,11 +972,14 @@ int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
         last_gemm[0] = BN; last_gemm[1] = C::kCtas; last_gemm[2] = ga.work.nsplit; last_gemm[3] = cluster;
         return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, cluster, tmA, tmB, tmO, ga, idesc);
     };
-    if constexpr (C::kClusterSlices) {
-        ga.work = plan_clusters(num_tiles, num_stages, slice);
-        if (ga.work.nsplit > 1) return launch(gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32, true>, ga.work.nsplit);
-    }
     ga.work = plan_work(num_tiles, num_stages, units, kMinSliceStages, kMinSavedStages, slice, kMaxSlicedItems / C::kCtas);
+    if constexpr (C::kClusterSlices) {
+        const WorkSplit cl = plan_clusters(num_tiles, num_stages, slice);
+        if (prefer_clusters(cl, ga.work, (int)ceil_div(g.Kc, C::kChunkElems))) {
+            ga.work = cl;
+            return launch(gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32, true>, cl.nsplit);
+        }
+    }
     if (ga.work.nsplit > 1 && !cleared)
         SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * C::kCtas * sizeof(uint32_t), st));
     return launch(gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32, false>, C::kCtas);
@@ -1120,9 +1135,9 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         auto stages = [&](int bn) {
             const int sms = sm_count(), tiles = (int)(ceil_div(Mo, CM) * ceil_div(No, bn)), per_tile = (int)ceil_div(Kc, stage_k);
             const bool slice = scale_mode == SCALE_VEC_B && g.partials;
-            const WorkSplit cl = plan_clusters(tiles, per_tile, slice && bn == 128);
-            if (cl.nsplit > 1) return (float)per_tile / cl.nsplit + kMinSavedStagesCluster;
             const WorkSplit sp = plan_work(tiles, per_tile, sms, kMinSliceStages, kMinSavedStages, slice);
+            const WorkSplit cl = plan_clusters(tiles, per_tile, slice && bn == 128);
+            if (prefer_clusters(cl, sp, (int)ceil_div(Kc, 128))) return (float)per_tile / cl.nsplit + kMinSavedStagesCluster;
             if (sp.nsplit > 1) return (float)(sp.split_first / sms) * per_tile + (float)per_tile / sp.nsplit + kMinSavedStages;
             return (float)ceil_div(tiles, sms) * per_tile;
         };

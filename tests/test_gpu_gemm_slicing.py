@@ -145,3 +145,19 @@ def test_clusters_of_three_leave_room(api, fmt):
         seen.add(slices)
     torch.cuda.synchronize()
     assert seen == {2, 3, 4}
+
+
+# Clusters, or more slices and the exchange through the workspace, by the length of the contraction: (chunks, tiles) -> (slices, CTAs of a
+# cluster), sums against the unsliced product as above.  (For 148 SMs in GPCs that hold more than 32 clusters of four.)
+@pytest.mark.parametrize("chunks,tiles,want", [(64, 45, (2, 2)), (118, 45, (3, 1)), (118, 42, (3, 1)), (118, 36, (3, 3)), (256, 36, (4, 1)), (256, 30, (4, 4))])
+def test_exchange_by_the_length_of_the_contraction(api, slicing, chunks, tiles, want):
+    M, K, N = 128 * chunks, 128, 128 * tiles
+    x, dy, a, b, keep = operands(api, M, K, N, FP8, FP8, chunks + tiles)
+    got = {}
+    for mode in (0, 1):
+        slicing(mode)
+        got[mode] = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32)
+    torch.cuda.synchronize()
+    assert api.snip_debug_last_gemm() == (128, 1, *want)
+    # the order of FP32 additions only, over at most 256 chunks (as in test_cluster_and_workspace_exchange, whose bound is for 65)
+    assert rel_fro(got[1].cpu().numpy(), got[0].cpu().numpy().astype(np.float64)) <= 2e-6
