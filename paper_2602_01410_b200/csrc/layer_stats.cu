@@ -456,13 +456,17 @@ extern "C" int snip_layer_stats(const snip_layer_tensors_t *t, uint32_t fmt_mask
             if (heavy) ++a.nheavy; else ++a.nlight;
         }
     }
-    // CTAs of each kind by their cost per 128x128 elements, measured: about 5 (1x128 and 128x1 tiles), 3 (128x128) and 1 (norm only)
+    // CTAs of each kind by their cost per 128x128 elements, measured: about 5 (1x128 and 128x1 tiles), 3 (128x128) and 1 (norm only).  FP4
+    // alone costs a little less than that (16384 x 4096 x 4096 136.6 us at 5 : 3 : 1, 132.2 us so; 8192 x 3200 x 9600 119.3, 116.8 us).
+    const bool f4_alone = fmt_mask == 4u;
     int64_t cost[2] = {0, 0};
     for (int i = 0; i < a.nheavy + a.nlight; ++i)
-        cost[i < a.nheavy ? 0 : 1] += (int64_t)a.t[i].nitems * (a.t[i].mode == MODE_ROWCOL ? 5 : a.t[i].mode == MODE_BLK ? 3 : 1);
+        cost[i < a.nheavy ? 0 : 1] += (int64_t)a.t[i].nitems * (a.t[i].mode == MODE_ROWCOL ? (f4_alone ? 47 : 50) : a.t[i].mode == MODE_BLK ? (f4_alone ? 29 : 30) : 10);
     a.light_ctas = a.nheavy == 0 ? grid : 0;
     if (a.nheavy && a.nlight) {
         a.light_ctas = (int32_t)(grid * cost[1] / (cost[0] + cost[1]));
+        // (past about 108 of 444 the launch takes 15-30 % longer, with any option: 512 x 8192 x 28672 179 us at 107, 239 us at 110)
+        if (f4_alone && a.light_ctas > grid * 6 / 25) a.light_ctas = grid * 6 / 25;
         if (a.light_ctas < 1) a.light_ctas = 1;
         if (a.light_ctas > grid - 1) a.light_ctas = grid - 1;
     }
