@@ -107,6 +107,7 @@ struct ChainLink {
     uint32_t *zero = nullptr;
     int32_t zero_words = 0;
     StatJobs *jobs = nullptr;   // quantizers append, the next GEMM takes them
+    int32_t *ctas = nullptr;    // [3], zero at first: what the chain's GEMMs under the paper's rule launched, in order
 };
 
 // One tensor of the two-output quantizer (quantize.cu: quantize_dual_impl, quantize_xwd_impl).

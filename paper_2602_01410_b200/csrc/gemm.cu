@@ -936,14 +936,35 @@ int max_clusters(int size)
 }
 
 // All tiles in slices, the slices of a tile in a cluster, where all clusters run at the same time and slicing saves what the exchange costs;
-// nsplit == 1: not so.  128-wide tiles on one CTA each.
-WorkSplit plan_clusters(int num_tiles, int num_stages, bool slice)
+// nsplit == 1: not so.  128-wide tiles on one CTA each.  In a chain the product starts beside others, on free_sms SMs: where its whole tiles
+// fit there and its slices do not, those that would wait for an SM cost more than a few stages saved (one layer, FP8, us whole / in two slices:
+// 3072 tokens 256 -> 4608 48.0 / 56.8, 1024 -> 1024 35.3 / 37.7; where neither fits, 3584 tokens 1152 -> 1024 44.2 / 41.1).
+WorkSplit plan_clusters(int num_tiles, int num_stages, bool slice, int free_sms)
 {
-    for (int ns = kMaxSlices; slice && ns > 1; --ns)
-        if (num_stages / ns >= kMinSliceStages && num_stages - num_stages / ns >= kMinSavedStagesCluster && num_tiles <= max_clusters(ns))
-            return {0, ns, num_tiles * ns};
+    for (int ns = kMaxSlices; slice && ns > 1; --ns) {
+        const int saved = num_stages - num_stages / ns;
+        if (num_stages / ns < kMinSliceStages || saved < kMinSavedStagesCluster || num_tiles > max_clusters(ns)) continue;
+        if (saved < kMinSavedStages && num_tiles <= free_sms && num_tiles * ns > free_sms) continue;
+        return {0, ns, num_tiles * ns};
+    }
     return {num_tiles, 1, num_tiles};
 }
+
+// SMs that a chain's third GEMM, the weight gradient, finds free when it starts (which is when all CTAs of the second one have started): all
+// but those on which a CTA of the second one had to wait for one of the first to end.  ctas: what the first two launched.
+int free_beside(const int32_t *ctas, int sms)
+{
+    const int late = ctas[1] - (sms - ctas[0]);
+    return late > 0 ? sms - late : sms;
+}
+
+// Host side of a launch.
+struct LaunchEnv {
+    bool cleared;       // status word and slice counters are zero when the kernel starts
+    int32_t free_sms;   // SMs that are free when it starts
+    int32_t *ctas;      // a chain's count of this GEMM's CTAs, or null
+    cudaStream_t st;
+};
 
 thread_local int last_gemm[4];   // see snip_debug_last_gemm
 
@@ -958,7 +979,7 @@ bool prefer_clusters(const WorkSplit &clusters, const WorkSplit &workspace, int 
 }
 
 template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32>
-int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc, bool cleared, cudaStream_t st)
+int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc, const LaunchEnv &env)
 {
     using C = Cfg<KIND, BN, SCALE, PAIR>;
     const int num_tiles = (int)(ceil_div(g.Mo, C::BM) * ceil_div(g.No, BN)), num_stages = (int)ceil_div(g.Kc, C::kStageK);
@@ -970,49 +991,50 @@ int launch_gemm(const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMa
         SNIP_CUDA_TRY(cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, C::kSmemBytes));
         const int grid = (ga.work.num_items < units ? ga.work.num_items : units) * C::kCtas;
         last_gemm[0] = BN; last_gemm[1] = C::kCtas; last_gemm[2] = ga.work.nsplit; last_gemm[3] = cluster;
-        return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, st, cluster, tmA, tmB, tmO, ga, idesc);
+        if (env.ctas) *env.ctas = grid;
+        return launch_chained(kern, grid, kGemmThreads, C::kSmemBytes, env.st, cluster, tmA, tmB, tmO, ga, idesc);
     };
     ga.work = plan_work(num_tiles, num_stages, units, kMinSliceStages, kMinSavedStages, slice, kMaxSlicedItems / C::kCtas);
     if constexpr (C::kClusterSlices) {
-        const WorkSplit cl = plan_clusters(num_tiles, num_stages, slice);
+        const WorkSplit cl = plan_clusters(num_tiles, num_stages, slice, env.free_sms);
         if (prefer_clusters(cl, ga.work, (int)ceil_div(g.Kc, C::kChunkElems))) {
             ga.work = cl;
             return launch(gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32, true>, cl.nsplit);
         }
     }
-    if (ga.work.nsplit > 1 && !cleared)
-        SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * C::kCtas * sizeof(uint32_t), st));
+    if (ga.work.nsplit > 1 && !env.cleared)
+        SNIP_CUDA_TRY(cudaMemsetAsync(g.counters, 0, (size_t)(num_tiles - ga.work.split_first) * kNumEpiWarps * C::kCtas * sizeof(uint32_t), env.st));
     return launch(gemm_kernel<KIND, BN, SCALE, PAIR, OUT_F32, false>, C::kCtas);
 }
 
 template <MmaKind KIND, int BN, int SCALE>
 int launch_gemm_form(bool pair, bool out_f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc,
-                     bool cleared, cudaStream_t st)
+                     const LaunchEnv &env)
 {
     if (pair)
-        return out_f32 ? launch_gemm<KIND, BN, SCALE, true, true>(tmA, tmB, tmO, g, idesc, cleared, st)
-                       : launch_gemm<KIND, BN, SCALE, true, false>(tmA, tmB, tmO, g, idesc, cleared, st);
-    return out_f32 ? launch_gemm<KIND, BN, SCALE, false, true>(tmA, tmB, tmO, g, idesc, cleared, st)
-                   : launch_gemm<KIND, BN, SCALE, false, false>(tmA, tmB, tmO, g, idesc, cleared, st);
+        return out_f32 ? launch_gemm<KIND, BN, SCALE, true, true>(tmA, tmB, tmO, g, idesc, env)
+                       : launch_gemm<KIND, BN, SCALE, true, false>(tmA, tmB, tmO, g, idesc, env);
+    return out_f32 ? launch_gemm<KIND, BN, SCALE, false, true>(tmA, tmB, tmO, g, idesc, env)
+                   : launch_gemm<KIND, BN, SCALE, false, false>(tmA, tmB, tmO, g, idesc, env);
 }
 template <MmaKind KIND, int BN>
 int launch_gemm_scale(int scale, bool pair, bool out_f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g,
-                      uint32_t idesc, bool cleared, cudaStream_t st)
+                      uint32_t idesc, const LaunchEnv &env)
 {
-    return scale == SCALE_BLOCK_B ? launch_gemm_form<KIND, BN, SCALE_BLOCK_B>(pair, out_f32, tmA, tmB, tmO, g, idesc, cleared, st)
-                                  : launch_gemm_form<KIND, BN, SCALE_VEC_B>(pair, out_f32, tmA, tmB, tmO, g, idesc, cleared, st);
+    return scale == SCALE_BLOCK_B ? launch_gemm_form<KIND, BN, SCALE_BLOCK_B>(pair, out_f32, tmA, tmB, tmO, g, idesc, env)
+                                  : launch_gemm_form<KIND, BN, SCALE_VEC_B>(pair, out_f32, tmA, tmB, tmO, g, idesc, env);
 }
 
 // 128-wide tiles, one CTA each.
 template <MmaKind KIND>
 int launch_gemm_narrow(int scale, bool out_f32, const CUtensorMap &tmA, const CUtensorMap &tmB, const CUtensorMap &tmO, const GemmArgs &g, uint32_t idesc,
-                       bool cleared, cudaStream_t st)
+                     const LaunchEnv &env)
 {
     if (scale == SCALE_BLOCK_B)
-        return out_f32 ? launch_gemm<KIND, 128, SCALE_BLOCK_B, false, true>(tmA, tmB, tmO, g, idesc, cleared, st)
-                       : launch_gemm<KIND, 128, SCALE_BLOCK_B, false, false>(tmA, tmB, tmO, g, idesc, cleared, st);
-    return out_f32 ? launch_gemm<KIND, 128, SCALE_VEC_B, false, true>(tmA, tmB, tmO, g, idesc, cleared, st)
-                   : launch_gemm<KIND, 128, SCALE_VEC_B, false, false>(tmA, tmB, tmO, g, idesc, cleared, st);
+        return out_f32 ? launch_gemm<KIND, 128, SCALE_BLOCK_B, false, true>(tmA, tmB, tmO, g, idesc, env)
+                       : launch_gemm<KIND, 128, SCALE_BLOCK_B, false, false>(tmA, tmB, tmO, g, idesc, env);
+    return out_f32 ? launch_gemm<KIND, 128, SCALE_VEC_B, false, true>(tmA, tmB, tmO, g, idesc, env)
+                   : launch_gemm<KIND, 128, SCALE_VEC_B, false, false>(tmA, tmB, tmO, g, idesc, env);
 }
 
 }  // namespace
@@ -1113,6 +1135,13 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     g.tx_skew = (uint32_t)g_tx_skew.load();
     g.wait_limit_ns = (uint64_t)g_wait_limit_ns.load();
     const bool f32 = out_dtype == SNIP_OUT_FP32;
+    LaunchEnv env = {w.cleared, sm_count(), nullptr, st};
+    if (link.ctas) {
+        int i = 0;
+        while (i < 2 && link.ctas[i]) ++i;
+        env.ctas = link.ctas + i;
+        if (i == 2) env.free_sms = free_beside(link.ctas, sm_count());
+    }
 
     // Pairs of CTAs on 256-row tiles halve a CTA's share of B and keep six stages instead of four: forward and input gradient 2-4 % faster
     // (FP8 16384x12288x4096 837 -> 808 us, 8192x8640x3200 248 -> 239 us, FP4 655 -> 635 us).  The weight gradient, whose promotion sets the pace,
@@ -1136,7 +1165,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
             const int sms = sm_count(), tiles = (int)(ceil_div(Mo, CM) * ceil_div(No, bn)), per_tile = (int)ceil_div(Kc, stage_k);
             const bool slice = scale_mode == SCALE_VEC_B && g.partials;
             const WorkSplit sp = plan_work(tiles, per_tile, sms, kMinSliceStages, kMinSavedStages, slice);
-            const WorkSplit cl = plan_clusters(tiles, per_tile, slice && bn == 128);
+            const WorkSplit cl = plan_clusters(tiles, per_tile, slice && bn == 128, env.free_sms);
             if (prefer_clusters(cl, sp, (int)ceil_div(Kc, 128))) return (float)per_tile / cl.nsplit + kMinSavedStagesCluster;
             if (sp.nsplit > 1) return (float)(sp.split_first / sms) * per_tile + (float)per_tile / sp.nsplit + kMinSavedStages;
             return (float)ceil_div(tiles, sms) * per_tile;
@@ -1166,8 +1195,8 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         if (rc) return rc;
         const uint32_t idesc = make_idesc_block_scaled(1, 1, CM * ctas, BN);
         g.stage_tx_bytes = (CM + BN / ctas) * 128 + g.tx_skew;
-        if (narrow) return launch_gemm_narrow<MmaKind::MXF4>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
-        return launch_gemm_scale<MmaKind::MXF4, 192>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
+        if (narrow) return launch_gemm_narrow<MmaKind::MXF4>(scale_mode, f32, tmA, tmB, tmO, g, idesc, env);
+        return launch_gemm_scale<MmaKind::MXF4, 192>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, env);
     }
     // FP8 x FP8, the mixed pairs and the FP4 x FP4 weight gradient over whole chunks: kind::f8f6f4; FP4 operands are expanded by
     // the TMA unit to one 16-byte-aligned group per 16 elements, which is the layout this MMA kind reads
@@ -1193,8 +1222,8 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // an FP4 operand expanded by the TMA unit occupies 128 B per row in shared memory but reports
     // only its 64 packed source bytes to the barrier
     g.stage_tx_bytes = CM * (a4 ? 64 : 128) + BN / ctas * (b4 ? 64 : 128) + g.tx_skew;
-    if (narrow) return launch_gemm_narrow<MmaKind::F8F6F4>(scale_mode, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
-    return launch_gemm_scale<MmaKind::F8F6F4, 256>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, w.cleared, st);
+    if (narrow) return launch_gemm_narrow<MmaKind::F8F6F4>(scale_mode, f32, tmA, tmB, tmO, g, idesc, env);
+    return launch_gemm_scale<MmaKind::F8F6F4, 256>(scale_mode, pair, f32, tmA, tmB, tmO, g, idesc, env);
 }
 
 }  // namespace snip

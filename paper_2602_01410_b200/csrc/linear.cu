@@ -329,7 +329,8 @@ extern "C" int snip_linear_fwd_bwd(const void *X, const void *W, const void *dY,
     quant.jobs = &jobs;
     quant.zero = static_cast<uint32_t *>(f.gws);
     quant.zero_words = gemm_ws_zero_words();
-    for (int i = 0; i < 3; ++i) mult[i].role = i ? CHAIN_BESIDE : CHAIN_AFTER;
+    int32_t ctas[3] = {0, 0, 0};
+    for (int i = 0; i < 3; ++i) { mult[i].role = i ? CHAIN_BESIDE : CHAIN_AFTER; mult[i].ctas = ctas; }
     mult[0].jobs = &jobs;
     GemmWs gw = gemm_ws(f.gws, gemm_ws_bytes_sliced());
     gw.cleared = true;

@@ -161,3 +161,25 @@ def test_exchange_by_the_length_of_the_contraction(api, slicing, chunks, tiles, 
     assert api.snip_debug_last_gemm() == (128, 1, *want)
     # the order of FP32 additions only, over at most 256 chunks (as in test_cluster_and_workspace_exchange, whose bound is for 65)
     assert rel_fro(got[1].cpu().numpy(), got[0].cpu().numpy().astype(np.float64)) <= 2e-6
+
+
+# In a layer the product starts beside the input gradient: (tokens, in, out), FP8 -> slices.  Whole tiles where they fit on the SMs that are
+# free then and slices do not; slices where neither fits, both fit, or the contraction is long.  (Counts are for 148 SMs.)
+@pytest.mark.parametrize("shape,slices", [((3072, 256, 4608), 1), ((3072, 1024, 1024), 1), ((3072, 4608, 256), 1), ((3584, 1152, 1024), 2),
+                                          ((3072, 512, 512), 3), ((5120, 256, 4608), 2)])
+def test_slices_of_a_product_that_starts_beside_others(api, shape, slices):
+    M, K, N = shape
+    rng = np.random.default_rng(sum(shape))
+    x, w, dy = to_dev(wl.make_x(rng, M, K, 0.01, 20.0)), to_dev(wl.make_w(rng, N, K)), to_dev(wl.make_dy(rng, M, N))
+    _, _, dw, _ = api.snip_linear_fwd_bwd(x, w, dy, FP8, FP8, FP8, api.OUT_FP32)
+    assert api.snip_debug_last_gemm()[:3] == (128, 1, slices)
+    api.snip_linear_wgrad(dy, x, FP8, FP8)
+    assert api.snip_debug_last_gemm()[2] > 1     # on its own it is sliced
+    api.snip_debug_set(api.DEBUG_GEMM_SLICING, 0)
+    try:
+        ref = api.snip_linear_wgrad(dy, x, FP8, FP8, api.OUT_FP32)[0]
+        torch.cuda.synchronize()
+    finally:
+        api.snip_debug_set(api.DEBUG_GEMM_SLICING, 1)
+    # the order of FP32 additions over at most 40 chunks (as above)
+    assert rel_fro(dw.cpu().numpy(), ref.cpu().numpy().astype(np.float64)) <= 1e-6
