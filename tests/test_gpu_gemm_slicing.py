@@ -101,19 +101,28 @@ def test_sliced_accumulate_garbage_workspace_and_minimum_workspace(api, slicing)
 
 # Both ways of adding the slices, forced: 128-wide tiles (kernel choice 3) whose slices are the CTAs of a cluster - two, three and four
 # of them, ragged tiles on both sides, contractions ending in a 64-wide tile, one group of a tile more for a CTA than for another - and
-# 256- / 192-wide tiles (choice 1), which exchange through the workspace.
+# 256- / 192-wide tiles (choice 1), which exchange through the workspace.  Partial sums in the workspace are there in the second case only.
 @pytest.mark.parametrize("fa,fb", [(FP8, FP8), (FP4, FP4)])
-@pytest.mark.parametrize("choice,shape", [(3, (3584, 1024, 1024)), (3, (6208, 704, 448)), (3, (8256, 192, 64)), (3, (8192, 1024, 512)), (1, (8192, 448, 320)), (1, (8256, 512, 256))])
+@pytest.mark.parametrize("choice,shape", [(3, (3584, 1024, 1024)), (3, (6208, 704, 448)), (3, (8256, 192, 64)), (3, (8192, 1024, 512)), (3, (4096, 768, 768)), (1, (8192, 448, 320)), (1, (8256, 512, 256))])
 def test_cluster_and_workspace_exchange(api, slicing, fa, fb, choice, shape):
     M, K, N = shape
     x, dy, a, b, keep = operands(api, M, K, N, fa, fb, 90 + choice + M + K + N)
     start = torch.randn(N, K, device="cuda")
+    ws = torch.full((api.snip_workspace_size(api.OP_WGRAD, M, N, K, fa, fb)[0],), 0xA5, dtype=torch.uint8, device="cuda")
+    partials = ws[8448:]   # behind status word and arrival counters
     api.snip_debug_set(api.DEBUG_GEMM_KERNEL, choice)
     try:
         outs = {}
         for mode in (0, 1, 1):
             slicing(mode)
-            f32 = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32)
+            f32 = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32, ws=ws)
+            width, _, slices, cluster = api.snip_debug_last_gemm()
+            assert (width == 128) == (choice == 3) and cluster == (slices if choice == 3 else 1)
+            # (6208 tokens in FP4: 25 stages of 256; 32 clusters of four are close to what the chip holds)
+            assert slices in ((1,) if mode == 0 else {(3584, 1024, 1024): (2,), (4096, 768, 768): (3,), (6208, 704, 448): (3 if fa == FP4 else 4,),
+                                                      (8192, 1024, 512): (3, 4)}.get(shape, (4,)))
+            torch.cuda.synchronize()
+            assert bool((partials == 0xA5).all()) == (choice == 3 or not outs)
             acc = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32, accumulate=True, out=start.clone())
             b16 = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_BF16)
             torch.cuda.synchronize()
@@ -183,3 +192,27 @@ def test_slices_of_a_product_that_starts_beside_others(api, shape, slices):
         api.snip_debug_set(api.DEBUG_GEMM_SLICING, 1)
     # the order of FP32 additions over at most 40 chunks (as above)
     assert rel_fro(dw.cpu().numpy(), ref.cpu().numpy().astype(np.float64)) <= 1e-6
+
+
+# 128-wide tiles that exchange through the workspace: more of them than SMs, so that only the last wave's are sliced (160 tiles: 148 and twelve,
+# these in three and four slices; ragged: 148 and twenty; a contraction that ends in a 64-wide tile, in FP4 stages of 256).
+@pytest.mark.parametrize("fa,fb", [(FP8, FP8), (FP4, FP4)])
+@pytest.mark.parametrize("shape,slices", [((3840, 640, 4096), 3), ((4096, 640, 4096), 4), ((4096, 704, 3520), 4), ((8256, 640, 4096), 4)])
+def test_last_wave_of_narrow_tiles(api, slicing, fa, fb, shape, slices):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("wave counts are for 148 SMs")
+    M, K, N = shape
+    x, dy, a, b, keep = operands(api, M, K, N, fa, fb, 600 + M + K + N)
+    ref = orc.linear_wgrad(dy, x, fa, fb)[0]
+    start = torch.randn(N, K, device="cuda")
+    api.snip_debug_set(api.DEBUG_GEMM_KERNEL, api.GEMM_KERNEL_NARROW)
+    try:
+        out = [api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32) for _ in range(3)]
+        plan = api.snip_debug_last_gemm()
+        acc = api.snip_gemm_quantized(api.OP_WGRAD, a, b, (N, K), api.OUT_FP32, accumulate=True, out=start.clone())
+        torch.cuda.synchronize()
+    finally:
+        api.snip_debug_set(api.DEBUG_GEMM_KERNEL, api.GEMM_KERNEL_AUTO)
+    assert plan == (128, 1, slices, 1)
+    assert rel_fro(out[0].cpu().numpy(), ref) <= 1e-5
+    assert torch.equal(out[1], out[0]) and torch.equal(out[2], out[0]) and torch.equal(acc, start + out[0])

@@ -39,7 +39,7 @@ def check_three(api, M, K, N, fa, fb, seed):
 
 
 # (M, K, N): the smallest; ragged rows, columns and contraction around a 128-wide tile; more narrow tiles than SMs;
-# a weight gradient in four slices
+# a weight gradient in four slices (FP4 x FP4, whose stages are twice as long where the contraction ends in a 64-wide tile: whole)
 @pytest.mark.parametrize("fa,fb", [(FP8, FP8), (FP4, FP4), (FP8, FP4), (FP4, FP8)])
 @pytest.mark.parametrize("shape", [(64, 64, 64), (192, 320, 448), (1088, 1472, 1984), (4160, 192, 256)])
 @pytest.mark.parametrize("choice", ["narrow", "auto"])

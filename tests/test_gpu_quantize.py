@@ -155,3 +155,53 @@ def test_power_of_two_scales_on_degenerate_tiles(api):
         assert np.array_equal(codes.cpu().numpy()[:q.packed().size].reshape(q.packed().shape), q.packed())
         assert np.array_equal(scales.cpu().numpy().reshape(q.scales.shape).view(np.uint32), q.scales.view(np.uint32))
         assert np.array_equal(sf.cpu().numpy(), orc.sf_atoms(q, False))
+
+
+def degenerate(name):
+    """Tensors whose error sums a scale's reciprocal weighs at the ends of its range: empty tiles (S = 1), subnormal ones (S = FLT_MAX), and
+    magnitudes whose squares are near the ends of binary32."""
+    rng = np.random.default_rng(19)
+    x = rng.standard_normal((256, 384)).astype(np.float32)
+    if name == "empty":
+        x[:128, :128] = 0.0
+        x[128:, 300] = 0.0
+        x[200] = 0.0
+    elif name == "large":
+        x *= np.float32(1e17)
+    elif name == "small":
+        x *= np.float32(1e-17)
+    bits = wl.to_bf16_bits(x)
+    if name == "subnormal":   # the sums are those of the other tiles: a subnormal one's are below binary32
+        bits[:128, :128] = 0x0001
+        bits[3, 5] = 0x8003
+        bits[200] = 0x0002
+    return bits
+
+
+@pytest.mark.parametrize("fmt", [FP8, FP4])
+@pytest.mark.parametrize("block,transposed", [(ROW, False), (COL, True), (BLK, False)])
+@pytest.mark.parametrize("name", ["empty", "subnormal", "large", "small"])
+def test_statistics_of_degenerate_tiles(api, name, block, transposed, fmt):
+    check_quantize(api, degenerate(name), fmt, block, transposed)
+
+
+@pytest.mark.parametrize("fmt", [FP8, FP4])
+@pytest.mark.parametrize("name", ["empty", "subnormal", "large", "small"])
+def test_layer_statistics_of_degenerate_tiles(api, name, fmt):
+    x = degenerate(name)
+    out = api.snip_layer_stats(X=to_dev(x), M=256, N=256, K=384, fmt_mask=1 << fmt)
+    w = api.snip_layer_stats(W=to_dev(x), M=256, N=256, K=384, fmt_mask=1 << fmt)
+    err, err_w = (t.cpu().numpy()[6:].reshape(3, 2, 3) for t in (out, w))
+    for got, block in ((err[0, fmt - 1, ROW], ROW), (err[0, fmt - 1, COL], COL), (err_w[1, fmt - 1, BLK], BLK)):
+        assert got == pytest.approx(orc.quantize(x, fmt, block).sumsq_err, rel=STATS_RTOL), block
+
+
+@pytest.mark.parametrize("formats", [(FP4, FP4), (FP8, FP4), (FP4, FP8)])
+@pytest.mark.parametrize("name", ["empty", "subnormal", "large", "small"])
+def test_two_outputs_statistics_of_degenerate_tiles(api, name, formats):
+    x = degenerate(name)
+    a, b = api.snip_quantize_dual(to_dev(x), api.DUAL_ROW_COLT, *formats)
+    torch.cuda.synchronize()
+    for got, fmt, block in ((a, formats[0], ROW), (b, formats[1], COL)):
+        ref, st = orc.quantize(x, fmt, block), api.stats_to_host(got["stats"][:24])
+        assert st["sumsq_x"] == pytest.approx(ref.sumsq_x, rel=STATS_RTOL) and st["sumsq_err"] == pytest.approx(ref.sumsq_err, rel=STATS_RTOL)

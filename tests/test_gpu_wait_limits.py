@@ -51,6 +51,8 @@ def test_chained_layer(api, hooks, kind, choice, shape):  # noqa: F811
     ws, step = layer(api, kind, *shape)
     api.snip_debug_set(api.DEBUG_GEMM_KERNEL, choice)
     want, during = check(api, hooks, ws, lambda: step(t, ws))
+    if shape[0] == 8192:
+        assert api.snip_debug_last_gemm()[2:] == ((4, 4) if choice == 0 else (4, 1))
     # the quantizers and their statistics are not held up
     assert torch.equal(during[3], want[3])
 
