@@ -1158,7 +1158,10 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // the pipeline stages that its SMs run one after the other (kMinSavedStages more where its last wave is sliced) times what a stage of a narrow
     // tile takes next to a wide one's: measured 0.64-0.68 forward and input gradient, 0.69-0.79 weight gradient.  FP4 against pairs 192 wide
     // 0.70-0.72 (8192 x 1536 outputs over 4096 features, us narrow / wide: 2 waves to 2 18.3 / 24.9, 5 to 4 41 / 46, 4 to 3 33.4 / 35.6, 11 to 8 87 / 89,
-    // 7 to 5 55.9 / 56.8, 3 to 2 25.8 / 25.0).
+    // 7 to 5 55.9 / 56.8, 3 to 2 25.8 / 25.0).  In a layer the next product takes over the SMs that a last wave leaves idle, so that whole waves
+    // count for less there and the line lies at 0.76 (one layer, us with it at 0.72 / 0.76: 8192 x 8640 -> 3200, 11 to 8, 714 / 706, 2816 x 2496 ->
+    // 3200, 4 to 3, 109.4 / 104.1, 4864 x 1920 -> 1792, 4 to 3, 92.5 / 94.1), and in the weight gradient, whose narrow stages take more (3264
+    // tokens, 2112 -> 3904 131.6 / 124.0 us).
     auto use_narrow = [&](int tile_n, int stage_k, float ratio) {
         if (choice != 0) return choice == 3;
         auto stages = [&](int bn) {
@@ -1185,7 +1188,7 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
         // warps' registers at once, and with half the operand bytes and a quarter of the tensor time it stays below the power
         // cap: 16384x12288x4096 755 -> 673 us, 8192x3200x8640 215 -> 193 us, 8192x2048x256 16.4 -> 14.5 us.  The weight gradient over
         // whole chunks takes the path below: with two operations per element the wider tile is as fast or faster.
-        const bool narrow = use_narrow(192, 256, 0.72f);
+        const bool narrow = use_narrow(192, 256, scale_mode == SCALE_BLOCK_B && !link.ctas ? 0.72f : 0.76f);
         const int BN = narrow ? 128 : 192;
         const bool pair = !narrow && use_pair(BN);
         const int ctas = pair ? 2 : 1;

@@ -88,3 +88,15 @@ def test_width_of_fp4_tiles_by_waves(api, row_tiles, width):
     api.snip_linear_fwd(X, W, FP4, FP4)
     torch.cuda.synchronize()
     assert api.snip_debug_last_gemm()[0] == width
+
+
+# ... and the FP4 weight gradient over a token count that ends in a 64-wide tile: 27 x 17 narrow or 27 x 12 wide tiles are four waves or three,
+# 192 columns; 20 x 11 or 20 x 8 are two either way, 128 columns.
+@pytest.mark.parametrize("rows,cols,width", [(27 * 128, 17 * 128, 192), (20 * 128, 11 * 128, 128)])
+def test_width_of_fp4_weight_gradient_tiles_by_waves(api, rows, cols, width):
+    if torch.cuda.get_device_properties(0).multi_processor_count != 148:
+        pytest.skip("wave counts are for 148 SMs")
+    DY, X = torch.randn(192, rows, device="cuda").bfloat16(), torch.randn(192, cols, device="cuda").bfloat16()
+    api.snip_linear_wgrad(DY, X, FP4, FP4)
+    torch.cuda.synchronize()
+    assert api.snip_debug_last_gemm()[0] == width
