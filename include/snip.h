@@ -267,10 +267,13 @@ int snip_quantize_mx(const void *x, int64_t rows, int64_t cols, int64_t ld, int 
 /*
  * Workspace bytes for one GEMM call of the given op and shape, and for the snip_linear_* call
  * of the same op (which also holds the quantized operands).  Host-only.  For SNIP_OP_WGRAD over
- * quantized operands gemm_bytes includes room (about 21 MB) that lets the kernel cut the tiles of
- * its last, partly filled wave over the SMs into slices of the contraction (their FP32 sums are
- * added in slice order, so results do not depend on timing); any GEMM also runs, unsliced, with
- * the 256-byte minimum.
+ * quantized operands gemm_bytes includes room (about 21 MB) that lets the kernel cut tiles into
+ * slices of the contraction where it would leave SMs idle: the tiles of its last, partly filled
+ * wave, or, of outputs with few tiles, all of them.  The slices' FP32 sums are added in slice order,
+ * so that results do not depend on timing; how many slices there are follows from the shape, the
+ * formats, the number of SMs and how the device groups them, and from whether the product is a call of its own or
+ * part of snip_linear_fwd_bwd.  Reruns on one device are bit-identical; devices that differ in this may
+ * add in a different order.  Any GEMM also runs, unsliced, with the 256-byte minimum.
  */
 int snip_workspace_size(int op, int64_t M, int64_t N, int64_t K, int fmt_a, int fmt_b,
                         size_t *gemm_bytes_host, size_t *linear_bytes_host);

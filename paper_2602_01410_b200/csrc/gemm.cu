@@ -14,7 +14,8 @@
 //                 (so the scaling overlaps the next chunk's MMAs, which write the other
 //                 tensor-memory buffer), then round and store the tile.
 // Three forms, chosen by shape in gemm_impl: 128-row tiles of 256 (192) or of 128 columns on one CTA, 256-row tiles on a
-// pair of CTAs (tcgen05.mma.cta_group::2; the leader's MMA warp and barriers serve both).
+// pair of CTAs (tcgen05.mma.cta_group::2; the leader's MMA warp and barriers serve both).  128-wide tiles of the weight gradient have a
+// fourth, in which the slices of a tile are the CTAs of a cluster.
 // All hand-offs use mbarriers with bounded waits; on a timeout the CTA raises a status word and
 // leaves cleanly (tensor memory is always released).
 #include <cuda.h>
@@ -671,7 +672,7 @@ gemm_kernel(const __grid_constant__ CUtensorMap tmA, const __grid_constant__ CUt
                 // A slice of a tile whose other slices are in this cluster (the CTA's only item).  The sums of fragment group gi belong to
                 // slice gi * nsl / G: every CTA writes the groups of the others into their stage memory, which no copy or MMA uses any
                 // more once all CTAs are here, and then adds its own groups in slice order and stores them.  Nothing is sent through L2
-                // and no CTA adds the whole tile: 8192 tokens x 256 x 2048 21.8 -> 17.6 us, 16384 x 512 x 1024 28.9 -> 24.1 us.  A CTA that gave
+                // and no CTA adds the whole tile: 8192 tokens x 256 x 2048 20.6 -> 16.5 us, 16384 x 512 x 1024 28.7 -> 22.9 us.  A CTA that gave
                 // up a wait takes part in both barriers all the same; before the second one it raises the abort flag of every CTA here, because
                 // none of them has the tile's sums then.
                 const int me = wi.slice, nsl = wi.nsl, per = (G + nsl - 1) / nsl;
@@ -1156,7 +1157,8 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // so that twice the tiles still are one wave (forward FP8 1024x2048x4096 18.0 -> 12.5 us, 8192x256x2048 11.2 -> 8.3 us, 512x512x512 6.6 -> 5.2
     // us; FP4 1024x4096x4096, two waves either way, 24.8 -> 18.6 us; weight gradient 8192x256x2048 28.6 -> 20.6 us).  A launch lasts as long as
     // the pipeline stages that its SMs run one after the other (kMinSavedStages more where its last wave is sliced) times what a stage of a narrow
-    // tile takes next to a wide one's: measured 0.64-0.68 forward and input gradient, 0.69-0.79 weight gradient.  FP4 against pairs 192 wide
+    // tile takes next to a wide one's: measured 0.64-0.68 forward and input gradient (one-CTA forms; against pairs FP8 is at 0.57-0.63 by now, three waves to two of
+    // 4096 features 29.8 us narrow, 32.3 us wide, and still goes by 0.68), 0.69-0.79 weight gradient.  FP4 against pairs 192 wide
     // 0.70-0.72 (8192 x 1536 outputs over 4096 features, us narrow / wide: 2 waves to 2 18.3 / 24.9, 5 to 4 41 / 46, 4 to 3 33.4 / 35.6, 11 to 8 87 / 89,
     // 7 to 5 55.9 / 56.8, 3 to 2 25.8 / 25.0).  In a layer the next product takes over the SMs that a last wave leaves idle, so that whole waves
     // count for less there and the line lies at 0.76 (one layer, us with it at 0.72 / 0.76: 8192 x 8640 -> 3200, 11 to 8, 714 / 706, 2816 x 2496 ->

@@ -5,13 +5,15 @@
 // registers.  The scheme-generation step needs the error of every option (Sec. 4.4), not only of
 // the format currently in use.
 //
-// One persistent launch for all six tensors, three CTAs of 256 threads per SM.  X, W and dY are bound by instruction issue and the FP32
-// pipe (three operations and a conversion per element and option), Y, dX and dW, of which only the norm is wanted, by HBM; so every SM
+// One persistent launch for all six tensors, three CTAs of 256 threads per SM.  X, W and dY are bound by instruction issue (66 % of the
+// slots, with two CTA barriers a tile; no pipe is full), Y, dX and dW, of which only the norm is wanted, by HBM; so every SM
 // works on both kinds at once, some CTAs on tiles of the first, some streaming the second.  Tiles are 128x128, each thread an 8x8
-// sub-block that it fetches itself (cp.async into a private slot, one tile ahead).  The arithmetic per option is the quantizer's: S =
-// FPX_MAX/amax (binary32 quotient, one division per tile and format, shared through shared memory), code = RNE_fmt(fl32(x*S)), error
-// term x - value(code)/S.  A reduction of the CTAs' sums follows.
-// Six tensors of an 8192 x 3200 x 9600 linear: 250 -> 147 us, X with four options 16384 x 4096: 98 -> 72 us (before: thirteen launches of one
+// sub-block that it fetches itself (cp.async into a private slot, one tile ahead).  Scales and codes are the quantizer's: S =
+// FPX_MAX/amax (binary32 quotient, one division per tile and format, shared through shared memory), code = RNE_fmt(fl32(x*S)); the error
+// term is x - value(code)/S for FP8 (per element pair a product, two packed FMAs, a conversion to the format and three back) and
+// value(code) - fl32(x*S) for FP4 (two additions for one of the FMAs and two of the conversions, weighed by S^-2 per tile line).  A
+// reduction of the CTAs' sums follows.
+// Six tensors of an 8192 x 3200 x 9600 linear: 250 -> 135 us, X with four options 16384 x 4096: 92 -> 68 us (before: thirteen launches of one
 // tile per CTA, every thread dividing for all of its rows and columns).
 #include <stddef.h>
 

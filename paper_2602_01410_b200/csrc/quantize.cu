@@ -143,14 +143,13 @@ struct ThreadStats {
 };
 
 // -1/S for the error term x - value(code)/S = x + value(code) * (-1/S).  Paper's rule: FP8: amax/FPX_MAX, which equals
-// 1/S to within one rounding; FP4, whose reciprocal weighs whole sums (kScaled below): the correctly rounded one of S.
-// Power-of-two rule: exact, from the exponent field.  For an empty tile the value is irrelevant (all codes are zero).
+// 1/S to within one rounding; FP4, whose reciprocal weighs whole sums (kScaledErr below): the correctly rounded one of S.
+// Power-of-two rule: exact, from the exponent field.  It has to be finite also for an empty tile, whose sums are zero (S is 1 there).
 template <int FMT>
 __device__ __forceinline__ float neg_inv(float amax, float s, int pow2)
 {
     if (FMT == SNIP_FMT_FP4_E2M1 && !pow2) return -__frcp_rn(s);
-    constexpr float kInvMax = (FMT == SNIP_FMT_FP8_E4M3) ? (1.0f / 448.0f) : (1.0f / 6.0f);
-    return pow2 ? __uint_as_float(0x80000000u | ((254u << 23) - __float_as_uint(s))) : -amax * kInvMax;
+    return pow2 ? __uint_as_float(0x80000000u | ((254u << 23) - __float_as_uint(s))) : -amax * (1.0f / 448.0f);
 }
 
 // Two binary32 products -> packed codes of an element pair (FP8: 16 bits, FP4: 8 bits) and, with STATS,

@@ -58,7 +58,7 @@ __device__ __forceinline__ bool elect_one()
     return pred != 0;
 }
 
-// ---- thread-block clusters (pairs of CTAs sharing one MMA) -------------------------------
+// ---- thread-block clusters (pairs of CTAs sharing one MMA; the two to four slices of a weight-gradient tile) ----
 __device__ __forceinline__ uint32_t cluster_ctarank()
 {
     uint32_t r;
@@ -72,7 +72,7 @@ __device__ __forceinline__ uint32_t mapa(uint32_t addr, uint32_t rank)
     asm volatile("mapa.shared::cluster.u32 %0, %1, %2;" : "=r"(r) : "r"(addr), "r"(rank));
     return r;
 }
-// All threads of both CTAs arrive and wait (hardware barrier; every path that reaches it is bounded).
+// All threads of the cluster's CTAs arrive and wait (hardware barrier; every path that reaches it is bounded).
 __device__ __forceinline__ void cluster_sync()
 {
     asm volatile("barrier.cluster.arrive.release.aligned;\n\tbarrier.cluster.wait.acquire.aligned;" ::: "memory");
@@ -85,7 +85,7 @@ __device__ __forceinline__ void mbar_arrive_cluster_relaxed(uint32_t cluster_add
     asm volatile("mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];" ::"r"(cluster_addr) : "memory");
 }
 // Arrivals by one lane of a converged warp, predicated by elect.sync: a `lane == 0` branch around the instruction, at the end of every
-// chunk of a GEMM, costs 2-6 % of its cycles.
+// chunk of a GEMM, costs 2-6 % of its cycles (but is the cheaper form between two groups of a chunk: see release_buffer in gemm.cu).
 __device__ __forceinline__ void mbar_arrive_cluster_relaxed_elected(uint32_t cluster_addr)
 {
     asm volatile("{\n\t.reg .pred p;\n\telect.sync _|p, 0xFFFFFFFF;\n\t@p mbarrier.arrive.relaxed.cluster.shared::cluster.b64 _, [%0];\n\t}" ::"r"(cluster_addr) : "memory");

@@ -2,7 +2,8 @@
 //
 // Item w < split_first is tile w over the whole contraction; the tiles from split_first on are cut into nsplit slices each, item
 // split_first + r * nsplit + j being slice j of tile split_first + r.  nsplit == 1: no slicing, num_items == number of tiles.  A
-// slice's FP32 sums go to the workspace; whoever delivers a sub-tile's last slice adds all of them in slice order.
+// slice's FP32 sums go to the workspace, and whoever delivers a sub-tile's last slice adds all of them in slice order; or the slices of a
+// tile are the CTAs of a cluster (then split_first is 0) and each adds its share of the tile, in slice order too (gemm.cu).
 #pragma once
 #include "common.cuh"
 
