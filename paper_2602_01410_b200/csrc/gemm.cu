@@ -975,8 +975,8 @@ thread_local int last_gemm[4];   // see snip_debug_last_gemm
 // 32.0 / 31.6, 256 44.7 / 41.6.
 bool prefer_clusters(const WorkSplit &clusters, const WorkSplit &workspace, int num_chunks)
 {
-    return clusters.nsplit > 1 && (float)num_chunks / clusters.nsplit + kMinSavedStagesCluster <=
-                                      (float)num_chunks / workspace.nsplit + (workspace.nsplit > 1 ? kWorkspaceExchangeChunks : 0);
+    if (clusters.nsplit == 1 || workspace.nsplit == 1) return clusters.nsplit > 1;   // (whole tiles: plan_clusters has weighed them)
+    return (float)num_chunks / clusters.nsplit + kMinSavedStagesCluster <= (float)num_chunks / workspace.nsplit + kWorkspaceExchangeChunks;
 }
 
 template <MmaKind KIND, int BN, int SCALE, bool PAIR, bool OUT_F32>

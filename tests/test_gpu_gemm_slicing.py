@@ -158,7 +158,7 @@ def test_clusters_of_three_leave_room(api, fmt):
 
 # Clusters, or more slices and the exchange through the workspace, by the length of the contraction: (chunks, tiles) -> (slices, CTAs of a
 # cluster), sums against the unsliced product as above.  (For 148 SMs in GPCs that hold more than 32 clusters of four.)
-@pytest.mark.parametrize("chunks,tiles,want", [(64, 45, (2, 2)), (118, 45, (3, 1)), (118, 42, (3, 1)), (118, 36, (3, 3)), (256, 36, (4, 1)), (256, 30, (4, 4))])
+@pytest.mark.parametrize("chunks,tiles,want", [(23, 10, (2, 2)), (22, 10, (1, 1)), (64, 45, (2, 2)), (118, 45, (3, 1)), (118, 42, (3, 1)), (118, 36, (3, 3)), (256, 36, (4, 1)), (256, 30, (4, 4))])
 def test_exchange_by_the_length_of_the_contraction(api, slicing, chunks, tiles, want):
     M, K, N = 128 * chunks, 128, 128 * tiles
     x, dy, a, b, keep = operands(api, M, K, N, FP8, FP8, chunks + tiles)
