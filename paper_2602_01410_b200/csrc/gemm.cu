@@ -1158,8 +1158,8 @@ int gemm_impl(int fmt_a, int fmt_b, const void *a_codes, const void *b_codes, in
     // us; FP4 1024x4096x4096, two waves either way, 24.8 -> 18.6 us; weight gradient 8192x256x2048 28.6 -> 20.6 us).  A launch lasts as long as
     // the pipeline stages that its SMs run one after the other (kMinSavedStages more where its last wave is sliced) times what a stage of a narrow
     // tile takes next to a wide one's: measured 0.64-0.68 forward and input gradient (one-CTA forms; against pairs FP8 is at 0.57-0.63 by now, three waves to two of
-    // 4096 features 29.8 us narrow, 32.3 us wide, and still goes by 0.68), 0.69-0.79 weight gradient.  FP4 against pairs 192 wide
-    // 0.70-0.72 (8192 x 1536 outputs over 4096 features, us narrow / wide: 2 waves to 2 18.3 / 24.9, 5 to 4 41 / 46, 4 to 3 33.4 / 35.6, 11 to 8 87 / 89,
+    // 4096 features 29.8 us narrow, 32.4 us wide, and still goes by 0.68), 0.69-0.79 weight gradient.  FP4 against pairs 192 wide
+    // 0.70-0.72 (1536 columns of 22-132 row tiles over 4096 features, us narrow / wide: 2 waves to 2 18.3 / 24.9, 5 to 4 41 / 46, 4 to 3 33.4 / 35.6, 11 to 8 87 / 89,
     // 7 to 5 55.9 / 56.8, 3 to 2 25.8 / 25.0).  In a layer the next product takes over the SMs that a last wave leaves idle, so that whole waves
     // count for less there and the line lies at 0.76 (one layer, us with it at 0.72 / 0.76: 8192 x 8640 -> 3200, 11 to 8, 714 / 706, 2816 x 2496 ->
     // 3200, 4 to 3, 109.4 / 104.1, 4864 x 1920 -> 1792, 4 to 3, 92.5 / 94.1), and in the weight gradient, whose narrow stages take more (3264
